@@ -125,15 +125,14 @@ struct hd_scan {
     int32_t *rec_buf = nullptr;   // 8 int32 arrays of rec_cap (coordinates, status, global list)
     int64_t rec_cap = 0;
     uint32_t *pair_buf = nullptr;  // lean walks (kLeanWords per pair), then the fallback list
-    hd::TileJob *jobs = nullptr;
-    int64_t job_cap = 0;
     hd::ScanDesc *desc_dev = nullptr;  // this scan's traversal descriptor
     hd::ScanDesc desc_host{};
     bool desc_dirty = true;
-    // 2 * ntiles tile totals, then the ingest blocks' pair counts per tile
+    // kGroups * ntiles tile totals, then the ingest blocks' pair counts per tile
     // (tile_count_words)
     uint32_t *tile_count = nullptr;
-    uint32_t *tile_cursor = nullptr;  // 2 * ntiles
+    uint32_t *tile_cursor = nullptr;  // kGroups * ntiles
+    unsigned long long *tile_events = nullptr;  // kGroups * ntiles
     int64_t *rows_scratch = nullptr;  // tile sums of the system-row offset scan
     int64_t rows_scratch_cap = 0;
     uint32_t *rows_bits = nullptr;    // the hull packed for the row passes
@@ -213,7 +212,7 @@ void free_scan(hd_scan *s)
 
     void *ptrs[] = {s->N, s->M, s->H1, s->H2, s->H3, s->bits_out, s->slice_key,
                     s->mt, s->slope, s->index, s->ctrl, s->rec_buf, s->staging,
-                    s->compact_blocks, s->d_count, s->compact_out, s->pair_buf, s->jobs,
+                    s->compact_blocks, s->d_count, s->compact_out, s->pair_buf, s->tile_events,
                     s->rows_scratch, s->rows_bits, s->thick_ws,
                     s->tile_count, s->tile_cursor, s->desc_dev};
     for (void *p : ptrs)
@@ -251,22 +250,16 @@ hd_status ensure_records(hd_scan *s, int64_t n, cudaStream_t st)
     HD_CUDA(cudaStreamSynchronize(st));
     if (s->rec_buf) cudaFree(s->rec_buf);
     if (s->pair_buf) cudaFree(s->pair_buf);
-    if (s->jobs) cudaFree(s->jobs);
     s->rec_buf = nullptr;
     s->pair_buf = nullptr;
-    s->jobs = nullptr;
     s->rec_cap = 0;
     bool ok = cudaMalloc(&s->rec_buf, sizeof(int32_t) * 8 *
                                           static_cast<size_t>(hd::records_stride(n))) == cudaSuccess;
     if (ok && s->tp.ntiles > 0) {
         const int64_t pair_cap = pairs_per_record(s->tp) * n;
-        const int64_t min_job = s->tp.job_size < hd::kMinJob ? s->tp.job_size : hd::kMinJob;
-        const int64_t job_cap = pair_cap / min_job + 2 * s->tp.ntiles + 1;
         ok = cudaMalloc(&s->pair_buf, sizeof(uint32_t) * (hd::kLeanWords + 3) *
-                                          static_cast<size_t>(pair_cap)) == cudaSuccess &&
-             cudaMalloc(&s->jobs, sizeof(hd::TileJob) * static_cast<size_t>(job_cap)) == cudaSuccess;
+                                          static_cast<size_t>(pair_cap)) == cudaSuccess;
         s->tp.pair_cap = pair_cap;
-        s->job_cap = job_cap;
     }
     if (!ok) {
         cudaGetLastError();
@@ -340,11 +333,11 @@ size_t ingest_blocks_max(const hd_scan *s)
            static_cast<size_t>(hd::kIngestBlocksPerSm);
 }
 
-// Words of tile_count: the 2 * ntiles totals, a column of pair counts per
-// tile and class for the most ingest blocks, then each block's pairs in all.
+// Words of tile_count: the kGroups * ntiles totals, a column of pair counts per
+// group and tile for the most ingest blocks, then each block's pairs in all.
 size_t tile_count_words(const hd_scan *s)
 {
-    const size_t cols = 2 * static_cast<size_t>(s->tp.ntiles);
+    const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
     return cols * (1 + ingest_blocks_max(s)) + ingest_blocks_max(s);
 }
 
@@ -359,6 +352,15 @@ hd::Pairs pairs_of(const hd_scan *s)
     p.fb = base ? reinterpret_cast<uint2 *>(base + hd::kLeanWords * cap) : nullptr;
     p.stage = base ? base + (hd::kLeanWords + 2) * cap : nullptr;
     return p;
+}
+
+hd::Buckets buckets_of(const hd_scan *s)
+{
+    hd::Buckets b;
+    b.count = s->tile_count;
+    b.first = s->tile_cursor;
+    b.events = s->tile_events;
+    return b;
 }
 
 // Tiles: one or more z-slices of the full x-y plane when they fit in the
@@ -403,9 +405,10 @@ void make_tile_plan(hd_scan *s)
     tp.job_size = s->tuning.job_size;  // <= 32767: int16 differences in the tiled traversal
     tp.refill = s->tuning.refill;
     tp.threads = s->tuning.threads;
-    // one 32-bit word per voxel (x-run and y-run difference counts in its
-    // two halves), plus a padding column and row for the ends of runs
-    tp.tile_words = (tp.tx + 1) * (tp.ty + 1) * tp.tz;
+    tp.thick = s->thick_k;
+    // one 32-bit word per voxel (tile_row_words in hd_geom.cuh)
+    // in whole 16-byte vectors
+    tp.tile_words = ((tp.tx + 1) * (tp.ty + 1) * tp.tz + 3) & ~3;
     auto magic = [](int t) {
         return t == 1 ? 0u : static_cast<unsigned>((1ull << 32) / static_cast<unsigned>(t)) + 1u;
     };
@@ -420,7 +423,7 @@ hd::ScanDesc make_desc(const hd_scan *s)
     hd::ScanDesc d{};
     d.tp = s->tp;
     d.pairs = pairs_of(s);
-    d.jobs = s->jobs;
+    d.buckets = buckets_of(s);
     d.ctrl = s->ctrl;
     d.N = s->N;
     d.M = s->M;
@@ -448,8 +451,8 @@ hd_status stage_prepare(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_
     const hd::Records rec = records_of(s, n);
     hd::TilePlan tp = s->tp;
     if (s->trace_grid <= 0) tp.ntiles = 0;
-    HD_CUDA(cudaMemsetAsync(&s->ctrl->njobs, 0, sizeof(hd::Ctrl) - offsetof(hd::Ctrl, njobs), st));
-    const size_t cols = 2 * static_cast<size_t>(s->tp.ntiles);
+    HD_CUDA(cudaMemsetAsync(&s->ctrl->n_global, 0, sizeof(hd::Ctrl) - offsetof(hd::Ctrl, n_global), st));
+    const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
     uint32_t *block_count = s->tile_count + cols;
     uint32_t *block_pairs = block_count + cols * ingest_blocks_max(s);
     const hd::Pairs pairs = pairs_of(s);
@@ -459,9 +462,8 @@ hd_status stage_prepare(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_
                               s->inputs_on_host ? 1 : 0, s->sm_count, st));
     s->launches += 1;
     if (tp.ntiles > 0) {
-        HD_CUDA(hd::launch_plan(tp, n, block_count, s->tile_count, s->tile_cursor, s->jobs, s->ctrl,
-                                s->sm_count, st));
-        HD_CUDA(hd::launch_scatter(tp, rec, n, s->ctrl, s->tile_cursor, block_count, block_pairs,
+        HD_CUDA(hd::launch_plan(tp, n, block_count, buckets_of(s), s->sm_count, st));
+        HD_CUDA(hd::launch_scatter(tp, rec, n, s->ctrl, buckets_of(s), block_count, block_pairs,
                                    pairs, s->sm_count, st));
         s->launches += 3;
     }
@@ -527,7 +529,7 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
     }
     if (s->thick_k > 0) {
         const hd::TilePlan &tp = s->tp;
-        if (tp.ntiles > 0 && tp.ntx == 1 && tp.nty == 1 && tp.tz == 1) {
+        if (tp.ntiles > 0 && s->trace_grid > 0 && tp.ntx == 1 && tp.nty == 1 && tp.tz == 1) {
             // thick rays on the tiled path: the same records and pairs,
             // dilated in the traversal
             hd_status r = upload_desc(s, st);
@@ -536,7 +538,8 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
             if (r != HD_OK) return r;
             HD_CUDA(hd::launch_thick_scan(s->desc_dev, &s->geom, records_of(s, n), s->ctrl, n,
                                           s->gq, s->thick_k, s->thick_ws, s->N, s->M,
-                                          tp.tile_words, tp.threads, s->sm_count, st));
+                                          tp.tile_words, tp.threads, s->trace_grid, s->sm_count,
+                                          st));
             s->launches += 4;
             return HD_OK;
         }
@@ -557,8 +560,8 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
     prof_end(s, 0, e0, st);
     cudaEvent_t e1 = prof_begin(s, st);
     if (s->tp.ntiles > 0 && s->trace_grid > 0) {
-        HD_CUDA(hd::launch_trace_tiles(s->desc_dev, 1, &s->ctrl->job_next, s->tp.tile_words,
-                                       s->tp.threads, s->trace_grid, st));
+        HD_CUDA(hd::launch_trace_tiles(s->desc_dev, 1, s->tp.tile_words, s->tp.threads,
+                                       s->trace_grid, st));
         s->launches += 1;
         if (s->profiling) s->trace_launches += 1;
     }
@@ -657,9 +660,12 @@ hd_status hd_scan_create(const hd_geometry *geom, const hd_params *params, hd_sc
     if (m & HD_MSC) alloc(reinterpret_cast<void **>(&s->H2), V);
     alloc(reinterpret_cast<void **>(&s->bits_out), sizeof(uint32_t) * s->words);
     make_tile_plan(s);
+    if (hd::init_ingest() != cudaSuccess || hd::init_scatter() != cudaSuccess) ok = false;
     if (s->tp.ntiles > 0) {
         alloc(reinterpret_cast<void **>(&s->tile_count), sizeof(uint32_t) * tile_count_words(s));
-        alloc(reinterpret_cast<void **>(&s->tile_cursor), sizeof(uint32_t) * 2 * s->tp.ntiles);
+        alloc(reinterpret_cast<void **>(&s->tile_cursor), sizeof(uint32_t) * hd::kGroups * s->tp.ntiles);
+        alloc(reinterpret_cast<void **>(&s->tile_events),
+              sizeof(unsigned long long) * hd::kGroups * s->tp.ntiles);
         const int per_sm = hd::trace_tiles_occupancy(s->tp.tile_words, s->tp.threads);
         s->trace_grid = per_sm > 0 ? per_sm * s->sm_count : 0;
     }
@@ -1038,6 +1044,8 @@ hd_status hd_scan_set_thick(hd_scan *scan, int32_t k)
         }
     }
     scan->thick_k = k;
+    scan->tp.thick = k;
+    scan->desc_dirty = true;
     if (k > 0) scan->euclid_d0 = 0.0f;
     return HD_OK;
 }
@@ -1058,7 +1066,11 @@ hd_status hd_scan_set_thick_distance(hd_scan *scan, float d0_mm)
         }
     }
     scan->euclid_d0 = d0_mm;
-    if (d0_mm > 0.0f) scan->thick_k = 0;
+    if (d0_mm > 0.0f) {
+        scan->thick_k = 0;
+        scan->tp.thick = 0;
+        scan->desc_dirty = true;
+    }
     return HD_OK;
 }
 
@@ -1075,20 +1087,24 @@ hd_status hd_scan_set_tuning(hd_scan *scan, const hd_tuning *t)
     if (!g.ok) return HD_ERR_CUDA;
     HD_CUDA(cudaDeviceSynchronize());
     // drop everything sized by the old plan; it regrows on the next add
-    void *old[] = {scan->tile_count, scan->tile_cursor, scan->rec_buf, scan->pair_buf, scan->jobs};
+    void *old[] = {scan->tile_count, scan->tile_cursor, scan->tile_events, scan->rec_buf,
+                   scan->pair_buf};
     for (void *p : old)
         if (p) cudaFree(p);
     scan->tile_count = scan->tile_cursor = nullptr;
+    scan->tile_events = nullptr;
     scan->rec_buf = nullptr;
     scan->pair_buf = nullptr;
-    scan->jobs = nullptr;
     scan->rec_cap = 0;
     scan->tuning = *t;
     make_tile_plan(scan);
     scan->trace_grid = 0;
     if (scan->tp.ntiles > 0) {
         if (cudaMalloc(&scan->tile_count, sizeof(uint32_t) * tile_count_words(scan)) != cudaSuccess ||
-            cudaMalloc(&scan->tile_cursor, sizeof(uint32_t) * 2 * scan->tp.ntiles) != cudaSuccess) {
+            cudaMalloc(&scan->tile_cursor, sizeof(uint32_t) * hd::kGroups * scan->tp.ntiles) !=
+                cudaSuccess ||
+            cudaMalloc(&scan->tile_events,
+                       sizeof(unsigned long long) * hd::kGroups * scan->tp.ntiles) != cudaSuccess) {
             cudaGetLastError();
             return HD_ERR_NOMEM;
         }
@@ -1195,7 +1211,6 @@ struct hd_batch {
     hd::ScanDesc *descs_dev = nullptr;  // kMaxBatch descriptors
     hd::ScanDesc *descs_pinned = nullptr;  // host staging of the table (pinned)
     cudaEvent_t descs_copied = nullptr;     // the last upload from descs_pinned is done
-    int *job_counter = nullptr;
     static constexpr int kSide = 8;
     cudaStream_t side[kSide] = {};
     cudaEvent_t fork = nullptr;
@@ -1221,7 +1236,6 @@ void free_batch(hd_batch *b)
     if (b->descs_dev) cudaFree(b->descs_dev);
     if (b->descs_pinned) cudaFreeHost(b->descs_pinned);
     if (b->descs_copied) cudaEventDestroy(b->descs_copied);
-    if (b->job_counter) cudaFree(b->job_counter);
     delete b;
 }
 
@@ -1268,9 +1282,7 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
     r = join();
     if (r != HD_OK) return r;
     if (any_tiled) {
-        HD_CUDA(cudaMemsetAsync(b->job_counter, 0, sizeof(int), st));
-        HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, b->job_counter, max_words,
-                                       b->threads, grid, st));
+        HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, st));
         *kernels += 1;
     }
     r = fork();
@@ -1314,7 +1326,6 @@ hd_status hd_batch_create(int32_t max_items, hd_batch **out)
     if (e == cudaSuccess)
         e = cudaMallocHost(&b->descs_pinned, sizeof(hd::ScanDesc) * hd::kMaxBatch);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->descs_copied, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc(&b->job_counter, sizeof(int));
     if (e != cudaSuccess) {
         note_cuda(e, "hd_batch_create");
         free_batch(b);

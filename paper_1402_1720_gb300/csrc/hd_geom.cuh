@@ -335,17 +335,39 @@ HD_HD int tile_range(const TilePlan &tp, const int32_t r[6], int lo[3], int hi[3
     return tile_range_z(tp, r, zlo, zhi, lo, hi);
 }
 
+// Orients a segment so that its major in-plane axis (the one with the larger
+// |D|, x when equal) moves + (A_i is a set of points, so swapping the ends
+// does not change it) and returns the type of its walks: bit 1 the major axis
+// is y, bit 0 the other in-plane axis moves -.
+HD_HD int orient_record(int32_t r[6])
+{
+    const int dx = r[3] - r[0], dy = r[4] - r[1];  // |G| < 2^30: no overflow
+    const int ax = dx < 0 ? -dx : dx, ay = dy < 0 ? -dy : dy;
+    const bool ymaj = ay > ax;
+    const bool flip = (ymaj ? dy : dx) < 0;
+    const int dm = ymaj ? dx : dy;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int32_t t = r[a];
+        r[a] = flip ? r[a + 3] : t;
+        r[a + 3] = flip ? t : r[a + 3];
+    }
+    return (ymaj ? 2 : 0) | ((flip ? dm > 0 : dm < 0) ? 1 : 0);
+}
+
 // A record's status word: bits 0-1 the path (0 no record, 1 tiled, 2
-// global), bit 2 the class (0 missed, 1 hit), bits 8-19 and 20-31 its first
-// and last slice (grid_z_range, computed once).
-HD_HD int32_t record_status(int path, int cls, int zlo, int zhi)
+// global), bits 2-4 its group (class + 2 type: the class, 0 missed or 1
+// hit, in bit 2, the walk type of orient_record in bits 3-4), bits 8-19 and 20-31 its first and last slice (grid_z_range, computed once).
+HD_HD int32_t record_status(int path, int cls, int type, int zlo, int zhi)
 {
     return static_cast<int32_t>(static_cast<uint32_t>(path) | (static_cast<uint32_t>(cls) << 2) |
+                                (static_cast<uint32_t>(type) << 3) |
                                 (static_cast<uint32_t>(zlo) << 8) |
                                 (static_cast<uint32_t>(zhi) << 20));
 }
 HD_HD int status_path(int32_t s) { return s & 3; }
 HD_HD int status_cls(int32_t s) { return (s >> 2) & 1; }
+HD_HD int status_group(int32_t s) { return (s >> 2) & 7; }  // class + 2 type
 HD_HD int status_zlo(int32_t s) { return (static_cast<uint32_t>(s) >> 8) & 0xfff; }
 HD_HD int status_zhi(int32_t s) { return static_cast<uint32_t>(s) >> 20; }
 
@@ -1294,6 +1316,132 @@ HD_HD bool tile_cursor_run(TileCursor &c, int &at_prev, int &at_cur)
     --c.kleft;
     c.rowb += c.rstep;
     return !last;
+}
+
+// ------------------------------------------------------------- event walk
+//
+// The tiled traversal's form of a lean walk whose major axis moves + (every
+// record is stored oriented that way).  Consecutive runs of such a walk share
+// a major index: run k ends at major index b in its row and run k + 1 begins at
+// b one row on (always in the same direction).  So instead of adding +1 where
+// each run begins and -1 past its end, the walk adds 1 to an event count E at
+// (row, b) for each change of row, and marks only its own first and last voxel
+// in P: one update per run where the two ends took two.  With the walks of a
+// tile sorted by type (major axis, row direction s), E and P decode together:
+//   count(m, row) = SP(m, row) + SE(m, row - s) - SE(m - 1, row)
+// SE and SP the prefix sums of E and P along the major axis (P is +1 at the
+// walk's first voxel, -1 just past its last).  A row of a walk holds at most
+// one event, so SE and SP stay within the pairs of a job (32767).
+//
+// Rays dilated by t voxels in-plane decode from the same events: the
+// dilated set's interval in a row runs from where the run t rows earlier began,
+// less t, to where the run t rows later ends, plus t, so
+//   count(m, row) = sum_{|j| <= t} SP(m, row + j)
+//                   + SE(m + t, row - (t + 1) s) - SE(m - t - 1, row + t s)
+// with P marked t before the first voxel and t past the last (clamped to the
+// row), SE read as 0 left of the row and as the row's total right of it.
+//
+// Layout: one word per voxel, E in the low and P in the high half (added as 1
+// and +-65536, so a row's prefix sum of words is SE + 65536 SP mod 2^32), the
+// major axis fastest, rows of W words (at least one past the voxels, for the
+// end marks), row = minor index + nminor * slice.
+
+// Words per row: one more than the voxels, rounded up to an odd number when
+// the box still fits in the (nx + 1)(ny + 1) words a tile is planned with, so
+// that the lanes of a warp that are in different rows at one major index hit
+// different banks.
+HD_HD int tile_row_words(int nmaj, int nminor)
+{
+    const int w = nmaj + 1;
+    return (w & 1) == 0 && nminor <= nmaj + 1 ? w + 1 : w;
+}
+
+// Packed event walk (kLeanWords words): |D_0|, |D_m| mod |D_0|, the Bresenham
+// remainder; then byte offsets from the tile's first word: of one event to the
+// next without the carry, of the first event, of the last place the end mark
+// can have, of the first mark; and the number of events (bit 31: no walk).
+HD_HD void event_pack(const LeanWalk &L, int nmaj, int nminor, int thick, uint32_t o[kLeanWords])
+{
+    const int W = tile_row_words(nmaj, nminor);
+    // events: the K' = min(K, ceil(X / |D_m|)) crossings k of minor 0 with
+    // J_k <= kmz, J_k = J_1 + floor(((k - 1) |D_m| + rem) / |D_0|) and
+    // X = (kmz - J_1 + 1) |D_0| - rem
+    int n = 0;
+    if (L.K > 0 && L.jn <= L.kmz) {
+        const long long X =
+            static_cast<long long>(L.kmz - L.jn + 1) * L.ad - static_cast<long long>(L.rem);
+        const long long am = static_cast<long long>(L.Qu) * L.ad + L.Ru;
+        const long long k = fdiv_small(X - 1, am) + 1;  // X >= 1: rem < |D_0|
+        n = k < L.K ? static_cast<int>(k) : L.K;
+    }
+    const int s = (L.fl & 2) ? 1 : -1;
+    const int row0 = L.row * W;
+    const int m0 = L.im0 - thick > 0 ? L.im0 - thick : 0;
+    const int j1 = L.jn < L.kmz ? L.jn : L.kmz;
+    const int rowk = row0 + s * n * W;
+    const int last = L.im0 + L.kmz + thick + 1;
+    o[0] = L.ad;
+    o[1] = L.Ru;
+    o[2] = L.rem;
+    o[3] = static_cast<uint32_t>(4 * (L.Qu + s * W));
+    o[4] = static_cast<uint32_t>(4 * (row0 + L.im0 + j1));
+    o[5] = static_cast<uint32_t>(4 * (rowk + (last < nmaj ? last : nmaj)));
+    o[6] = static_cast<uint32_t>(4 * (row0 + m0));
+    o[7] = static_cast<uint32_t>(n);
+}
+
+// A packed event walk with no voxel.
+HD_HD void event_pack_empty(uint32_t o[kLeanWords])
+{
+    for (int i = 0; i < kLeanWords; ++i) o[i] = 0;
+    o[7] = 0x80000000u;
+}
+
+// An event walk in progress; addresses are byte offsets from a base the
+// caller chooses (such as the tile's shared-memory address).
+struct EventCursor {
+    unsigned ad, Ru, rem;
+    int addr;  // of the next event
+    int step;  // to the one after it, without the carry
+    int left;  // events left
+    int endl;  // the last address the end mark can have
+};
+
+// Starts a packed walk; *first receives the address of its first mark.
+// False when there is no walk (no events left then either).
+HD_HD bool event_start(const uint32_t o[kLeanWords], int base, EventCursor &c, int &first)
+{
+    c.ad = o[0];
+    c.Ru = o[1];
+    c.rem = o[2];
+    c.step = static_cast<int>(o[3]);
+    c.addr = base + static_cast<int>(o[4]);
+    c.endl = base + static_cast<int>(o[5]);
+    first = base + static_cast<int>(o[6]);
+    const bool walk = static_cast<int>(o[7]) >= 0;
+    c.left = walk ? static_cast<int>(o[7]) : 0;
+    return walk;
+}
+
+// Moves past one event.
+HD_HD void event_next(EventCursor &c)
+{
+    c.rem += c.Ru;
+    const bool carry = c.rem >= c.ad;
+    c.addr += c.step;
+    if (carry) {
+        c.rem -= c.ad;
+        c.addr += 4;
+    }
+    --c.left;
+}
+
+// Address of the end mark once no event is left (the cursor then stands at
+// the event that would follow, in the last row); thick4 = 4 (t + 1).
+HD_HD int event_end(const EventCursor &c, int thick4)
+{
+    const int e = c.addr + thick4;
+    return e < c.endl ? e : c.endl;
 }
 
 // Packed run-walk state: 16 32-bit words, so a walk prepared by one kernel

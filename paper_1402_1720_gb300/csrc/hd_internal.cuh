@@ -10,7 +10,8 @@ namespace hd {
 
 constexpr int64_t kQ16 = 65536;
 constexpr int kMaxN = 4096;
-constexpr int kMaxTiles = 2048;       // tiles per class for the shared-memory path
+constexpr int kMaxTiles = 2048;       // tiles per group for the shared-memory path
+constexpr int kGroups = 8;            // groups of records: class + 2 * walk type (hd_geom.cuh)
 constexpr int kTraceThreads = 512;    // threads per block of the tiled traversal
 constexpr int kTileSmemBytes = 224 * 1024;  // shared memory per block for a private tile
 
@@ -30,16 +31,14 @@ struct GeomQ {
     unsigned long long mx, my, mz;  // floor(2^64 / (2 s)): division by multiply-high
 };
 
-// Device-side counters of one scan.  The block from njobs to the end is
+// Device-side counters of one scan.  The block from n_global to the end is
 // cleared before every chunk of histories.
 struct Ctrl {
     unsigned long long n_in, n_miss, n_hit, n_none, n_reject;
     unsigned long long steps_miss, steps_hit;
     unsigned long long pairs_general;  // pairs sent to the fallback list (cumulative)
     unsigned long long runs;           // runs walked by the tiled pass (cumulative)
-    int njobs;                // jobs of the tiled traversal
     unsigned int n_global;    // records listed for the global path (Records::glist)
-    int job_next;             // next job to hand out
     unsigned int n_fallback;  // records traversed by the global-memory path
     unsigned int n_pair_fallback;  // entries of the pair fallback list
     unsigned int fb_next;          // next fallback entry to hand out
@@ -90,20 +89,21 @@ struct TilePlan {
     int nx, ny, nz;
     int tx, ty, tz;     // tile size in voxels
     int ntx, nty, ntz;  // tiles per axis
-    int ntiles;         // tiles per class (0: tiled path off)
+    int ntiles;         // tiles per group (0: tiled path off)
     int max_tiles;      // records touching more tiles take the global path
     int pairs_per_record;  // pair budget per history (pair_cap = this * slots)
-    int job_size;       // pairs per job
+    int job_size;       // most pairs between two flushes of a tile
     long long pair_cap;
     int tile_words;     // 32-bit words of shared memory per block
     int refill;         // idle lanes that trigger a warp refill
     int threads;        // threads per block of the traversal (256, 512, 768, 1024)
+    int thick;          // in-plane dilation of the walks, voxels (0: thin paths)
     unsigned mtx, mty, mtz;  // floor(2^32 / t) + 1 (0 when t = 1): division by a tile size
 };
 
-// (record, tile) pairs sorted by tile: the packed lean walk of the record
-// clipped to the tile, 32 bytes per pair (two uint4: one 32-byte sector;
-// class and tile come from the job).  A pair whose walk has no lean form
+// (record, tile) pairs sorted by group and tile: the packed event walk of the
+// record clipped to the tile, 32 bytes per pair (two uint4: one 32-byte
+// sector; group and tile come from the job).  A pair whose walk has no lean form
 // (a tie, a pending start, or a z crossing inside the tile) holds instead
 // its tile-local endpoints, tile and class, marked empty for the lean pass,
 // and its position goes to the fallback list; traversal blocks that run out
@@ -124,25 +124,25 @@ constexpr int kMaxRecordTiles = 32;
 constexpr int kRecordTileBits = 5;
 static_assert(kMaxRecordTiles == 1 << kRecordTileBits, "tile index bits");
 
-struct TileJob {
-    int tile;   // tile id within its class
-    int cls;    // 0 missed (N), 1 hit (M)
-    int start;  // pair range [start, end)
-    int end;
+// The buckets of a chunk: its pairs by group and tile (bucket group * ntiles +
+// tile), kGroups ntiles of each.
+struct Buckets {
+    uint32_t *count;             // pairs
+    uint32_t *first;             // the bucket's first pair
+    unsigned long long *events;  // events of their walks (hd_geom.cuh)
 };
 
 // Everything the traversal kernel needs about one scan; a batch passes a
-// table of these and one job counter for all of them.
+// table of these.
 struct ScanDesc {
     TilePlan tp;
     Pairs pairs;
-    const TileJob *jobs;
-    Ctrl *ctrl;  // njobs of the scan (read) and its step counters (added to)
+    Buckets buckets;
+    Ctrl *ctrl;  // the scan's counters (added to) and fallback list (read)
     uint32_t *N, *M;
 };
 
 constexpr int kMaxBatch = 64;  // scans per batched traversal launch
-constexpr int kMinJob = 8192;  // smallest job the plan makes (pairs), unless the tuning is lower
 
 struct Inputs {
     const float *angle, *u_in, *v_in, *u_out, *v_out, *wepl;
@@ -151,7 +151,7 @@ struct Inputs {
 // ---- launchers (stream-ordered; return the launch's cudaError_t) ----
 
 // Classification, records and pair counts of a chunk.  block_count (null
-// when tp.ntiles is 0) receives, per tile-class column c (2 tp.ntiles of
+// when tp.ntiles is 0) receives, per group-tile column c (kGroups tp.ntiles of
 // them) and ingest block b, the pairs of that block's records in that tile
 // at [c * blocks + b]; block_pairs[b] the block's pairs in all, listed in
 // stage (Pairs::stage).  Each block keeps to a pair budget of
@@ -164,26 +164,25 @@ cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cor
                           cudaStream_t s);
 
 // Per column: the exclusive prefix over blocks of block_count (in place) and
-// the column total into tile_count; then the plan (tile offsets into
-// tile_cursor, the job table).
+// the column total into buckets.count; then the buckets' first pairs, and
+// their events cleared.
 cudaError_t launch_plan(const TilePlan &tp, int64_t n, uint32_t *block_count,
-                        uint32_t *tile_count, uint32_t *tile_cursor, TileJob *jobs, Ctrl *ctrl,
-                        int sm_count, cudaStream_t s);
+                        const Buckets &buckets, int sm_count, cudaStream_t s);
 
 // Counting sort of the (record, tile) pairs by tile, with the walk set-up of
 // each pair; block b of the chunk split takes the block_pairs[b] pairs that
-// ingest block b listed and writes those of tile c from
-// tile_cursor[c] + block_count[c * blocks + b] on.
+// ingest block b listed and writes those of bucket c from
+// buckets.first[c] + block_count[c * blocks + b] on, adding their events.
 cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ctrl *ctrl,
-                           const uint32_t *tile_cursor, const uint32_t *block_count,
+                           const Buckets &buckets, const uint32_t *block_count,
                            const uint32_t *block_pairs, const Pairs &pairs, int sm_count,
                            cudaStream_t s);
 
-// Persistent traversal over the jobs of nscans scans (descs on the device),
-// handed out through *job_counter (zero before the launch).  smem_words is
-// the largest tile of the scans; threads is 256, 512, 768 or 1024.
-cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int *job_counter,
-                               int smem_words, int threads, int grid, cudaStream_t s);
+// Traversal of the pairs of nscans scans (descs on the device) by `grid`
+// resident blocks.  tile_words is the largest tile of the scans; threads is
+// 256, 512, 768 or 1024.
+cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
+                               int grid, cudaStream_t s);
 
 // Global-memory traversal of the records whose path is 2 (or of every
 // record when all_records is set); upper is the chunk's slot count.
@@ -191,12 +190,17 @@ cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, c
                                 uint32_t *N, uint32_t *M, int all_records,
                                 int sm_count, cudaStream_t s);
 
+// Once per device, before the first launch there: the shared memory ingest and
+// scatter may use for the most tiles a plan can have.
+cudaError_t init_ingest();
+cudaError_t init_scatter();
+
 cudaError_t launch_classify(const float *wepl, int64_t n, float tau_l, float tau_h,
                             uint8_t *cls, cudaStream_t s);
 
-// Blocks per SM the tiled traversal can keep resident with this much shared
-// memory per block and this many threads (0 when the launch is impossible).
-int trace_tiles_occupancy(int smem_words, int threads);
+// Blocks per SM the tiled traversal can keep resident with tiles of this many
+// words and this many threads (0 when the launch is impossible).
+int trace_tiles_occupancy(int tile_words, int threads);
 
 struct DecideArgs {
     int32_t nx, ny, nz;

@@ -1,7 +1,7 @@
 // Bucketing of the (record, tile) pairs of a chunk for the tiled traversal,
 // after ingest has counted, per ingest block, its pairs in each tile:
 //   bases    per tile, exclusive scan over the blocks -> each block's offset
-//   plan     exclusive scan of the tile totals -> tile offsets, job table
+//   plan     exclusive scan of the totals -> each bucket's first pair
 //   scatter  counting sort of the pairs by tile: block b of the ingest split
 //            writes its pairs from its offsets, with each pair's walk set-up
 #include <cooperative_groups.h>
@@ -49,7 +49,7 @@ __device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *s_warp
 }
 
 
-// One warp per tile-class column: the exclusive prefix over the ingest
+// One warp per group-tile column: the exclusive prefix over the ingest
 // blocks of their pair counts (in place) and the column's total.
 __global__ void __launch_bounds__(256) bases_kernel(int ncols, int nblocks, uint32_t *counts,
                                                     uint32_t *totals)
@@ -69,71 +69,38 @@ __global__ void __launch_bounds__(256) bases_kernel(int ncols, int nblocks, uint
     if (lane == 0) totals[c] = run;
 }
 
-// One block: tile offsets (exclusive scan of the counts), cursors for the
-// scatter, and the job table (chunks of one tile's pairs).  The job size
-// adapts to the amount of work: at most tp.job_size pairs, and small enough
-// that there are about three jobs per SM (not below kMinJob, so a job's
-// flush stays small against its walks; two or four per SM, or a smaller
-// floor, measured slower).
-__global__ void __launch_bounds__(1024) plan_kernel(TilePlan tp, const uint32_t *tile_count,
-                                                    uint32_t *tile_cursor, TileJob *jobs,
-                                                    Ctrl *ctrl, int sm_count)
+// One block: the buckets' first pairs (exclusive scan of their counts).
+__global__ void __launch_bounds__(1024) plan_kernel(int nt, Buckets buckets)
 {
     __shared__ unsigned s_warp[33];
-    __shared__ unsigned s_js;
-    const int nt = 2 * tp.ntiles;
     const int per = (nt + blockDim.x - 1) / blockDim.x;
     const int t0 = threadIdx.x * per;
     unsigned my_pairs = 0;
-    for (int t = t0; t < t0 + per && t < nt; ++t) my_pairs += tile_count[t];
+    for (int t = t0; t < t0 + per && t < nt; ++t) my_pairs += buckets.count[t];
     unsigned tot_pairs;
     unsigned off = block_excl_scan(my_pairs, s_warp, tot_pairs);
-    if (threadIdx.x == 0) {
-        const unsigned want = (tot_pairs + 3u * sm_count - 1u) / (3u * sm_count);
-        unsigned js = want < static_cast<unsigned>(tp.job_size) ? want : tp.job_size;
-        if (js < static_cast<unsigned>(kMinJob)) js = kMinJob;
-        if (js > static_cast<unsigned>(tp.job_size)) js = tp.job_size;
-        s_js = js;
-    }
-    __syncthreads();
-    const unsigned js = s_js;
-    unsigned my_jobs = 0;
-    for (int t = t0; t < t0 + per && t < nt; ++t) my_jobs += (tile_count[t] + js - 1) / js;
-    unsigned tot_jobs;
-    unsigned joff = block_excl_scan(my_jobs, s_warp, tot_jobs);
     for (int t = t0; t < t0 + per && t < nt; ++t) {
-        const unsigned c = tile_count[t];
-        tile_cursor[t] = off;
-        for (unsigned s = 0; s < c; s += js) {
-            TileJob j;
-            j.tile = t % tp.ntiles;
-            j.cls = t / tp.ntiles;
-            j.start = static_cast<int>(off + s);
-            j.end = static_cast<int>(off + (s + js < c ? s + js : c));
-            jobs[joff++] = j;
-        }
-        off += c;
-    }
-    if (threadIdx.x == 0) {
-        ctrl->njobs = static_cast<int>(tot_jobs);
-        ctrl->job_next = 0;
+        buckets.first[t] = off;
+        buckets.events[t] = 0;
+        off += buckets.count[t];
     }
 }
 
-// The general set-up of one (record, tile) pair: its packed lean walk, an
+// The general set-up of one (record, tile) pair: its packed event walk, an
 // empty walk, or (returns true) the general form for the fallback list.
 __device__ __noinline__ bool general_setup(const int32_t gi[3], const int32_t go[3], int dx,
-                                           int dy, int dz, int tile, int cls, uint4 &p0,
-                                           uint4 &p1)
+                                           int dy, int dz, int thick, int tile, int cls,
+                                           uint4 &p0, uint4 &p1)
 {
     RunWalk w;
     LeanWalk L;
     uint32_t pk[kLeanWords];
     bool fallback = false;
     if (!run_begin(w, gi, go, dx, dy, dz)) {
-        lean_pack_empty(pk);
+        event_pack_empty(pk);
     } else if (lean_of(w, L)) {
-        lean_pack(L, pk);
+        const bool ymaj = (L.fl >> 2) & 1;
+        event_pack(L, ymaj ? dy : dx, ymaj ? dx : dy, thick, pk);
     } else {
         // walked from the fallback list by the general run walk
         general_pack(gi, go, tile, cls, pk);
@@ -149,20 +116,23 @@ __device__ __noinline__ bool general_setup(const int32_t gi[3], const int32_t go
 // tile_start[c] + block_base[c * blocks + b] on (a shared-memory cursor per
 // tile orders them within the block).
 __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
-    TilePlan tp, Records rec, int64_t per_block, const uint32_t *tile_start,
-    const uint32_t *block_base, const uint32_t *block_pairs, Ctrl *ctrl, Pairs pairs)
+    TilePlan tp, Records rec, int64_t per_block, Buckets buckets, const uint32_t *block_base,
+    const uint32_t *block_pairs, Ctrl *ctrl, Pairs pairs)
 {
     extern __shared__ uint32_t s_mem[];
-    const int nt = 2 * tp.ntiles;
-    uint32_t *s_base = s_mem;       // this block's first position in each tile
-    uint32_t *s_next = s_mem + nt;  // pairs written per tile so far
+    const int nt = kGroups * tp.ntiles;
+    uint32_t *s_base = s_mem;       // this block's first position in each bucket
+    uint32_t *s_next = s_mem + nt;  // pairs written per bucket so far
+    uint32_t *s_events = s_next + nt;  // and the events of their walks
     for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-        s_base[t] = tile_start[t] + block_base[static_cast<size_t>(t) * gridDim.x + blockIdx.x];
+        s_base[t] = buckets.first[t] + block_base[static_cast<size_t>(t) * gridDim.x + blockIdx.x];
         s_next[t] = 0;
+        s_events[t] = 0;
     }
     __syncthreads();
     const int64_t h0 = static_cast<int64_t>(blockIdx.x) * per_block;
     const unsigned npairs = block_pairs[blockIdx.x];
+    unsigned runs = 0;
     const uint32_t *list = pairs.stage + static_cast<int64_t>(blockIdx.x) * per_block * tp.pairs_per_record;
     for (unsigned e = threadIdx.x; e < npairs; e += kScatterThreads) {
         const uint32_t code = list[e];
@@ -187,7 +157,8 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
             y = lo[1] + (j / ex) % ey;
             z = lo[2] + j / (ex * ey);
         }
-        const int t = cls * tp.ntiles + x + tp.ntx * (y + tp.nty * z);
+        const int tile = x + tp.ntx * (y + tp.nty * z);
+        const int t = status_group(stw) * tp.ntiles + tile;
         const uint32_t pos = s_base[t] + atomicAdd(&s_next[t], 1u);
         // set up the walk of this record clipped to this tile
         const int x0 = x * tp.tx, y0 = y * tp.ty, z0 = z * tp.tz;
@@ -206,17 +177,22 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
             const int rl = slab_lean(gi, go, dx, dy, L);
             uint32_t pk[kLeanWords];
             if (rl == 1) {
-                lean_pack(L, pk);
+                const bool ymaj = (L.fl >> 2) & 1;
+                event_pack(L, ymaj ? dy : dx, ymaj ? dx : dy, tp.thick, pk);
             } else if (rl == 0) {
-                lean_pack_empty(pk);
+                event_pack_empty(pk);
             } else {
-                general_pack(gi, go, t - cls * tp.ntiles, cls, pk);
+                general_pack(gi, go, tile, cls, pk);
                 fallback = true;
             }
             p0 = make_uint4(pk[0], pk[1], pk[2], pk[3]);
             p1 = make_uint4(pk[4], pk[5], pk[6], pk[7]);
         } else {
-            fallback = general_setup(gi, go, dx, dy, dz, t - cls * tp.ntiles, cls, p0, p1);
+            fallback = general_setup(gi, go, dx, dy, dz, tp.thick, tile, cls, p0, p1);
+        }
+        if (static_cast<int>(p1.w) >= 0) {
+            runs += p1.w + 1u;  // a walk's runs: one more than its events
+            if (p1.w != 0u) atomicAdd(&s_events[t], p1.w);
         }
         pairs.v[2 * static_cast<size_t>(pos)] = p0;
         pairs.v[2 * static_cast<size_t>(pos) + 1] = p1;
@@ -233,33 +209,47 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
             pairs.fb[at] = make_uint2(pos, 0u);
         }
     }
+    // runs of the chunk's thin walks, for the statistics
+    unsigned long long all = tp.thick > 0 ? 0u : runs;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(kFull, all, o);
+    if ((threadIdx.x & 31u) == 0 && all) atomicAdd(&ctrl->runs, all);
+    __syncthreads();
+    for (int t = threadIdx.x; t < nt; t += blockDim.x)
+        if (s_events[t])
+            atomicAdd(&buckets.events[t], static_cast<unsigned long long>(s_events[t]));
 }
 
 }  // namespace
 
 cudaError_t launch_plan(const TilePlan &tp, int64_t n, uint32_t *block_count,
-                        uint32_t *tile_count, uint32_t *tile_cursor, TileJob *jobs, Ctrl *ctrl,
-                        int sm_count, cudaStream_t s)
+                        const Buckets &buckets, int sm_count, cudaStream_t s)
 {
-    const int ncols = 2 * tp.ntiles;
+    const int ncols = kGroups * tp.ntiles;
     const ChunkSplit sp = chunk_split(n, sm_count);
     bases_kernel<<<static_cast<unsigned>((ncols + 7) / 8), 256, 0, s>>>(ncols, sp.blocks,
-                                                                        block_count, tile_count);
-    plan_kernel<<<1, 1024, 0, s>>>(tp, tile_count, tile_cursor, jobs, ctrl,
-                                   sm_count > 0 ? sm_count : 1);
+                                                                        block_count,
+                                                                        buckets.count);
+    plan_kernel<<<1, 1024, 0, s>>>(ncols, buckets);
     return cudaGetLastError();
 }
 
+cudaError_t init_scatter()
+{
+    return cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                static_cast<int>(sizeof(uint32_t)) * 3 * kGroups * kMaxTiles);
+}
+
 cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ctrl *ctrl,
-                           const uint32_t *tile_cursor, const uint32_t *block_count,
+                           const Buckets &buckets, const uint32_t *block_count,
                            const uint32_t *block_pairs, const Pairs &pairs, int sm_count,
                            cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const ChunkSplit sp = chunk_split(n, sm_count);
-    const size_t smem = sizeof(uint32_t) * 4 * static_cast<size_t>(tp.ntiles);
+    const size_t smem = sizeof(uint32_t) * 3 * kGroups * static_cast<size_t>(tp.ntiles);
     scatter_kernel<<<static_cast<unsigned>(sp.blocks), kScatterThreads, smem, s>>>(
-        tp, rec, sp.per_block, tile_cursor, block_count, block_pairs, ctrl, pairs);
+        tp, rec, sp.per_block, buckets, block_count, block_pairs, ctrl, pairs);
     return cudaGetLastError();
 }
 

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "hd_geom.cuh"
+#include "hd_fallback.cuh"
 #include "hd_thick.cuh"
 
 namespace hd {
@@ -204,6 +205,95 @@ __global__ void __launch_bounds__(kThickThreads) thick_kernel(Inputs in, int64_t
     }
 }
 
+// The fallback pairs (no event walk), a warp per pair: the lanes walk their
+// strips of the slice (warp_strip) and gather the walk's run of each row (first
+// and last major index) in shared memory, then take the target rows, each the
+// union of the runs within k rows grown by k, voxel by voxel into N or M (the
+// pairs are few: a pass over difference arrays would cost more than all of
+// them).
+constexpr int kFbWarps = 2;  // warps per block, each with 16 KB for kMaxN / 2 rows
+
+__global__ void __launch_bounds__(32 * kFbWarps) thick_fallback_kernel(
+    const ScanDesc *__restrict__ dp, int k)
+{
+    __shared__ int s_lo[kFbWarps][kMaxN / 2], s_hi[kFbWarps][kMaxN / 2];
+    const int lane = static_cast<int>(threadIdx.x & 31u);
+    int *const rlo = s_lo[threadIdx.x >> 5], *const rhi = s_hi[threadIdx.x >> 5];
+    const ScanDesc &d = *dp;
+    const unsigned nf = d.ctrl->n_pair_fallback;
+    const TilePlan tp = d.tp;
+    for (;;) {
+        if (nf == 0) return;
+        unsigned i = 0;
+        if (lane == 0) i = atomicAdd(&d.ctrl->fb_next, 1u);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        if (i >= nf) return;
+        int32_t gi[3], go[3];
+        const uint32_t id = load_general(d.pairs, d.pairs.fb[i].x, gi, go);
+        const int cls = static_cast<int>(id & 1u);
+        const int z = static_cast<int>(id >> 1);  // tiles are whole slices
+        const bool ymaj = abs(go[1] - gi[1]) > abs(go[0] - gi[0]);
+        const int nminor = ymaj ? tp.nx : tp.ny, nmaj = ymaj ? tp.ny : tp.nx;
+        // the rows of the walk in pieces that fit the buffer, k rows of
+        // overlap on either side
+        const int piece = kMaxN / 2 - 2 * k;
+        for (int t0 = 0; t0 < nminor; t0 += piece) {
+            const int r0 = max(t0 - k, 0), r1 = min(t0 + piece + k, nminor);
+            for (int r = r0 + lane; r < r1; r += 32) {
+                rlo[r - r0] = nmaj;
+                rhi[r - r0] = -1;
+            }
+            __syncwarp();
+            int dx = tp.nx, dy = tp.ny, ox = 0, oy = 0;
+            int32_t a[3], b[3];
+            RunWalk w;
+            if (warp_strip(gi, go, dx, dy, ox, oy, a, b) && run_begin(w, a, b, dx, dy, 1)) {
+                // in a narrow strip the walk's own axes may be the other way
+                // round only for equal |D|, where both are x-major
+                const int om = ymaj ? oy : ox, on = ymaj ? ox : oy;
+                int row, lo, hi;
+                while (run_next(w, row, lo, hi)) {
+                    const int r = row + on;
+                    if (r >= r0 && r < r1) {
+                        atomicMin(&rlo[r - r0], lo + om);
+                        atomicMax(&rhi[r - r0], hi + om);
+                    }
+                }
+            }
+            __syncwarp();
+            uint32_t *const vol =
+                (cls == 0 ? d.N : d.M) + static_cast<int64_t>(z) * tp.nx * tp.ny;
+            const int64_t mstep = ymaj ? tp.nx : 1, tstep = ymaj ? 1 : tp.nx;
+            for (int t = t0 + lane; t < min(t0 + piece, nminor); t += 32) {
+                int lo = nmaj, hi = -1;
+                for (int r = max(t - k, 0); r <= min(t + k, nminor - 1); ++r) {
+                    lo = min(lo, rlo[r - r0]);
+                    hi = max(hi, rhi[r - r0]);
+                }
+                if (hi >= 0) {
+                    for (int m = max(lo - k, 0); m <= min(hi + k, nmaj - 1); ++m)
+                        atomicAdd(vol + t * tstep + m * mstep, 1u);
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
+// Whether a chunk has records on the global path (it nearly never does: then
+// clearing their difference arrays and summing the rows, 20 MB each way and
+// 0.4 ms on the head-sized grid, is skipped).
+__device__ __forceinline__ bool thick_left_over(const Ctrl *ctrl) { return ctrl->n_global != 0; }
+
+__global__ void __launch_bounds__(kThickThreads) thick_clear_kernel(uint4 *ws, int64_t n,
+                                                                    const Ctrl *ctrl)
+{
+    if (!thick_left_over(ctrl)) return;
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        ws[i] = make_uint4(0, 0, 0, 0);
+}
+
 // The records of a chunk that take the global path (status 2: too many
 // tiles, or beyond the pair budget): each walked whole over the grid into the
 // global difference arrays; voxel memberships added to the scan's counters.
@@ -233,8 +323,9 @@ __global__ void __launch_bounds__(kThickThreads) thick_records_kernel(Records re
 
 __global__ void __launch_bounds__(kThickThreads) thick_rows_kernel(
     const int32_t *__restrict__ diff, int64_t rows, int nmaj, int stride_maj, int nminor,
-    int64_t plane, int major_is_y, uint32_t *__restrict__ out)
+    int64_t plane, int major_is_y, uint32_t *__restrict__ out, const Ctrl *__restrict__ ctrl)
 {
+    if (ctrl != nullptr && !thick_left_over(ctrl)) return;
     const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (r >= rows || out == nullptr) return;
     const int64_t z = r / nminor;
@@ -304,9 +395,9 @@ cudaError_t launch_thick(const Inputs &in, int64_t n, const hd_geometry *geom, c
         if (!out) continue;
         const int64_t rx = int64_t(geom->ny) * geom->nz, ry = int64_t(geom->nx) * geom->nz;
         thick_rows_kernel<<<static_cast<unsigned>((rx + 255) / 256), 256, 0, st>>>(
-            ws.dx[c], rx, geom->nx, 1, geom->ny, plane, 0, out);
+            ws.dx[c], rx, geom->nx, 1, geom->ny, plane, 0, out, nullptr);
         thick_rows_kernel<<<static_cast<unsigned>((ry + 255) / 256), 256, 0, st>>>(
-            ws.dy[c], ry, geom->ny, geom->nx, geom->nx, plane, 1, out);
+            ws.dy[c], ry, geom->ny, geom->nx, geom->nx, plane, 1, out, nullptr);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && (stats || intervals)) {
@@ -335,9 +426,10 @@ ThickDiff thick_diff_of(const hd_geometry *geom, void *workspace)
     return td;
 }
 
-// Adds the global difference arrays to N and M (row prefix sums).
+// Adds the global difference arrays to N and M (row prefix sums); with ctrl,
+// only when its chunk has records on the global path.
 static cudaError_t launch_thick_rows(const hd_geometry *geom, const ThickWs &ws, uint32_t *N,
-                                     uint32_t *M, cudaStream_t st)
+                                     uint32_t *M, const Ctrl *ctrl, cudaStream_t st)
 {
     const int64_t plane = int64_t(geom->nx) * geom->ny;
     for (int c = 0; c < 2; ++c) {
@@ -345,9 +437,9 @@ static cudaError_t launch_thick_rows(const hd_geometry *geom, const ThickWs &ws,
         if (!out) continue;
         const int64_t rx = int64_t(geom->ny) * geom->nz, ry = int64_t(geom->nx) * geom->nz;
         thick_rows_kernel<<<static_cast<unsigned>((rx + 255) / 256), 256, 0, st>>>(
-            ws.dx[c], rx, geom->nx, 1, geom->ny, plane, 0, out);
+            ws.dx[c], rx, geom->nx, 1, geom->ny, plane, 0, out, ctrl);
         thick_rows_kernel<<<static_cast<unsigned>((ry + 255) / 256), 256, 0, st>>>(
-            ws.dy[c], ry, geom->ny, geom->nx, geom->nx, plane, 1, out);
+            ws.dy[c], ry, geom->ny, geom->nx, geom->nx, plane, 1, out, ctrl);
     }
     return cudaGetLastError();
 }
@@ -358,7 +450,7 @@ cudaError_t launch_thick_finish(const hd_geometry *geom, void *workspace, uint32
 {
     ThickWs ws{};
     thick_layout(geom, workspace, &ws);
-    cudaError_t e = launch_thick_rows(geom, ws, N, M, st);
+    cudaError_t e = launch_thick_rows(geom, ws, N, M, nullptr, st);
     if (e == cudaSuccess && (stats || intervals)) {
         thick_stats_kernel<<<1, 32, 0, st>>>(ws.stats, stats, intervals);
         e = cudaGetLastError();
@@ -369,24 +461,26 @@ cudaError_t launch_thick_finish(const hd_geometry *geom, void *workspace, uint32
 cudaError_t launch_thick_scan(const ScanDesc *desc_dev, const hd_geometry *geom,
                               const Records &rec, Ctrl *ctrl, int64_t upper, const GeomQ &g,
                               int k, void *workspace, uint32_t *N, uint32_t *M, int smem_words,
-                              int threads, int sm_count, cudaStream_t st)
+                              int threads, int grid, int sm_count, cudaStream_t st)
 {
     ThickWs ws{};
     const size_t need = thick_layout(geom, workspace, &ws);
     const ThickDiff td = thick_diff_of(geom, workspace);
-    cudaError_t e = cudaMemsetAsync(workspace, 0, need, st);
-    if (e == cudaSuccess)
-        e = launch_trace_thick(desc_dev, &ctrl->job_next, k, td, smem_words, threads,
-                               sm_count > 0 ? sm_count : 1, st);
+    cudaError_t e = launch_trace_tiles(desc_dev, 1, smem_words, threads, grid, st);
     if (e == cudaSuccess && upper > 0) {
         int64_t blocks = (upper + kThickThreads - 1) / kThickThreads;
         const int64_t cap = int64_t(sm_count > 0 ? sm_count : 1) * 8;
         if (blocks > cap) blocks = cap;
+        // the workspace is a multiple of 256 bytes (thick_layout)
+        thick_clear_kernel<<<static_cast<unsigned>(cap), kThickThreads, 0, st>>>(
+            static_cast<uint4 *>(workspace), static_cast<int64_t>(need / 16), ctrl);
+        thick_fallback_kernel<<<static_cast<unsigned>(sm_count > 0 ? 4 * sm_count : 4), 32 * kFbWarps, 0,
+                                st>>>(desc_dev, k);
         thick_records_kernel<<<static_cast<unsigned>(blocks), kThickThreads, 0, st>>>(rec, ctrl, g,
                                                                                       k, td);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = launch_thick_rows(geom, ws, N, M, st);
+    if (e == cudaSuccess) e = launch_thick_rows(geom, ws, N, M, ctrl, st);
     return e;
 }
 

@@ -1,10 +1,9 @@
 // Shared-memory privatised traversal: the grid is cut into tiles whose
 // counters fit in one block's shared memory, every (record, tile) pair is
 // walked with the exact traversal clipped to the tile, and each block adds
-// its private tile into N or M once per job.  Persistent blocks take jobs
-// (ranges of one tile's pairs, made in hd_scatter.cu); warps refill idle
-// lanes from the job's pair range, so lanes do not wait for the longest
-// path.
+// its private tile into N or M once per part of a bucket (the pairs of one
+// group and tile, sorted in hd_scatter.cu) that it has walked; warps refill
+// idle lanes from the parts' pairs, so lanes do not wait for the longest path.
 #include "hd_fallback.cuh"
 
 namespace hd {
@@ -12,30 +11,22 @@ namespace hd {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kRunsPerStep = 8;  // runs a traversal lane walks between refill checks
+constexpr int kEventsPerStep = 8;  // events a traversal lane walks between refill checks
 
 // ---------------------------------------------------------------- traversal
 //
-// A block's private tile holds one 32-bit word per voxel of the tile box,
-// laid out x fastest with one padding column and one padding row:
-// word(x, y, z) = x + Wx (y + Hy z), Wx = dx + 1, Hy = dy + 1.  Its low
-// 16 bits are the difference counts of runs along x, its high 16 bits those
-// of runs along y (z is never a run axis: it is always a minor one).  A run
-// lo..hi adds +1 (x runs) or +65536 (y runs) at its first voxel and the
-// negative just past its last one, which for a run ending at the box's edge
-// is the padding column or row, so no run needs a bounds test.  Each job
-// covers at most 32767 pairs, so every difference and every prefix sum of
-// either half stays inside int16, and a word read as lo + 65536 hi (mod
-// 2^32) decodes exactly even after carries between the halves.  Rows of
-// words are an odd number of words apart (for the 200-voxel planes here),
-// so lanes walking parallel paths at the same major index hit distinct
-// banks.
-
-__device__ __forceinline__ void load_lean(const Pairs &pairs, int idx, uint4 &a, uint4 &b)
-{
-    a = __ldg(&pairs.v[2 * static_cast<size_t>(idx)]);
-    b = __ldg(&pairs.v[2 * static_cast<size_t>(idx) + 1]);
-}
+// A block's private tile holds one 32-bit word per voxel of the tile box in
+// the layout of event walks (hd_geom.cuh): all walks of a bucket have one type,
+// so the tile's fast axis is their major axis, the low half of a word counts
+// the row changes that leave a run there and the high half the walks' first
+// and last marks.  A part has at most 32767 pairs, so every prefix sum of
+// either half stays inside 16 bits.
+//
+// Bound: integer issue of the event loop and the refills, one shared atomic
+// per run (3.4 voxels on the head-sized scan).  The form before, +1 and -1 at
+// the two ends of each run, took two and about three times the integer steps
+// per run: head-sized scan (9e6 histories) 0.683 -> 0.407 ms, large streamed
+// scan 0.288 -> 0.186 ms per chunk, with the balance and the flush below.
 
 // Shared-memory reduction (no value returned) at a shared-space byte address.
 __device__ __forceinline__ void smem_red_add(int addr, uint32_t v)
@@ -43,258 +34,617 @@ __device__ __forceinline__ void smem_red_add(int addr, uint32_t v)
     asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v));
 }
 
-// Walks the pairs [start, start + total) of a job into the block's tile:
-// each lane walks one pair and holds the packed lean walk of its next one
-// (loaded a refill ahead, so starting a walk never waits on memory).  A
-// refill happens once enough lanes are idle; then every idle lane with a
-// prefetched pair starts it and fetches another, the pair index coming from
-// the block's counter *s_next.  Adds the runs walked to `runs`.
-__device__ __forceinline__ void walk_job(uint32_t *tile, int dx, int dy, int dz,
-                                         const Pairs &pairs, int start, int total, int refill,
-                                         unsigned *s_next, unsigned &runs)
+// Event u of a step of cnt events: counted at the cursor, which then moves on
+// (event_next without the count of events left); nothing when u >= cnt.
+// Predicated by hand: the loop the compiler made of "leave when the walk ends"
+// took about 16 instructions and a reconvergence per event, this takes 7.
+__device__ __forceinline__ void event_step(EventCursor &c, int u, int cnt)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, q;\n\t"
+        "setp.gt.s32 p, %3, %4;\n\t"
+        "@p red.shared.add.u32 [%0], 1;\n\t"
+        "@p add.u32 %1, %1, %5;\n\t"
+        "setp.ge.and.u32 q, %1, %2, p;\n\t"
+        "@p add.s32 %0, %0, %6;\n\t"
+        "@q sub.u32 %1, %1, %2;\n\t"
+        "@q add.s32 %0, %0, 4;\n\t"
+        "}"
+        : "+r"(c.addr), "+r"(c.rem)
+        : "r"(c.ad), "r"(cnt), "r"(u), "r"(c.Ru), "r"(c.step)
+        : "memory");
+}
+
+// One block's part of a bucket.  Pairs lie in the order of their histories (by
+// gantry angle), so the lengths of their walks drift along a bucket; slots
+// take them in pieces of 32 (a warp's walks stay alike) from kCols places of
+// the bucket in turn, so that a range of slots samples all of it and ranges
+// of equal size cost about the same: slot p is pair
+// 32 ((v % kCols) rows + v / kCols) + p % 32, v = p / 32 (none when that is
+// past the bucket's count).
+//
+// Parts are walked in groups: as many consecutive ones as have room for their
+// tiles side by side in shared memory are walked together and then flushed, so
+// that the block waits for its last walks once per group (about 14 000 cycles,
+// as long as the walks of 1 300 pairs) and not once per part.
+constexpr int kCols = 16;
+struct TilePart {
+    const uint4 *first_pair;  // the bucket's first pair
+    int scan;
+    int tile;    // tile id within its group
+    int group;   // bit 0 the class (missed: N, hit: M), bits 1-2 the walk type
+    int count;   // the bucket's pairs
+    int start;   // slots [start, end)
+    int end;
+    int words;   // of its tile
+    int offset;  // of the tile in the block's shared memory, in words
+    int slot0;   // slots of the group before this part's
+};
+
+__device__ __forceinline__ int slot_rows(int count) { return (count + 32 * kCols - 1) / (32 * kCols); }
+
+// A lane's next walk, loaded ahead.
+struct NextWalk {
+    uint4 a, b;
+    int base;  // its tile's offset in bytes
+    bool have;
+};
+
+// The walk in slot r of the group of `n` parts: none past the pairs of a part.
+__device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, NextWalk &nw)
+{
+    int j = 0;
+    while (j + 1 < n && r >= parts[j + 1].slot0) ++j;
+    const TilePart &t = parts[j];
+    const int p = t.start + r - t.slot0;
+    const int v = p >> 5;
+    const int k = 32 * ((v & (kCols - 1)) * slot_rows(t.count) + v / kCols) + (p & 31);
+    nw.base = 4 * t.offset;
+    if (k < t.count) {
+        nw.a = __ldg(t.first_pair + 2 * static_cast<size_t>(k));
+        nw.b = __ldg(t.first_pair + 2 * static_cast<size_t>(k) + 1);
+    } else {
+        nw.b.w = 0x80000000u;
+    }
+}
+
+// The first walks of a group of `total` slots, a lane its own slot.  Loaded
+// before the flush that precedes them, which hides their latency.
+__device__ __forceinline__ void first_walks(const TilePart *parts, int n, int total, NextWalk &nw)
+{
+    nw.have = static_cast<int>(threadIdx.x) < total;
+    if (nw.have) load_slot(parts, n, static_cast<int>(threadIdx.x), nw);
+}
+
+// Walks the `total` slots of a group of parts into the block's tiles: each
+// lane walks one pair and holds the packed walk of its next one (loaded a
+// refill ahead, so starting a walk never waits on memory).  A refill happens
+// once enough lanes are idle: they mark the ends of their finished walks, and
+// those with a prefetched pair start it and fetch another, the slot coming
+// from the block's counter *s_next (blockDim.x at the start: the first walks
+// are the lanes' own, see first_walks).  Between refills the warp only counts
+// events.  Out of line, so that nothing else in the kernel takes its registers.
+__device__ __noinline__ void walk_parts(uint32_t *tiles, int thick, const TilePart *parts, int n,
+                                        int total, int refill, unsigned *s_next, NextWalk nw)
 {
     const unsigned lane = threadIdx.x & 31u;
-    const int sbase = static_cast<int>(__cvta_generic_to_shared(tile));
-    TileCursor c;
-    bool active = false;
-    uint4 na = make_uint4(0, 0, 0, 0), nb = na;
-    int nidx = -1;
-    {
-        unsigned base = 0;
-        if (lane == 0) base = atomicAdd(s_next, 32u);
-        base = __shfl_sync(kFull, base, 0);
-        const unsigned r = base + lane;
-        if (r < static_cast<unsigned>(total)) {
-            nidx = start + static_cast<int>(r);
-            load_lean(pairs, nidx, na, nb);
-        }
-    }
+    const int sbase = static_cast<int>(__cvta_generic_to_shared(tiles));
+    const int thick4 = 4 * (thick + 1);
+    EventCursor c;
+    c.ad = c.Ru = c.rem = 0u;
+    c.addr = c.step = c.left = c.endl = 0;
+    bool unmarked = false;  // the walk's end is still to be marked
     for (;;) {
-        const unsigned want = __ballot_sync(kFull, !active && nidx >= 0);
-        const unsigned busy = __ballot_sync(kFull, active);
-        if ((want | busy) == 0) break;
-        if (want != 0 && (__popc(want) >= static_cast<unsigned>(refill) || busy == 0)) {
-            if (!active && nidx >= 0) {
-                const uint32_t o[kLeanWords] = {na.x, na.y, na.z, na.w, nb.x, nb.y, nb.z, nb.w};
-                active = tile_cursor_start(o, dx, dy, dz, sbase, c);
-                // runs of a walk = its minor-0 crossings left at the start
-                // minus those left after its last run (see tile_cursor_run)
-                if (active) runs += static_cast<unsigned>(c.kleft);
-                nidx = -1;
-            }
-            unsigned base = 0;
-            const unsigned nw = __popc(want);
-            if (lane == 0) base = atomicAdd(s_next, nw);
-            base = __shfl_sync(kFull, base, 0);
-            if (want & (1u << lane)) {
-                const unsigned r = base + __popc(want & ((1u << lane) - 1u));
-                if (r < static_cast<unsigned>(total)) {
-                    nidx = start + static_cast<int>(r);
-                    load_lean(pairs, nidx, na, nb);
+        const unsigned idle = __ballot_sync(kFull, c.left == 0);
+        if (__popc(idle) >= refill) {
+            const unsigned want = __ballot_sync(kFull, c.left == 0 && nw.have);
+            if (c.left == 0) {
+                if (unmarked) smem_red_add(event_end(c, thick4), 0xffff0000u);
+                unmarked = false;
+                if (nw.have) {
+                    const uint32_t o[kLeanWords] = {nw.a.x, nw.a.y, nw.a.z, nw.a.w,
+                                                    nw.b.x, nw.b.y, nw.b.z, nw.b.w};
+                    int first;
+                    unmarked = event_start(o, sbase + nw.base, c, first);
+                    if (unmarked) smem_red_add(first, 65536u);
+                    nw.have = false;
                 }
             }
-            continue;
-        }
-        // up to kRunsPerStep runs before the warp checks for refills again.
-        // A lane whose walk ends leaves the loop (predicating it instead was
-        // 25 % slower), and an unroll by 2 measured best (full unrolling,
-        // none, 6, 12 or 16 runs: 5-27 % slower on the head-200 scan).
-        if (active) {
-#pragma unroll 2
-            for (int u = 0; u < kRunsPerStep; ++u) {
-                int at_prev, at_cur;
-                active = tile_cursor_run(c, at_prev, at_cur);
-                smem_red_add(at_prev, c.vprev);
-                smem_red_add(at_cur, c.vcur);
-                if (!active) {
-                    runs -= static_cast<unsigned>(c.kleft);
-                    break;
+            if (want != 0) {
+                unsigned base = 0;
+                if (lane == 0) base = atomicAdd(s_next, __popc(want));
+                base = __shfl_sync(kFull, base, 0);
+                if (want & (1u << lane)) {
+                    const unsigned r = base + __popc(want & ((1u << lane) - 1u));
+                    nw.have = r < static_cast<unsigned>(total);
+                    if (nw.have) load_slot(parts, n, static_cast<int>(r), nw);
                 }
+            } else if (idle == kFull) {
+                break;
             }
         }
+        const int cnt = min(c.left, kEventsPerStep);
+#pragma unroll
+        for (int u = 0; u < kEventsPerStep; ++u) event_step(c, u, cnt);
+        c.left -= cnt;
     }
 }
 
-// Flush of a job's tile into vol (the scan's N or M) and zeroing of the
-// tile for the next job: (1) warps take rows, decode each word into two
-// plain int16 halves and prefix-sum the low halves along x; (2) warps take
-// columns and prefix-sum the high halves along y; (3) every voxel adds the
-// sum of its two halves to vol (one global atomic per nonzero voxel) and
-// every word, padding included, is cleared.
-__device__ __forceinline__ void flush_tile(uint32_t *tile, int dx, int dy, int dz, uint32_t *vol,
-                                           int nx, int ny, int x0, int y0, int z0)
+// A warp's inclusive prefix sums of a row of W <= 32 kPer words: word
+// lane kPer + i in v[i] (kPer odd: the lanes read from 32 banks).  `after`:
+// the tile's words from the row's start on.  When there are 32 kPer of them,
+// those past the row's end are read too: they come after the row's and are
+// dropped.
+template <int kPer>
+__device__ __forceinline__ void row_prefix(const uint32_t *row, int W, int after,
+                                           uint32_t (&v)[kPer])
 {
-    const unsigned lane = threadIdx.x & 31u;
-    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    const int Wx = dx + 1, Hy = dy + 1;
-    // (1) rows along x: decode, then inclusive prefix of the low halves
-    {
-        const int chunk = (dx + 31) >> 5;
-        for (int r = warp; r < dy * dz; r += nwarps) {
-            const int y = r % dy, z = r / dy;
-            uint32_t *row = tile + Wx * (y + Hy * z);
-            const int b = lane * chunk;
-            const int e = min(b + chunk, dx);
-            int acc = 0;
-            for (int i = b; i < e; ++i) acc += static_cast<int16_t>(row[i] & 0xffffu);
-            int incl = acc;
+    const int lane = static_cast<int>(threadIdx.x & 31u);
+    const int b = lane * kPer;
+    if (after >= 32 * kPer) {
 #pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(kFull, incl, o);
-                if (lane >= static_cast<unsigned>(o)) incl += t;
-            }
-            int run = incl - acc;
-            for (int i = b; i < e; ++i) {
-                const uint32_t w = row[i];
-                const int lo = static_cast<int16_t>(w & 0xffffu);
-                const int hi = static_cast<int>(w - static_cast<uint32_t>(lo)) >> 16;
-                run += lo;
-                row[i] = (static_cast<uint32_t>(run) & 0xffffu) | (static_cast<uint32_t>(hi) << 16);
+        for (int i = 0; i < kPer; ++i) v[i] = row[b + i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) v[i] = b + i < W ? row[b + i] : 0u;
+    }
+#pragma unroll
+    for (int i = 1; i < kPer; ++i) v[i] += v[i - 1];
+    uint32_t incl = v[kPer - 1];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= o) incl += t;
+    }
+    const uint32_t before = incl - v[kPer - 1];
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) v[i] += before;
+}
+
+// Adds a count to a voxel unless it is zero (predicated: no branch).
+__device__ __forceinline__ void add_count(uint32_t *v, uint32_t c)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.u32 p, %1, 0;\n\t"
+        "@p red.global.add.u32 [%0], %1;\n\t"
+        "}" ::"l"(v),
+        "r"(c)
+        : "memory");
+}
+
+// Where a tile's counts go: the volume's voxel (0, 0, 0) of the tile, and its
+// grid's extents.
+struct FlushTo {
+    uint32_t *vol;
+    int nx, ny;
+    __device__ __forceinline__ uint32_t *line(int y, int z) const
+    {
+        return vol + static_cast<long long>(nx) * (y + static_cast<long long>(ny) * z);
+    }
+};
+
+// Flush of thin walks whose rows fit 32 kPer words.  A warp takes a band of
+// rows in walk order and keeps each row's prefix sums in registers for the
+// next one, so a word is read once for its count (modulo 2^16, where counts
+// lie, SP + SE' - SE is one three-operand sum of the words), written back as a
+// count, and read, cleared and added to the volume by lanes along x: about 100
+// instructions per 200-voxel row, where separate prefix, decode and clear
+// passes took 240 (issue-bound: 21 000 to 9 000 cycles per 200 x 200 tile).
+template <int kPer>
+__device__ __noinline__ void flush_rows(uint32_t *tile, int dx, int dy, int dz, bool ymaj, int s,
+                                        int W, FlushTo to)
+{
+    const int lane = static_cast<int>(threadIdx.x & 31u);
+    const int warp = static_cast<int>(threadIdx.x >> 5), nwarps = static_cast<int>(blockDim.x >> 5);
+    const int nmaj = ymaj ? dy : dx, nminor = ymaj ? dx : dy;
+    const int rows = nminor * dz;
+    const int band = (rows + nwarps - 1) / nwarps;
+    const int a = min(warp * band, rows), e = min(a + band, rows);
+    const int i0 = s > 0 ? 0 : nminor - 1;  // a slice's first row in walk order
+    int r = s > 0 ? a : e - 1;
+    int z = dz == 1 ? 0 : r / nminor, i = r - z * nminor;
+    uint32_t pv[kPer];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) pv[k] = 0u;
+    // the row before the band belongs to another warp, which overwrites it
+    if (a < e && i != i0) row_prefix<kPer>(tile + W * (r - s), W, W * (rows - (r - s)), pv);
+    __syncthreads();
+    for (int n = a; n < e; ++n, r += s) {
+        uint32_t *row = tile + W * r;
+        if (i == i0) {
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) pv[k] = 0u;
+        }
+        uint32_t v[kPer];
+        // what follows the row may be rewritten meanwhile: harmless, it is dropped
+        row_prefix<kPer>(row, W, W * (rows - r), v);
+        uint32_t left = __shfl_up_sync(kFull, v[kPer - 1], 1);
+        if (lane == 0) left = 0u;
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            const int m = lane * kPer + k;
+            const uint32_t c = ((v[k] >> 16) + pv[k] - left) & 0xffffu;
+            left = v[k];
+            pv[k] = v[k];
+            if (m < W) row[m] = m < nmaj ? c : 0u;
+        }
+        if (!ymaj) {
+            __syncwarp();
+            uint32_t *out = to.line(i, z) + lane;
+            uint32_t c[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) c[k] = lane + 32 * k < dx ? row[lane + 32 * k] : 0u;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                if (lane + 32 * k < dx) row[lane + 32 * k] = 0u;
+                add_count(out + 32 * k, c[k]);
             }
         }
-        // (the padding column and row are never read: step 3 clears them)
-    }
-    __syncthreads();
-    // (2) columns along y: inclusive prefix of the (decoded) high halves
-    {
-        const int chunk = (dy + 31) >> 5;
-        for (int col = warp; col < dx * dz; col += nwarps) {
-            const int x = col % dx, z = col / dx;
-            uint32_t *base = tile + x + Wx * Hy * z;
-            const int b = lane * chunk;
-            const int e = min(b + chunk, dy);
-            int acc = 0;
-            for (int i = b; i < e; ++i) acc += static_cast<int>(base[Wx * i]) >> 16;
-            int incl = acc;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int t = __shfl_up_sync(kFull, incl, o);
-                if (lane >= static_cast<unsigned>(o)) incl += t;
-            }
-            int run = incl - acc;
-            for (int i = b; i < e; ++i) {
-                const uint32_t w = base[Wx * i];
-                run += static_cast<int>(w) >> 16;
-                base[Wx * i] = (w & 0xffffu) | (static_cast<uint32_t>(run) << 16);
-            }
+        // the next row in walk order
+        i += s;
+        if (i < 0) {
+            i = nminor - 1;
+            --z;
+        } else if (i == nminor) {
+            i = 0;
+            ++z;
         }
     }
-    __syncthreads();
-    // (3) add to the volume and clear every word of the box, a warp per row
-    // of words (padding row included), its lanes along x
-    for (int r = warp; r < Hy * dz; r += nwarps) {
-        const int y = r % Hy, z = r / Hy;
-        uint32_t *row = tile + Wx * r;
-        const bool real = y < dy;
-        const long long g0 =
-            x0 + static_cast<long long>(nx) * ((y0 + y) + static_cast<long long>(ny) * (z0 + z));
-        for (int x = static_cast<int>(lane); x < Wx; x += 32) {
-            const uint32_t w = row[x];
-            row[x] = 0u;
-            if (real && x < dx) {
-                const int v = static_cast<int>(w & 0xffffu) + static_cast<int>(w >> 16);
-                if (v) atomicAdd(&vol[g0 + x], static_cast<uint32_t>(v));
+    if (ymaj) {
+        __syncthreads();
+        for (int l = warp; l < dy * dz; l += nwarps) {
+            const int zz = dz == 1 ? 0 : l / dy, y = l - zz * dy;
+            uint32_t *out = to.line(y, zz) + lane;
+            uint32_t *line = tile + y + W * nminor * zz + W * lane;
+            for (int x = lane; x - lane < dx; x += 128, out += 128, line += 128 * W) {
+                uint32_t c[4];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) c[k] = x + 32 * k < dx ? line[32 * k * W] : 0u;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    if (x + 32 * k < dx) line[32 * k * W] = 0u;
+                    add_count(out + 32 * k, c[k]);
+                }
             }
         }
     }
 }
 
-// No job left: the pairs without a lean form (the fallback lists), walked
-// with the general run walk in global memory, 32 entries per warp claim, so
-// blocks that finish their last job early take them.  Out of line, so its
-// registers do not weigh on the lean walk loop.
+// In-place inclusive prefix sum of a row of any length by a warp.
+__device__ __forceinline__ void prefix_row(uint32_t *row, int W)
+{
+    const int lane = static_cast<int>(threadIdx.x & 31u);
+    uint32_t carry = 0;
+    for (int w0 = 0; w0 < W; w0 += 32) {
+        uint32_t v = w0 + lane < W ? row[w0 + lane] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t t = __shfl_up_sync(kFull, v, o);
+            if (lane >= o) v += t;
+        }
+        v += carry;
+        if (w0 + lane < W) row[w0 + lane] = v;
+        carry = __shfl_sync(kFull, v, 31);
+    }
+}
+
+// The count of voxel m of a dilated row from the prefix-summed tile (see the
+// event walks in hd_geom.cuh); i is the row's minor index, s the walks' row
+// direction, `row` its first word.
+__device__ __forceinline__ int thick_count(const uint32_t *row, int W, int m, int nmaj, int i,
+                                           int nminor, int s, int thick)
+{
+    int v = 0;
+    const int j0 = max(-thick, -i), j1 = min(thick, nminor - 1 - i);
+    for (int j = j0; j <= j1; ++j) v += static_cast<int>(row[m + j * W]) >> 16;
+    const int ia = i - (thick + 1) * s, ib = i + thick * s;
+    if (ia >= 0 && ia < nminor)
+        v += static_cast<int>(row[min(m + thick, nmaj) - (thick + 1) * s * W] & 0xffffu);
+    if (ib >= 0 && ib < nminor && m - thick > 0)
+        v -= static_cast<int>(row[m - thick - 1 + thick * s * W] & 0xffffu);
+    return v;
+}
+
+// Flush of dilated walks, and of rows longer than flush_rows takes: prefix
+// sums in place, each voxel's count from its neighbours' words, then clearing.
+__device__ __noinline__ void flush_general(uint32_t *tile, int dx, int dy, int dz, bool ymaj, int s,
+                                           int W, int thick, FlushTo to)
+{
+    const int lane = static_cast<int>(threadIdx.x & 31u);
+    const int warp = static_cast<int>(threadIdx.x >> 5), nwarps = static_cast<int>(blockDim.x >> 5);
+    const int nmaj = ymaj ? dy : dx, nminor = ymaj ? dx : dy;
+    for (int r = warp; r < nminor * dz; r += nwarps) prefix_row(tile + W * r, W);
+    __syncthreads();
+    // a warp per line of voxels along x; mx, my: words from a voxel to the next
+    const int mx = ymaj ? W : 1, my = ymaj ? 1 : W;
+    for (int l = warp; l < dy * dz; l += nwarps) {
+        const int z = dz == 1 ? 0 : l / dy, y = l - z * dy;
+        uint32_t *out = to.line(y, z);
+        const uint32_t *line = tile + my * y + W * nminor * z;
+        for (int x = lane; x < dx; x += 32) {
+            const int i = ymaj ? x : y, m = ymaj ? y : x;
+            add_count(out + x, static_cast<uint32_t>(thick_count(line + mx * x - m, W, m, nmaj, i,
+                                                                 nminor, s, thick)));
+        }
+    }
+    __syncthreads();
+    // the tile starts on a 16-byte boundary and is planned in whole vectors
+    uint4 *t4 = reinterpret_cast<uint4 *>(tile);
+    for (int w = static_cast<int>(threadIdx.x); w < (W * nminor * dz + 3) >> 2; w += blockDim.x)
+        t4[w] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// Adds the tile's counts to the volume (one global atomic per nonzero voxel,
+// lanes along x whichever axis the rows follow) and clears it for the next job.
+__device__ __forceinline__ void flush_tile(uint32_t *tile, int dx, int dy, int dz, int type,
+                                           int thick, uint32_t *vol, int nx, int ny, int x0,
+                                           int y0, int z0)
+{
+    const bool ymaj = (type & 2) != 0;
+    const int s = (type & 1) ? -1 : 1;
+    const int nmaj = ymaj ? dy : dx, nminor = ymaj ? dx : dy;
+    const int W = tile_row_words(nmaj, nminor);
+    const FlushTo to{vol + x0 + static_cast<long long>(nx) * (y0 + static_cast<long long>(ny) * z0),
+                     nx, ny};
+    if (thick > 0 || W > 32 * 13) flush_general(tile, dx, dy, dz, ymaj, s, W, thick, to);
+    else if (W <= 32 * 3) flush_rows<3>(tile, dx, dy, dz, ymaj, s, W, to);
+    else if (W <= 32 * 5) flush_rows<5>(tile, dx, dy, dz, ymaj, s, W, to);
+    else if (W <= 32 * 7) flush_rows<7>(tile, dx, dy, dz, ymaj, s, W, to);
+    else if (W <= 32 * 9) flush_rows<9>(tile, dx, dy, dz, ymaj, s, W, to);
+    else flush_rows<13>(tile, dx, dy, dz, ymaj, s, W, to);
+}
+
+// The pairs without an event walk (the fallback lists), walked with the general
+// run walk in global memory, a warp per pair, by the blocks as they run out of
+// parts.  Out of line, so its registers do not weigh on the event loop.
 __device__ __noinline__ void walk_fallback_lists(const ScanDesc *__restrict__ descs, int nscans)
 {
-    const unsigned lane = threadIdx.x & 31u;
     for (int k = 0; k < nscans; ++k) {
         const ScanDesc &d = descs[k];
+        if (d.tp.thick > 0) continue;  // dilated by a kernel of their own
         const unsigned nf = d.ctrl->n_pair_fallback;
         if (nf == 0) continue;
-        uint32_t *const N = d.N;
-        uint32_t *const M = d.M;
         for (;;) {
-            unsigned base = 0;
-            if (lane == 0) base = atomicAdd(&d.ctrl->fb_next, 32u);
-            base = __shfl_sync(kFull, base, 0);
-            if (base >= nf) break;
-            const unsigned i = base + lane;
-            if (i < nf) {
-                const uint32_t pos = d.pairs.fb[i].x;
-                uint4 a, b;
-                load_lean(d.pairs, static_cast<int>(pos), a, b);
-                const int32_t gi[3] = {static_cast<int32_t>(a.x), static_cast<int32_t>(a.y),
-                                       static_cast<int32_t>(a.z)};
-                const int32_t go[3] = {static_cast<int32_t>(a.w), static_cast<int32_t>(b.x),
-                                       static_cast<int32_t>(b.z)};
-                GlobalVisit v;
-                v.vol = (b.w & 1u) == 0 ? N : M;
-                walk_tile_global(d.tp, gi, go, static_cast<int>(b.w >> 1), v);
-            }
+            unsigned i = 0;
+            if ((threadIdx.x & 31u) == 0) i = atomicAdd(&d.ctrl->fb_next, 1u);
+            i = __shfl_sync(kFull, i, 0);
+            if (i >= nf) break;
+            int32_t gi[3], go[3];
+            const uint32_t id = load_general(d.pairs, d.pairs.fb[i].x, gi, go);
+            GlobalVisit v;
+            v.vol = (id & 1u) == 0 ? d.N : d.M;
+            walk_tile_global(d.tp, gi, go, static_cast<int>(id >> 1), v);
+            __syncwarp();
         }
     }
+}
+
+// Cost of a bucket in event units: its events, kPairCost per walk (its start,
+// marks and loads), and for its flush kFlushCost per word of the tile and
+// kPartCost besides (fits over the parts of the head-sized and the large
+// streamed scan).
+constexpr unsigned kPairCost = 9, kFlushCost = 4, kPartCost = 10000;
+constexpr int kPartList = 32;  // parts a block lists at a time
+
+__device__ __forceinline__ unsigned long long flush_cost(int tile_words)
+{
+    return kPartCost + static_cast<unsigned long long>(kFlushCost) * static_cast<unsigned>(tile_words);
+}
+
+struct BucketCost {
+    unsigned long long cost;  // 0: no pairs
+    unsigned count;
+};
+
+__device__ __forceinline__ BucketCost bucket_cost(const ScanDesc &d, int t)
+{
+    BucketCost b;
+    b.count = d.buckets.count[t];
+    b.cost = b.count == 0 ? 0ull
+                          : d.buckets.events[t] +
+                                static_cast<unsigned long long>(kPairCost) * b.count +
+                                flush_cost(d.tp.tile_words);
+    return b;
+}
+
+// Where the boundary at cost x of the launch falls in a bucket whose cost
+// begins at p: pieces of 32 slots before it (0 .. all).  A part worth less
+// than its own flush goes to the neighbour.
+__device__ __forceinline__ int boundary_slot(const BucketCost &b, int tile_words,
+                                             unsigned long long p, unsigned long long x)
+{
+    const int pieces = kCols * slot_rows(static_cast<int>(b.count));
+    const unsigned long long f = flush_cost(tile_words);
+    if (x <= p + f) return 0;
+    if (x + f >= p + b.cost) return 32 * pieces;
+    return 32 * static_cast<int>((x - p) * static_cast<unsigned long long>(pieces) / b.cost);
+}
+
+// Exclusive block scan of one 64-bit value per thread (blockDim.x <= 1024).
+__device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long long v,
+                                                                unsigned long long *s_warp,
+                                                                unsigned long long &total)
+{
+    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    unsigned long long incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(kFull, incl, o);
+        if (lane >= static_cast<unsigned>(o)) incl += t;
+    }
+    __syncthreads();  // the last use of s_warp is over
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
+    // every warp scans the warps' sums for itself
+    unsigned long long w = lane < nw ? s_warp[lane] : 0ull;
+    const unsigned long long own = w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long t = __shfl_up_sync(kFull, w, o);
+        if (lane >= static_cast<unsigned>(o)) w += t;
+    }
+    total = __shfl_sync(kFull, w, 31);
+    return __shfl_sync(kFull, w - own, wid) + incl - v;
 }
 
 }  // namespace
 
-// Persistent traversal: blocks take jobs (one tile's range of pairs) from
-// the job counter until none is left, walk them into their shared-memory
-// tile and flush it; then they walk the fallback lists.  max_words is the
-// largest tile of the scans (the dynamic shared memory of the launch).
+// The traversal: the buckets of all scans laid end to end by cost, one equal
+// stretch per block (static: the costs are counted, not estimated, so the
+// blocks end within a few per cent of each other, and a bucket is flushed once
+// per block that has a part of it; a queue of four jobs per SM flushed twice
+// as often and left the SMs 10 % apart).  Each part is walked into the block's
+// shared-memory tile and flushed; then the blocks walk the fallback lists.
+// smem_words: the dynamic shared memory of the launch, at least the
+// largest tile of the scans.
 template <int kThreads>
 __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
-    const ScanDesc *__restrict__ descs, int nscans, int *job_counter, int max_words)
+    const ScanDesc *__restrict__ descs, int nscans, int smem_words)
 {
-    extern __shared__ uint32_t tile[];
-    __shared__ int s_job, s_scan;
+    extern __shared__ __align__(16) uint32_t tile[];
     __shared__ unsigned s_next;
-    __shared__ int s_prefix[kMaxBatch + 1];
-    const unsigned lane = threadIdx.x & 31u;
-    // jobs of scan k are the global job numbers [s_prefix[k], s_prefix[k+1])
+    __shared__ int s_first[kMaxBatch + 1];
+    __shared__ TilePart s_parts[kPartList];
+    __shared__ int s_group[kPartList + 1];  // first part of each group
+    __shared__ int s_slots[kPartList];      // slots of each group
+    __shared__ int s_ngroups;
+    __shared__ unsigned long long s_warp[32];
+    // buckets of scan k are the launch's buckets [s_first[k], s_first[k + 1])
     if (threadIdx.x == 0) {
         int acc = 0;
         for (int k = 0; k < nscans; ++k) {
-            s_prefix[k] = acc;
-            acc += descs[k].ctrl->njobs;
+            s_first[k] = acc;
+            acc += kGroups * descs[k].tp.ntiles;
         }
-        s_prefix[nscans] = acc;
+        s_first[nscans] = acc;
     }
     // each flush clears its box: the tile starts cleared once
-    for (int w = threadIdx.x; w < max_words; w += blockDim.x) tile[w] = 0u;
+    for (int w = threadIdx.x; w < smem_words >> 2; w += blockDim.x)
+        reinterpret_cast<uint4 *>(tile)[w] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    const int total_jobs = s_prefix[nscans];
-    for (;;) {
-        if (threadIdx.x == 0) {
-            const int J = atomicAdd(job_counter, 1);
-            int k = 0;
-            while (k + 1 < nscans && s_prefix[k + 1] <= J) ++k;
-            s_job = J;
-            s_scan = k;
-            s_next = 0;
+    const int nb = s_first[nscans];
+    const int per = (nb + kThreads - 1) / kThreads;
+    const int i0 = min(static_cast<int>(threadIdx.x) * per, nb), i1 = min(i0 + per, nb);
+    // the thread's buckets i0 .. i1 - 1: visit(scan, bucket within it)
+    auto each = [&](auto visit) {
+        int k = 0;
+        for (int i = i0; i < i1; ++i) {
+            while (i >= s_first[k + 1]) ++k;
+            visit(k, i - s_first[k]);
+        }
+    };
+    unsigned long long mine = 0, total;
+    each([&](int k, int t) { mine += bucket_cost(descs[k], t).cost; });
+    const unsigned long long before = block_excl_scan64(mine, s_warp, total);
+    // the block's stretch: an equal share, but worth about two flushes
+    unsigned long long blocks = total / (2ull * flush_cost(descs[0].tp.tile_words)) + 1ull;
+    if (blocks > gridDim.x) blocks = gridDim.x;
+    const unsigned long long share = (total + blocks - 1ull) / blocks;
+    const unsigned long long x0 = share * blockIdx.x, x1 = x0 + share;
+    // the parts of the thread's buckets in that stretch, each at most
+    // job_size pairs (in whole pieces): count, then list
+    auto parts = [&](auto take) {
+        unsigned long long p = before;
+        each([&](int k, int t) {
+            const ScanDesc &d = descs[k];
+            const BucketCost b = bucket_cost(d, t);
+            if (b.cost != 0 && p < x1 && p + b.cost > x0) {
+                const int s0 = x0 > p ? boundary_slot(b, d.tp.tile_words, p, x0) : 0;
+                const int s1 = x1 < p + b.cost ? boundary_slot(b, d.tp.tile_words, p, x1)
+                                               : 32 * kCols * slot_rows(static_cast<int>(b.count));
+                const int most = d.tp.job_size & ~31;
+                for (int s = s0; s < s1; s += most)
+                    take(k, t, static_cast<int>(b.count), s, min(s + most, s1));
+            }
+            p += b.cost;
+        });
+    };
+    unsigned long long nmine = 0, nparts;
+    parts([&](int, int, int, int, int) { ++nmine; });
+    const unsigned long long rank0 = block_excl_scan64(nmine, s_warp, nparts);
+    for (unsigned long long j0 = 0; j0 < nparts; j0 += kPartList) {
+        if (nmine != 0) {
+            unsigned long long r = rank0;
+            parts([&](int k, int t, int count, int s0, int s1) {
+                if (r >= j0 && r < j0 + kPartList) {
+                    TilePart &j = s_parts[r - j0];
+                    const ScanDesc &d = descs[k];
+                    j.first_pair = d.pairs.v + 2 * static_cast<size_t>(d.buckets.first[t]);
+                    j.scan = k;
+                    j.tile = t % d.tp.ntiles;
+                    j.group = t / d.tp.ntiles;
+                    j.count = count;
+                    j.start = s0;
+                    j.end = s1;
+                    j.words = d.tp.tile_words;
+                }
+                ++r;
+            });
         }
         __syncthreads();
-        if (s_job >= total_jobs) break;
-        const ScanDesc &d = descs[s_scan];
-        const TilePlan tp = d.tp;
-        const TileJob job = d.jobs[s_job - s_prefix[s_scan]];
-        const int tix = job.tile % tp.ntx;
-        const int tiy = (job.tile / tp.ntx) % tp.nty;
-        const int tiz = job.tile / (tp.ntx * tp.nty);
-        const int x0 = tix * tp.tx, y0 = tiy * tp.ty, z0 = tiz * tp.tz;
-        const int dx = min(tp.tx, tp.nx - x0), dy = min(tp.ty, tp.ny - y0),
-                  dz = min(tp.tz, tp.nz - z0);
-        unsigned runs = 0;
-        walk_job(tile, dx, dy, dz, d.pairs, job.start,
-                 job.end - job.start, tp.refill, &s_next, runs);
+        if (threadIdx.x == 0) {
+            const int here = static_cast<int>(nparts - j0 < kPartList ? nparts - j0 : kPartList);
+            int g = 0, words = 0, slots = 0;
+            s_group[0] = 0;
+            for (int q = 0; q < here; ++q) {
+                TilePart &j = s_parts[q];
+                if (q > s_group[g] && words + j.words > smem_words) {
+                    s_slots[g] = slots;
+                    s_group[++g] = q;
+                    words = slots = 0;
+                }
+                j.offset = words;
+                j.slot0 = slots;
+                words += j.words;
+                slots += j.end - j.start;
+            }
+            s_slots[g] = slots;
+            s_group[++g] = here;
+            s_ngroups = g;
+        }
         __syncthreads();
-        flush_tile(tile, dx, dy, dz, job.cls == 0 ? d.N : d.M, tp.nx, tp.ny, x0, y0, z0);
-        // runs walked by this job, added to its scan's counter
-        unsigned long long ru = runs;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) ru += __shfl_xor_sync(kFull, ru, o);
-        if (lane == 0 && ru) atomicAdd(&d.ctrl->runs, ru);
+        const int ngroups = s_ngroups;
+        NextWalk nw;
+        nw.a = nw.b = make_uint4(0, 0, 0, 0);
+        nw.base = 0;
+        first_walks(s_parts, s_group[1], s_slots[0], nw);
+        for (int g = 0; g < ngroups; ++g) {
+            const int q0 = s_group[g], q1 = s_group[g + 1];
+            if (threadIdx.x == 0) s_next = blockDim.x;
+            __syncthreads();
+            const TilePlan &tp0 = descs[s_parts[q0].scan].tp;
+            walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, &s_next, nw);
+            if (g + 1 < ngroups)
+                first_walks(s_parts + q1, s_group[g + 2] - q1, s_slots[g + 1], nw);
+            __syncthreads();
+            for (int q = q0; q < q1; ++q) {
+                const TilePart &j = s_parts[q];
+                const ScanDesc &d = descs[j.scan];
+                const TilePlan &tp = d.tp;
+                const int tix = j.tile % tp.ntx;
+                const int tiy = (j.tile / tp.ntx) % tp.nty;
+                const int tiz = j.tile / (tp.ntx * tp.nty);
+                const int bx = tix * tp.tx, by = tiy * tp.ty, bz = tiz * tp.tz;
+                flush_tile(tile + j.offset, min(tp.tx, tp.nx - bx), min(tp.ty, tp.ny - by),
+                           min(tp.tz, tp.nz - bz), j.group >> 1, tp.thick,
+                           (j.group & 1) == 0 ? d.N : d.M, tp.nx, tp.ny, bx, by, bz);
+            }
+        }
         __syncthreads();
     }
     walk_fallback_lists(descs, nscans);
+}
+
+// Shared memory of a launch whose largest tile has this many words: room for
+// up to eight tiles.
+static int trace_smem_words(int tile_words)
+{
+    const int n = kTileSmemBytes / 4 / tile_words;
+    return tile_words * (n < 1 ? 1 : (n > 8 ? 8 : n));
 }
 
 template <int kThreads>
@@ -318,8 +668,9 @@ int occupancy_of(int smem_words)
     return nb;
 }
 
-int trace_tiles_occupancy(int smem_words, int threads)
+int trace_tiles_occupancy(int tile_words, int threads)
 {
+    const int smem_words = trace_smem_words(tile_words);
     switch (threads) {
     case 256: return occupancy_of<256>(smem_words);
     case 512: return occupancy_of<512>(smem_words);
@@ -329,24 +680,25 @@ int trace_tiles_occupancy(int smem_words, int threads)
     }
 }
 
-cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int *job_counter,
-                               int smem_words, int threads, int grid, cudaStream_t s)
+cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
+                               int grid, cudaStream_t s)
 {
-    if (nscans < 1 || nscans > kMaxBatch || smem_words * 4 > kTileSmemBytes)
+    if (nscans < 1 || nscans > kMaxBatch || tile_words * 4 > kTileSmemBytes)
         return cudaErrorInvalidValue;
+    const int smem_words = trace_smem_words(tile_words);
     const size_t smem = static_cast<size_t>(smem_words) * 4;
     switch (threads) {
     case 256:
-        trace_tiles_kernel<256><<<grid, 256, smem, s>>>(descs, nscans, job_counter, smem_words);
+        trace_tiles_kernel<256><<<grid, 256, smem, s>>>(descs, nscans, smem_words);
         break;
     case 512:
-        trace_tiles_kernel<512><<<grid, 512, smem, s>>>(descs, nscans, job_counter, smem_words);
+        trace_tiles_kernel<512><<<grid, 512, smem, s>>>(descs, nscans, smem_words);
         break;
     case 768:
-        trace_tiles_kernel<768><<<grid, 768, smem, s>>>(descs, nscans, job_counter, smem_words);
+        trace_tiles_kernel<768><<<grid, 768, smem, s>>>(descs, nscans, smem_words);
         break;
     case 1024:
-        trace_tiles_kernel<1024><<<grid, 1024, smem, s>>>(descs, nscans, job_counter, smem_words);
+        trace_tiles_kernel<1024><<<grid, 1024, smem, s>>>(descs, nscans, smem_words);
         break;
     default: return cudaErrorInvalidValue;
     }

@@ -115,8 +115,9 @@ __device__ __forceinline__ void admit_and_write(const TilePlan &tp, const Record
                                                 Ctrl *ctrl, uint32_t *s_hist, unsigned *s_demand,
                                                 unsigned budget, int64_t h0, int64_t i,
                                                 int64_t i1, uint32_t *stage, int cls,
-                                                const int32_t r[6])
+                                                int32_t r[6])
 {
+    const int type = orient_record(r);
     int tcount = 0;
     int zlo = 0, zhi = 0;
     bool ok = false;
@@ -161,7 +162,7 @@ __device__ __forceinline__ void admit_and_write(const TilePlan &tp, const Record
     if (i >= i1) return;
     int32_t st = 0;
     if (ok) {
-        st = record_status(path, cls - 1, zlo, zhi);
+        st = record_status(path, cls - 1, type, zlo, zhi);
         if (path == 1) {
             int lo[3], hi[3];
             if (tp.ntx == 1 && tp.nty == 1) {
@@ -172,7 +173,7 @@ __device__ __forceinline__ void admit_and_write(const TilePlan &tp, const Record
             } else {
                 tile_range_z(tp, r, zlo, zhi, lo, hi);
             }
-            const int off = (cls - 1) * tp.ntiles;
+            const int off = (cls - 1 + 2 * type) * tp.ntiles;
             for (int z = lo[2]; z <= hi[2]; ++z)
                 for (int y = lo[1]; y <= hi[1]; ++y)
                     for (int x = lo[0]; x <= hi[0]; ++x)
@@ -202,9 +203,9 @@ __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
     int use_miss, int use_hit, TilePlan tp, Records rec, Ctrl *ctrl, uint32_t *block_count,
     uint32_t *block_pairs, uint32_t *stage)
 {
-    extern __shared__ uint32_t s_hist[];  // 2 * ntiles counters
+    extern __shared__ uint32_t s_hist[];  // kGroups * ntiles counters
     __shared__ unsigned s_demand, s_total;
-    const int nh = 2 * tp.ntiles;
+    const int nh = kGroups * tp.ntiles;
     for (int t = threadIdx.x; t < nh; t += blockDim.x) s_hist[t] = 0;
     if (threadIdx.x == 0) {
         s_demand = 0;
@@ -348,7 +349,7 @@ cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cor
     const bool tiled = tp.ntiles > 0 && block_count && block_pairs && stage;
     TilePlan tpl = tp;
     if (!tiled) tpl.ntiles = 0;
-    const size_t smem = sizeof(uint32_t) * 2 * static_cast<size_t>(tpl.ntiles);
+    const size_t smem = sizeof(uint32_t) * kGroups * static_cast<size_t>(tpl.ntiles);
     uint32_t *bc = tiled ? block_count : nullptr;
     uint32_t *bp = tiled ? block_pairs : nullptr;
     uint32_t *sg = tiled ? stage : nullptr;
@@ -365,6 +366,17 @@ cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cor
             in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl, bc,
             bp, sg);
     return cudaGetLastError();
+}
+
+cudaError_t init_ingest()
+{
+    const int most = static_cast<int>(sizeof(uint32_t)) * kGroups * kMaxTiles;
+    cudaError_t e = cudaFuncSetAttribute(ingest_kernel<true>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(ingest_kernel<false>,
+                                 cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    return e;
 }
 
 cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, const GeomQ &g,

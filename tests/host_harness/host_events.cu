@@ -1,0 +1,84 @@
+// Host build of the event walks (hd_geom.cuh) for tests/test_host_events.py.
+#include <vector>
+
+#include "../../paper_1402_1720_gb300/csrc/hd_geom.cuh"
+
+// The event walk of the oriented segment in a box of dx x dy x dz voxels,
+// dilated by `thick`: its updates applied to plain counters in the tile's
+// layout, decoded by the definition (prefix sums along the major axis), the
+// voxels with a nonzero count returned box-linear (x fastest).  direct: the
+// one-slice set-up the scatter uses (dz = 1), else the general one.  Returns
+// -1 when the walk has no event form, -2 an update outside the box's words or
+// in another row than its walk's, -3 a voxel counted other than once.
+extern "C" int hx_events(const int32_t *seg, int dx, int dy, int dz, int thick, int direct,
+                         int32_t *out, int *nruns)
+{
+    int32_t r[6];
+    for (int a = 0; a < 6; ++a) r[a] = seg[a];
+    const int type = hd::orient_record(r);
+    const int32_t gi[3] = {r[0], r[1], r[2]}, go[3] = {r[3], r[4], r[5]};
+    const bool ymaj = (type & 2) != 0;
+    const int s = (type & 1) ? -1 : 1;
+    const int nmaj = ymaj ? dy : dx, nmin = ymaj ? dx : dy;
+    const int W = hd::tile_row_words(nmaj, nmin);
+    if (nmin * W * dz > (dx + 1) * (dy + 1) * dz) return -2;
+    *nruns = 0;
+    hd::LeanWalk L;
+    if (direct) {
+        const int rl = hd::slab_lean(gi, go, dx, dy, L);
+        if (rl == 0) return 0;
+        if (rl < 0) return -1;
+    } else {
+        hd::RunWalk w;
+        if (!hd::run_begin(w, gi, go, dx, dy, dz)) return 0;
+        if (!hd::lean_of(w, L)) return -1;
+    }
+    const bool moves = gi[0] != go[0] || gi[1] != go[1];
+    if (((L.fl >> 2) & 1) != (ymaj ? 1 : 0) || (moves && !(L.fl & 1))) return -4;
+    uint32_t o[hd::kLeanWords];
+    hd::event_pack(L, nmaj, nmin, thick, o);
+    const int words = nmin * W * dz;
+    std::vector<int> E(words, 0), P(words, 0);
+    hd::EventCursor c;
+    int first;
+    if (!hd::event_start(o, 0, c, first)) return -2;
+    auto ok = [&](int at) { return at >= 0 && at / 4 < words && (at & 3) == 0; };
+    if (!ok(first)) return -2;
+    P[first / 4] += 1;
+    int row = first / 4 / W;
+    *nruns = c.left + 1;
+    while (c.left) {
+        if (!ok(c.addr) || c.addr / 4 / W != row || c.addr / 4 % W >= nmaj) return -2;
+        E[c.addr / 4] += 1;
+        hd::event_next(c);
+        row += s;
+    }
+    const int end = hd::event_end(c, 4 * (thick + 1));
+    if (!ok(end) || end / 4 / W != row) return -2;
+    P[end / 4] -= 1;
+    std::vector<int> SE(words), SP(words);
+    for (int q = 0; q < nmin * dz; ++q) {
+        int e = 0, p = 0;
+        for (int m = 0; m < W; ++m) {
+            SE[q * W + m] = e += E[q * W + m];
+            SP[q * W + m] = p += P[q * W + m];
+        }
+    }
+    int n = 0;
+    for (int z = 0; z < dz; ++z)
+        for (int y = 0; y < dy; ++y)
+            for (int x = 0; x < dx; ++x) {
+                const int i = ymaj ? x : y, m = ymaj ? y : x;
+                int v = 0;
+                for (int j = -thick; j <= thick; ++j)
+                    if (i + j >= 0 && i + j < nmin) v += SP[(i + j + nmin * z) * W + m];
+                const int ia = i - (thick + 1) * s, ib = i + thick * s;
+                if (ia >= 0 && ia < nmin)
+                    v += SE[(ia + nmin * z) * W + (m + thick < nmaj ? m + thick : nmaj)];
+                if (ib >= 0 && ib < nmin && m - thick - 1 >= 0)
+                    v -= SE[(ib + nmin * z) * W + m - thick - 1];
+                if (v != 0 && v != 1) return -3;
+                if (v) out[n++] = x + dx * (y + dy * z);
+            }
+    return n;
+}

@@ -1,0 +1,80 @@
+"""Event walks (hd_geom.cuh), compiled for the host, against the CPU oracle's
+voxel sets: one update per change of row and two marks per walk decode to the
+set itself and to the set dilated in-plane, on adversarial segments (ties,
+planes, box edges) and generic ones.  Runs without a GPU."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from tests.test_oracle_pins import _random_segments
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+SRC = os.path.join(HERE, "host_harness", "host_events.cu")
+I32P = ctypes.POINTER(ctypes.c_int32)
+
+
+@pytest.fixture(scope="module")
+def hx(tmp_path_factory):
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(nvcc):
+        pytest.skip("nvcc not available")
+    out = str(tmp_path_factory.mktemp("hx") / "libhostevents.so")
+    subprocess.check_call([nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-shared",
+                           "-gencode", "arch=compute_103a,code=sm_103a",
+                           "-diag-suppress", "20014", "-o", out, SRC,
+                           "-I", os.path.join(HERE, "..", "include")])
+    return ctypes.CDLL(out)
+
+
+def _generic(rng, n, dims):
+    """Segments across the box in every direction, ends inside and outside."""
+    d = np.array(dims)
+    for _ in range(n):
+        span = rng.choice([0.1, 1.0, 3.0])
+        a = rng.uniform(-0.6, 1.6, 3) * d
+        b = a + rng.uniform(-1.0, 1.0, 3) * d * span * np.array([1.0, 1.0, rng.choice([0.02, 1.0])])
+        yield [np.round(65536 * v).astype(np.int32) for v in (a, b)]
+
+
+def _dilate(v, dims, t):
+    if t == 0 or v.size == 0:
+        return np.sort(v)
+    nx, ny, nz = dims
+    vol = np.zeros((nz, ny, nx), bool)
+    vol.reshape(-1)[v] = True
+    out = vol.copy()
+    for dy in range(-t, t + 1):
+        for dx in range(-t, t + 1):
+            s = vol[:, max(0, -dy):ny - max(0, dy), max(0, -dx):nx - max(0, dx)]
+            if s.size:
+                out[:, max(0, dy):ny - max(0, -dy), max(0, dx):nx - max(0, -dx)] |= s
+    return np.flatnonzero(out.reshape(-1))
+
+
+@pytest.mark.parametrize("dims,direct", [((5, 4, 1), 1), ((1, 1, 1), 1), ((1, 7, 1), 1),
+                                         ((9, 1, 1), 1), ((40, 30, 1), 1), ((17, 64, 1), 1),
+                                         ((12, 11, 3), 0), ((40, 30, 2), 0)])
+def test_event_walks_equal_oracle(oracle_mod, hx, dims, direct):
+    rng = np.random.default_rng(sum(dims) + 3)
+    segs = list(_random_segments(rng, 1500, dims)) + list(_generic(rng, 1500, dims))
+    seen = 0
+    for a, b in segs:
+        seg = np.concatenate([a, b]).astype(np.int32)
+        ref = oracle_mod.voxel_set(np.asarray(a, np.int32), np.asarray(b, np.int32), *dims)
+        for t in (0, 1, 3):
+            if t and dims[2] > 1:
+                continue
+            out = np.zeros(int(np.prod(dims)), np.int32)
+            runs = ctypes.c_int(0)
+            n = hx.hx_events(seg.ctypes.data_as(I32P), *dims, t, direct, out.ctypes.data_as(I32P),
+                             ctypes.byref(runs))
+            if n == -1:
+                continue
+            assert n >= 0, (n, seg.tolist(), t)
+            seen += n > 0
+            assert np.array_equal(out[:n], _dilate(ref, dims, t)), (seg.tolist(), t)
+    assert seen > 300
