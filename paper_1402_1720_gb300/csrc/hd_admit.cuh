@@ -1,0 +1,108 @@
+// Admission of records to the tiled path, shared by the ingest kernels: the
+// pair budget of a block, its tile histogram, its pair list, and the records at
+// their histories' slots.
+#pragma once
+
+#include "hd_geom.cuh"
+
+namespace hd {
+namespace {
+
+__device__ __forceinline__ unsigned warp_sum_u32(unsigned v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+__device__ __forceinline__ unsigned warp_incl_scan(unsigned v)
+{
+    const unsigned lane = threadIdx.x & 31u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= static_cast<unsigned>(o)) v += t;
+    }
+    return v;
+}
+
+// Decide the path of each lane's record (tiled within the block's pair
+// budget, else global; ok false: no record), count its tiles in the block
+// histogram, list its pairs in the block's share of stage, and write it at its
+// history's slot i (when i < i1).  tcount: its tiles (-1: not for the tiled
+// path); tiles(lo, hi) gives their box.  Budget reservations are per warp on a
+// shared-memory counter, so the block never waits at a barrier.  The pairs
+// the budget admits fill the list from its start without gaps: the
+// reservations tile [0, total) in the order of their ends, and only the one
+// record that straddles the budget, and the records after it, are turned
+// away (they take the global path, exact either way).
+template <class TilesT>
+__device__ __forceinline__ void reserve_and_write(const TilePlan &tp, const Records &rec, Ctrl *ctrl,
+                                                  uint32_t *s_hist, unsigned *s_demand,
+                                                  unsigned budget, int64_t h0, int64_t i,
+                                                  int64_t i1, uint32_t *stage, int cls, int type,
+                                                  bool ok, int tcount, int zlo, int zhi,
+                                                  const int32_t r[6], const TilesT &tiles)
+{
+    const unsigned demand = ok && tcount > 0 ? static_cast<unsigned>(tcount) : 0u;
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned incl = warp_incl_scan(demand);
+    const unsigned tot = __shfl_sync(0xffffffffu, incl, 31);
+    unsigned wbase = 0;
+    if (lane == 31 && tot) wbase = atomicAdd(s_demand, tot);
+    wbase = __shfl_sync(0xffffffffu, wbase, 31);
+    const unsigned long long end = static_cast<unsigned long long>(wbase) + incl;
+    const int path = ok ? (demand > 0 && end <= budget ? 1 : 2) : 0;
+    if (rec.glist) {
+        // the global path's list: one counter update per warp
+        const unsigned gm = __ballot_sync(0xffffffffu, path == 2);
+        if (gm) {
+            const int lead = __ffs(gm) - 1;
+            unsigned gb = 0;
+            if (static_cast<int>(lane) == lead) gb = atomicAdd(&ctrl->n_global, __popc(gm));
+            gb = __shfl_sync(0xffffffffu, gb, lead);
+            if (path == 2) rec.glist[gb + __popc(gm & ((1u << lane) - 1u))] = static_cast<int32_t>(i);
+        }
+    }
+    if (i >= i1) return;
+    int32_t st = 0;
+    if (ok) {
+        st = record_status(path, cls, type, zlo, zhi);
+        if (path == 1) {
+            int lo[3], hi[3];
+            tiles(lo, hi);
+            const int off = (cls + 2 * type) * tp.ntiles;
+            for (int z = lo[2]; z <= hi[2]; ++z)
+                for (int y = lo[1]; y <= hi[1]; ++y)
+                    for (int x = lo[0]; x <= hi[0]; ++x)
+                        atomicAdd(&s_hist[off + x + tp.ntx * (y + tp.nty * z)], 1u);
+            // the record's pairs hold positions end - c .. end - 1 of the
+            // block's list (all below its budget)
+            const uint32_t code = static_cast<uint32_t>(i - h0) << kRecordTileBits;
+            const unsigned first = static_cast<unsigned>(end) - demand;
+            for (int j = 0; j < tcount; ++j) stage[first + j] = code | static_cast<uint32_t>(j);
+        }
+#pragma unroll
+        for (int a = 0; a < 6; ++a) rec.g[a][i] = r[a];
+    }
+    rec.status[i] = st;
+}
+
+// The end of an ingest block: its pair counts per bucket and in all.
+__device__ __forceinline__ void write_block_counts(int nh, const uint32_t *s_hist, unsigned *s_total,
+                                                   uint32_t *block_count, uint32_t *block_pairs)
+{
+    __syncthreads();
+    unsigned mine = 0;
+    for (int t = threadIdx.x; t < nh; t += blockDim.x) {
+        block_count[static_cast<size_t>(t) * gridDim.x + blockIdx.x] = s_hist[t];
+        mine += s_hist[t];
+    }
+    mine = warp_sum_u32(mine);
+    if ((threadIdx.x & 31u) == 0 && mine) atomicAdd(s_total, mine);
+    __syncthreads();
+    if (threadIdx.x == 0) block_pairs[blockIdx.x] = *s_total;
+}
+
+}  // namespace
+}  // namespace hd

@@ -138,6 +138,7 @@ struct hd_scan {
     uint32_t *rows_bits = nullptr;    // the hull packed for the row passes
     int32_t thick_k = 0;             // thick rays: in-plane dilation (0 = thin paths)
     float euclid_d0 = 0.0f;          // thick rays by Euclidean distance, mm (0 = off)
+    int euclid_pairs = 0;            // their pairs per record on the tiled path (0: not taken)
     void *thick_ws = nullptr;        // their difference arrays
     bool inputs_on_host = false;  // the chunk being added is read in place from host memory
     float *staging = nullptr;  // copied host inputs: 6 columns of staging_half floats
@@ -341,6 +342,15 @@ size_t tile_count_words(const hd_scan *s)
     return cols * (1 + ingest_blocks_max(s)) + ingest_blocks_max(s);
 }
 
+// Pairs of Euclidean thick rays that the pair buffer holds: kSliceWords words
+// each, a word of the list of open rows (two words per entry) and one of the
+// blocks' pair lists.
+int64_t euclid_pair_cap(const hd_scan *s)
+{
+    const int64_t words = (hd::kLeanWords + 3) * static_cast<int64_t>(s->tp.pair_cap);
+    return words / (hd::kSliceWords + 2) & ~int64_t(3);
+}
+
 hd::Pairs pairs_of(const hd_scan *s)
 {
     hd::Pairs p;
@@ -351,6 +361,14 @@ hd::Pairs pairs_of(const hd_scan *s)
     p.v = reinterpret_cast<uint4 *>(base);
     p.fb = base ? reinterpret_cast<uint2 *>(base + hd::kLeanWords * cap) : nullptr;
     p.stage = base ? base + (hd::kLeanWords + 2) * cap : nullptr;
+    p.fb_cap = 0;
+    if (s->euclid_pairs > 0) {
+        // Euclidean thick rays: the same buffer in their layout
+        const size_t c = static_cast<size_t>(euclid_pair_cap(s));
+        p.fb = base ? reinterpret_cast<uint2 *>(base + hd::kSliceWords * c) : nullptr;
+        p.fb_cap = static_cast<uint32_t>(c / 2);
+        p.stage = base ? base + (hd::kSliceWords + 1) * c : nullptr;
+    }
     return p;
 }
 
@@ -422,6 +440,7 @@ hd::ScanDesc make_desc(const hd_scan *s)
 {
     hd::ScanDesc d{};
     d.tp = s->tp;
+    if (s->euclid_pairs > 0) d.tp.pairs_per_record = s->euclid_pairs;
     d.pairs = pairs_of(s);
     d.buckets = buckets_of(s);
     d.ctrl = s->ctrl;
@@ -518,8 +537,35 @@ int finalize_launches(const hd_scan *scan) { return (scan->params.methods & HD_S
 hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st)
 {
     if (s->euclid_d0 > 0.0f) {
-        // Euclidean thick rays: a warp per history over the rows of its capsule
         const uint32_t m = s->params.methods;
+        if (s->euclid_pairs > 0 && s->trace_grid > 0) {
+            // Euclidean thick rays on the tiled path, in chunks whose pairs
+            // fit the buffer
+            hd_status r = upload_desc(s, st);
+            if (r != HD_OK) return r;
+            const int64_t most = euclid_pair_cap(s) / s->euclid_pairs & ~int64_t(3);
+            const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
+            uint32_t *block_count = s->tile_count + cols;
+            uint32_t *block_pairs = block_count + cols * ingest_blocks_max(s);
+            // equal chunks
+            const int64_t parts = most > 0 ? (n + most - 1) / most : 0;
+            const int64_t per = parts > 0 ? ((n + parts - 1) / parts + 3) & ~int64_t(3) : 0;
+            for (int64_t off = 0; per > 0 && off < n; off += per) {
+                const int64_t c = n - off < per ? n - off : per;
+                const hd::Inputs part{in.angle + off, in.u_in + off,  in.v_in + off,
+                                      in.u_out + off, in.v_out + off, in.wepl + off};
+                HD_CUDA(cudaMemsetAsync(&s->ctrl->n_global, 0,
+                                        sizeof(hd::Ctrl) - offsetof(hd::Ctrl, n_global), st));
+                HD_CUDA(hd::launch_euclid_scan(
+                    s->desc_dev, s->desc_host, part, c, &s->geom, s->gq, s->cordic,
+                    s->params.wepl_miss_lt, s->params.wepl_hit_gt, (m & (HD_SC | HD_MSC)) ? 1 : 0,
+                    (m & HD_SM) ? 1 : 0, s->euclid_d0, records_of(s, c), block_count, block_pairs,
+                    s->thick_ws, s->trace_grid, s->sm_count, st));
+                s->launches += 12;
+            }
+            if (per > 0) return HD_OK;
+        }
+        // other plans: a warp per history over the rows of its capsule
         HD_CUDA(hd::launch_euclid(in, n, &s->geom, s->gq, s->cordic, s->params.wepl_miss_lt,
                                   s->params.wepl_hit_gt, (m & (HD_SC | HD_MSC)) ? 1 : 0,
                                   (m & HD_SM) ? 1 : 0, s->euclid_d0, s->thick_ws, s->N, s->M,
@@ -660,7 +706,9 @@ hd_status hd_scan_create(const hd_geometry *geom, const hd_params *params, hd_sc
     if (m & HD_MSC) alloc(reinterpret_cast<void **>(&s->H2), V);
     alloc(reinterpret_cast<void **>(&s->bits_out), sizeof(uint32_t) * s->words);
     make_tile_plan(s);
-    if (hd::init_ingest() != cudaSuccess || hd::init_scatter() != cudaSuccess) ok = false;
+    if (hd::init_ingest() != cudaSuccess || hd::init_scatter() != cudaSuccess ||
+        hd::init_euclid() != cudaSuccess)
+        ok = false;
     if (s->tp.ntiles > 0) {
         alloc(reinterpret_cast<void **>(&s->tile_count), sizeof(uint32_t) * tile_count_words(s));
         alloc(reinterpret_cast<void **>(&s->tile_cursor), sizeof(uint32_t) * hd::kGroups * s->tp.ntiles);
@@ -1046,7 +1094,10 @@ hd_status hd_scan_set_thick(hd_scan *scan, int32_t k)
     scan->thick_k = k;
     scan->tp.thick = k;
     scan->desc_dirty = true;
-    if (k > 0) scan->euclid_d0 = 0.0f;
+    if (k > 0) {
+        scan->euclid_d0 = 0.0f;
+        scan->euclid_pairs = 0;
+    }
     return HD_OK;
 }
 
@@ -1069,8 +1120,10 @@ hd_status hd_scan_set_thick_distance(hd_scan *scan, float d0_mm)
     if (d0_mm > 0.0f) {
         scan->thick_k = 0;
         scan->tp.thick = 0;
-        scan->desc_dirty = true;
     }
+    scan->euclid_pairs =
+        d0_mm > 0.0f ? hd::euclid_pairs_per_record(&scan->geom, d0_mm, scan->tp) : 0;
+    scan->desc_dirty = true;
     return HD_OK;
 }
 
@@ -1098,6 +1151,9 @@ hd_status hd_scan_set_tuning(hd_scan *scan, const hd_tuning *t)
     scan->rec_cap = 0;
     scan->tuning = *t;
     make_tile_plan(scan);
+    scan->euclid_pairs = scan->euclid_d0 > 0.0f
+                             ? hd::euclid_pairs_per_record(&scan->geom, scan->euclid_d0, scan->tp)
+                             : 0;
     scan->trace_grid = 0;
     if (scan->tp.ntiles > 0) {
         if (cudaMalloc(&scan->tile_count, sizeof(uint32_t) * tile_count_words(scan)) != cudaSuccess ||

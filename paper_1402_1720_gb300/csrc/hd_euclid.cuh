@@ -574,5 +574,256 @@ HD_HD void k_range(const CapF &cf, int a, int blo2, int bhi2, int &klo, int &khi
     khi = min_i(bhi2, static_cast<int>(floorf(hi)));
 }
 
+// ------------------------------------------------------ rows of one slice
+//
+// The tiled form takes a history's rows one slice (fixed k) at a time.  When
+// every centre of the grid projects onto the segment's interior (the trackers
+// stand outside the grid), the capsule is a cylinder there, and its rows have
+// a closed form: with h^2 = u_1^2 + u_2^2, row a of the slice lies at the
+// signed distance e R from the line in the plane of axes 1 and 2, linear in a,
+// and its voxels are the indices within Kr sqrt(1 - e^2) of a centre f, linear
+// in a too (f in index units, Kr = R |u| / (h 2 s_0)).  Both linear functions
+// start from exact 64-bit products at the first row, so their float errors are
+// relative to their own values.
+//
+// Certainty (eps = 2^-24).  Per row e is off by at most de = 16 eps (|e_0| +
+// n |e_a|) over the n rows (u, step and the reciprocals each add a rounding or
+// two of their own size: 11 in all), f by at most 16 eps (|f_0| + n |f_a| + 2
+// |A_0 - c_0| / (2 s_0)), so 1 - e^2 is off by at most dq = 4 de + 4 eps for |e|
+// near 1 or less, its root by dq / root, and the ends by E0 + Kd / root in all,
+// E0 the bound for f and 16 eps Kr for the roundings of Kr, of the root and of
+// the ends themselves, Kd = Kr dq.  When both ends give the same index over that
+// range, and 1 - e^2 is above 4 dq (or below -dq: no voxel), the row's voxels
+// are certain; the other rows (about 0.3 %) go to the exact search.
+struct SliceRows {
+    float e0, ea;  // e of the first row, and its change per row
+    float f0, fa;  // f, in index units of the tile
+    float Kr, E0, Kd, dq;
+    int row;  // the first row, in rows of the tile
+    int n;    // rows
+};
+
+constexpr float kEps = 5.9604644775390625e-8f;  // 2^-24
+
+// Where a record's rows can lie: false when no voxel centre of the grid is
+// inside; else the slices klo .. khi and the extent of axis y (ylo .. yhi, for
+// tiles that are strips), and whether the closed form above holds.  In float,
+// widened by 2^-14 S, far beyond its roundings.
+HD_HD bool euclid_range(const GeomQ &g, const long long W[6], long long R, int &klo, int &khi,
+                        int &ylo, int &yhi, bool &closed)
+{
+    const float P[3] = {static_cast<float>(2 * W[0]), static_cast<float>(2 * W[1]),
+                        static_cast<float>(2 * W[2])};
+    const float D[3] = {static_cast<float>(2 * (W[3] - W[0])), static_cast<float>(2 * (W[4] - W[1])),
+                        static_cast<float>(2 * (W[5] - W[2]))};
+    const float H[3] = {static_cast<float>((g.nx - 1LL) * g.sx), static_cast<float>((g.ny - 1LL) * g.sy),
+                        static_cast<float>((g.nz - 1LL) * g.sz)};
+    const float Rf = static_cast<float>(R);
+    float S = Rf, uu = 0.0f, dmin = 0.0f, dmax = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        S += H[a] + fabsf(P[a]) + fabsf(D[a]);
+        uu = fmaf(D[a], D[a], uu);
+        const float lo = (-H[a] - P[a]) * D[a], hi = (H[a] - P[a]) * D[a];
+        dmin += fminf(lo, hi);
+        dmax += fmaxf(lo, hi);
+    }
+    const float m = S * (1.0f / 16384.0f);
+    const float mu = m * (fabsf(D[0]) + fabsf(D[1]) + fabsf(D[2]));
+    // off both in-plane axes (h > 0 either way round) and interior
+    closed = W[0] != W[3] && W[1] != W[4] && dmin > mu && dmax < uu - mu;
+    float t0 = 0.0f, t1 = 1.0f;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+        const float L = H[a] + Rf + m;
+        if (D[a] == 0.0f) {
+            if (fabsf(P[a]) > L) return false;
+            continue;
+        }
+        const float i = 1.0f / D[a];
+        const float ta = (-L - P[a]) * i, tb = (L - P[a]) * i;
+        t0 = fmaxf(t0, fminf(ta, tb));
+        t1 = fminf(t1, fmaxf(ta, tb));
+    }
+    if (t0 > t1) return false;
+    const float z0 = fmaf(t0, D[2], P[2]), z1 = fmaf(t1, D[2], P[2]);
+    const float iz = 0.5f / static_cast<float>(g.sz), iy = 0.5f / static_cast<float>(g.sy);
+    const float kl = (fminf(z0, z1) - Rf - m + H[2]) * iz - 0.01f;
+    const float kh = (fmaxf(z0, z1) + Rf + m + H[2]) * iz + 0.01f;
+    if (kh < 0.0f || kl > static_cast<float>(g.nz - 1)) return false;
+    klo = static_cast<int>(ceilf(fmaxf(kl, 0.0f)));
+    khi = static_cast<int>(floorf(fminf(kh, static_cast<float>(g.nz - 1))));
+    const float y0 = fmaf(t0, D[1], P[1]), y1 = fmaf(t1, D[1], P[1]);
+    const float yl = (fminf(y0, y1) - Rf - m + H[1]) * iy - 0.01f;
+    const float yh = (fmaxf(y0, y1) + Rf + m + H[1]) * iy + 0.01f;
+    if (yh < 0.0f || yl > static_cast<float>(g.ny - 1)) return false;
+    ylo = static_cast<int>(ceilf(fmaxf(yl, 0.0f)));
+    yhi = static_cast<int>(floorf(fminf(yh, static_cast<float>(g.ny - 1))));
+    return klo <= khi && ylo <= yhi;
+}
+
+// The rows of slice k in a tile of `rows` rows from index a0 on, its row
+// indices 0 .. len - 1 starting at m0 (a record with the closed form).
+// False when none can have a voxel.
+HD_HD bool slice_rows(const GeomQ &g, const int32_t W[6], long long R, int k, int a0, int rows,
+                      int m0, int len, SliceRows &r)
+{
+    const int dx = W[3] - W[0], dy = W[4] - W[1];
+    const bool ymaj = (dy < 0 ? -dy : dy) > (dx < 0 ? -dx : dx);
+    const int n0 = ymaj ? g.ny : g.nx, n1 = ymaj ? g.nx : g.ny;
+    const int s0 = static_cast<int>(ymaj ? g.sy : g.sx), s1 = static_cast<int>(ymaj ? g.sx : g.sy);
+    const int A0 = 2 * (ymaj ? W[1] : W[0]), A1 = 2 * (ymaj ? W[0] : W[1]), A2 = 2 * W[2];
+    const int u0 = 2 * (ymaj ? dy : dx), u1 = 2 * (ymaj ? dx : dy), u2 = 2 * (W[5] - W[2]);
+    auto mul = [](int a, int b) { return static_cast<long long>(a) * b; };
+    const float uf0 = static_cast<float>(u0), uf1 = static_cast<float>(u1),
+                uf2 = static_cast<float>(u2);
+    const float h2 = static_cast<float>(mul(u1, u1) + mul(u2, u2));
+    const float uu = static_cast<float>(mul(u0, u0) + mul(u1, u1) + mul(u2, u2));
+    const float ih2 = rcp_rn(h2), is0 = rcp_rn(static_cast<float>(2 * s0));
+    const float Rf = static_cast<float>(R);
+#ifdef __CUDA_ARCH__
+    const float ih = __frsqrt_rn(h2), ul = __fsqrt_rn(uu);
+#else
+    const float ih = 1.0f / std::sqrt(h2), ul = std::sqrt(uu);
+#endif
+    const float ihR = ih * rcp_rn(Rf);
+    const float st1 = static_cast<float>(2 * s1);
+    r.Kr = ul * ih * Rf * is0;
+    r.ea = st1 * uf2 * ihR;
+    r.fa = uf0 * uf1 * ih2 * st1 * is0;
+    const int wz = (2 * k + 1 - g.nz) * static_cast<int>(g.sz) - A2;
+    const int c0 = (1 - n0) * s0;
+    const float off = static_cast<float>(A0 - c0) * is0;
+    auto at = [&](int a, float &e, float &f) {
+        const int wc = (2 * a + 1 - n1) * s1 - A1;
+        e = static_cast<float>(mul(wc, u2) - mul(wz, u1)) * ihR;
+        f = uf0 * (static_cast<float>(mul(wc, u1) + mul(wz, u2)) * ih2) * is0 + off -
+            static_cast<float>(m0);
+    };
+    // the rows whose |e| can be at most 1 and whose voxels can reach the tile:
+    // float ranges widened by half a row, cut to the tile
+    float e, f;
+    at(a0, e, f);
+    float lo = 0.0f, hi = static_cast<float>(rows - 1);
+    if (fabsf(r.ea) * (hi + 1.0f) > 1e-6f) {
+        const float i = 1.0f / r.ea;
+        const float x = (-1.0001f - e) * i, y = (1.0001f - e) * i;
+        lo = fmaxf(lo, fminf(x, y) - 0.5f);
+        hi = fminf(hi, fmaxf(x, y) + 0.5f);
+    } else if (fabsf(e) > 1.001f) {
+        return false;
+    }
+    if (fabsf(r.fa) > 1e-3f) {
+        const float i = 1.0f / r.fa, w = r.Kr + 1.0f;
+        const float x = (-w - f) * i, y = (static_cast<float>(len - 1) + w - f) * i;
+        lo = fmaxf(lo, fminf(x, y) - 0.5f);
+        hi = fminf(hi, fmaxf(x, y) + 0.5f);
+    }
+    if (!(lo <= hi)) return false;
+    const int b0 = static_cast<int>(ceilf(lo)), b1 = static_cast<int>(floorf(hi));
+    if (b0 > b1) return false;
+    at(a0 + b0, r.e0, r.f0);
+    r.row = b0;
+    r.n = b1 - b0 + 1;
+    const float n = static_cast<float>(r.n);
+    const float de = 16.0f * kEps * (fabsf(r.e0) + n * fabsf(r.ea));
+    r.dq = 4.0f * de + 4.0f * kEps;
+    r.E0 = 16.0f * kEps * (2.0f * fabsf(off) + fabsf(static_cast<float>(m0)) + fabsf(r.f0) +
+                           n * fabsf(r.fa) + 1.0f + r.Kr);
+    r.Kd = r.Kr * r.dq;
+    return true;
+}
+
+// x rounded up and down to a whole number, |x| < 2^22, plus 1.5 2^23.
+constexpr float kWhole = 12582912.0f;
+HD_HD float whole_up(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __fadd_ru(x, kWhole);
+#else
+    return std::ceil(x) + kWhole;
+#endif
+}
+HD_HD float whole_down(float x)
+{
+#ifdef __CUDA_ARCH__
+    return __fadd_rd(x, kWhole);
+#else
+    return std::floor(x) + kWhole;
+#endif
+}
+HD_HD float rsqrt_est(float x)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+#else
+    return 1.0f / std::sqrt(x);
+#endif
+}
+
+// Row i of the slice: its first and last index (whole_up form, cut to the tile's
+// 0 .. len - 1, top = kWhole + len - 1), empty when lo > hi.  False when the row
+// is not certain.
+HD_HD bool slice_row(const SliceRows &r, float i, float top, float &lo, float &hi)
+{
+    const float e = fmaf(i, r.ea, r.e0);
+    const float q = fmaf(-e, e, 1.0f);
+    const float rs = rsqrt_est(fmaxf(q, r.dq));
+    const float hw = r.Kr * (q * rs);
+    const float c = fmaf(i, r.fa, r.f0);
+    const float tol = fmaf(r.Kd, rs, r.E0);
+    const float big = 1048576.0f;
+    const float x = fminf(fmaxf(c - hw, -big), big), y = fminf(fmaxf(c + hw, -big), big);
+    const float x0 = whole_up(x - tol), x1 = whole_up(x + tol);
+    const float y0 = whole_down(y - tol), y1 = whole_down(y + tol);
+    lo = fmaxf(x0, kWhole);
+    hi = fminf(y0, top);
+    const bool sure = (x0 == x1 && y0 == y1 && q > 4.0f * r.dq) || q < -r.dq;
+    if (q < 0.0f) hi = kWhole - 1.0f;  // the row misses the cylinder
+    return sure;
+}
+
+// A row of a tile left to the exact search: a + 2^12 k + 2^24 strip (the tile's
+// place along y; rows along y are cut to it).
+HD_HD uint32_t row_code(int a, int k, int strip)
+{
+    return static_cast<uint32_t>(a) | (static_cast<uint32_t>(k) << 12) |
+           (static_cast<uint32_t>(strip) << 24);
+}
+
+// The exact search of one listed row of the record in `slot`, its voxels added
+// to N or M one by one.
+__device__ __noinline__ void exact_row(const RowsArgs &ra, const ScanDesc &d, uint32_t slot,
+                                       uint32_t code)
+{
+    const GeomQ &g = ra.g;
+    long long W[6];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) W[q] = ra.rec.g[q][slot];
+    const int cls = status_cls(ra.rec.status[slot]);
+    long long A[3], B[3];
+    bool ymaj;
+    int blo[3], bhi[3];
+    float S;
+    if (!capsule_frame(g, W, ra.R, A, B, ymaj, blo, bhi, S)) return;
+    CapX cx;
+    capx_of(g, A, B, ymaj, ra.R, cx);
+    const CapF cf = capf_of(cx, S, ra.R);
+    const int a = static_cast<int>(code & 0xfffu), k = static_cast<int>((code >> 12) & 0xfffu);
+    int lo, hi;
+    if (!row_interval(cf, cx, a, k, lo, hi)) return;
+    uint32_t *vol = (cls ? d.M : d.N) + static_cast<size_t>(k) * g.nx * g.ny;
+    if (ymaj) {
+        const int y0 = static_cast<int>(code >> 24) * d.tp.ty;
+        lo = max_i(lo, y0);
+        hi = min_i(hi, min_i(y0 + d.tp.ty, g.ny) - 1);
+        for (int m = lo; m <= hi; ++m) atomicAdd(vol + a + static_cast<size_t>(g.nx) * m, 1u);
+    } else {
+        for (int m = lo; m <= hi; ++m) atomicAdd(vol + m + static_cast<size_t>(g.nx) * a, 1u);
+    }
+}
+
 }  // namespace
 }  // namespace hd

@@ -116,7 +116,13 @@ struct Pairs {
     // record's slot less the block's first slot, times kMaxRecordTiles,
     // plus the pair's tile index within the record.
     uint32_t *stage;
+    // Euclidean thick rays use the same buffer with kSliceWords words per pair
+    // in v, and fb as the list of the rows left to the exact search (fb_cap
+    // entries: the record's slot; row, slice and strip, see row_code).
+    uint32_t fb_cap;
 };
+
+constexpr int kSliceWords = 12;
 
 // Tiles a record may touch on the tiled path (its box of tiles; more take
 // the global path), and the bits of a tile index within a record.
@@ -143,6 +149,15 @@ struct ScanDesc {
 };
 
 constexpr int kMaxBatch = 64;  // scans per batched traversal launch
+
+// What the exact search of a row of Euclidean thick rays needs: the geometry,
+// R = 2 q16(d_0), and the chunk's records (world endpoints, mm * 2^16).
+struct RowsArgs {
+    static constexpr bool kRows = true;
+    GeomQ g;
+    long long R;
+    Records rec;
+};
 
 struct Inputs {
     const float *angle, *u_in, *v_in, *u_out, *v_out, *wepl;
@@ -183,6 +198,10 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
 // 256, 512, 768 or 1024.
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
                                int grid, cudaStream_t s);
+
+// The same over the pairs of Euclidean thick rays of one scan (hd_euclid.cu).
+cudaError_t launch_trace_rows(const ScanDesc *desc, int tile_words, int threads, int grid,
+                              const RowsArgs &ra, cudaStream_t s);
 
 // Global-memory traversal of the records whose path is 2 (or of every
 // record when all_records is set); upper is the chunk's slot count.

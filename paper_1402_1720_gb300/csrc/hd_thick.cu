@@ -458,29 +458,44 @@ cudaError_t launch_thick_finish(const hd_geometry *geom, void *workspace, uint32
     return e;
 }
 
+cudaError_t launch_thick_clear(const hd_geometry *geom, void *workspace, const Ctrl *ctrl,
+                               int sm_count, cudaStream_t st)
+{
+    // the workspace is a multiple of 256 bytes (thick_layout)
+    const int64_t need = static_cast<int64_t>(thick_workspace_bytes(geom));
+    thick_clear_kernel<<<static_cast<unsigned>(sm_count > 0 ? 8 * sm_count : 8), kThickThreads, 0, st>>>(
+        static_cast<uint4 *>(workspace), need / 16, ctrl);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_thick_left(const hd_geometry *geom, void *workspace, uint32_t *N, uint32_t *M,
+                              const Ctrl *ctrl, cudaStream_t st)
+{
+    ThickWs ws{};
+    thick_layout(geom, workspace, &ws);
+    return launch_thick_rows(geom, ws, N, M, ctrl, st);
+}
+
 cudaError_t launch_thick_scan(const ScanDesc *desc_dev, const hd_geometry *geom,
                               const Records &rec, Ctrl *ctrl, int64_t upper, const GeomQ &g,
                               int k, void *workspace, uint32_t *N, uint32_t *M, int smem_words,
                               int threads, int grid, int sm_count, cudaStream_t st)
 {
-    ThickWs ws{};
-    const size_t need = thick_layout(geom, workspace, &ws);
     const ThickDiff td = thick_diff_of(geom, workspace);
     cudaError_t e = launch_trace_tiles(desc_dev, 1, smem_words, threads, grid, st);
     if (e == cudaSuccess && upper > 0) {
         int64_t blocks = (upper + kThickThreads - 1) / kThickThreads;
         const int64_t cap = int64_t(sm_count > 0 ? sm_count : 1) * 8;
         if (blocks > cap) blocks = cap;
-        // the workspace is a multiple of 256 bytes (thick_layout)
-        thick_clear_kernel<<<static_cast<unsigned>(cap), kThickThreads, 0, st>>>(
-            static_cast<uint4 *>(workspace), static_cast<int64_t>(need / 16), ctrl);
+        e = launch_thick_clear(geom, workspace, ctrl, sm_count, st);
+        if (e != cudaSuccess) return e;
         thick_fallback_kernel<<<static_cast<unsigned>(sm_count > 0 ? 4 * sm_count : 4), 32 * kFbWarps, 0,
                                 st>>>(desc_dev, k);
         thick_records_kernel<<<static_cast<unsigned>(blocks), kThickThreads, 0, st>>>(rec, ctrl, g,
                                                                                       k, td);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = launch_thick_rows(geom, ws, N, M, ctrl, st);
+    if (e == cudaSuccess) e = launch_thick_left(geom, workspace, N, M, ctrl, st);
     return e;
 }
 

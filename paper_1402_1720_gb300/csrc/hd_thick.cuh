@@ -113,6 +113,26 @@ cudaError_t launch_thick(const Inputs &in, int64_t n, const hd_geometry *geom, c
                          unsigned long long *stats, int64_t *intervals, int sm_count,
                          cudaStream_t st);
 
+// For a tiled pass with a scan's counters: clears the difference arrays, and adds
+// them to N and M (either may be null), when its chunk has records on the
+// global path; nothing otherwise.
+cudaError_t launch_thick_clear(const hd_geometry *geom, void *workspace, const Ctrl *ctrl,
+                               int sm_count, cudaStream_t st);
+cudaError_t launch_thick_left(const hd_geometry *geom, void *workspace, uint32_t *N, uint32_t *M,
+                              const Ctrl *ctrl, cudaStream_t st);
+
+// Euclidean thick rays of a scan on the tiled path (hd_euclid.cu): pairs per
+// record to plan with (0: the tiled path does not take this scan), and one
+// chunk of histories, at most desc.pairs' capacity / that many.
+cudaError_t init_euclid();
+int euclid_pairs_per_record(const hd_geometry *geom, float d0, const TilePlan &tp);
+cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, const Inputs &in,
+                               int64_t n, const hd_geometry *geom, const GeomQ &g,
+                               const Cordic &cd, float tau_l, float tau_h, int use_miss,
+                               int use_hit, float d0, const Records &rec, uint32_t *block_count,
+                               uint32_t *block_pairs, void *workspace, int grid, int sm_count,
+                               cudaStream_t st);
+
 // Euclidean thick rays (hd_euclid.cu): clears the workspace, adds the sets
 // A_i(d0) = {v : centre of v within d0 mm of L_i} of n histories to N and M
 // (either may be null when its class is not used), and, when `stats` is not

@@ -4,6 +4,7 @@
 // its private tile into N or M once per part of a bucket (the pairs of one
 // group and tile, sorted in hd_scatter.cu) that it has walked; warps refill
 // idle lanes from the parts' pairs, so lanes do not wait for the longest path.
+#include "hd_euclid.cuh"
 #include "hd_fallback.cuh"
 
 namespace hd {
@@ -27,6 +28,11 @@ constexpr int kEventsPerStep = 8;  // events a traversal lane walks between refi
 // the two ends of each run, took two and about three times the integer steps
 // per run: head-sized scan (9e6 histories) 0.683 -> 0.407 ms, large streamed
 // scan 0.288 -> 0.186 ms per chunk, with the balance and the flush below.
+
+// What the kernel of the thin and dilated walks needs besides the scans: nothing.
+struct NoRows {
+    static constexpr bool kRows = false;
+};
 
 // Shared-memory reduction (no value returned) at a shared-space byte address.
 __device__ __forceinline__ void smem_red_add(int addr, uint32_t v)
@@ -84,15 +90,18 @@ struct TilePart {
 
 __device__ __forceinline__ int slot_rows(int count) { return (count + 32 * kCols - 1) / (32 * kCols); }
 
-// A lane's next walk, loaded ahead.
+// A lane's next walk, loaded ahead: kVec 16-byte words per pair.
+template <int kVec>
 struct NextWalk {
-    uint4 a, b;
+    uint4 v[kVec];
     int base;  // its tile's offset in bytes
     bool have;
+    bool walk;  // false: a slot past its bucket's pairs
 };
 
 // The walk in slot r of the group of `n` parts: none past the pairs of a part.
-__device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, NextWalk &nw)
+template <int kVec>
+__device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, NextWalk<kVec> &nw)
 {
     int j = 0;
     while (j + 1 < n && r >= parts[j + 1].slot0) ++j;
@@ -101,17 +110,18 @@ __device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, N
     const int v = p >> 5;
     const int k = 32 * ((v & (kCols - 1)) * slot_rows(t.count) + v / kCols) + (p & 31);
     nw.base = 4 * t.offset;
-    if (k < t.count) {
-        nw.a = __ldg(t.first_pair + 2 * static_cast<size_t>(k));
-        nw.b = __ldg(t.first_pair + 2 * static_cast<size_t>(k) + 1);
-    } else {
-        nw.b.w = 0x80000000u;
+    nw.walk = k < t.count;
+    if (nw.walk) {
+#pragma unroll
+        for (int q = 0; q < kVec; ++q) nw.v[q] = __ldg(t.first_pair + kVec * static_cast<size_t>(k) + q);
     }
 }
 
 // The first walks of a group of `total` slots, a lane its own slot.  Loaded
 // before the flush that precedes them, which hides their latency.
-__device__ __forceinline__ void first_walks(const TilePart *parts, int n, int total, NextWalk &nw)
+template <int kVec>
+__device__ __forceinline__ void first_walks(const TilePart *parts, int n, int total,
+                                            NextWalk<kVec> &nw)
 {
     nw.have = static_cast<int>(threadIdx.x) < total;
     if (nw.have) load_slot(parts, n, static_cast<int>(threadIdx.x), nw);
@@ -126,7 +136,8 @@ __device__ __forceinline__ void first_walks(const TilePart *parts, int n, int to
 // are the lanes' own, see first_walks).  Between refills the warp only counts
 // events.  Out of line, so that nothing else in the kernel takes its registers.
 __device__ __noinline__ void walk_parts(uint32_t *tiles, int thick, const TilePart *parts, int n,
-                                        int total, int refill, unsigned *s_next, NextWalk nw)
+                                        int total, int refill, unsigned *s_next,
+                                        NextWalk<2> nw, const ScanDesc &, const NoRows &)
 {
     const unsigned lane = threadIdx.x & 31u;
     const int sbase = static_cast<int>(__cvta_generic_to_shared(tiles));
@@ -143,10 +154,10 @@ __device__ __noinline__ void walk_parts(uint32_t *tiles, int thick, const TilePa
                 if (unmarked) smem_red_add(event_end(c, thick4), 0xffff0000u);
                 unmarked = false;
                 if (nw.have) {
-                    const uint32_t o[kLeanWords] = {nw.a.x, nw.a.y, nw.a.z, nw.a.w,
-                                                    nw.b.x, nw.b.y, nw.b.z, nw.b.w};
-                    int first;
-                    unmarked = event_start(o, sbase + nw.base, c, first);
+                    const uint32_t o[kLeanWords] = {nw.v[0].x, nw.v[0].y, nw.v[0].z, nw.v[0].w,
+                                                    nw.v[1].x, nw.v[1].y, nw.v[1].z, nw.v[1].w};
+                    int first = 0;
+                    if (nw.walk) unmarked = event_start(o, sbase + nw.base, c, first);
                     if (unmarked) smem_red_add(first, 65536u);
                     nw.have = false;
                 }
@@ -168,6 +179,105 @@ __device__ __noinline__ void walk_parts(uint32_t *tiles, int thick, const TilePa
 #pragma unroll
         for (int u = 0; u < kEventsPerStep; ++u) event_step(c, u, cnt);
         c.left -= cnt;
+    }
+}
+
+// One row of a slice walk (slice_row): its interval's +1 and -1 in the row at
+// `at` (a byte address less 4 kWhole's bits, so that the whole_up form of an
+// index is added to it directly); nothing unless `on`.
+__device__ __forceinline__ void row_step(int at, float lo, float hi, bool on)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        ".reg .b32 a, b;\n\t"
+        "setp.ne.s32 p, %3, 0;\n\t"
+        "shl.b32 a, %1, 2;\n\t"
+        "shl.b32 b, %2, 2;\n\t"
+        "add.s32 a, a, %0;\n\t"
+        "add.s32 b, b, %0;\n\t"
+        "@p red.shared.add.u32 [a], 1;\n\t"
+        "@p red.shared.add.u32 [b+4], -1;\n\t"
+        "}" ::"r"(at),
+        "r"(__float_as_int(lo)), "r"(__float_as_int(hi)), "r"(on ? 1 : 0)
+        : "memory");
+}
+
+constexpr int kRowsPerStep = 4;  // rows a lane takes between refill checks
+
+// walk_parts for Euclidean thick rays: a lane takes the rows of one history in
+// one slice, one after the other, each a closed form of about 35 instructions
+// (slice_row) and two shared atomics.  The rows the closed form leaves open go
+// to the scan's list, or are searched at once when that is full.
+__device__ __noinline__ void walk_parts(uint32_t *tiles, int, const TilePart *parts, int n, int total,
+                                        int refill, unsigned *s_next, NextWalk<3> nw,
+                                        const ScanDesc &d, const RowsArgs &ra)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    const int sbase = static_cast<int>(__cvta_generic_to_shared(tiles)) -
+                      static_cast<int>(0x4B400000u << 2);
+    SliceRows c{};
+    float i = 0.0f, top = 0.0f;
+    int left = 0, at = 0, step = 0;
+    uint32_t slot = 0, code = 0;
+    for (;;) {
+        const unsigned idle = __ballot_sync(kFull, left == 0);
+        if (__popc(idle) >= refill) {
+            const unsigned want = __ballot_sync(kFull, left == 0 && nw.have);
+            if (left == 0 && nw.have) {
+                if (nw.walk) {
+                    c.e0 = __uint_as_float(nw.v[0].x);
+                    c.ea = __uint_as_float(nw.v[0].y);
+                    c.f0 = __uint_as_float(nw.v[0].z);
+                    c.fa = __uint_as_float(nw.v[0].w);
+                    c.Kr = __uint_as_float(nw.v[1].x);
+                    c.E0 = __uint_as_float(nw.v[1].y);
+                    c.Kd = __uint_as_float(nw.v[1].z);
+                    c.dq = __uint_as_float(nw.v[1].w);
+                    left = static_cast<int>(nw.v[2].x >> 16);
+                    at = sbase + nw.base + 4 * static_cast<int>(nw.v[2].x & 0xffffu);
+                    top = __int_as_float(0x4B400000 + static_cast<int>(nw.v[2].y & 0xffffu) - 1);
+                    step = 4 * static_cast<int>(nw.v[2].y >> 16);
+                    slot = nw.v[2].z;
+                    code = nw.v[2].w;
+                    i = 0.0f;
+                }
+                nw.have = false;
+            }
+            if (want != 0) {
+                unsigned base = 0;
+                if (lane == 0) base = atomicAdd(s_next, __popc(want));
+                base = __shfl_sync(kFull, base, 0);
+                if (want & (1u << lane)) {
+                    const unsigned r = base + __popc(want & ((1u << lane) - 1u));
+                    nw.have = r < static_cast<unsigned>(total);
+                    if (nw.have) load_slot(parts, n, static_cast<int>(r), nw);
+                }
+            } else if (idle == kFull) {
+                break;
+            }
+        }
+        const int cnt = min(left, kRowsPerStep);
+        unsigned open = 0;  // rows of this step left to the exact search
+#pragma unroll
+        for (int u = 0; u < kRowsPerStep; ++u) {
+            float lo, hi;
+            const bool sure = slice_row(c, i, top, lo, hi);
+            const bool on = u < cnt;
+            row_step(at, lo, hi, on && sure && lo <= hi);
+            if (on && !sure) open |= 1u << u;
+            i += 1.0f;
+            at += step;
+        }
+        left -= cnt;
+        while (open != 0) {
+            const int u = __ffs(open) - 1;
+            open &= open - 1;
+            const uint32_t row = code + static_cast<uint32_t>(static_cast<int>(i) - kRowsPerStep + u);
+            const unsigned k = atomicAdd(&d.ctrl->n_pair_fallback, 1u);
+            if (k < d.pairs.fb_cap) d.pairs.fb[k] = make_uint2(slot, row);
+            else exact_row(ra, d, slot, row);
+        }
     }
 }
 
@@ -232,8 +342,9 @@ struct FlushTo {
 // lie, SP + SE' - SE is one three-operand sum of the words), written back as a
 // count, and read, cleared and added to the volume by lanes along x: about 100
 // instructions per 200-voxel row, where separate prefix, decode and clear
-// passes took 240 (issue-bound: 21 000 to 9 000 cycles per 200 x 200 tile).
-template <int kPer>
+// passes took 240.  kPlain: the words are difference counts along the rows, and
+// their prefix sums the counts (Euclidean thick rays).
+template <int kPer, bool kPlain>
 __device__ __noinline__ void flush_rows(uint32_t *tile, int dx, int dy, int dz, bool ymaj, int s,
                                         int W, FlushTo to)
 {
@@ -250,7 +361,7 @@ __device__ __noinline__ void flush_rows(uint32_t *tile, int dx, int dy, int dz, 
 #pragma unroll
     for (int k = 0; k < kPer; ++k) pv[k] = 0u;
     // the row before the band belongs to another warp, which overwrites it
-    if (a < e && i != i0) row_prefix<kPer>(tile + W * (r - s), W, W * (rows - (r - s)), pv);
+    if (!kPlain && a < e && i != i0) row_prefix<kPer>(tile + W * (r - s), W, W * (rows - (r - s)), pv);
     __syncthreads();
     for (int n = a; n < e; ++n, r += s) {
         uint32_t *row = tile + W * r;
@@ -267,7 +378,7 @@ __device__ __noinline__ void flush_rows(uint32_t *tile, int dx, int dy, int dz, 
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
             const int m = lane * kPer + k;
-            const uint32_t c = ((v[k] >> 16) + pv[k] - left) & 0xffffu;
+            const uint32_t c = kPlain ? v[k] : ((v[k] >> 16) + pv[k] - left) & 0xffffu;
             left = v[k];
             pv[k] = v[k];
             if (m < W) row[m] = m < nmaj ? c : 0u;
@@ -350,7 +461,9 @@ __device__ __forceinline__ int thick_count(const uint32_t *row, int W, int m, in
 }
 
 // Flush of dilated walks, and of rows longer than flush_rows takes: prefix
-// sums in place, each voxel's count from its neighbours' words, then clearing.
+// sums in place, each voxel's count from its neighbours' words (or its own,
+// kPlain), then clearing.
+template <bool kPlain>
 __device__ __noinline__ void flush_general(uint32_t *tile, int dx, int dy, int dz, bool ymaj, int s,
                                            int W, int thick, FlushTo to)
 {
@@ -367,8 +480,9 @@ __device__ __noinline__ void flush_general(uint32_t *tile, int dx, int dy, int d
         const uint32_t *line = tile + my * y + W * nminor * z;
         for (int x = lane; x < dx; x += 32) {
             const int i = ymaj ? x : y, m = ymaj ? y : x;
-            add_count(out + x, static_cast<uint32_t>(thick_count(line + mx * x - m, W, m, nmaj, i,
-                                                                 nminor, s, thick)));
+            add_count(out + x, kPlain ? line[mx * x]
+                                      : static_cast<uint32_t>(thick_count(
+                                            line + mx * x - m, W, m, nmaj, i, nminor, s, thick)));
         }
     }
     __syncthreads();
@@ -380,6 +494,7 @@ __device__ __noinline__ void flush_general(uint32_t *tile, int dx, int dy, int d
 
 // Adds the tile's counts to the volume (one global atomic per nonzero voxel,
 // lanes along x whichever axis the rows follow) and clears it for the next job.
+template <bool kPlain>
 __device__ __forceinline__ void flush_tile(uint32_t *tile, int dx, int dy, int dz, int type,
                                            int thick, uint32_t *vol, int nx, int ny, int x0,
                                            int y0, int z0)
@@ -390,12 +505,12 @@ __device__ __forceinline__ void flush_tile(uint32_t *tile, int dx, int dy, int d
     const int W = tile_row_words(nmaj, nminor);
     const FlushTo to{vol + x0 + static_cast<long long>(nx) * (y0 + static_cast<long long>(ny) * z0),
                      nx, ny};
-    if (thick > 0 || W > 32 * 13) flush_general(tile, dx, dy, dz, ymaj, s, W, thick, to);
-    else if (W <= 32 * 3) flush_rows<3>(tile, dx, dy, dz, ymaj, s, W, to);
-    else if (W <= 32 * 5) flush_rows<5>(tile, dx, dy, dz, ymaj, s, W, to);
-    else if (W <= 32 * 7) flush_rows<7>(tile, dx, dy, dz, ymaj, s, W, to);
-    else if (W <= 32 * 9) flush_rows<9>(tile, dx, dy, dz, ymaj, s, W, to);
-    else flush_rows<13>(tile, dx, dy, dz, ymaj, s, W, to);
+    if ((!kPlain && thick > 0) || W > 32 * 13) flush_general<kPlain>(tile, dx, dy, dz, ymaj, s, W, thick, to);
+    else if (W <= 32 * 3) flush_rows<3, kPlain>(tile, dx, dy, dz, ymaj, s, W, to);
+    else if (W <= 32 * 5) flush_rows<5, kPlain>(tile, dx, dy, dz, ymaj, s, W, to);
+    else if (W <= 32 * 7) flush_rows<7, kPlain>(tile, dx, dy, dz, ymaj, s, W, to);
+    else if (W <= 32 * 9) flush_rows<9, kPlain>(tile, dx, dy, dz, ymaj, s, W, to);
+    else flush_rows<13, kPlain>(tile, dx, dy, dz, ymaj, s, W, to);
 }
 
 // The pairs without an event walk (the fallback lists), walked with the general
@@ -427,6 +542,7 @@ __device__ __noinline__ void walk_fallback_lists(const ScanDesc *__restrict__ de
 // marks and loads), and for its flush kFlushCost per word of the tile and
 // kPartCost besides (fits over the parts of the head-sized and the large
 // streamed scan).
+// For Euclidean thick rays the events are rows, each about five times the work.
 constexpr unsigned kPairCost = 9, kFlushCost = 4, kPartCost = 10000;
 constexpr int kPartList = 32;  // parts a block lists at a time
 
@@ -440,12 +556,12 @@ struct BucketCost {
     unsigned count;
 };
 
-__device__ __forceinline__ BucketCost bucket_cost(const ScanDesc &d, int t)
+__device__ __forceinline__ BucketCost bucket_cost(const ScanDesc &d, int t, bool rows)
 {
     BucketCost b;
     b.count = d.buckets.count[t];
     b.cost = b.count == 0 ? 0ull
-                          : d.buckets.events[t] +
+                          : (rows ? 5ull : 1ull) * d.buckets.events[t] +
                                 static_cast<unsigned long long>(kPairCost) * b.count +
                                 flush_cost(d.tp.tile_words);
     return b;
@@ -501,10 +617,12 @@ __device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long lo
 // shared-memory tile and flushed; then the blocks walk the fallback lists.
 // smem_words: the dynamic shared memory of the launch, at least the
 // largest tile of the scans.
-template <int kThreads>
+template <int kThreads, class RowsT>
 __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
-    const ScanDesc *__restrict__ descs, int nscans, int smem_words)
+    const ScanDesc *__restrict__ descs, int nscans, int smem_words, const RowsT ra)
 {
+    constexpr bool kRows = RowsT::kRows;
+    constexpr int kVec = kRows ? kSliceWords / 4 : kLeanWords / 4;
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ unsigned s_next;
     __shared__ int s_first[kMaxBatch + 1];
@@ -538,7 +656,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         }
     };
     unsigned long long mine = 0, total;
-    each([&](int k, int t) { mine += bucket_cost(descs[k], t).cost; });
+    each([&](int k, int t) { mine += bucket_cost(descs[k], t, kRows).cost; });
     const unsigned long long before = block_excl_scan64(mine, s_warp, total);
     // the block's stretch: an equal share, but worth about two flushes
     unsigned long long blocks = total / (2ull * flush_cost(descs[0].tp.tile_words)) + 1ull;
@@ -551,7 +669,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         unsigned long long p = before;
         each([&](int k, int t) {
             const ScanDesc &d = descs[k];
-            const BucketCost b = bucket_cost(d, t);
+            const BucketCost b = bucket_cost(d, t, kRows);
             if (b.cost != 0 && p < x1 && p + b.cost > x0) {
                 const int s0 = x0 > p ? boundary_slot(b, d.tp.tile_words, p, x0) : 0;
                 const int s1 = x1 < p + b.cost ? boundary_slot(b, d.tp.tile_words, p, x1)
@@ -573,7 +691,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
                 if (r >= j0 && r < j0 + kPartList) {
                     TilePart &j = s_parts[r - j0];
                     const ScanDesc &d = descs[k];
-                    j.first_pair = d.pairs.v + 2 * static_cast<size_t>(d.buckets.first[t]);
+                    j.first_pair = d.pairs.v + kVec * static_cast<size_t>(d.buckets.first[t]);
                     j.scan = k;
                     j.tile = t % d.tp.ntiles;
                     j.group = t / d.tp.ntiles;
@@ -608,16 +726,15 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         }
         __syncthreads();
         const int ngroups = s_ngroups;
-        NextWalk nw;
-        nw.a = nw.b = make_uint4(0, 0, 0, 0);
-        nw.base = 0;
+        NextWalk<kVec> nw{};
         first_walks(s_parts, s_group[1], s_slots[0], nw);
         for (int g = 0; g < ngroups; ++g) {
             const int q0 = s_group[g], q1 = s_group[g + 1];
             if (threadIdx.x == 0) s_next = blockDim.x;
             __syncthreads();
             const TilePlan &tp0 = descs[s_parts[q0].scan].tp;
-            walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, &s_next, nw);
+            walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, &s_next, nw,
+                       descs[s_parts[q0].scan], ra);
             if (g + 1 < ngroups)
                 first_walks(s_parts + q1, s_group[g + 2] - q1, s_slots[g + 1], nw);
             __syncthreads();
@@ -629,14 +746,14 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
                 const int tiy = (j.tile / tp.ntx) % tp.nty;
                 const int tiz = j.tile / (tp.ntx * tp.nty);
                 const int bx = tix * tp.tx, by = tiy * tp.ty, bz = tiz * tp.tz;
-                flush_tile(tile + j.offset, min(tp.tx, tp.nx - bx), min(tp.ty, tp.ny - by),
+                flush_tile<kRows>(tile + j.offset, min(tp.tx, tp.nx - bx), min(tp.ty, tp.ny - by),
                            min(tp.tz, tp.nz - bz), j.group >> 1, tp.thick,
                            (j.group & 1) == 0 ? d.N : d.M, tp.nx, tp.ny, bx, by, bz);
             }
         }
         __syncthreads();
     }
-    walk_fallback_lists(descs, nscans);
+    if (!kRows) walk_fallback_lists(descs, nscans);
 }
 
 // Shared memory of a launch whose largest tile has this many words: room for
@@ -652,15 +769,18 @@ int occupancy_of(int smem_words)
 {
     // allow the largest tile once, so launches (also inside graph capture)
     // need no attribute change
-    if (cudaFuncSetAttribute(trace_tiles_kernel<kThreads>,
+    if (cudaFuncSetAttribute(trace_tiles_kernel<kThreads, NoRows>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
-        cudaSuccess) {
+            cudaSuccess ||
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, RowsArgs>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
+            cudaSuccess) {
         cudaGetLastError();
         return 0;
     }
     int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, trace_tiles_kernel<kThreads>, kThreads,
-                                                      static_cast<size_t>(smem_words) * 4) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, trace_tiles_kernel<kThreads, NoRows>,
+                                                      kThreads, static_cast<size_t>(smem_words) * 4) !=
         cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -680,8 +800,9 @@ int trace_tiles_occupancy(int tile_words, int threads)
     }
 }
 
-cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
-                               int grid, cudaStream_t s)
+template <class RowsT>
+static cudaError_t launch_trace(const ScanDesc *descs, int nscans, int tile_words, int threads,
+                                int grid, const RowsT &ra, cudaStream_t s)
 {
     if (nscans < 1 || nscans > kMaxBatch || tile_words * 4 > kTileSmemBytes)
         return cudaErrorInvalidValue;
@@ -689,20 +810,32 @@ cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words
     const size_t smem = static_cast<size_t>(smem_words) * 4;
     switch (threads) {
     case 256:
-        trace_tiles_kernel<256><<<grid, 256, smem, s>>>(descs, nscans, smem_words);
+        trace_tiles_kernel<256, RowsT><<<grid, 256, smem, s>>>(descs, nscans, smem_words, ra);
         break;
     case 512:
-        trace_tiles_kernel<512><<<grid, 512, smem, s>>>(descs, nscans, smem_words);
+        trace_tiles_kernel<512, RowsT><<<grid, 512, smem, s>>>(descs, nscans, smem_words, ra);
         break;
     case 768:
-        trace_tiles_kernel<768><<<grid, 768, smem, s>>>(descs, nscans, smem_words);
+        trace_tiles_kernel<768, RowsT><<<grid, 768, smem, s>>>(descs, nscans, smem_words, ra);
         break;
     case 1024:
-        trace_tiles_kernel<1024><<<grid, 1024, smem, s>>>(descs, nscans, smem_words);
+        trace_tiles_kernel<1024, RowsT><<<grid, 1024, smem, s>>>(descs, nscans, smem_words, ra);
         break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
+}
+
+cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
+                               int grid, cudaStream_t s)
+{
+    return launch_trace(descs, nscans, tile_words, threads, grid, NoRows{}, s);
+}
+
+cudaError_t launch_trace_rows(const ScanDesc *desc, int tile_words, int threads, int grid,
+                              const RowsArgs &ra, cudaStream_t s)
+{
+    return launch_trace(desc, 1, tile_words, threads, grid, ra, s);
 }
 
 }  // namespace hd

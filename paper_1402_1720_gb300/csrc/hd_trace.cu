@@ -19,18 +19,12 @@
 // just after t, so a mixed tie visits the corner voxel between the two.
 // The walk starts at the parameter where the segment enters the grid box
 // (exact rational), so voxels outside the grid cost nothing.
+#include "hd_admit.cuh"
 #include "hd_fallback.cuh"
 
 namespace hd {
 
 namespace {
-
-__device__ __forceinline__ unsigned warp_sum_u32(unsigned v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // ------------------------------------------------------------------ ingest
 
@@ -91,26 +85,8 @@ __device__ __forceinline__ int ingest_one(const GeomQ &g, const Cordic &cd, floa
 }
 
 
-__device__ __forceinline__ unsigned warp_incl_scan(unsigned v)
-{
-    const unsigned lane = threadIdx.x & 31u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= static_cast<unsigned>(o)) v += t;
-    }
-    return v;
-}
-
-// Decide the path of each lane's record (tiled within the block's pair
-// budget, else global), count its tiles in the block histogram, list its
-// pairs in the block's share of stage, and write it at its history's slot
-// i (when i < i1; cls 0: no record).  Budget reservations are per warp on a
-// shared-memory counter, so the block never waits at a barrier.  The pairs
-// the budget admits fill the list from its start without gaps: the
-// reservations tile [0, total) in the order of their ends, and only the one
-// record that straddles the budget, and the records after it, are turned
-// away (they take the global path, exact either way).
+// The path of each lane's record and its place in the pair list (see
+// reserve_and_write), from the tiles its segment can touch.
 __device__ __forceinline__ void admit_and_write(const TilePlan &tp, const Records &rec,
                                                 Ctrl *ctrl, uint32_t *s_hist, unsigned *s_demand,
                                                 unsigned budget, int64_t h0, int64_t i,
@@ -118,76 +94,34 @@ __device__ __forceinline__ void admit_and_write(const TilePlan &tp, const Record
                                                 int32_t r[6])
 {
     const int type = orient_record(r);
-    int tcount = 0;
+    int c = 0;
     int zlo = 0, zhi = 0;
-    bool ok = false;
-    if (cls != 0) {
-        int c = 0;
-        if (grid_z_range(tp, r, zlo, zhi)) {
-            if (tp.ntx == 1 && tp.nty == 1) {
-                // whole-plane tiles: the part inside the grid's x-y extent
-                // meets every plane tile of its slices
-                const unsigned m = tp.mtz;
-                const int t0 = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zlo), m)) : zlo;
-                const int t1 = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zhi), m)) : zhi;
-                c = t1 - t0 + 1;
-            } else {
-                int lo[3], hi[3];
-                c = tile_range_z(tp, r, zlo, zhi, lo, hi);
-            }
-        }
-        ok = c != 0;  // else no voxel of the grid: nothing to traverse
-        tcount = (tp.ntiles > 0 && c <= tp.max_tiles) ? c : -1;
-    }
-    const unsigned demand = ok && tcount > 0 ? static_cast<unsigned>(tcount) : 0u;
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned incl = warp_incl_scan(demand);
-    const unsigned tot = __shfl_sync(0xffffffffu, incl, 31);
-    unsigned wbase = 0;
-    if (lane == 31 && tot) wbase = atomicAdd(s_demand, tot);
-    wbase = __shfl_sync(0xffffffffu, wbase, 31);
-    const unsigned long long end = static_cast<unsigned long long>(wbase) + incl;
-    const int path = ok ? (demand > 0 && end <= budget ? 1 : 2) : 0;
-    if (rec.glist) {
-        // the global path's list: one counter update per warp
-        const unsigned gm = __ballot_sync(0xffffffffu, path == 2);
-        if (gm) {
-            const int lead = __ffs(gm) - 1;
-            unsigned gb = 0;
-            if (static_cast<int>(lane) == lead) gb = atomicAdd(&ctrl->n_global, __popc(gm));
-            gb = __shfl_sync(0xffffffffu, gb, lead);
-            if (path == 2) rec.glist[gb + __popc(gm & ((1u << lane) - 1u))] = static_cast<int32_t>(i);
-        }
-    }
-    if (i >= i1) return;
-    int32_t st = 0;
-    if (ok) {
-        st = record_status(path, cls - 1, type, zlo, zhi);
-        if (path == 1) {
+    if (cls != 0 && grid_z_range(tp, r, zlo, zhi)) {
+        if (tp.ntx == 1 && tp.nty == 1) {
+            // whole-plane tiles: the part inside the grid's x-y extent
+            // meets every plane tile of its slices
+            const unsigned m = tp.mtz;
+            const int t0 = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zlo), m)) : zlo;
+            const int t1 = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zhi), m)) : zhi;
+            c = t1 - t0 + 1;
+        } else {
             int lo[3], hi[3];
-            if (tp.ntx == 1 && tp.nty == 1) {
-                const unsigned m = tp.mtz;
-                lo[0] = hi[0] = lo[1] = hi[1] = 0;
-                lo[2] = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zlo), m)) : zlo;
-                hi[2] = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zhi), m)) : zhi;
-            } else {
-                tile_range_z(tp, r, zlo, zhi, lo, hi);
-            }
-            const int off = (cls - 1 + 2 * type) * tp.ntiles;
-            for (int z = lo[2]; z <= hi[2]; ++z)
-                for (int y = lo[1]; y <= hi[1]; ++y)
-                    for (int x = lo[0]; x <= hi[0]; ++x)
-                        atomicAdd(&s_hist[off + x + tp.ntx * (y + tp.nty * z)], 1u);
-            // the record's pairs hold positions end - c .. end - 1 of the
-            // block's list (all below its budget)
-            const uint32_t code = static_cast<uint32_t>(i - h0) << kRecordTileBits;
-            const unsigned first = static_cast<unsigned>(end) - demand;
-            for (int j = 0; j < tcount; ++j) stage[first + j] = code | static_cast<uint32_t>(j);
+            c = tile_range_z(tp, r, zlo, zhi, lo, hi);
         }
-#pragma unroll
-        for (int a = 0; a < 6; ++a) rec.g[a][i] = r[a];
     }
-    rec.status[i] = st;
+    // no tile: no voxel of the grid, nothing to traverse
+    const int tcount = tp.ntiles > 0 && c <= tp.max_tiles ? c : -1;
+    reserve_and_write(tp, rec, ctrl, s_hist, s_demand, budget, h0, i, i1, stage, cls - 1, type,
+                      c != 0, tcount, zlo, zhi, r, [&](int lo[3], int hi[3]) {
+                          if (tp.ntx == 1 && tp.nty == 1) {
+                              const unsigned m = tp.mtz;
+                              lo[0] = hi[0] = lo[1] = hi[1] = 0;
+                              lo[2] = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zlo), m)) : zlo;
+                              hi[2] = m ? static_cast<int>(umulhi32(static_cast<unsigned>(zhi), m)) : zhi;
+                          } else {
+                              tile_range_z(tp, r, zlo, zhi, lo, hi);
+                          }
+                      });
 }
 
 // One block per range of the chunk split.  Inputs in device memory: one
@@ -286,16 +220,7 @@ __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
         if (a4) atomicAdd(&ctrl->n_reject, static_cast<unsigned long long>(a4));
     }
     if (block_count == nullptr) return;
-    __syncthreads();
-    unsigned mine = 0;
-    for (int t = threadIdx.x; t < nh; t += blockDim.x) {
-        block_count[static_cast<size_t>(t) * gridDim.x + blockIdx.x] = s_hist[t];
-        mine += s_hist[t];
-    }
-    mine = warp_sum_u32(mine);
-    if ((threadIdx.x & 31u) == 0 && mine) atomicAdd(&s_total, mine);
-    __syncthreads();
-    if (threadIdx.x == 0) block_pairs[blockIdx.x] = s_total;
+    write_block_counts(nh, s_hist, &s_total, block_count, block_pairs);
 }
 
 // ---------------------------------------------------------------- traversal
