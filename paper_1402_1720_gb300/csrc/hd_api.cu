@@ -52,6 +52,9 @@ struct DeviceGuard {
 constexpr int64_t kChunk = int64_t(1) << 25;  // histories per internal launch sequence
 // a block's slot offsets (below the chunk size) fit a pair-list entry
 static_assert(kChunk <= (int64_t(1) << (32 - hd::kRecordTileBits)), "pair-list entry width");
+// Words of a pair of Euclidean thick rays: its rows, a word of the list of open
+// rows (two words per entry) and one of the blocks' pair lists.
+constexpr int64_t kEuclidPairWords = hd::kSliceWords + 2;
 constexpr int64_t kMaxScanHistories = 4294967295LL;
 
 // theta_i = round(atan(2^-i) * 180/pi * 2^30), K = round(2^30 prod (1 + 2^-2i)^-1/2),
@@ -124,6 +127,7 @@ struct hd_scan {
     int trace_grid = 0;
     int32_t *rec_buf = nullptr;   // 8 int32 arrays of rec_cap (coordinates, status, global list)
     int64_t rec_cap = 0;
+    int64_t pair_words = 0;        // of pair_buf
     uint32_t *pair_buf = nullptr;  // lean walks (kLeanWords per pair), then the fallback list
     hd::ScanDesc *desc_dev = nullptr;  // this scan's traversal descriptor
     hd::ScanDesc desc_host{};
@@ -258,8 +262,24 @@ hd_status ensure_records(hd_scan *s, int64_t n, cudaStream_t st)
                                           static_cast<size_t>(hd::records_stride(n))) == cudaSuccess;
     if (ok && s->tp.ntiles > 0) {
         const int64_t pair_cap = pairs_per_record(s->tp) * n;
-        ok = cudaMalloc(&s->pair_buf, sizeof(uint32_t) * (hd::kLeanWords + 3) *
-                                          static_cast<size_t>(pair_cap)) == cudaSuccess;
+        s->pair_words = (hd::kLeanWords + 3) * pair_cap;
+        if (s->euclid_pairs > 0) {
+            // one chunk's pairs when they are not too many (16 M: 0.9 GB)
+            const int64_t want = (s->euclid_pairs * n < (int64_t(1) << 24) ? s->euclid_pairs * n + 4
+                                                                           : int64_t(1) << 24) *
+                                     kEuclidPairWords +
+                                 hd::kOpenLists;
+            if (want > s->pair_words) s->pair_words = want;
+        }
+        ok = cudaMalloc(&s->pair_buf, sizeof(uint32_t) * static_cast<size_t>(s->pair_words)) ==
+             cudaSuccess;
+        if (!ok && s->pair_words > (hd::kLeanWords + 3) * pair_cap) {
+            // smaller chunks
+            cudaGetLastError();
+            s->pair_words = (hd::kLeanWords + 3) * pair_cap;
+            ok = cudaMalloc(&s->pair_buf, sizeof(uint32_t) * static_cast<size_t>(s->pair_words)) ==
+                 cudaSuccess;
+        }
         s->tp.pair_cap = pair_cap;
     }
     if (!ok) {
@@ -342,13 +362,11 @@ size_t tile_count_words(const hd_scan *s)
     return cols * (1 + ingest_blocks_max(s)) + ingest_blocks_max(s);
 }
 
-// Pairs of Euclidean thick rays that the pair buffer holds: kSliceWords words
-// each, a word of the list of open rows (two words per entry) and one of the
-// blocks' pair lists.
+// Pairs of Euclidean thick rays that the pair buffer holds.
 int64_t euclid_pair_cap(const hd_scan *s)
 {
-    const int64_t words = (hd::kLeanWords + 3) * static_cast<int64_t>(s->tp.pair_cap);
-    return words / (hd::kSliceWords + 2) & ~int64_t(3);
+    const int64_t c = (s->pair_words - hd::kOpenLists) / kEuclidPairWords & ~int64_t(3);
+    return c > 0 ? c : 0;
 }
 
 hd::Pairs pairs_of(const hd_scan *s)
@@ -362,12 +380,15 @@ hd::Pairs pairs_of(const hd_scan *s)
     p.fb = base ? reinterpret_cast<uint2 *>(base + hd::kLeanWords * cap) : nullptr;
     p.stage = base ? base + (hd::kLeanWords + 2) * cap : nullptr;
     p.fb_cap = 0;
+    p.fb_count = nullptr;
     if (s->euclid_pairs > 0) {
         // Euclidean thick rays: the same buffer in their layout
         const size_t c = static_cast<size_t>(euclid_pair_cap(s));
+        const int lists = s->trace_grid > 0 ? s->trace_grid : 1;
         p.fb = base ? reinterpret_cast<uint2 *>(base + hd::kSliceWords * c) : nullptr;
-        p.fb_cap = static_cast<uint32_t>(c / 2);
+        p.fb_cap = static_cast<uint32_t>(c / 2 / static_cast<size_t>(lists));
         p.stage = base ? base + (hd::kSliceWords + 1) * c : nullptr;
+        p.fb_count = base ? base + (hd::kSliceWords + 2) * c : nullptr;
     }
     return p;
 }
@@ -538,12 +559,13 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
 {
     if (s->euclid_d0 > 0.0f) {
         const uint32_t m = s->params.methods;
-        if (s->euclid_pairs > 0 && s->trace_grid > 0) {
+        if (s->euclid_pairs > 0 && s->trace_grid > 0 && s->trace_grid <= hd::kOpenLists) {
             // Euclidean thick rays on the tiled path, in chunks whose pairs
             // fit the buffer
             hd_status r = upload_desc(s, st);
             if (r != HD_OK) return r;
-            const int64_t most = euclid_pair_cap(s) / s->euclid_pairs & ~int64_t(3);
+            int64_t most = euclid_pair_cap(s) / s->euclid_pairs & ~int64_t(3);
+            if (most > (int64_t(1) << 23)) most = int64_t(1) << 23;  // a slot's bits in open_code
             const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
             uint32_t *block_count = s->tile_count + cols;
             uint32_t *block_pairs = block_count + cols * ingest_blocks_max(s);

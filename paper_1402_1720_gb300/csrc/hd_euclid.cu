@@ -14,7 +14,7 @@
 // records without the closed form (trackers inside the grid, axis-parallel
 // paths, too many tiles) to the kernel below, which the standalone
 // accumulation and other plans use for every history.  Head-sized scan,
-// 2.7e6 histories, d_0 = 2.5 mm, all hulls: 12.46 -> 2.22 ms.
+// 2.7e6 histories, d_0 = 2.5 mm, all hulls: 12.46 -> 1.46 ms.
 //
 // euclid_kernel.  A warp takes groups of 32 consecutive histories (so each lane's
 // gantry cos/sin rarely change); each lane classifies one history and sets
@@ -373,6 +373,7 @@ __global__ void __launch_bounds__(kSetupThreads, 2) euclid_setup_kernel(
         SliceRows r{};
         if (!slice_rows(ra.g, w, ra.R, k, a0, rows, m0, len, r)) r.n = 0;
         const int W = tile_row_words(len, rows);
+        const unsigned long long open = open_code(static_cast<uint32_t>(slot), a0 + r.row, k, 0, y);
         uint4 *out = pairs.v + (kSliceWords / 4) * static_cast<size_t>(pos);
         out[0] = make_uint4(__float_as_uint(r.e0), __float_as_uint(r.ea), __float_as_uint(r.f0),
                             __float_as_uint(r.fa));
@@ -380,7 +381,8 @@ __global__ void __launch_bounds__(kSetupThreads, 2) euclid_setup_kernel(
                             __float_as_uint(r.dq));
         out[2] = make_uint4(static_cast<uint32_t>(r.row * W) | (static_cast<uint32_t>(r.n) << 16),
                             static_cast<uint32_t>(len) | (static_cast<uint32_t>(W) << 16),
-                            static_cast<uint32_t>(slot), row_code(a0 + r.row, k, y));
+                            static_cast<uint32_t>(open),
+                            static_cast<uint32_t>(open >> 32));
         if (r.n > 0) atomicAdd(&s_events[t], static_cast<uint32_t>(r.n));
     }
     __syncthreads();
@@ -389,15 +391,21 @@ __global__ void __launch_bounds__(kSetupThreads, 2) euclid_setup_kernel(
             atomicAdd(&buckets.events[t], static_cast<unsigned long long>(s_events[t]));
 }
 
-// The rows the tiled pass left to the exact search, a thread each.
+// What the tiled pass left open, a thread each: kOpenParts blocks per part of the
+// list (a block's of that pass).
+constexpr int kOpenParts = 8;
+
 __global__ void __launch_bounds__(128) euclid_open_kernel(const ScanDesc *__restrict__ dp, RowsArgs ra)
 {
     const ScanDesc &d = *dp;
-    const unsigned listed = d.ctrl->n_pair_fallback;
+    const unsigned part = blockIdx.x / kOpenParts;
+    const unsigned listed = d.pairs.fb_count[part];
     const unsigned n = listed < d.pairs.fb_cap ? listed : d.pairs.fb_cap;
-    for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        const uint2 e = d.pairs.fb[k];
-        exact_row(ra, d, e.x, e.y);
+    const uint2 *list = d.pairs.fb + static_cast<size_t>(part) * d.pairs.fb_cap;
+    for (unsigned k = (blockIdx.x % kOpenParts) * blockDim.x + threadIdx.x; k < n;
+         k += kOpenParts * blockDim.x) {
+        const uint2 e = list[k];
+        settle_open(ra, d, e.x, static_cast<int>(e.y));
     }
 }
 
@@ -445,7 +453,7 @@ int euclid_pairs_per_record(const hd_geometry *geom, float d0, const TilePlan &t
 {
     const double k = std::ceil(2.0 * d0 / geom->sz) + 2.0;  // slices of a nearly flat path
     const double p = k * (tp.nty > 2 ? 2 : tp.nty);
-    if (tp.ntiles <= 0 || tp.ntx != 1 || tp.tz != 1 || tp.nty > 256 || 2 * q16_of(d0) < 2 ||
+    if (tp.ntiles <= 0 || tp.ntx != 1 || tp.tz != 1 || tp.nty > kOpenStrips || 2 * q16_of(d0) < 2 ||
         p > kMaxRecordTiles)
         return 0;
     return static_cast<int>(p);
@@ -474,8 +482,7 @@ cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, c
         tp, ra, sp.per_block, desc.buckets, block_count, block_pairs, desc.pairs);
     e = launch_trace_rows(desc_dev, tp.tile_words, tp.threads, grid, ra, st);
     if (e != cudaSuccess) return e;
-    euclid_open_kernel<<<static_cast<unsigned>(sm_count > 0 ? 8 * sm_count : 8), 128, 0, st>>>(desc_dev,
-                                                                                               ra);
+    euclid_open_kernel<<<static_cast<unsigned>(grid * kOpenParts), 128, 0, st>>>(desc_dev, ra);
     // the records of the global path, when there are any
     e = launch_thick_clear(geom, workspace, desc.ctrl, sm_count, st);
     if (e != cudaSuccess) return e;

@@ -46,6 +46,7 @@
 
 #include <cmath>
 #include <cstdint>
+#include <cstring>
 
 #include "hd_geom.cuh"
 
@@ -447,9 +448,9 @@ HD_HD long long floor_div(long long v, long long s)
 // as world_cs gives them) and R = 2 q16(d_0): the doubled endpoints A, B in
 // the permuted frame, whether rows run along y (else x), the index box of
 // the rows that can meet the capsule on axes 1 and 2 ([blo, bhi]; false when
-// empty), and S of the float filter.
+// empty; not computed for null pointers), and S of the float filter.
 HD_HD bool capsule_frame(const GeomQ &g, const long long W[6], long long R, long long A[3],
-                         long long B[3], bool &ymaj, int blo[3], int bhi[3], float &S)
+                         long long B[3], bool &ymaj, int *blo, int *bhi, float &S)
 {
     long long P[3], Q[3];
     for (int q = 0; q < 3; ++q) {
@@ -479,6 +480,7 @@ HD_HD bool capsule_frame(const GeomQ &g, const long long W[6], long long R, long
         s += (w0 > w1 ? w0 : w1) + abs_ll(B[q] - A[q]);
     }
     S = static_cast<float>(s);
+    if (blo == nullptr) return true;
     // index box of the capsule on axes 1 and 2: centres within
     // [min(A, B) - R, max(A, B) + R], widened by one
 #pragma unroll
@@ -588,13 +590,16 @@ HD_HD void k_range(const CapF &cf, int a, int blo2, int bhi2, int &klo, int &khi
 //
 // Certainty (eps = 2^-24).  Per row e is off by at most de = 16 eps (|e_0| +
 // n |e_a|) over the n rows (u, step and the reciprocals each add a rounding or
-// two of their own size: 11 in all), f by at most 16 eps (|f_0| + n |f_a| + 2
-// |A_0 - c_0| / (2 s_0)), so 1 - e^2 is off by at most dq = 4 de + 4 eps for |e|
+// two of their own size: 11 in all), f by at most 16 eps (|f_0| + n |f_a| + |m_0|
+// + |off|) (off the midpoint's index: 3 eps of its own size, and the rest,
+// u_0 g / h^2, 8 eps of at most the sum of the others), so 1 - e^2 is off by at most dq = 4 de + 4 eps for |e|
 // near 1 or less, its root by dq / root, and the ends by E0 + Kd / root in all,
 // E0 the bound for f and 16 eps Kr for the roundings of Kr, of the root and of
-// the ends themselves, Kd = Kr dq.  When both ends give the same index over that
-// range, and 1 - e^2 is above 4 dq (or below -dq: no voxel), the row's voxels
-// are certain; the other rows (about 0.3 %) go to the exact search.
+// the ends themselves, Kd = Kr dq.  With 1 - e^2 above 4 dq the indices that lie
+// inside over that whole range are certain, and those that lie inside over a
+// part of it only, at most one at either end unless the range is wide, take the
+// exact test one by one (about 0.15 % of the rows have one); below -dq the row
+// has no voxel; the few rows in between go to the exact search.
 struct SliceRows {
     float e0, ea;  // e of the first row, and its change per row
     float f0, fa;  // f, in index units of the tile
@@ -672,7 +677,10 @@ HD_HD bool slice_rows(const GeomQ &g, const int32_t W[6], long long R, int k, in
     const bool ymaj = (dy < 0 ? -dy : dy) > (dx < 0 ? -dx : dx);
     const int n0 = ymaj ? g.ny : g.nx, n1 = ymaj ? g.nx : g.ny;
     const int s0 = static_cast<int>(ymaj ? g.sy : g.sx), s1 = static_cast<int>(ymaj ? g.sx : g.sy);
-    const int A0 = 2 * (ymaj ? W[1] : W[0]), A1 = 2 * (ymaj ? W[0] : W[1]), A2 = 2 * W[2];
+    // measured from the segment's midpoint (near the grid, so that f's parts are
+    // no larger than the grid): the doubled coordinates of the ends' sum
+    const int A0 = ymaj ? W[1] + W[4] : W[0] + W[3], A1 = ymaj ? W[0] + W[3] : W[1] + W[4],
+              A2 = W[2] + W[5];
     const int u0 = 2 * (ymaj ? dy : dx), u1 = 2 * (ymaj ? dx : dy), u2 = 2 * (W[5] - W[2]);
     auto mul = [](int a, int b) { return static_cast<long long>(a) * b; };
     const float uf0 = static_cast<float>(u0), uf1 = static_cast<float>(u1),
@@ -728,7 +736,7 @@ HD_HD bool slice_rows(const GeomQ &g, const int32_t W[6], long long R, int k, in
     const float n = static_cast<float>(r.n);
     const float de = 16.0f * kEps * (fabsf(r.e0) + n * fabsf(r.ea));
     r.dq = 4.0f * de + 4.0f * kEps;
-    r.E0 = 16.0f * kEps * (2.0f * fabsf(off) + fabsf(static_cast<float>(m0)) + fabsf(r.f0) +
+    r.E0 = 16.0f * kEps * (fabsf(off) + fabsf(static_cast<float>(m0)) + fabsf(r.f0) +
                            n * fabsf(r.fa) + 1.0f + r.Kr);
     r.Kd = r.Kr * r.dq;
     return true;
@@ -752,6 +760,22 @@ HD_HD float whole_down(float x)
     return std::floor(x) + kWhole;
 #endif
 }
+HD_HD float mul_rn(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fmul_rn(a, b);
+#else
+    return a * b;
+#endif
+}
+HD_HD float add_rn(float a, float b)
+{
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
 HD_HD float rsqrt_est(float x)
 {
 #ifdef __CUDA_ARCH__
@@ -763,65 +787,119 @@ HD_HD float rsqrt_est(float x)
 #endif
 }
 
-// Row i of the slice: its first and last index (whole_up form, cut to the tile's
-// 0 .. len - 1, top = kWhole + len - 1), empty when lo > hi.  False when the row
-// is not certain.
-HD_HD bool slice_row(const SliceRows &r, float i, float top, float &lo, float &hi)
+// Row i of the slice, in whole_up form (kWhole plus the index in the tile): the
+// indices x1 .. y0 are certainly inside, those below x0 and above y1 certainly
+// not.  Returns 1 - e^2: the row has no voxel below -dq, and is open up to 4 dq.
+HD_HD float slice_row(const SliceRows &r, float i, float &x0, float &x1, float &y0, float &y1)
 {
     const float e = fmaf(i, r.ea, r.e0);
     const float q = fmaf(-e, e, 1.0f);
     const float rs = rsqrt_est(fmaxf(q, r.dq));
-    const float hw = r.Kr * (q * rs);
+    // products and sums rounded one by one: every copy of this function in a
+    // kernel gives the same ends
+    const float hw = mul_rn(r.Kr, mul_rn(q, rs));
     const float c = fmaf(i, r.fa, r.f0);
     const float tol = fmaf(r.Kd, rs, r.E0);
     const float big = 1048576.0f;
-    const float x = fminf(fmaxf(c - hw, -big), big), y = fminf(fmaxf(c + hw, -big), big);
-    const float x0 = whole_up(x - tol), x1 = whole_up(x + tol);
-    const float y0 = whole_down(y - tol), y1 = whole_down(y + tol);
-    lo = fmaxf(x0, kWhole);
-    hi = fminf(y0, top);
-    const bool sure = (x0 == x1 && y0 == y1 && q > 4.0f * r.dq) || q < -r.dq;
-    if (q < 0.0f) hi = kWhole - 1.0f;  // the row misses the cylinder
-    return sure;
+    const float x = fminf(fmaxf(add_rn(c, -hw), -big), big);
+    const float y = fminf(fmaxf(add_rn(c, hw), -big), big);
+    x0 = whole_up(add_rn(x, -tol));
+    x1 = whole_up(add_rn(x, tol));
+    y0 = whole_down(add_rn(y, -tol));
+    y1 = whole_down(add_rn(y, tol));
+    return q;
 }
 
-// A row of a tile left to the exact search: a + 2^12 k + 2^24 strip (the tile's
-// place along y; rows along y are cut to it).
-HD_HD uint32_t row_code(int a, int k, int strip)
+// A pair's row code in 64 bits: the record's slot (23 bits), row a, slice k and an
+// index of the row within the tile (12 bits each), the tile's strip along y
+// (4 bits; rows along y begin at it).
+constexpr int kOpenSlots = 1 << 23, kOpenStrips = 16;
+HD_HD unsigned long long open_code(uint32_t slot, int a, int k, int m, int strip)
 {
-    return static_cast<uint32_t>(a) | (static_cast<uint32_t>(k) << 12) |
-           (static_cast<uint32_t>(strip) << 24);
+    return static_cast<unsigned long long>(slot) | (static_cast<unsigned long long>(a) << 23) |
+           (static_cast<unsigned long long>(k) << 35) | (static_cast<unsigned long long>(m) << 47) |
+           (static_cast<unsigned long long>(strip) << 59);
 }
 
-// The exact search of one listed row of the record in `slot`, its voxels added
-// to N or M one by one.
-__device__ __noinline__ void exact_row(const RowsArgs &ra, const ScanDesc &d, uint32_t slot,
-                                       uint32_t code)
+// The pair's packed rows: the closed form, the tile's row length less one in
+// whole_up form, and the code of its first row.
+HD_HD void slice_unpack(const uint4 v[3], SliceRows &r, float &top, unsigned long long &code)
+{
+    auto f = [](uint32_t x) {
+#ifdef __CUDA_ARCH__
+        return __uint_as_float(x);
+#else
+        float y;
+        memcpy(&y, &x, 4);
+        return y;
+#endif
+    };
+    r.e0 = f(v[0].x);
+    r.ea = f(v[0].y);
+    r.f0 = f(v[0].z);
+    r.fa = f(v[0].w);
+    r.Kr = f(v[1].x);
+    r.E0 = f(v[1].y);
+    r.Kd = f(v[1].z);
+    r.dq = f(v[1].w);
+    r.n = static_cast<int>(v[2].x >> 16);
+    top = kWhole + static_cast<float>(static_cast<int>(v[2].y & 0xffffu) - 1);
+    code = v[2].z | (static_cast<unsigned long long>(v[2].w) << 32);
+}
+
+// Settles exactly what row i of the pair at `pos` leaves open (see slice_row): the
+// indices x0 .. x1 - 1 and y0 + 1 .. y1, each once, or the whole row, inside the
+// tile; its voxels added to N or M one by one.  The closed form is recomputed
+// from the pair, so its ends are those the traversal saw.
+__device__ __noinline__ void settle_open(const RowsArgs &ra, const ScanDesc &d, uint32_t pos, int i)
 {
     const GeomQ &g = ra.g;
+    SliceRows r{};
+    float top;
+    unsigned long long code;
+    {
+        const uint4 *p = d.pairs.v + (kSliceWords / 4) * static_cast<size_t>(pos);
+        const uint4 v[3] = {p[0], p[1], p[2]};
+        slice_unpack(v, r, top, code);
+    }
+    float x0, x1, y0, y1;
+    const float q = slice_row(r, static_cast<float>(i), x0, x1, y0, y1);
+    const uint32_t slot = static_cast<uint32_t>(code & (kOpenSlots - 1));
+    const int a = static_cast<int>((code >> 23) & 0xfffu) + i;
+    const int k = static_cast<int>((code >> 35) & 0xfffu);
+    const int strip = static_cast<int>((code >> 59) & (kOpenStrips - 1));
     long long W[6];
 #pragma unroll
-    for (int q = 0; q < 6; ++q) W[q] = ra.rec.g[q][slot];
+    for (int w = 0; w < 6; ++w) W[w] = ra.rec.g[w][slot];
     const int cls = status_cls(ra.rec.status[slot]);
     long long A[3], B[3];
     bool ymaj;
-    int blo[3], bhi[3];
     float S;
-    if (!capsule_frame(g, W, ra.R, A, B, ymaj, blo, bhi, S)) return;
+    capsule_frame(g, W, ra.R, A, B, ymaj, nullptr, nullptr, S);
     CapX cx;
     capx_of(g, A, B, ymaj, ra.R, cx);
-    const CapF cf = capf_of(cx, S, ra.R);
-    const int a = static_cast<int>(code & 0xfffu), k = static_cast<int>((code >> 12) & 0xfffu);
-    int lo, hi;
-    if (!row_interval(cf, cx, a, k, lo, hi)) return;
-    uint32_t *vol = (cls ? d.M : d.N) + static_cast<size_t>(k) * g.nx * g.ny;
-    if (ymaj) {
-        const int y0 = static_cast<int>(code >> 24) * d.tp.ty;
-        lo = max_i(lo, y0);
-        hi = min_i(hi, min_i(y0 + d.tp.ty, g.ny) - 1);
-        for (int m = lo; m <= hi; ++m) atomicAdd(vol + a + static_cast<size_t>(g.nx) * m, 1u);
-    } else {
-        for (int m = lo; m <= hi; ++m) atomicAdd(vol + m + static_cast<size_t>(g.nx) * a, 1u);
+    const int m0 = ymaj ? strip * d.tp.ty : 0;
+    uint32_t *line = (cls ? d.M : d.N) + static_cast<size_t>(k) * g.nx * g.ny +
+                     (ymaj ? static_cast<size_t>(a) : static_cast<size_t>(g.nx) * a);
+    const size_t step = ymaj ? g.nx : 1;
+    if (!(q > 4.0f * r.dq)) {
+        const CapF cf = capf_of(cx, S, ra.R);
+        int lo, hi;
+        if (!row_interval(cf, cx, a, k, lo, hi)) return;
+        lo = max_i(lo, m0);
+        hi = min_i(hi, m0 + static_cast<int>(top - kWhole));
+        for (int m = lo; m <= hi; ++m) atomicAdd(line + step * m, 1u);
+        return;
+    }
+    float p = fmaxf(x0, kWhole);
+    const float p1 = fminf(x1 - 1.0f, fminf(y1, top));
+    const float q0 = fmaxf(fmaxf(y0 + 1.0f, x1), kWhole), q1 = fminf(y1, top);
+    if (p > p1) p = q0;  // nearly always one index at one end
+    while (p <= p1 || (p >= q0 && p <= q1)) {
+        const int m = m0 + static_cast<int>(p - kWhole);
+        if (F_exact(cx, a, k, m) <= cx.T) atomicAdd(line + step * m, 1u);
+        p += 1.0f;
+        if (p > p1 && p < q0) p = q0;
     }
 }
 

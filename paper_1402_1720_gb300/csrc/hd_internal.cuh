@@ -117,10 +117,13 @@ struct Pairs {
     // plus the pair's tile index within the record.
     uint32_t *stage;
     // Euclidean thick rays use the same buffer with kSliceWords words per pair
-    // in v, and fb as the list of the rows left to the exact search (fb_cap
-    // entries: the record's slot; row, slice and strip, see row_code).
+    // in v, and fb as the lists of what their closed form leaves open, one per
+    // traversal block: fb_count entries in each (the pair, the row in it), room
+    // for fb_cap.
     uint32_t fb_cap;
+    uint32_t *fb_count;
 };
+constexpr int kOpenLists = 2048;  // most blocks of that traversal
 
 constexpr int kSliceWords = 12;
 

@@ -76,7 +76,8 @@ __device__ __forceinline__ void event_step(EventCursor &c, int u, int cnt)
 // as long as the walks of 1 300 pairs) and not once per part.
 constexpr int kCols = 16;
 struct TilePart {
-    const uint4 *first_pair;  // the bucket's first pair
+    const uint4 *pairs;  // the scan's pairs
+    uint32_t first;      // the bucket's first one
     int scan;
     int tile;    // tile id within its group
     int group;   // bit 0 the class (missed: N, hit: M), bits 1-2 the walk type
@@ -94,7 +95,8 @@ __device__ __forceinline__ int slot_rows(int count) { return (count + 32 * kCols
 template <int kVec>
 struct NextWalk {
     uint4 v[kVec];
-    int base;  // its tile's offset in bytes
+    int base;      // its tile's offset in bytes
+    uint32_t pos;  // the pair
     bool have;
     bool walk;  // false: a slot past its bucket's pairs
 };
@@ -112,8 +114,9 @@ __device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, N
     nw.base = 4 * t.offset;
     nw.walk = k < t.count;
     if (nw.walk) {
+        nw.pos = t.first + static_cast<uint32_t>(k);
 #pragma unroll
-        for (int q = 0; q < kVec; ++q) nw.v[q] = __ldg(t.first_pair + kVec * static_cast<size_t>(k) + q);
+        for (int q = 0; q < kVec; ++q) nw.v[q] = __ldg(t.pairs + kVec * static_cast<size_t>(nw.pos) + q);
     }
 }
 
@@ -203,12 +206,12 @@ __device__ __forceinline__ void row_step(int at, float lo, float hi, bool on)
         : "memory");
 }
 
-constexpr int kRowsPerStep = 4;  // rows a lane takes between refill checks
+constexpr int kRowsPerStep = 8;  // rows a lane takes between refill checks (4: 6 % slower)
 
 // walk_parts for Euclidean thick rays: a lane takes the rows of one history in
 // one slice, one after the other, each a closed form of about 35 instructions
-// (slice_row) and two shared atomics.  The rows the closed form leaves open go
-// to the scan's list, or are searched at once when that is full.
+// (slice_row) and two shared atomics.  What the closed form leaves open goes to
+// the scan's list, or is settled at once when that is full.
 __device__ __noinline__ void walk_parts(uint32_t *tiles, int, const TilePart *parts, int n, int total,
                                         int refill, unsigned *s_next, NextWalk<3> nw,
                                         const ScanDesc &d, const RowsArgs &ra)
@@ -219,27 +222,19 @@ __device__ __noinline__ void walk_parts(uint32_t *tiles, int, const TilePart *pa
     SliceRows c{};
     float i = 0.0f, top = 0.0f;
     int left = 0, at = 0, step = 0;
-    uint32_t slot = 0, code = 0;
+    uint32_t pos = 0;  // the pair
     for (;;) {
         const unsigned idle = __ballot_sync(kFull, left == 0);
         if (__popc(idle) >= refill) {
             const unsigned want = __ballot_sync(kFull, left == 0 && nw.have);
             if (left == 0 && nw.have) {
                 if (nw.walk) {
-                    c.e0 = __uint_as_float(nw.v[0].x);
-                    c.ea = __uint_as_float(nw.v[0].y);
-                    c.f0 = __uint_as_float(nw.v[0].z);
-                    c.fa = __uint_as_float(nw.v[0].w);
-                    c.Kr = __uint_as_float(nw.v[1].x);
-                    c.E0 = __uint_as_float(nw.v[1].y);
-                    c.Kd = __uint_as_float(nw.v[1].z);
-                    c.dq = __uint_as_float(nw.v[1].w);
-                    left = static_cast<int>(nw.v[2].x >> 16);
+                    unsigned long long code;
+                    slice_unpack(nw.v, c, top, code);
+                    left = c.n;
+                    pos = nw.pos;
                     at = sbase + nw.base + 4 * static_cast<int>(nw.v[2].x & 0xffffu);
-                    top = __int_as_float(0x4B400000 + static_cast<int>(nw.v[2].y & 0xffffu) - 1);
                     step = 4 * static_cast<int>(nw.v[2].y >> 16);
-                    slot = nw.v[2].z;
-                    code = nw.v[2].w;
                     i = 0.0f;
                 }
                 nw.have = false;
@@ -258,14 +253,15 @@ __device__ __noinline__ void walk_parts(uint32_t *tiles, int, const TilePart *pa
             }
         }
         const int cnt = min(left, kRowsPerStep);
-        unsigned open = 0;  // rows of this step left to the exact search
+        unsigned open = 0;  // rows of this step with something left open
 #pragma unroll
         for (int u = 0; u < kRowsPerStep; ++u) {
-            float lo, hi;
-            const bool sure = slice_row(c, i, top, lo, hi);
-            const bool on = u < cnt;
-            row_step(at, lo, hi, on && sure && lo <= hi);
-            if (on && !sure) open |= 1u << u;
+            float x0, x1, y0, y1;
+            const float q = slice_row(c, i, x0, x1, y0, y1);
+            const float lo = fmaxf(x1, kWhole), hi = fminf(y0, top);
+            const bool on = u < cnt, closed = q > 4.0f * c.dq;
+            row_step(at, lo, hi, on && closed && lo <= hi);
+            if (on && !((closed && x0 == x1 && y0 == y1) || q < -c.dq)) open |= 1u << u;
             i += 1.0f;
             at += step;
         }
@@ -273,10 +269,14 @@ __device__ __noinline__ void walk_parts(uint32_t *tiles, int, const TilePart *pa
         while (open != 0) {
             const int u = __ffs(open) - 1;
             open &= open - 1;
-            const uint32_t row = code + static_cast<uint32_t>(static_cast<int>(i) - kRowsPerStep + u);
-            const unsigned k = atomicAdd(&d.ctrl->n_pair_fallback, 1u);
-            if (k < d.pairs.fb_cap) d.pairs.fb[k] = make_uint2(slot, row);
-            else exact_row(ra, d, slot, row);
+            // to the block's list, or settled at once when that is full
+            const int row = static_cast<int>(i) + u - kRowsPerStep;
+            const unsigned n = atomicAdd(s_next + 1, 1u);
+            if (n < d.pairs.fb_cap)
+                d.pairs.fb[static_cast<size_t>(blockIdx.x) * d.pairs.fb_cap + n] =
+                    make_uint2(pos, static_cast<uint32_t>(row));
+            else
+                settle_open(ra, d, pos, row);
         }
     }
 }
@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     constexpr bool kRows = RowsT::kRows;
     constexpr int kVec = kRows ? kSliceWords / 4 : kLeanWords / 4;
     extern __shared__ __align__(16) uint32_t tile[];
-    __shared__ unsigned s_next;
+    __shared__ unsigned s_next[2];  // the next slot; entries of the block's list of open rows
     __shared__ int s_first[kMaxBatch + 1];
     __shared__ TilePart s_parts[kPartList];
     __shared__ int s_group[kPartList + 1];  // first part of each group
@@ -633,6 +633,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     __shared__ unsigned long long s_warp[32];
     // buckets of scan k are the launch's buckets [s_first[k], s_first[k + 1])
     if (threadIdx.x == 0) {
+        s_next[1] = 0;
         int acc = 0;
         for (int k = 0; k < nscans; ++k) {
             s_first[k] = acc;
@@ -691,7 +692,8 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
                 if (r >= j0 && r < j0 + kPartList) {
                     TilePart &j = s_parts[r - j0];
                     const ScanDesc &d = descs[k];
-                    j.first_pair = d.pairs.v + kVec * static_cast<size_t>(d.buckets.first[t]);
+                    j.pairs = d.pairs.v;
+                    j.first = d.buckets.first[t];
                     j.scan = k;
                     j.tile = t % d.tp.ntiles;
                     j.group = t / d.tp.ntiles;
@@ -730,10 +732,10 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         first_walks(s_parts, s_group[1], s_slots[0], nw);
         for (int g = 0; g < ngroups; ++g) {
             const int q0 = s_group[g], q1 = s_group[g + 1];
-            if (threadIdx.x == 0) s_next = blockDim.x;
+            if (threadIdx.x == 0) s_next[0] = blockDim.x;
             __syncthreads();
             const TilePlan &tp0 = descs[s_parts[q0].scan].tp;
-            walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, &s_next, nw,
+            walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, s_next, nw,
                        descs[s_parts[q0].scan], ra);
             if (g + 1 < ngroups)
                 first_walks(s_parts + q1, s_group[g + 2] - q1, s_slots[g + 1], nw);
@@ -753,7 +755,11 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         }
         __syncthreads();
     }
-    if (!kRows) walk_fallback_lists(descs, nscans);
+    if (kRows) {
+        if (threadIdx.x == 0) descs[0].pairs.fb_count[blockIdx.x] = s_next[1];
+    } else {
+        walk_fallback_lists(descs, nscans);
+    }
 }
 
 // Shared memory of a launch whose largest tile has this many words: room for
@@ -764,6 +770,11 @@ static int trace_smem_words(int tile_words)
     return tile_words * (n < 1 ? 1 : (n > 8 ? 8 : n));
 }
 
+// Threads of the traversal of Euclidean thick rays: its row loop wants about 100
+// registers; 1024 threads leave it 64 (head-sized grid, 2.7e6 histories, 2.5 mm,
+// whole scan, in three chunks: 2.00 ms at 1024, 1.84 at 512, 2.23 at 256).
+static constexpr int rows_threads(int threads) { return threads > 512 ? 512 : threads; }
+
 template <int kThreads>
 int occupancy_of(int smem_words)
 {
@@ -772,7 +783,7 @@ int occupancy_of(int smem_words)
     if (cudaFuncSetAttribute(trace_tiles_kernel<kThreads, NoRows>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, RowsArgs>,
+        cudaFuncSetAttribute(trace_tiles_kernel<rows_threads(kThreads), RowsArgs>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess) {
         cudaGetLastError();
@@ -835,7 +846,7 @@ cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words
 cudaError_t launch_trace_rows(const ScanDesc *desc, int tile_words, int threads, int grid,
                               const RowsArgs &ra, cudaStream_t s)
 {
-    return launch_trace(desc, 1, tile_words, threads, grid, ra, s);
+    return launch_trace(desc, 1, tile_words, rows_threads(threads), grid, ra, s);
 }
 
 }  // namespace hd

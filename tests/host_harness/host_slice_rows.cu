@@ -54,17 +54,25 @@ extern "C" long long hx_slice_rows(const long long *W, int nx, int ny, int nz, f
                 if (part) return -2;
                 continue;
             }
-            float fl, fh;
-            const float top = hd::kWhole + static_cast<float>(len - 1);
-            if (!hd::slice_row(r, static_cast<float>(a - r.row), top, fl, fh)) {
+            float x0, x1, y0, y1;
+            const float q = hd::slice_row(r, static_cast<float>(a - r.row), x0, x1, y0, y1);
+            if (!(q > 4.0f * r.dq) && !(q < -r.dq)) {
                 ++*open;
                 continue;
             }
             ++certain;
-            const bool got = fl <= fh;
-            if (got != part) return -1;
-            if (got && (static_cast<int>(fl - hd::kWhole) != tl || static_cast<int>(fh - hd::kWhole) != th))
-                return -1;
+            if (q < 0.0f) {
+                if (part) return -1;
+                continue;
+            }
+            if (x0 != x1 || y0 != y1) ++*open;
+            // x1 .. y0 inside, below x0 and above y1 outside (tile indices)
+            for (int m = 0; m < len; ++m) {
+                const float f = hd::kWhole + static_cast<float>(m);
+                const bool in = have && m >= lo - m0 && m <= hi - m0;
+                if (f >= x1 && f <= y0 && !in) return -1;
+                if ((f < x0 || f > y1) && in) return -1;
+            }
         }
     }
     return certain;
