@@ -49,18 +49,6 @@ HD_HD unsigned umulhi32(unsigned a, unsigned b)
 #endif
 }
 
-// floor(n / d) for d >= 2, |n| < 2^62, with m = floor(2^64 / d): the
-// multiply-high quotient is low by at most one, fixed by one comparison.
-HD_HD long long floordiv_magic(long long n, unsigned long long d, unsigned long long m)
-{
-    const bool neg = n < 0;
-    const unsigned long long u =
-        neg ? static_cast<unsigned long long>(-(n + 1)) : static_cast<unsigned long long>(n);
-    unsigned long long q = umulhi64(u, m);
-    if (u - q * d >= d) ++q;
-    return neg ? -1 - static_cast<long long>(q) : static_cast<long long>(q);
-}
-
 // Q16 of a value known to satisfy |x| < 4096: the 32-bit conversion rounds
 // exactly as the 64-bit one does.
 HD_HD int q16_small(float x)
@@ -142,6 +130,39 @@ HD_HD long long fdiv_small(long long a, long long b)
     if (r >= b) ++q;
     return q;
 }
+// Approximate reciprocal of b > 0 (within two units of the last place).
+HD_HD float rcp_int(int b)
+{
+#ifdef __CUDA_ARCH__
+    return __fdividef(1.0f, static_cast<float>(b));
+#else
+    return 1.0f / static_cast<float>(b);
+#endif
+}
+
+// floor(a / b) and its remainder for 0 < b < 2^31, |a / b| < 2^20, rb =
+// rcp_int(b): the estimate is within one of the floor (relative error below
+// 2^-21), so one step each way settles it; the remainder is one 32 x 32
+// product, and a divisor used twice has its reciprocal taken once.
+HD_HD int fdiv32(long long a, int b, float rb, long long &rem)
+{
+#ifdef __CUDA_ARCH__
+    int q = __float2int_rd(__ll2float_rn(a) * rb);
+#else
+    int q = static_cast<int>(std::floor(static_cast<float>(a) * rb));
+#endif
+    rem = a - static_cast<long long>(q) * static_cast<long long>(b);
+    if (rem < 0) {
+        --q;
+        rem += b;
+    }
+    if (rem >= b) {
+        ++q;
+        rem -= b;
+    }
+    return q;
+}
+
 // Rotation-mode CORDIC of an angle in degrees * 2^16: cos and sin * 2^30.
 HD_HD void cordic_cs(long long a_q16, const Cordic &cd, long long &c, long long &s)
 {
@@ -176,11 +197,18 @@ HD_HD void cordic_cs(long long a_q16, const Cordic &cd, long long &c, long long 
 }
 
 // Grid coordinate (voxel units, Q16) of a world coordinate w (mm, Q16):
-// floor((2 w + n s) 2^16 / (2 s)), the division done by multiply-high.
-HD_HD long long to_grid(long long w, int n, long long s_q, unsigned long long m)
+// floor((2 w + n s) 2^16 / (2 s)) = floor((2 w + n s) 2^15 / s).  The numerator
+// N = 2 w + n s lies within 1.61e9 in magnitude (|w| < 2^29, n s <= 2^29), so N
+// plus the bias is an unsigned 32-bit n', and floor(n' M / 2^54) with M =
+// floor(2^69 / s) + 1 is the quotient exactly: its error n' / 2^54 stays below
+// 1 / s (n' < 2^32, s <= 2^22).  Two 32 x 32 products, where a 64-bit
+// multiply-high division took about four times the instructions.
+HD_HD long long to_grid(int w, const GridDiv &d)
 {
-    return floordiv_magic((2 * w + static_cast<long long>(n) * s_q) * kQ16,
-                          static_cast<unsigned long long>(2 * s_q), m);
+    const uint32_t n = static_cast<uint32_t>(2 * w + d.ns) + d.bias;
+    const unsigned long long lo = static_cast<unsigned long long>(n) * d.mlo;
+    const unsigned long long hi = static_cast<unsigned long long>(n) * d.mhi + (lo >> 32);
+    return static_cast<long long>(hi >> 22) - d.off;
 }
 
 // Host-side construction of the fixed-point geometry.
@@ -194,13 +222,22 @@ inline GeomQ make_geomq(int nx, int ny, int nz, float sx, float sy, float sz, fl
     g.sy = llrint(static_cast<double>(sy) * 65536.0);
     g.sz = llrint(static_cast<double>(sz) * 65536.0);
     g.T = llrint(static_cast<double>(T) * 65536.0);
-    auto magic = [](long long s) {
-        const unsigned __int128 one = static_cast<unsigned __int128>(1) << 64;
-        return static_cast<unsigned long long>(one / static_cast<unsigned long long>(2 * s));
+    auto axis = [](int n, long long s) {
+        GridDiv d;
+        const unsigned long long m = static_cast<unsigned long long>(
+                                         (static_cast<unsigned __int128>(1) << 69) /
+                                         static_cast<unsigned long long>(s)) + 1;
+        d.mlo = static_cast<uint32_t>(m);
+        d.mhi = static_cast<uint32_t>(m >> 32);
+        d.ns = static_cast<int32_t>(n * s);
+        const long long k = (1620000000LL + s - 1) / s;  // >= the largest |N|
+        d.bias = static_cast<uint32_t>(k * s);
+        d.off = k << 15;
+        return d;
     };
-    g.mx = magic(g.sx);
-    g.my = magic(g.sy);
-    g.mz = magic(g.sz);
+    g.dx = axis(nx, g.sx);
+    g.dy = axis(ny, g.sy);
+    g.dz = axis(nz, g.sz);
     return g;
 }
 
@@ -234,16 +271,16 @@ HD_HD bool endpoints_cs(const GeomQ &g, long long c, long long s, float ui, floa
         return false;
     long long W[6];
     world_cs(g, c, s, ui, vi, uo, vo, W);
-    const long long G[6] = {to_grid(W[0], g.nx, g.sx, g.mx), to_grid(W[1], g.ny, g.sy, g.my),
-                            to_grid(W[2], g.nz, g.sz, g.mz), to_grid(W[3], g.nx, g.sx, g.mx),
-                            to_grid(W[4], g.ny, g.sy, g.my), to_grid(W[5], g.nz, g.sz, g.mz)};
-    const long long lim = 1LL << 30;
+    const GridDiv *const d[3] = {&g.dx, &g.dy, &g.dz};
+    bool ok = true;
 #pragma unroll
     for (int a = 0; a < 6; ++a) {
-        if (G[a] >= lim || G[a] <= -lim) return false;
-        out[a] = static_cast<int32_t>(G[a]);
+        const long long G = to_grid(static_cast<int>(W[a]), *d[a % 3]);
+        // |G| < 2^30
+        ok = ok && static_cast<unsigned long long>(G + ((1LL << 30) - 1)) < (1ULL << 31) - 1;
+        out[a] = static_cast<int32_t>(G);
     }
-    return true;
+    return ok;
 }
 
 // Grid Q16 endpoints of one history; false when the history is rejected.
@@ -256,40 +293,44 @@ HD_HD bool endpoints(const GeomQ &g, const Cordic &cd, float ang, float ui, floa
     return endpoints_cs(g, c, s, ui, vi, uo, vo, out);
 }
 
-// The slices the part of a segment inside the grid's x-y extent can touch:
-// the parameter interval [t_lo, t_hi] of the segment r (grid Q16) inside
-// [0, nx) x [0, ny) (closed at its ends, exact rationals), and the z
-// indices at its two ends, ordered and clamped to the grid.  A superset of
-// the slices that hold voxels of the segment (z is monotone along it);
-// false when the segment misses the grid.
+// The slices the part of a segment inside the grid's x-y extent can touch: a
+// superset of the slices that hold voxels of the segment (z is monotone along
+// it); false when the segment misses the grid (it then has no voxel at all,
+// though a segment that barely misses it may get slices).  In float, the extent
+// widened by 16 eps (eps = 2^-24) of the numbers that enter a parameter, whose
+// roundings are below 8 eps of them, and z by 8 eps of its own (exact rationals
+// took three times the instructions and gave the same slices but for one in a
+// thousand).
 HD_HD bool grid_z_range(const TilePlan &tp, const int32_t r[6], int &zlo, int &zhi)
 {
-    // t_lo = nl / dl, t_hi = nh / dh (den > 0)
-    long long nl = 0, dl = 1, nh = 1, dh = 1;
-    const int H[2] = {tp.nx << 16, tp.ny << 16};
+    const float eps = 5.9604644775390625e-8f;
+    float t0 = 0.0f, t1 = 1.0f;
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
-        const long long p = r[a], d = static_cast<long long>(r[a + 3]) - r[a];
-        long long en = 0, ed = 1, xn = 1, xd = 1;  // entry and exit parameters
-        if (d > 0) {
-            if (p >= H[a] || p + d < 0) return false;
-            if (p < 0) { en = -p; ed = d; }
-            if (p + d > H[a]) { xn = H[a] - p; xd = d; }
-        } else if (d < 0) {
-            if (p < 0 || p + d >= H[a]) return false;
-            if (p >= H[a]) { en = p - H[a]; ed = -d; }
-            if (p + d < 0) { xn = p; xd = -d; }
-        } else if (p < 0 || p >= H[a]) {
-            return false;
+        const float H = static_cast<float>((a == 0 ? tp.nx : tp.ny) << 16);
+        const float p = static_cast<float>(r[a]);
+        const int di = r[a + 3] - r[a];
+        const float d = static_cast<float>(di);
+        const float m = fmaf(16.0f * eps, fabsf(p) + fabsf(d) + H, 1.0f);
+        if (di == 0) {
+            if (p < -m || p > H + m) return false;
+        } else {
+#ifdef __CUDA_ARCH__
+            const float i = __frcp_rn(d);
+#else
+            const float i = 1.0f / d;
+#endif
+            const float ta = (-m - p) * i, tb = (H + m - p) * i;
+            t0 = fmaxf(t0, fminf(ta, tb));
+            t1 = fminf(t1, fmaxf(ta, tb));
         }
-        if (en * dl > nl * ed) { nl = en; dl = ed; }
-        if (xn * dh < nh * xd) { nh = xn; dh = xd; }
     }
-    if (nl * dh > nh * dl) return false;
-    const long long z = r[2], dz = static_cast<long long>(r[5]) - r[2];
-    int z0 = static_cast<int>(floordiv_small(z * dl + nl * dz, dl << 16));
-    int z1 = static_cast<int>(floordiv_small(z * dh + nh * dz, dh << 16));
-    if (z0 > z1) { const int t = z0; z0 = z1; z1 = t; }
+    if (t0 > t1) return false;
+    const float z = static_cast<float>(r[2]), dz = static_cast<float>(r[5] - r[2]);
+    const float za = fmaf(t0, dz, z), zb = fmaf(t1, dz, z);
+    const float m = fmaf(8.0f * eps, fabsf(z) + fabsf(dz), 1.0f);
+    const int z0 = static_cast<int>(floorf((fminf(za, zb) - m) * (1.0f / 65536.0f)));
+    const int z1 = static_cast<int>(floorf((fmaxf(za, zb) + m) * (1.0f / 65536.0f)));
     if (z1 < 0 || z0 >= tp.nz) return false;
     zlo = z0 < 0 ? 0 : z0;
     zhi = z1 >= tp.nz ? tp.nz - 1 : z1;
@@ -991,6 +1032,7 @@ HD_HD int slab_lean(const int32_t gi[3], const int32_t go[3], int nx, int ny, Le
     int idx[3];
     bool onp[3];
     const long long den = static_cast<long long>(tQ) << 16;
+    const float rQ = rcp_int(static_cast<int>(tQ));
     // the entry point's coordinate along each axis, P tQ + tN D over den
     // (also right for the entry axis and when the segment starts inside)
 #pragma unroll
@@ -1000,9 +1042,9 @@ HD_HD int slab_lean(const int32_t gi[3], const int32_t go[3], int nx, int ny, Le
             idx[2] = num < 0 ? -1 : (num >= den ? 1 : 0);
             onp[2] = num == 0 || num == den;
         } else {
-            const long long q = fdiv_small(num >> 16, static_cast<long long>(tQ));
-            idx[a] = static_cast<int>(q);
-            onp[a] = num == q * den;
+            long long rem;
+            idx[a] = fdiv32(num >> 16, static_cast<int>(tQ), rQ, rem);
+            onp[a] = rem == 0 && (num & 0xffff) == 0;
         }
     }
 #pragma unroll
@@ -1068,18 +1110,20 @@ HD_HD int slab_lean(const int32_t gi[3], const int32_t go[3], int nx, int ny, Le
             q0 = kQBig;
             rh0 = 1;
         } else {
-            const long long q = fdiv_small(dh, static_cast<long long>(a0));
-            q0 = static_cast<int>(q);
-            rh0 = static_cast<unsigned>(dh - q * static_cast<long long>(a0));
+            long long rem;
+            q0 = fdiv32(dh, static_cast<int>(a0), rcp_int(static_cast<int>(a0)), rem);
+            rh0 = static_cast<unsigned>(rem);
         }
     }
+    const float r1 = act1 ? rcp_int(static_cast<int>(a1)) : 0.0f;
     if (act1) {
         if ((d1 & 0xffff) == 0) return -1;  // z may tie with the major axis
         const long long dh = d1 >> 16;
         if (float_of(dh) >= 1048576.0f * static_cast<float>(a1)) {
             q1 = kQBig;
         } else {
-            q1 = static_cast<int>(fdiv_small(dh, static_cast<long long>(a1)));
+            long long rem;
+            q1 = fdiv32(dh, static_cast<int>(a1), r1, rem);
         }
     }
     if (q0 < -1 || q1 < -1) return -1;
@@ -1099,8 +1143,10 @@ HD_HD int slab_lean(const int32_t gi[3], const int32_t go[3], int nx, int ny, Le
             if (float_of(num) >= (static_cast<float>(kc0) + 2.0f) * float_of(step)) {
                 kz = kc0;
             } else {
-                const long long q = fdiv_small(num, step) + 1;
-                kz = q < kc0 ? static_cast<int>(q) : kc0;
+                // floor(num / (a1 2^16)) = floor(floor(num / 2^16) / a1)
+                long long rem;
+                const int q = fdiv32(num >> 16, static_cast<int>(a1), r1, rem) + 1;
+                kz = q < kc0 ? q : kc0;
             }
         }
     }
@@ -1371,8 +1417,9 @@ HD_HD void event_pack(const LeanWalk &L, int nmaj, int nminor, int thick, uint32
         const long long X =
             static_cast<long long>(L.kmz - L.jn + 1) * L.ad - static_cast<long long>(L.rem);
         const long long am = static_cast<long long>(L.Qu) * L.ad + L.Ru;
-        const long long k = fdiv_small(X - 1, am) + 1;  // X >= 1: rem < |D_0|
-        n = k < L.K ? static_cast<int>(k) : L.K;
+        long long rem;  // X >= 1: L.rem < |D_0|
+        const int k = fdiv32(X - 1, static_cast<int>(am), rcp_int(static_cast<int>(am)), rem) + 1;
+        n = k < L.K ? k : L.K;
     }
     const int s = (L.fl & 2) ? 1 : -1;
     const int row0 = L.row * W;

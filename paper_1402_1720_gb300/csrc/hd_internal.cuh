@@ -22,13 +22,23 @@ struct Cordic {
     long long K;
 };
 
+// One axis of the map from world to grid coordinates: the voxel size s and the
+// extent n s (mm * 2^16), floor(2^69 / s) + 1 in two words, and a multiple of s
+// that makes every numerator positive, with its quotient.
+struct GridDiv {
+    int32_t ns;
+    uint32_t mlo, mhi;
+    uint32_t bias;
+    long long off;
+};
+
 // Geometry in the fixed-point units the kernels use.
 struct GeomQ {
     int32_t nx, ny, nz;
     int32_t pad;
     long long sx, sy, sz;  // voxel sizes, mm * 2^16
     long long T;           // tracker half-separation, mm * 2^16
-    unsigned long long mx, my, mz;  // floor(2^64 / (2 s)): division by multiply-high
+    GridDiv dx, dy, dz;    // world to grid coordinates (to_grid in hd_geom.cuh)
 };
 
 // Device-side counters of one scan.  The block from n_global to the end is

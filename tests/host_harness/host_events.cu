@@ -3,6 +3,20 @@
 
 #include "../../paper_1402_1720_gb300/csrc/hd_geom.cuh"
 
+// to_grid against floor((2 w + n s) 2^16 / (2 s)) in 128 bits; mismatches.
+extern "C" long long hx_to_grid(int n, float s, const int32_t *w, long long count)
+{
+    const hd::GeomQ g = hd::make_geomq(n, n, n, s, s, s, 1.0f);
+    long long bad = 0;
+    for (long long i = 0; i < count; ++i) {
+        const __int128 num = (2 * (__int128)w[i] + (__int128)n * g.sx) * 65536, den = 2 * g.sx;
+        __int128 q = num / den;
+        if (num % den != 0 && num < 0) --q;
+        if ((__int128)hd::to_grid(w[i], g.dx) != q) ++bad;
+    }
+    return bad;
+}
+
 // The event walk of the oriented segment in a box of dx x dy x dz voxels,
 // dilated by `thick`: its updates applied to plain counters in the tile's
 // layout, decoded by the definition (prefix sums along the major axis), the

@@ -78,3 +78,18 @@ def test_event_walks_equal_oracle(oracle_mod, hx, dims, direct):
             seen += n > 0
             assert np.array_equal(out[:n], _dilate(ref, dims, t)), (seg.tolist(), t)
     assert seen > 300
+
+
+@pytest.mark.parametrize("n,s", [(4096, 1 / 64), (128, 64.0), (4096, 2.0), (1, 64.0), (200, 1.0),
+                                 (181, 0.93), (64, 0.015640259), (127, 63.99998)])
+def test_grid_coordinate_is_exact(hx, n, s):
+    """The two-product division of the world-to-grid map equals the floor over
+    the whole range of world coordinates, at multiples of the voxel size too."""
+    rng = np.random.default_rng(n)
+    hx.hx_to_grid.restype = ctypes.c_longlong
+    sq = int(round(s * 65536))
+    w = np.concatenate([rng.integers(-2 ** 29, 2 ** 29, 200000), np.arange(-2 ** 29, -2 ** 29 + 99),
+                        np.arange(2 ** 29 - 99, 2 ** 29), rng.integers(-2 ** 29 // sq, 2 ** 29 // sq,
+                                                                       20000) * sq // 2])
+    w = np.ascontiguousarray(w, dtype=np.int32)
+    assert hx.hx_to_grid(n, ctypes.c_float(s), w.ctypes.data_as(I32P), ctypes.c_longlong(w.size)) == 0
