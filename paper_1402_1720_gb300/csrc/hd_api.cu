@@ -140,6 +140,8 @@ struct hd_scan {
     int64_t *rows_scratch = nullptr;  // tile sums of the system-row offset scan
     int64_t rows_scratch_cap = 0;
     uint32_t *rows_bits = nullptr;    // the hull packed for the row passes
+    uint32_t *rows_walks = nullptr;   // a chunk's path walks for them
+    int64_t rows_walks_cap = 0;
     int32_t thick_k = 0;             // thick rays: in-plane dilation (0 = thin paths)
     float euclid_d0 = 0.0f;          // thick rays by Euclidean distance, mm (0 = off)
     int euclid_pairs = 0;            // their pairs per record on the tiled path (0: not taken)
@@ -218,7 +220,7 @@ void free_scan(hd_scan *s)
     void *ptrs[] = {s->N, s->M, s->H1, s->H2, s->H3, s->bits_out, s->slice_key,
                     s->mt, s->slope, s->index, s->ctrl, s->rec_buf, s->staging,
                     s->compact_blocks, s->d_count, s->compact_out, s->pair_buf, s->tile_events,
-                    s->rows_scratch, s->rows_bits, s->thick_ws,
+                    s->rows_scratch, s->rows_bits, s->rows_walks, s->thick_ws,
                     s->tile_count, s->tile_cursor, s->desc_dev};
     for (void *p : ptrs)
         if (p) cudaFree(p);
@@ -917,25 +919,55 @@ hd_status hd_scan_system_rows(hd_scan *scan, int32_t method, const float *angle_
     }
     const uint8_t *hull = mask_of(scan, method);
     if (!scan->rows_bits) {
-        if (cudaMalloc(&scan->rows_bits, sizeof(uint32_t) * static_cast<size_t>(scan->words)) !=
+        if (cudaMalloc(&scan->rows_bits, sizeof(uint32_t) * static_cast<size_t>(scan->words + 1)) !=
             cudaSuccess) {
             cudaGetLastError();
             scan->rows_bits = nullptr;
             return HD_ERR_NOMEM;
         }
     }
+    const int64_t chunk = n < hd::kRowsChunk ? n : hd::kRowsChunk;
+    if (chunk > scan->rows_walks_cap) {
+        HD_CUDA(cudaStreamSynchronize(st));
+        if (scan->rows_walks) cudaFree(scan->rows_walks);
+        scan->rows_walks = nullptr;
+        scan->rows_walks_cap = 0;
+        // the walks, then the passes' counters
+        if (cudaMalloc(&scan->rows_walks, sizeof(uint32_t) * hd::kPathWords *
+                                              static_cast<size_t>(chunk) + 64) != cudaSuccess) {
+            cudaGetLastError();
+            return HD_ERR_NOMEM;
+        }
+        scan->rows_walks_cap = chunk;
+    }
     HD_CUDA(hd::launch_pack_bits(hull, scan->V, scan->rows_bits, st));
-    const hd::Inputs in{angle_deg, u_in, v_in, u_out, v_out, nullptr};
-    HD_CUDA(hd::launch_rows_count(in, n, scan->gq, scan->cordic, hull, scan->rows_bits, row_ptr,
-                                  scan->sm_count, st));
+    unsigned *counters = scan->rows_walks + hd::kPathWords * scan->rows_walks_cap;
+    auto setup = [&](int64_t off, int64_t c) {
+        const hd::Inputs in{angle_deg + off, u_in + off, v_in + off, u_out + off, v_out + off, nullptr};
+        return hd::launch_rows_setup(in, c, scan->gq, scan->cordic, scan->rows_walks, scan->sm_count,
+                                     st);
+    };
+    for (int64_t off = 0; off < n; off += chunk) {
+        const int64_t c = n - off < chunk ? n - off : chunk;
+        HD_CUDA(setup(off, c));
+        HD_CUDA(hd::launch_rows_count(scan->rows_walks, c, scan->gq, scan->rows_bits, counters,
+                                      row_ptr + off, off == 0, scan->sm_count, st));
+    }
     HD_CUDA(hd::launch_rows_scan(row_ptr + 1, n, scan->rows_scratch, st));
     int64_t total = 0;
     HD_CUDA(cudaMemcpyAsync(&total, row_ptr + n, sizeof(int64_t), cudaMemcpyDeviceToHost, st));
     HD_CUDA(cudaStreamSynchronize(st));
     *nnz = total;
     if (total > capacity) return HD_ERR_RANGE;
-    HD_CUDA(hd::launch_rows_emit(in, n, scan->gq, scan->cordic, hull, scan->rows_bits, row_ptr,
-                                 cols, scan->sm_count, st));
+    for (int64_t off = 0; off < n; off += chunk) {
+        const int64_t c = n - off < chunk ? n - off : chunk;
+        if (n > chunk) {  // else the count pass' walks are still there
+            HD_CUDA(setup(off, c));
+            HD_CUDA(cudaMemsetAsync(counters, 0, 2 * sizeof(unsigned), st));
+        }
+        HD_CUDA(hd::launch_rows_emit(scan->rows_walks, c, scan->gq, scan->rows_bits, counters,
+                                     row_ptr + off, cols, scan->sm_count, st));
+    }
     return HD_OK;
 }
 

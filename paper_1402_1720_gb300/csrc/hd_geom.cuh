@@ -888,6 +888,235 @@ HD_HD void walk_path(const int32_t r[6], int nx, int ny, int nz, VisitT &visit)
     }
 }
 
+// -------------------------------------------------------------- path walk
+//
+// The whole-grid walk of one path as runs in path order, for segments with no
+// tie (nearly all): both minors cross between two major crossings, never at
+// the same parameter as one, and never together.  Counting major crossings
+// from the start, minor 0's next crossing comes after jn of them and z's after
+// jz (Bresenham steps of 32-bit integers, as in the lean walks below); when
+// both fall between the same two, the sign of e12 (advanced from the crossings
+// so far, only then) tells which comes first.  These are exactly the runs
+// run_next produces; a run costs about 20 instructions where the general step,
+// with its 64-bit order term and its saturated quotients, took about 90.
+struct PathWalk {
+    unsigned ad, Ru, rem;     // |D_0|, |D_m| mod |D_0|, Bresenham remainder
+    unsigned adz, Ruz, remz;  // the same for z
+    int jn, Qu, jz, Quz;      // next crossings, and |D_m| div |D_c| (capped)
+    int km, kc, kz;           // valid crossings left: major in all, minor 0, z
+    int im0;                  // major index of the first voxel
+    uint32_t vb;              // voxel of major index 0 in the current row
+    int fl;                   // bit 0 major +, 1 minor 0 +, 2 z +, 3 major is y
+    long long e12;            // order of minor 0 against z at the start (< 0: minor 0 first)
+    int c0, z0;               // kc and kz at the start
+    int s;                    // major crossings before the current run
+};
+constexpr int kPathWords = 16;  // packed size (64 bytes)
+
+// The path walk of gi -> go (grid Q16) over the grid: 1, 0 (no voxel), or -1
+// (a tie, or no in-plane motion: the general run walk).  The set-up is
+// slab_lean's with z an axis like the others.
+HD_HD int path_lean(const int32_t gi[3], const int32_t go[3], int nx, int ny, int nz, PathWalk &L)
+{
+    const int P[3] = {gi[0], gi[1], gi[2]};
+    const int D[3] = {go[0] - gi[0], go[1] - gi[1], go[2] - gi[2]};
+    const int n[3] = {nx, ny, nz};
+    if (D[0] == 0 && D[1] == 0) return -1;
+    unsigned tN = 0, tQ = 1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int H = n[a] << 16;
+        unsigned cN = 0, cQ = 1;
+        bool cand = false;
+        if (D[a] > 0) {
+            if (P[a] >= H) return 0;
+            if (P[a] < 0) { cN = static_cast<unsigned>(-P[a]); cQ = static_cast<unsigned>(D[a]); cand = true; }
+        } else if (D[a] < 0) {
+            if (P[a] < 0) return 0;
+            if (P[a] >= H) { cN = static_cast<unsigned>(P[a] - H); cQ = static_cast<unsigned>(-D[a]); cand = true; }
+        } else if (P[a] < 0 || P[a] >= H) {
+            return 0;
+        }
+        if (cand && static_cast<unsigned long long>(cN) * tQ > static_cast<unsigned long long>(tN) * cQ) {
+            tN = cN;
+            tQ = cQ;
+        }
+    }
+    if (tN > tQ) return 0;
+    int idx[3];
+    bool onp[3];
+    const float rQ = rcp_int(static_cast<int>(tQ));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const long long num = static_cast<long long>(P[a]) * tQ + static_cast<long long>(tN) * D[a];
+        long long rem;
+        idx[a] = fdiv32(num >> 16, static_cast<int>(tQ), rQ, rem);
+        onp[a] = rem == 0 && (num & 0xffff) == 0;
+    }
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        if ((D[a] > 0 && idx[a] >= n[a]) || (D[a] < 0 && idx[a] < 0)) return 0;
+    // an axis moving - that enters through its upper face (see slab_lean)
+    int out = -1;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        if (idx[a] >= n[a]) {
+            if (out >= 0) return -1;
+            out = a;
+        }
+    }
+    if (out >= 0) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            if (a != out && D[a] < 0 && onp[a]) return -1;
+            if (a == out) idx[a] -= 1;
+        }
+    }
+    int nm[3], k[3];
+    unsigned A[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const int f = go[a] >> 16;
+        const bool pos = D[a] > 0, neg = D[a] < 0;
+        A[a] = pos ? static_cast<unsigned>(D[a]) : (neg ? static_cast<unsigned>(-D[a]) : 0u);
+        nm[a] = pos ? ((idx[a] + 1) << 16) - P[a] : (neg ? P[a] - (idx[a] << 16) : 1);
+        k[a] = pos ? (f < n[a] - 1 ? f : n[a] - 1) - idx[a] : (neg ? idx[a] - (f > 0 ? f : 0) : 0);
+    }
+    if (k[0] < 0 || k[1] < 0 || k[2] < 0) return 0;  // the walk ends where it enters
+    const bool ymaj = A[1] > A[0];
+    const unsigned am = ymaj ? A[1] : A[0], a0 = ymaj ? A[0] : A[1], a1 = A[2];
+    const long long nmm = ymaj ? nm[1] : nm[0], nmc = ymaj ? nm[0] : nm[1], nmz = nm[2];
+    // minor against the major axis: the quotient and remainder of its first
+    // crossing, and of the step to the next
+    auto minor = [&](unsigned a, long long d, int &j, unsigned &rem, int &Qu, unsigned &Ru) {
+        j = kQBig;
+        rem = 0;
+        Qu = kQBig;
+        Ru = 0;
+        if (a == 0) return true;
+        if ((d & 0xffff) == 0) return false;  // may tie with the major axis
+        const unsigned qu = am / a;
+        Qu = qu >= (1u << 20) ? kQBig : static_cast<int>(qu);
+        Ru = am - qu * a;
+        const long long dh = d >> 16;
+        if (float_of(dh) < 1048576.0f * static_cast<float>(a)) {
+            long long rm;
+            const int q = fdiv32(dh, static_cast<int>(a), rcp_int(static_cast<int>(a)), rm);
+            if (q < -1) return false;
+            j = q + 1;
+            rem = static_cast<unsigned>(rm);
+        }
+        return true;
+    };
+    if (!minor(a0, nmc * am - nmm * a0, L.jn, L.rem, L.Qu, L.Ru)) return -1;
+    if (!minor(a1, nmz * am - nmm * a1, L.jz, L.remz, L.Quz, L.Ruz)) return -1;
+    L.e12 = a0 == 0 ? 1 : (a1 == 0 ? -1 : nmc * a1 - nmz * a0);
+    if (a0 != 0 && a1 != 0 && (L.e12 & 0xffff) == 0) return -1;  // the minors may tie
+    constexpr int kCap = 16383, kQuCap = 8192;  // beyond any box: never reached
+    L.jn = L.jn < kCap ? L.jn : kCap;
+    L.jz = L.jz < kCap ? L.jz : kCap;
+    L.Qu = L.Qu < kQuCap ? L.Qu : kQuCap;
+    L.Quz = L.Quz < kQuCap ? L.Quz : kQuCap;
+    L.ad = a0 != 0 ? a0 : 1u;
+    L.adz = a1 != 0 ? a1 : 1u;
+    L.km = ymaj ? k[1] : k[0];
+    L.kc = L.c0 = ymaj ? k[0] : k[1];
+    L.kz = L.z0 = k[2];
+    L.im0 = ymaj ? idx[1] : idx[0];
+    L.vb = static_cast<uint32_t>(ymaj ? idx[0] : nx * idx[1]) +
+           static_cast<uint32_t>(nx) * static_cast<uint32_t>(ny) * static_cast<uint32_t>(idx[2]);
+    L.fl = ((ymaj ? D[1] : D[0]) > 0 ? 1 : 0) | ((ymaj ? D[0] : D[1]) > 0 ? 2 : 0) |
+           (D[2] > 0 ? 4 : 0) | (ymaj ? 8 : 0);
+    L.s = 0;
+    return 1;
+}
+
+HD_HD void path_pack(const PathWalk &L, uint32_t o[kPathWords])
+{
+    o[0] = L.ad;
+    o[1] = L.Ru;
+    o[2] = L.rem;
+    o[3] = L.adz;
+    o[4] = L.Ruz;
+    o[5] = L.remz;
+    o[6] = static_cast<uint32_t>(L.jn) | (static_cast<uint32_t>(L.Qu) << 16);
+    o[7] = static_cast<uint32_t>(L.jz) | (static_cast<uint32_t>(L.Quz) << 16);
+    o[8] = static_cast<uint32_t>(L.km) | (static_cast<uint32_t>(L.kc) << 16);
+    o[9] = static_cast<uint32_t>(L.kz) | (static_cast<uint32_t>(L.im0) << 16);
+    o[10] = L.vb;
+    o[11] = static_cast<uint32_t>(L.fl);
+    o[12] = static_cast<uint32_t>(static_cast<unsigned long long>(L.e12) & 0xffffffffull);
+    o[13] = static_cast<uint32_t>(static_cast<unsigned long long>(L.e12) >> 32);
+    o[14] = o[15] = 0;
+}
+
+HD_HD void path_unpack(const uint32_t o[kPathWords], PathWalk &L)
+{
+    L.ad = o[0];
+    L.Ru = o[1];
+    L.rem = o[2];
+    L.adz = o[3];
+    L.Ruz = o[4];
+    L.remz = o[5];
+    L.jn = static_cast<int>(o[6] & 0xffffu);
+    L.Qu = static_cast<int>(o[6] >> 16);
+    L.jz = static_cast<int>(o[7] & 0xffffu);
+    L.Quz = static_cast<int>(o[7] >> 16);
+    L.km = static_cast<int>(o[8] & 0xffffu);
+    L.kc = L.c0 = static_cast<int>(o[8] >> 16);
+    L.kz = L.z0 = static_cast<int>(o[9] & 0xffffu);
+    L.im0 = static_cast<int>(o[9] >> 16);
+    L.vb = o[10];
+    L.fl = static_cast<int>(o[11]);
+    L.e12 = static_cast<long long>((static_cast<unsigned long long>(o[13]) << 32) | o[12]);
+    L.s = 0;
+}
+
+// When minor 0 and z both cross between the same two major crossings: whether z
+// does first.
+HD_HD bool path_z_first(const PathWalk &L)
+{
+    return L.e12 + ((static_cast<long long>(L.c0 - L.kc) * L.adz) << 16) -
+               ((static_cast<long long>(L.z0 - L.kz) * L.ad) << 16) >
+           0;
+}
+
+// The current run: vb the voxel of major index 0 in its row, a .. b its major
+// indices in path order (a > b when the major axis moves -).  Returns whether
+// more runs follow.
+HD_HD bool path_run(PathWalk &L, int nx, int plane, uint32_t &vb, int &a, int &b)
+{
+    const int j = L.jn < L.jz ? L.jn : L.jz;
+    const bool out = j > L.km;
+    const int e = out ? L.km : j;
+    vb = L.vb;
+    a = (L.fl & 1) ? L.im0 + L.s : L.im0 - L.s;
+    b = (L.fl & 1) ? L.im0 + e : L.im0 - e;
+    if (out) return false;
+    bool zc = L.jz < L.jn;
+    if (L.jz == L.jn) zc = path_z_first(L);
+    L.s = e;
+    if (!zc) {
+        if (L.kc == 0) return false;
+        --L.kc;
+        const int st = (L.fl & 8) ? 1 : nx;
+        L.vb += static_cast<uint32_t>((L.fl & 2) ? st : -st);
+        L.rem += L.Ru;
+        const bool carry = L.rem >= L.ad;
+        L.rem = carry ? L.rem - L.ad : L.rem;
+        L.jn += L.Qu + (carry ? 1 : 0);
+    } else {
+        if (L.kz == 0) return false;
+        --L.kz;
+        L.vb += static_cast<uint32_t>((L.fl & 4) ? plane : -plane);
+        L.remz += L.Ruz;
+        const bool carry = L.remz >= L.adz;
+        L.remz = carry ? L.remz - L.adz : L.remz;
+        L.jz += L.Quz + (carry ? 1 : 0);
+    }
+    return true;
+}
+
 // ---------------------------------------------------------- lean run walk
 //
 // Most walks inside a one-voxel-deep tile are "lean": the in-plane minor

@@ -17,6 +17,36 @@ extern "C" long long hx_to_grid(int n, float s, const int32_t *w, long long coun
     return bad;
 }
 
+// The path walk (through pack and unpack) against the general run walk, run by
+// run: returns its runs, 0 when neither has a voxel, -1 when it declines, -2
+// when only one of them has a voxel, -3 when a run differs.
+extern "C" int hx_path(const int32_t *gi, const int32_t *go, int nx, int ny, int nz)
+{
+    hd::PathWalk P;
+    hd::RunWalk w;
+    const int r = hd::path_lean(gi, go, nx, ny, nz, P);
+    const bool have = hd::run_begin(w, gi, go, nx, ny, nz);
+    if (r < 0) return -1;
+    if (r == 0) return have ? -2 : 0;
+    if (!have) return -2;
+    uint32_t o[hd::kPathWords];
+    hd::path_pack(P, o);
+    hd::path_unpack(o, P);
+    const bool ymaj = (w.flags >> 5) & 1, plus = w.flags & 1;
+    int row, lo, hi, n = 0;
+    bool more = true;
+    while (hd::run_next(w, row, lo, hi)) {
+        if (!more) return -3;
+        uint32_t vb;
+        int a, b;
+        more = hd::path_run(P, nx, nx * ny, vb, a, b);
+        const uint32_t base = ymaj ? row % nx + nx * ny * (row / nx) : nx * row;
+        if (vb != base || a != (plus ? lo : hi) || b != (plus ? hi : lo)) return -3;
+        ++n;
+    }
+    return more ? -3 : n;
+}
+
 // The event walk of the oriented segment in a box of dx x dy x dz voxels,
 // dilated by `thick`: its updates applied to plain counters in the tile's
 // layout, decoded by the definition (prefix sums along the major axis), the

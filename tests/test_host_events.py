@@ -80,6 +80,22 @@ def test_event_walks_equal_oracle(oracle_mod, hx, dims, direct):
     assert seen > 300
 
 
+@pytest.mark.parametrize("dims", [(5, 4, 3), (1, 1, 1), (7, 1, 2), (40, 30, 20), (9, 1, 1),
+                                  (64, 64, 8), (17, 200, 3)])
+def test_path_walk_equals_run_walk(hx, dims):
+    """Every run of the path walk is the general run walk's, in order; it
+    declines only ties and paths without in-plane motion."""
+    rng = np.random.default_rng(sum(dims) + 5)
+    generic = list(_generic(rng, 4000, dims))
+    taken = 0
+    for k, (a, b) in enumerate(generic + list(_random_segments(rng, 4000, dims))):
+        n = hx.hx_path(np.asarray(a, np.int32).ctypes.data_as(I32P),
+                       np.asarray(b, np.int32).ctypes.data_as(I32P), *dims)
+        assert n >= -1, (n, np.asarray(a).tolist(), np.asarray(b).tolist())
+        taken += n >= 0 and k < len(generic)
+    assert taken > 0.95 * len(generic)
+
+
 @pytest.mark.parametrize("n,s", [(4096, 1 / 64), (128, 64.0), (4096, 2.0), (1, 64.0), (200, 1.0),
                                  (181, 0.93), (64, 0.015640259), (127, 63.99998)])
 def test_grid_coordinate_is_exact(hx, n, s):
