@@ -5,16 +5,22 @@
 // is missed and its line is carved in every slice it covers; the carved
 // image is averaged over a window in each slice and thresholded.
 //
-// Four stream-ordered kernels, all integer arithmetic:
-//   binned_stats_kernel  one thread per history: 7 64-bit atomics into its
-//                        bin's row of the table (n, S and Q of 3 values)
-//   binned_cut_kernel    one thread per history: the 3 sigma test in 128-bit
-//                        integers against the finished statistics, kept n
-//                        and kept WEPL sum by 2 atomics
-//   binned_carve_kernel  one block per (angle bin, slice): the lines of the
-//                        block's missed bins walked run by run into a bitmap
-//                        of the slice in shared memory, merged into the
-//                        volume bitmap with one atomicAnd per changed word
+// Stream-ordered kernels, all integer arithmetic.  Two passes over the
+// histories, each in one of two forms:
+//   binned_stats_tiles_kernel, binned_cut_tiles_kernel  a block per SM takes
+//                        consecutive histories and keeps the bins of one gantry
+//                        angle in shared memory (histories arrive angle by
+//                        angle); the finished table goes out with one atomic per
+//                        bin and word.  Sums of n, S and Q of 3 values; then the
+//                        3 sigma test against bounds taken once per bin
+//   binned_stats_kernel, binned_cut_kernel  one thread per history, 7 and 2
+//                        64-bit atomics into its bin's row of the table: few
+//                        histories, or an angle's bins beyond shared memory
+// and the image:
+//   binned_carve_kernel  one block per (angle bin, vertical bin): the lines of
+//                        the block's missed bins walked run by run into a bitmap
+//                        in shared memory, merged into the volume bitmap of each
+//                        slice of the bin with one atomicAnd per changed word
 //   binned_filter_kernel one thread per voxel: the window count of uncarved
 //                        voxels, the hull byte and the carved byte
 #include <cmath>
@@ -28,7 +34,14 @@ struct BinQ {
     int n_ang, n_u, n_v, k;
     long long ang_q, u_q, v_q, u_lo_q, v_lo_q;  // Q16 degrees and mm
     long long miss_q8;                          // 1/256 mm
+    float r_ang, r_u, r_v;                      // rcp_int of twice the bin sizes
     int w, min_count;
+};
+
+// Slices z0 .. z1 - 1 share the lines of vertical bin iv; count: the bin's
+// statistics are counted with this group (the first of its bin).
+struct SliceGroup {
+    int iv, z0, z1, count;
 };
 
 namespace {
@@ -41,30 +54,64 @@ constexpr int kCtrWords = 8;
 constexpr int kMaxSmemWords = 48 * 1024;  // slice bitmaps up to 192 KB in shared memory
 constexpr long long kFull = 360LL * 65536;
 
-__device__ __forceinline__ long long q8_of(float x) { return __float2ll_rn(x * 256.0f); }
+__device__ __forceinline__ int q8_of(float x) { return __float2int_rn(x * 256.0f); }
 
-// Bin of one history, -1 when it is not binned; x receives WEPL, lateral and
-// vertical slope in 1/256 mm.
-__device__ __forceinline__ long long bin_of(const BinQ &b, float ang, float ui, float vi, float uo,
-                                            float vo, float wepl, long long x[3])
+// floor(a / b) for |a| < 2^30, 0 < b < 2^30 and |a / b| < 2^18, rb = rcp_int(b):
+// the float quotient is within one of it.
+__device__ __forceinline__ int bin_div(int a, int b, float rb)
 {
-    if (!(fabsf(ang) < 1048576.0f) || !(fabsf(wepl) < 1024.0f)) return -1;
+    int q = __float2int_rd(static_cast<float>(a) * rb);
+    const int r = a - q * b;
+    if (r < 0) --q;
+    if (r >= b) ++q;
+    return q;
+}
+
+struct BinAt {
+    int ia, iu, iv;
+    int x[3];  // WEPL (|.| <= 2^18), lateral and vertical slope (< 2^18) in 1/256 mm
+};
+
+// Angle bin of an angle with |ang| < 2^20.
+__device__ __forceinline__ int angle_bin(const BinQ &b, float ang)
+{
+    int a;
+    if (ang >= 0.0f && ang < 360.0f) {
+        a = __float2int_rn(ang * 65536.0f);
+        if (a == static_cast<int>(kFull)) a = 0;
+    } else {
+        const long long t = q16_of(ang);  // |t| < 2^36: a small quotient
+        a = static_cast<int>(t - floordiv_small(t, kFull) * kFull);
+    }
+    const int q = static_cast<int>(b.ang_q);
+    const int ia = bin_div(2 * a + q, 2 * q, b.r_ang);  // nearest centre
+    return ia == b.n_ang ? 0 : ia;
+}
+
+// Bin of one history; false when it is not binned.  All in 32 bits: u and v in
+// Q16 stay below 2^28, twice a bin size and twice a lower edge below 2^29.
+__device__ __forceinline__ bool bin_of(const BinQ &b, float ang, float ui, float vi, float uo,
+                                       float vo, float wepl, BinAt &o)
+{
+    if (!(fabsf(ang) < 1048576.0f) || !(fabsf(wepl) < 1024.0f)) return false;
     if (!(fabsf(ui) < 4096.0f) || !(fabsf(vi) < 4096.0f) || !(fabsf(uo) < 4096.0f) ||
         !(fabsf(vo) < 4096.0f))
-        return -1;
-    x[0] = q8_of(wepl);
-    x[1] = q8_of(uo) - q8_of(ui);
-    x[2] = q8_of(vo) - q8_of(vi);
-    if (llabs(x[1]) >= 1024 * 256 || llabs(x[2]) >= 1024 * 256) return -1;
-    long long a = q16_of(ang);  // |a| < 2^36: the quotients below are small
-    a -= floordiv_small(a, kFull) * kFull;
-    long long ia = floordiv_small(2 * a + b.ang_q, 2 * b.ang_q);  // nearest centre
-    if (ia == b.n_ang) ia = 0;
-    const long long u2 = q16_of(ui) + q16_of(uo), v2 = q16_of(vi) + q16_of(vo);
-    const long long iu = floordiv_small(u2 - 2 * b.u_lo_q, 2 * b.u_q);
-    const long long iv = floordiv_small(v2 - 2 * b.v_lo_q, 2 * b.v_q);
-    if (iu < 0 || iu >= b.n_u || iv < 0 || iv >= b.n_v) return -1;
-    return ia + static_cast<long long>(b.n_ang) * (iu + static_cast<long long>(b.n_u) * iv);
+        return false;
+    o.x[0] = q8_of(wepl);
+    o.x[1] = q8_of(uo) - q8_of(ui);
+    o.x[2] = q8_of(vo) - q8_of(vi);
+    if (abs(o.x[1]) >= 1024 * 256 || abs(o.x[2]) >= 1024 * 256) return false;
+    o.ia = angle_bin(b, ang);
+    const int u2 = q16_small(ui) + q16_small(uo) - 2 * static_cast<int>(b.u_lo_q);
+    const int v2 = q16_small(vi) + q16_small(vo) - 2 * static_cast<int>(b.v_lo_q);
+    o.iu = bin_div(u2, 2 * static_cast<int>(b.u_q), b.r_u);
+    o.iv = bin_div(v2, 2 * static_cast<int>(b.v_q), b.r_v);
+    return o.iu >= 0 && o.iu < b.n_u && o.iv >= 0 && o.iv < b.n_v;
+}
+
+__device__ __forceinline__ long long row_of(const BinQ &b, const BinAt &o)
+{
+    return o.ia + static_cast<long long>(b.n_ang) * (o.iu + static_cast<long long>(b.n_u) * o.iv);
 }
 
 // x within k population standard deviations of a bin holding n values of
@@ -90,61 +137,398 @@ __device__ __forceinline__ void warp_add(unsigned long long v, unsigned long lon
     if ((threadIdx.x & 31) == 0 && v != 0) atomicAdd(dst, v);
 }
 
-__global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_stats_kernel(Inputs in, int64_t n, BinQ b,
-                                                                   unsigned long long *acc,
-                                                                   unsigned long long *ctr)
+__device__ __forceinline__ unsigned long long u64_of(int x)
 {
-    unsigned long long binned = 0;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += stride) {
-        long long x[3];
-        const long long bi = bin_of(b, in.angle[i], in.u_in[i], in.v_in[i], in.u_out[i],
-                                    in.v_out[i], in.wepl[i], x);
-        if (bi < 0) continue;
-        unsigned long long *a = acc + kAccWords * bi;
-        atomicAdd(a, 1ull);
+    return static_cast<unsigned long long>(static_cast<long long>(x));
+}
+
+// The six sums of one history into its bin's row.
+__device__ __forceinline__ void add_sums(unsigned long long *a, const int x[3])
+{
 #pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            atomicAdd(a + 1 + q, static_cast<unsigned long long>(x[q]));
-            atomicAdd(a + 4 + q, static_cast<unsigned long long>(x[q] * x[q]));
-        }
-        ++binned;
+    for (int q = 0; q < 3; ++q) {
+        atomicAdd(a + 1 + q, u64_of(x[q]));
+        atomicAdd(a + 4 + q, static_cast<unsigned long long>(static_cast<long long>(x[q]) * x[q]));
     }
+}
+
+// The 3 sigma test of one history against its bin's finished statistics
+// (words 0-6, while other threads add to words 7 and 8).
+__device__ __forceinline__ bool keep_of(const BinQ &b, const unsigned long long *a, const int x[3])
+{
+    const long long cnt = static_cast<long long>(a[0]);
+    bool keep = true;
+#pragma unroll
+    for (int q = 0; q < 3; ++q)
+        keep = keep && within(cnt, static_cast<long long>(a[1 + q]),
+                              static_cast<long long>(a[4 + q]), x[q], b.k);
+    return keep;
+}
+
+// Histories i, i + stride, .. below end without a table, those of vertical bins
+// v0 .. v1 - 1: seven and two atomics each.  kAtOnce of them are in flight.
+template <int kAtOnce>
+__device__ __forceinline__ void load_histories(const Inputs &in, int64_t i, int64_t end,
+                                               int64_t stride, float h[kAtOnce][6])
+{
+#pragma unroll
+    for (int k = 0; k < kAtOnce; ++k) {
+        const int64_t j = i + k * stride;
+        h[k][0] = 2097152.0f;  // not binned
+        if (j < end) {
+            h[k][0] = __ldg(in.angle + j);
+            h[k][1] = __ldg(in.u_in + j);
+            h[k][2] = __ldg(in.v_in + j);
+            h[k][3] = __ldg(in.u_out + j);
+            h[k][4] = __ldg(in.v_out + j);
+            h[k][5] = __ldg(in.wepl + j);
+        }
+    }
+}
+
+template <int kAtOnce>
+__device__ __forceinline__ unsigned stats_direct(const Inputs &in, int64_t i, int64_t end,
+                                                 int64_t stride, const BinQ &b, int v0, int v1,
+                                                 unsigned long long *acc)
+{
+    unsigned binned = 0;
+    for (; i < end; i += kAtOnce * stride) {
+        float h[kAtOnce][6];
+        load_histories<kAtOnce>(in, i, end, stride, h);
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            BinAt o;
+            if (!bin_of(b, h[k][0], h[k][1], h[k][2], h[k][3], h[k][4], h[k][5], o)) continue;
+            if (o.iv < v0 || o.iv >= v1) continue;
+            unsigned long long *a = acc + kAccWords * row_of(b, o);
+            atomicAdd(a, 1ull);
+            add_sums(a, o.x);
+            ++binned;
+        }
+    }
+    return binned;
+}
+
+template <int kAtOnce>
+__device__ __forceinline__ unsigned cut_direct(const Inputs &in, int64_t i, int64_t end,
+                                               int64_t stride, const BinQ &b, int v0, int v1,
+                                               unsigned long long *acc)
+{
+    unsigned cut = 0;
+    for (; i < end; i += kAtOnce * stride) {
+        float h[kAtOnce][6];
+        load_histories<kAtOnce>(in, i, end, stride, h);
+        unsigned long long *a[kAtOnce];
+        unsigned long long w[kAtOnce][7];
+        int x[kAtOnce][3];
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            BinAt o;
+            a[k] = nullptr;
+            if (!bin_of(b, h[k][0], h[k][1], h[k][2], h[k][3], h[k][4], h[k][5], o)) continue;
+            if (o.iv < v0 || o.iv >= v1) continue;
+            a[k] = acc + kAccWords * row_of(b, o);
+#pragma unroll
+            for (int f = 0; f < 7; ++f) w[k][f] = a[k][f];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) x[k][q] = o.x[q];
+        }
+#pragma unroll
+        for (int k = 0; k < kAtOnce; ++k) {
+            if (a[k] == nullptr) continue;
+            if (!keep_of(b, w[k], x[k])) {
+                ++cut;
+                continue;
+            }
+            atomicAdd(a[k] + 7, 1ull);
+            atomicAdd(a[k] + 8, u64_of(x[k][0]));
+        }
+    }
+    return cut;
+}
+
+__global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_stats_kernel(
+    Inputs in, int64_t n, BinQ b, unsigned long long *acc, unsigned long long *ctr)
+{
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    warp_add(stats_direct<1>(in, i, n, static_cast<int64_t>(gridDim.x) * blockDim.x, b, 0, b.n_v, acc),
+             ctr + 0);
+}
+
+__global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_cut_kernel(
+    Inputs in, int64_t n, BinQ b, unsigned long long *acc, unsigned long long *ctr)
+{
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    warp_add(cut_direct<1>(in, i, n, static_cast<int64_t>(gridDim.x) * blockDim.x, b, 0, b.n_v, acc),
+             ctr + 1);
+}
+
+// ---- the passes with an angle's bins in shared memory ----
+//
+// Bound: shared-memory atomics (ten per history, random banks) and integer issue.
+// Head grid, 9e6 histories: statistics 365 -> 97 us, cuts 250 -> 112 us (7 and 2
+// 64-bit atomics per history in L2 before, and 128-bit tests for each).
+
+constexpr int kTileThreads = 768;   // one block per SM
+constexpr int kTileUnroll = 2;      // histories per thread and chunk, the next chunk's in flight
+constexpr int kTileChunk = kTileThreads * kTileUnroll;
+constexpr int kStatsWords = 10;     // n, S x 3, Q low 18 bits x 3, Q high x 3
+constexpr int kCutWords = 8;        // bounds x 6, kept n, kept sum
+constexpr int kTileBytes = 224000;  // of the 227 KB a block can have
+// Sums of one flush's histories per bin: beyond this many in a bin the rest of
+// its values go straight to the table.  2^18 times it stays below 2^31.
+constexpr unsigned kTileCount = 8191;
+constexpr int kMaxWindows = 4;
+// Histories per bin of an angle and block that pay for a table (head grid, 4544
+// bins an angle: at 1.1 million histories in all 245 us with it, 228 without; at
+// 1.8 million 265 and 279).
+constexpr int kTileFill = 2;
+
+// The window of vertical bins a block keeps (n_v split into n_win windows of
+// rows bins each, a block per window and segment of histories).
+struct BinTiles {
+    int n_win, rows;
+};
+
+// Chunks of kTileThreads * kTileUnroll consecutive histories; the table holds
+// the angle bin of a chunk's first history, and a chunk that begins with another
+// angle changes it.  Where angles come in no order a table buys nothing: chunks
+// whose first, middle and last history lie in three angles change nothing, and a
+// block that meets many of them hands its histories to the direct loop.
+struct TileAngle {
+    int cur = -1, stray = 0, chunks = 0;
+    // next: the angle to change to; s: the three histories' angles
+    __device__ __forceinline__ bool due(const BinQ &b, const float s[3], int &next)
+    {
+        ++chunks;
+        next = fabsf(s[0]) < 1048576.0f ? angle_bin(b, s[0]) : cur;
+        if (next == cur) return false;
+        if (s[0] != s[1] && s[1] != s[2]) {
+            ++stray;
+            return false;
+        }
+        return true;
+    }
+    __device__ __forceinline__ bool lost() const { return stray > 2 + chunks / 4; }
+};
+
+// Columns of this thread's histories of the chunk at c0; past i1 an angle that is
+// not binned.
+__device__ __forceinline__ void load_chunk(const Inputs &in, int64_t c0, int64_t i1,
+                                           float h[kTileUnroll][6], float s[3])
+{
+    if (c0 >= i1) return;
+    s[0] = __ldg(in.angle + c0);
+    s[1] = __ldg(in.angle + min(c0 + kTileChunk / 2, i1 - 1));
+    s[2] = __ldg(in.angle + min(c0 + kTileChunk, i1) - 1);
+    load_histories<kTileUnroll>(in, c0 + threadIdx.x, i1, kTileThreads, h);
+}
+
+__global__ void __launch_bounds__(kTileThreads) binned_stats_tiles_kernel(Inputs in, int64_t n,
+                                                                          BinQ b, BinTiles t,
+                                                                          unsigned long long *acc,
+                                                                          unsigned long long *ctr)
+{
+    extern __shared__ uint32_t s_tab[];  // word f of bin e at f * E + e
+    const int win = blockIdx.x % t.n_win, seg = blockIdx.x / t.n_win, n_seg = gridDim.x / t.n_win;
+    const int64_t i0 = n * seg / n_seg, i1 = n * (seg + 1) / n_seg;
+    const int v0 = win * t.rows, v1 = min(b.n_v, v0 + t.rows);
+    const int E = b.n_u * (v1 - v0);
+    for (int e = threadIdx.x; e < kStatsWords * E; e += kTileThreads) s_tab[e] = 0u;
+    unsigned long long binned = 0;
+    TileAngle ang;
+    auto flush = [&]() {
+        __syncthreads();
+        if (ang.cur >= 0) {
+            for (int e = threadIdx.x; e < E; e += kTileThreads) {
+                const uint32_t c = s_tab[e];
+                if (c == 0u) continue;
+                unsigned long long *a =
+                    acc + kAccWords * (ang.cur + static_cast<long long>(b.n_ang) *
+                                                     (e + static_cast<long long>(b.n_u) * v0));
+                atomicAdd(a, static_cast<unsigned long long>(c));
+                s_tab[e] = 0u;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    uint32_t *const S = s_tab + (1 + q) * E + e, *const L = S + 3 * E,
+                                   *const H = S + 6 * E;
+                    atomicAdd(a + 1 + q, u64_of(static_cast<int>(*S)));
+                    atomicAdd(a + 4 + q, (static_cast<unsigned long long>(*H) << 18) + *L);
+                    *S = *L = *H = 0u;
+                }
+            }
+        }
+        __syncthreads();
+    };
+    float ahead[kTileUnroll][6] = {}, sample[3] = {};
+    load_chunk(in, i0, i1, ahead, sample);
+    int64_t c0 = i0;
+    for (; c0 < i1 && !ang.lost(); c0 += kTileChunk) {
+        int next;
+        if (ang.due(b, sample, next)) {
+            flush();
+            ang.cur = next;
+        }
+        float h[kTileUnroll][6];
+#pragma unroll
+        for (int k = 0; k < kTileUnroll; ++k)
+#pragma unroll
+            for (int f = 0; f < 6; ++f) h[k][f] = ahead[k][f];
+        load_chunk(in, c0 + kTileChunk, i1, ahead, sample);
+#pragma unroll
+        for (int k = 0; k < kTileUnroll; ++k) {
+            BinAt o;
+            if (!bin_of(b, h[k][0], h[k][1], h[k][2], h[k][3], h[k][4], h[k][5], o)) continue;
+            if (o.iv < v0 || o.iv >= v1) continue;
+            ++binned;
+            if (o.ia != ang.cur) {
+                unsigned long long *a = acc + kAccWords * row_of(b, o);
+                atomicAdd(a, 1ull);
+                add_sums(a, o.x);
+                continue;
+            }
+            const int e = o.iu + b.n_u * (o.iv - v0);
+            if (atomicAdd(s_tab + e, 1u) >= kTileCount) {
+                add_sums(acc + kAccWords * row_of(b, o), o.x);
+                continue;
+            }
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                uint32_t *const S = s_tab + (1 + q) * E + e;
+                atomicAdd(S, static_cast<uint32_t>(o.x[q]));
+                const unsigned long long x2 =
+                    static_cast<unsigned long long>(static_cast<long long>(o.x[q]) * o.x[q]);
+                atomicAdd(S + 3 * E, static_cast<uint32_t>(x2) & 0x3ffffu);
+                const uint32_t hi = static_cast<uint32_t>(x2 >> 18);
+                if (hi != 0u) atomicAdd(S + 6 * E, hi);
+            }
+        }
+    }
+    flush();
+    binned += stats_direct<2>(in, c0 + threadIdx.x, i1, kTileThreads, b, v0, v1, acc);
     warp_add(binned, ctr + 0);
 }
 
-// Reads words 0-6 of a bin row (fixed since the statistics phase ended)
-// while other threads add to words 7 and 8.
-__global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_cut_kernel(Inputs in, int64_t n, BinQ b,
-                                                                 unsigned long long *acc,
-                                                                 unsigned long long *ctr)
+// The test of within() as |x - m| <= r with m = S / n and r = k sqrt(n Q - S^2) / n
+// in float: m is off by less than 3 2^-24 of 2^18 and the difference by half a
+// unit of 2^19, together less than kCutSlack, and r by less than kCutEps of itself.  A
+// value inside by both margins is kept, one outside by both is cut, the rest
+// take the test in integers.  Empty bins keep everything (r infinite); a variance
+// that wrapped below zero leaves all to the integers (r a NaN).  (Integer bounds
+// per bin needed exact roots and divisions: 29 of the pass's 82 million warp
+// instructions.)
+constexpr float kCutSlack = 0.25f, kCutEps = 3.814697265625e-6f;  // 2^-18
+
+__device__ __forceinline__ float2 cut_limits(int k, const unsigned long long *a, int q)
 {
-    unsigned long long cut = 0;
-    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-         i += stride) {
-        long long x[3];
-        const long long bi = bin_of(b, in.angle[i], in.u_in[i], in.v_in[i], in.u_out[i],
-                                    in.v_out[i], in.wepl[i], x);
-        if (bi < 0) continue;
-        unsigned long long *a = acc + kAccWords * bi;
-        const long long cnt = static_cast<long long>(a[0]);
-        bool keep = true;
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            keep = keep && within(cnt, static_cast<long long>(a[1 + q]),
-                                  static_cast<long long>(a[4 + q]), x[q], b.k);
-        if (!keep) {
-            ++cut;
-            continue;
-        }
-        atomicAdd(a + 7, 1ull);
-        atomicAdd(a + 8, static_cast<unsigned long long>(x[0]));
+    const unsigned long long n = a[0];
+    const long long S = static_cast<long long>(a[1 + q]), Q = static_cast<long long>(a[4 + q]);
+    if (n == 0) return make_float2(0.0f, INFINITY);
+    float var;
+    if (n < 8192) {  // n Q and S^2 below 2^62
+        var = __ll2float_rn(static_cast<long long>(n) * Q - S * S);
+    } else {
+        const __int128 v = static_cast<__int128>(n) * Q - static_cast<__int128>(S) * S;
+        var = __ll2float_rn(static_cast<long long>(v >> 62)) * 4611686018427387904.0f +
+              __ll2float_rn(static_cast<long long>(v & ((static_cast<__int128>(1) << 62) - 1)));
     }
+    const float fn = __ull2float_rn(n);
+    return make_float2(__fdiv_rn(__ll2float_rn(S), fn),
+                       __fdiv_rn(static_cast<float>(k) * __fsqrt_rn(var), fn));
+}
+
+__global__ void __launch_bounds__(kTileThreads) binned_cut_tiles_kernel(Inputs in, int64_t n, BinQ b,
+                                                                        BinTiles t,
+                                                                        unsigned long long *acc,
+                                                                        unsigned long long *ctr)
+{
+    extern __shared__ uint32_t s_tab[];  // limits of the 3 values, kept n, kept sum
+    float2 *const s_lim = reinterpret_cast<float2 *>(s_tab);
+    const int win = blockIdx.x % t.n_win, seg = blockIdx.x / t.n_win, n_seg = gridDim.x / t.n_win;
+    const int64_t i0 = n * seg / n_seg, i1 = n * (seg + 1) / n_seg;
+    const int v0 = win * t.rows, v1 = min(b.n_v, v0 + t.rows);
+    const int E = b.n_u * (v1 - v0);
+    unsigned long long cut = 0;
+    TileAngle ang;
+    auto row_at = [&](int e) {
+        return acc + kAccWords * (ang.cur + static_cast<long long>(b.n_ang) *
+                                                (e + static_cast<long long>(b.n_u) * v0));
+    };
+    auto flush = [&]() {
+        __syncthreads();
+        if (ang.cur >= 0) {
+            for (int e = threadIdx.x; e < E; e += kTileThreads) {
+                const uint32_t c = s_tab[6 * E + e];
+                if (c == 0u) continue;
+                unsigned long long *a = row_at(e);
+                atomicAdd(a + 7, static_cast<unsigned long long>(c));
+                atomicAdd(a + 8, u64_of(static_cast<int>(s_tab[7 * E + e])));
+            }
+        }
+    };
+    float ahead[kTileUnroll][6] = {}, sample[3] = {};
+    load_chunk(in, i0, i1, ahead, sample);
+    int64_t c0 = i0;
+    for (; c0 < i1 && !ang.lost(); c0 += kTileChunk) {
+        int next;
+        if (ang.due(b, sample, next)) {
+            flush();
+            ang.cur = next;
+            for (int e = threadIdx.x; e < E; e += kTileThreads) {
+                const unsigned long long *a = row_at(e);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) s_lim[q * E + e] = cut_limits(b.k, a, q);
+                s_tab[6 * E + e] = s_tab[7 * E + e] = 0u;
+            }
+            __syncthreads();
+        }
+        float h[kTileUnroll][6];
+#pragma unroll
+        for (int k = 0; k < kTileUnroll; ++k)
+#pragma unroll
+            for (int f = 0; f < 6; ++f) h[k][f] = ahead[k][f];
+        load_chunk(in, c0 + kTileChunk, i1, ahead, sample);
+#pragma unroll
+        for (int k = 0; k < kTileUnroll; ++k) {
+            BinAt o;
+            if (!bin_of(b, h[k][0], h[k][1], h[k][2], h[k][3], h[k][4], h[k][5], o)) continue;
+            if (o.iv < v0 || o.iv >= v1) continue;
+            if (o.ia != ang.cur) {
+                unsigned long long *a = acc + kAccWords * row_of(b, o);
+                if (!keep_of(b, a, o.x)) {
+                    ++cut;
+                    continue;
+                }
+                atomicAdd(a + 7, 1ull);
+                atomicAdd(a + 8, u64_of(o.x[0]));
+                continue;
+            }
+            const int e = o.iu + b.n_u * (o.iv - v0);
+            bool keep = true, out = false;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const float2 lim = s_lim[q * E + e];
+                const float d = fabsf(static_cast<float>(o.x[q]) - lim.x);
+                keep = keep && d <= lim.y * (1.0f - kCutEps) - kCutSlack;
+                out = out || d > lim.y * (1.0f + kCutEps) + kCutSlack;
+            }
+            if (!keep && !out) keep = keep_of(b, row_at(e), o.x);
+            if (!keep) {
+                ++cut;
+                continue;
+            }
+            if (atomicAdd(s_tab + 6 * E + e, 1u) >= kTileCount)
+                atomicAdd(row_at(e) + 8, u64_of(o.x[0]));
+            else
+                atomicAdd(s_tab + 7 * E + e, static_cast<uint32_t>(o.x[0]));
+        }
+    }
+    flush();
+    cut += cut_direct<2>(in, c0 + threadIdx.x, i1, kTileThreads, b, v0, v1, acc);
     warp_add(cut, ctr + 1);
 }
 
+// Bins used and missed, where the carving blocks do not count them.
 __global__ void __launch_bounds__(kBinThreads) binned_bins_kernel(const unsigned long long *acc,
                                                                   int64_t nb, long long miss_q8,
                                                                   unsigned long long *ctr)
@@ -189,19 +573,22 @@ __device__ __forceinline__ void clear_run(uint32_t *img, bool ymaj, int row, int
 }
 
 // Host-computed line tables: centre angle of each angle bin, lateral centre
-// of each u bin, centre height and vertical bin (or -1) of each slice.
+// of each u bin, centre height of each slice, and the groups of slices.
 struct LineTables {
     const float *ang_c, *u_c, *zc;
-    const int *slice_bin;
+    const SliceGroup *groups;
 };
 
 constexpr int kMaxLinesPerBlock = 1024;  // lateral bins a block lists at once
 
-// One block per (angle bin, slice): the block's missed bins are listed in
-// shared memory, then each thread walks lines from the list.  A line lies at
-// the slice's centre height, so its walk is clipped to the slice (a box one
+// One block per (angle bin, group of slices): the block's missed bins are
+// listed in shared memory, then each thread walks lines from the list.  A line
+// lies at a slice's centre height, so its walk is clipped to the slice (a box one
 // voxel deep) and is lean unless a crossing ties with another: the runs then
-// come from the closed-form cursor, otherwise from the general run walk.
+// come from the closed-form cursor, otherwise from the general run walk.  The
+// lines of one vertical bin differ between its slices in their height alone, and a
+// height inside the slice crosses nothing: one walk serves every slice of a group
+// (slices of 2.5 mm in bins of 5 mm: 154 -> 108 us on the head grid).
 template <bool kShared>
 __global__ void __launch_bounds__(kCarveThreads) binned_carve_kernel(
     const unsigned long long *acc, BinQ b, GeomQ g, Cordic cd, LineTables t, uint32_t *bits,
@@ -211,15 +598,16 @@ __global__ void __launch_bounds__(kCarveThreads) binned_carve_kernel(
     __shared__ int s_list[kMaxLinesPerBlock];
     __shared__ int s_warp[kCarveThreads / 32];
     __shared__ long long s_cs[2];
-    const int ia = blockIdx.x, z = blockIdx.y;
-    const int iv = t.slice_bin[z];
-    if (iv < 0) return;  // the same for the whole block
+    const int ia = blockIdx.x;
+    const SliceGroup grp = t.groups[blockIdx.y];
+    const int iv = grp.iv, z = grp.z0;
+    const bool empty = grp.z1 == grp.z0;  // no slice: the bin is only counted
     uint32_t *gimg = bits + static_cast<size_t>(z) * wps;
     uint32_t *img = kShared ? sm : gimg;
     if (kShared)
         for (int w = threadIdx.x; w < wps; w += blockDim.x) sm[w] = 0xffffffffu;
     const uint32_t plane = static_cast<uint32_t>(g.nx) * static_cast<uint32_t>(g.ny);
-    const float zc = t.zc[z];
+    const float zc = empty ? 0.0f : t.zc[z];
     if (threadIdx.x == 0) {  // the block's gantry cos and sin, once
         long long c, sn;
         cordic_cs(q16_of(t.ang_c[ia]), cd, c, sn);
@@ -227,7 +615,7 @@ __global__ void __launch_bounds__(kCarveThreads) binned_carve_kernel(
         s_cs[1] = sn;
     }
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
-    unsigned long long lines = 0, outside = 0;
+    unsigned long long lines = 0, outside = 0, used = 0, missed = 0;
     for (int base = 0; base < b.n_u; base += kMaxLinesPerBlock) {
         // the chunk's missed bins, listed in lateral order (neighbouring
         // lanes then walk neighbouring, similar lines)
@@ -239,7 +627,13 @@ __global__ void __launch_bounds__(kCarveThreads) binned_carve_kernel(
             if (iu < end) {
                 const long long bi = ia + static_cast<long long>(b.n_ang) *
                                               (iu + static_cast<long long>(b.n_u) * iv);
-                miss = bin_missed(acc + kAccWords * bi, b.miss_q8);
+                const unsigned long long *a = acc + kAccWords * bi;
+                miss = bin_missed(a, b.miss_q8);
+                if (grp.count) {
+                    used += a[0] != 0 ? 1 : 0;
+                    missed += miss ? 1 : 0;
+                }
+                miss = miss && !empty;
             }
             const unsigned bal = __ballot_sync(0xffffffffu, miss);
             if (lane == 0) s_warp[warp] = __popc(bal);
@@ -289,11 +683,16 @@ __global__ void __launch_bounds__(kCarveThreads) binned_carve_kernel(
     if (kShared) {
         for (int w = threadIdx.x; w < wps; w += blockDim.x) {
             const uint32_t m = sm[w];
-            if (m != 0xffffffffu) atomicAnd(gimg + w, m);
+            if (m != 0xffffffffu)
+                for (int k = 0; k < grp.z1 - grp.z0; ++k)
+                    atomicAnd(gimg + static_cast<size_t>(k) * wps + w, m);
         }
     }
-    warp_add(lines, ctr + 4);
-    warp_add(outside, ctr + 5);
+    const unsigned long long slices = static_cast<unsigned long long>(grp.z1 - grp.z0);
+    warp_add(used, ctr + 2);
+    warp_add(missed, ctr + 3);
+    warp_add(lines * slices, ctr + 4);
+    warp_add(outside * slices, ctr + 5);
 }
 
 // Window count of uncarved voxels in each slice (outside the grid counts as
@@ -307,22 +706,22 @@ __global__ void __launch_bounds__(256) binned_filter_kernel(const uint32_t *bits
     const int z = blockIdx.z;
     if (x >= nx || y >= ny) return;
     const uint32_t *img = bits + static_cast<size_t>(z) * wps;
-    auto bit = [&](int X, int Y) {
-        const uint32_t l = static_cast<uint32_t>(X) + static_cast<uint32_t>(nx) * Y;
-        return static_cast<int>((__ldg(img + (l >> 5)) >> (l & 31u)) & 1u);
-    };
+    // a row of the window is at most 15 consecutive bits, in one word or two
+    const int xl = max(x - r, 0), width = min(x + r, nx - 1) - xl + 1;
+    const uint32_t wmask = (1u << width) - 1u;
     int c = 0;
-    for (int dy = -r; dy <= r; ++dy) {
-        const int Y = y + dy;
-        if (Y < 0 || Y >= ny) continue;
-        for (int dx = -r; dx <= r; ++dx) {
-            const int X = x + dx;
-            if (X >= 0 && X < nx) c += bit(X, Y);
-        }
+    uint32_t own = 0u;
+    for (int Y = max(y - r, 0); Y <= min(y + r, ny - 1); ++Y) {
+        const uint32_t l = static_cast<uint32_t>(xl) + static_cast<uint32_t>(nx) * Y;
+        const int w = static_cast<int>(l >> 5);
+        const uint32_t row = __funnelshift_r(__ldg(img + w), __ldg(img + min(w + 1, wps - 1)),
+                                             l & 31u) & wmask;
+        c += __popc(row);
+        if (Y == y) own = row >> (x - xl);
     }
     const size_t v = static_cast<size_t>(x) + static_cast<size_t>(nx) * (y + static_cast<size_t>(ny) * z);
     mask[v] = c >= min_count ? 1 : 0;
-    carved[v] = static_cast<uint8_t>(bit(x, y));
+    carved[v] = static_cast<uint8_t>(own & 1u);
 }
 
 int grid_for(int64_t n, int sm_count, int per_sm = 8)
@@ -354,7 +753,9 @@ struct hd_binned {
     uint32_t *bits = nullptr;           // nz x wps carved bitmap (1 = not carved)
     uint8_t *mask = nullptr, *carved = nullptr;
     float *tables = nullptr;  // n_ang angle centres, n_u lateral centres, nz heights
-    int *slice_bin = nullptr;
+    hd::SliceGroup *groups = nullptr;
+    int n_groups = 0;
+    bool count_apart = false;  // the bins are counted by binned_bins_kernel
     int phase = 0;  // 0 statistics, 1 cuts, 2 finalised
 };
 
@@ -413,6 +814,9 @@ hd_status make_binq(const hd_binned_params *p, hd::BinQ &b)
     b.v_q = fixed_of(p->v_bin_mm, 65536.0);
     b.u_lo_q = fixed_of(p->u_lo_mm, 65536.0);
     b.v_lo_q = fixed_of(p->v_lo_mm, 65536.0);
+    b.r_ang = hd::rcp_int(static_cast<int>(2 * b.ang_q));
+    b.r_u = hd::rcp_int(static_cast<int>(2 * b.u_q));
+    b.r_v = hd::rcp_int(static_cast<int>(2 * b.v_q));
     b.k = p->k_sigma;
     b.miss_q8 = fixed_of(p->miss_wepl_mm, 256.0);
     b.w = p->window;
@@ -436,13 +840,15 @@ void free_binned(hd_binned *b)
     if (b->mask) cudaFree(b->mask);
     if (b->carved) cudaFree(b->carved);
     if (b->tables) cudaFree(b->tables);
-    if (b->slice_bin) cudaFree(b->slice_bin);
+    if (b->groups) cudaFree(b->groups);
     delete b;
 }
 
-// Every input pointer must be readable by the device.
-hd_status check_inputs(const float *const *p, int k)
+// Every input pointer must be readable by the device; host: some input lies in
+// host memory.
+hd_status check_inputs(const float *const *p, int k, bool &host)
 {
+    host = false;
     for (int i = 0; i < k; ++i) {
         if (!p[i]) return HD_ERR_ARG;
         cudaPointerAttributes at{};
@@ -451,8 +857,25 @@ hd_status check_inputs(const float *const *p, int k)
             return HD_ERR_ARG;
         }
         if (at.type == cudaMemoryTypeUnregistered) return HD_ERR_ARG;
+        if (at.type != cudaMemoryTypeDevice) host = true;
     }
     return HD_OK;
+}
+
+// How a pass of n histories keeps an angle's bins in shared memory (words 32-bit
+// words each); n_win 0 when it does not: more than four windows (each reads every
+// history again), host inputs read twice, or too few histories to fill and empty
+// a block's table.
+hd::BinTiles tiles_of(const hd_binned *b, int64_t n, int words, bool host)
+{
+    const int64_t bins = hd::kTileBytes / (4 * words);
+    const int64_t rows = bins / b->bq.n_u;
+    if (rows < 1) return {0, 0};
+    const int64_t n_win = (b->bq.n_v + rows - 1) / rows;
+    if (n_win > (host ? 1 : hd::kMaxWindows) || n_win > b->sm_count) return {0, 0};
+    const int64_t per_angle = int64_t(b->bq.n_u) * b->bq.n_v;
+    if (n < per_angle * b->sm_count * hd::kTileFill) return {0, 0};
+    return {static_cast<int>(n_win), static_cast<int>((b->bq.n_v + n_win - 1) / n_win)};
 }
 
 hd_status pass(hd_binned *b, const float *angle_deg, const float *u_in, const float *v_in,
@@ -462,11 +885,23 @@ hd_status pass(hd_binned *b, const float *angle_deg, const float *u_in, const fl
     if (n < 0) return HD_ERR_ARG;
     if (n == 0) return HD_OK;
     const float *p[6] = {angle_deg, u_in, v_in, u_out, v_out, wepl};
-    const hd_status v = check_inputs(p, 6);
+    bool host;
+    const hd_status v = check_inputs(p, 6, host);
     if (v != HD_OK) return v;
     const hd::Inputs in{angle_deg, u_in, v_in, u_out, v_out, wepl};
+    const int words = cut ? hd::kCutWords : hd::kStatsWords;
+    const hd::BinTiles t = tiles_of(b, n, words, host);
     const int grid = hd::grid_for(n, b->sm_count, hd::kPassBlocksPerSm);  // one wave
-    if (cut)
+    if (t.n_win > 0) {
+        const unsigned blocks = static_cast<unsigned>(b->sm_count / t.n_win * t.n_win);
+        const size_t smem = sizeof(uint32_t) * words * size_t(b->bq.n_u) * t.rows;
+        if (cut)
+            hd::binned_cut_tiles_kernel<<<blocks, hd::kTileThreads, smem, st>>>(in, n, b->bq, t,
+                                                                              b->acc, b->ctr);
+        else
+            hd::binned_stats_tiles_kernel<<<blocks, hd::kTileThreads, smem, st>>>(in, n, b->bq, t,
+                                                                                b->acc, b->ctr);
+    } else if (cut)
         hd::binned_cut_kernel<<<grid, hd::kBinThreads, 0, st>>>(in, n, b->bq, b->acc, b->ctr);
     else
         hd::binned_stats_kernel<<<grid, hd::kBinThreads, 0, st>>>(in, n, b->bq, b->acc, b->ctr);
@@ -541,10 +976,12 @@ hd_status hd_binned_create(const hd_geometry *geom, const hd_binned_params *para
     const int nz = geom->nz;
     const size_t nt = static_cast<size_t>(bq.n_ang) + bq.n_u + nz;
     float *tab = new (std::nothrow) float[nt];
-    int *sb = new (std::nothrow) int[nz];
-    if (!tab || !sb) {
+    b->count_apart = bq.n_v > 2 * nz + 64;
+    hd::SliceGroup *grp = new (std::nothrow)
+        hd::SliceGroup[size_t(nz) + (b->count_apart ? 0 : size_t(bq.n_v))];
+    if (!tab || !grp) {
         delete[] tab;
-        delete[] sb;
+        delete[] grp;
         delete b;
         return HD_ERR_NOMEM;
     }
@@ -553,12 +990,36 @@ hd_status hd_binned_create(const hd_geometry *geom, const hd_binned_params *para
     for (int iu = 0; iu < bq.n_u; ++iu)
         tab[bq.n_ang + iu] = static_cast<float>(
             static_cast<double>(2 * bq.u_lo_q + (2LL * iu + 1) * bq.u_q) / (2.0 * 65536.0));
+    // groups: a bin's slices (heights rise with z) together while the heights lie
+    // inside their slices and a bitmap in shared memory collects the lines; bins
+    // without slices have an empty group, unless they are so many that counting
+    // them takes a kernel of its own
+    int ng = 0, next_iv = 0;
+    bool open = false;
     for (int z = 0; z < nz; ++z) {
         const long long c2 = (2LL * z + 1 - nz) * b->gq.sz;
-        tab[bq.n_ang + bq.n_u + z] = static_cast<float>(static_cast<double>(c2) / (2.0 * 65536.0));
+        const float zc = static_cast<float>(static_cast<double>(c2) / (2.0 * 65536.0));
+        tab[bq.n_ang + bq.n_u + z] = zc;
         const long long iv = floordiv_host(c2 - 2 * bq.v_lo_q, 2 * bq.v_q);
-        sb[z] = (iv >= 0 && iv < bq.n_v) ? static_cast<int>(iv) : -1;
+        if (iv < 0 || iv >= bq.n_v) continue;
+        const long long at = std::fabs(zc) < 4096.0f
+                                 ? hd::to_grid(hd::q16_small(zc), b->gq.dz) - (int64_t(z) << 16) : 0;
+        const bool inside = at > 0 && at < 65536 && b->wps <= hd::kMaxSmemWords;
+        if (inside && open && grp[ng - 1].iv == iv) {
+            grp[ng - 1].z1 = z + 1;
+            continue;
+        }
+        if (next_iv <= iv) {
+            while (!b->count_apart && next_iv < iv) grp[ng++] = {next_iv++, 0, 0, 1};
+            grp[ng++] = {static_cast<int>(iv), z, z + 1, b->count_apart ? 0 : 1};
+            next_iv = static_cast<int>(iv) + 1;
+        } else {
+            grp[ng++] = {static_cast<int>(iv), z, z + 1, 0};
+        }
+        open = inside;
     }
+    while (!b->count_apart && next_iv < bq.n_v) grp[ng++] = {next_iv++, 0, 0, 1};
+    b->n_groups = ng;
     bool ok = true;
     auto alloc = [&](void **p, size_t bytes) {
         if (!ok) return;
@@ -574,11 +1035,11 @@ hd_status hd_binned_create(const hd_geometry *geom, const hd_binned_params *para
     alloc(reinterpret_cast<void **>(&b->mask), size_t(b->V));
     alloc(reinterpret_cast<void **>(&b->carved), size_t(b->V));
     alloc(reinterpret_cast<void **>(&b->tables), sizeof(float) * nt);
-    alloc(reinterpret_cast<void **>(&b->slice_bin), sizeof(int) * nz);
+    alloc(reinterpret_cast<void **>(&b->groups), sizeof(hd::SliceGroup) * (ng > 0 ? ng : 1));
     if (ok) {
         cudaError_t c = cudaMemcpy(b->tables, tab, sizeof(float) * nt, cudaMemcpyHostToDevice);
         if (c == cudaSuccess)
-            c = cudaMemcpy(b->slice_bin, sb, sizeof(int) * nz, cudaMemcpyHostToDevice);
+            c = cudaMemcpy(b->groups, grp, sizeof(hd::SliceGroup) * ng, cudaMemcpyHostToDevice);
         if (c == cudaSuccess)
             c = cudaMemset(b->acc, 0, sizeof(unsigned long long) * hd::kAccWords * b->nb);
         if (c == cudaSuccess) c = cudaMemset(b->ctr, 0, sizeof(unsigned long long) * hd::kCtrWords);
@@ -586,13 +1047,13 @@ hd_status hd_binned_create(const hd_geometry *geom, const hd_binned_params *para
         if (c != cudaSuccess) {
             hd::note_cuda_error(c, "hd_binned_create: initialise");
             delete[] tab;
-            delete[] sb;
+            delete[] grp;
             free_binned(b);
             return HD_ERR_CUDA;
         }
     }
     delete[] tab;
-    delete[] sb;
+    delete[] grp;
     if (!ok) {
         free_binned(b);
         return HD_ERR_NOMEM;
@@ -602,7 +1063,13 @@ hd_status hd_binned_create(const hd_geometry *geom, const hd_binned_params *para
     if (cudaFuncSetAttribute(hd::binned_carve_kernel<true>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(sizeof(uint32_t) * hd::kMaxSmemWords)) !=
-        cudaSuccess) {
+            cudaSuccess ||
+        cudaFuncSetAttribute(hd::binned_stats_tiles_kernel,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, hd::kTileBytes) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(hd::binned_cut_tiles_kernel,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, hd::kTileBytes) !=
+            cudaSuccess) {
         cudaGetLastError();
         free_binned(b);
         return HD_ERR_CUDA;
@@ -668,19 +1135,22 @@ hd_status hd_binned_finalize(hd_binned *b, void *stream)
     const int nz = b->geom.nz;
     HB_CUDA(cudaMemsetAsync(b->ctr + 2, 0, sizeof(unsigned long long) * 4, st));
     HB_CUDA(cudaMemsetAsync(b->bits, 0xff, sizeof(uint32_t) * size_t(b->wps) * nz, st));
-    hd::binned_bins_kernel<<<hd::grid_for(b->nb, b->sm_count), hd::kBinThreads, 0, st>>>(
-        b->acc, b->nb, b->bq.miss_q8, b->ctr);
+    if (b->count_apart)
+        hd::binned_bins_kernel<<<hd::grid_for(b->nb, b->sm_count), hd::kBinThreads, 0, st>>>(
+            b->acc, b->nb, b->bq.miss_q8, b->ctr);
     HB_CUDA(cudaGetLastError());
     const hd::LineTables t{b->tables, b->tables + b->bq.n_ang, b->tables + b->bq.n_ang + b->bq.n_u,
-                           b->slice_bin};
-    const dim3 cg(static_cast<unsigned>(b->bq.n_ang), static_cast<unsigned>(nz));
-    if (b->wps <= hd::kMaxSmemWords)
-        hd::binned_carve_kernel<true><<<cg, hd::kCarveThreads, sizeof(uint32_t) * b->wps, st>>>(
-            b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr);
-    else
-        hd::binned_carve_kernel<false><<<cg, hd::kCarveThreads, 0, st>>>(
-            b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr);
-    HB_CUDA(cudaGetLastError());
+                           b->groups};
+    const dim3 cg(static_cast<unsigned>(b->bq.n_ang), static_cast<unsigned>(b->n_groups));
+    if (b->n_groups > 0) {
+        if (b->wps <= hd::kMaxSmemWords)
+            hd::binned_carve_kernel<true><<<cg, hd::kCarveThreads, sizeof(uint32_t) * b->wps, st>>>(
+                b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr);
+        else
+            hd::binned_carve_kernel<false><<<cg, hd::kCarveThreads, 0, st>>>(
+                b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr);
+        HB_CUDA(cudaGetLastError());
+    }
     const dim3 fb(32, 8);
     const dim3 fg(static_cast<unsigned>((b->geom.nx + 31) / 32),
                   static_cast<unsigned>((b->geom.ny + 7) / 8), static_cast<unsigned>(nz));
