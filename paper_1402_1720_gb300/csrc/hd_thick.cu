@@ -305,9 +305,9 @@ __global__ void __launch_bounds__(kThickThreads) thick_records_kernel(Records re
     const int64_t total = rec.glist ? static_cast<int64_t>(ctrl->n_global) : rec.cap;
     ThickRing rg;
     unsigned vox[2] = {0, 0};
-    for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < total;
-         k += stride) {
-        const int64_t i = rec.glist ? static_cast<int64_t>(rec.glist[k]) : k;
+    for (int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; q < total;
+         q += stride) {
+        const int64_t i = rec.glist ? static_cast<int64_t>(rec.glist[q]) : q;
         const int32_t stw = rec.status[i];
         if (status_path(stw) != 2) continue;
         const int32_t gi[3] = {rec.g[0][i], rec.g[1][i], rec.g[2][i]};
