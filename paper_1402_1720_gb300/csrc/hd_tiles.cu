@@ -567,14 +567,22 @@ __device__ __forceinline__ BucketCost bucket_cost(const ScanDesc &d, int t, bool
     return b;
 }
 
+// Blocks of its own for a bucket, about two flushes' worth of work each.
+__device__ __forceinline__ unsigned long long own_blocks(const BucketCost &b, int tile_words)
+{
+    const unsigned long long f = 2ull * flush_cost(tile_words);
+    return (b.cost + f - 1ull) / f;
+}
+
 // Where the boundary at cost x of the launch falls in a bucket whose cost
 // begins at p: pieces of 32 slots before it (0 .. all).  A part worth less
-// than its own flush goes to the neighbour.
+// than its own flush goes to the neighbour (tile_words -1: costs are blocks,
+// and a boundary stays where it falls).
 __device__ __forceinline__ int boundary_slot(const BucketCost &b, int tile_words,
                                              unsigned long long p, unsigned long long x)
 {
     const int pieces = kCols * slot_rows(static_cast<int>(b.count));
-    const unsigned long long f = flush_cost(tile_words);
+    const unsigned long long f = tile_words < 0 ? 0ull : flush_cost(tile_words);
     if (x <= p + f) return 0;
     if (x + f >= p + b.cost) return 32 * pieces;
     return 32 * static_cast<int>((x - p) * static_cast<unsigned long long>(pieces) / b.cost);
@@ -658,22 +666,42 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     };
     unsigned long long mine = 0, total;
     each([&](int k, int t) { mine += bucket_cost(descs[k], t, kRows).cost; });
-    const unsigned long long before = block_excl_scan64(mine, s_warp, total);
+    unsigned long long before = block_excl_scan64(mine, s_warp, total);
     // the block's stretch: an equal share, but worth about two flushes
     unsigned long long blocks = total / (2ull * flush_cost(descs[0].tp.tile_words)) + 1ull;
-    if (blocks > gridDim.x) blocks = gridDim.x;
-    const unsigned long long share = (total + blocks - 1ull) / blocks;
-    const unsigned long long x0 = share * blockIdx.x, x1 = x0 + share;
+    unsigned long long share = 0, x0 = 0, x1 = 0;
+    // a launch too small for that on every block: whole blocks for each bucket
+    // instead, one for about two flushes' worth (a block of two small buckets
+    // flushes twice, 11 000 cycles each)
+    bool own = blocks < gridDim.x;  // the same in all blocks and threads
+    if (own) {
+        unsigned long long m = 0, all;
+        each([&](int k, int t) { m += own_blocks(bucket_cost(descs[k], t, kRows), descs[k].tp.tile_words); });
+        const unsigned long long b = block_excl_scan64(m, s_warp, all);
+        own = all <= gridDim.x;
+        if (own) {
+            before = b;
+            share = 1ull;
+        }
+    }
+    if (!own) {
+        if (blocks > gridDim.x) blocks = gridDim.x;
+        share = (total + blocks - 1ull) / blocks;
+    }
+    x0 = share * blockIdx.x;
+    x1 = x0 + share;
     // the parts of the thread's buckets in that stretch, each at most
     // job_size pairs (in whole pieces): count, then list
     auto parts = [&](auto take) {
         unsigned long long p = before;
         each([&](int k, int t) {
             const ScanDesc &d = descs[k];
-            const BucketCost b = bucket_cost(d, t, kRows);
+            BucketCost b = bucket_cost(d, t, kRows);
+            if (own) b.cost = own_blocks(b, d.tp.tile_words);
             if (b.cost != 0 && p < x1 && p + b.cost > x0) {
-                const int s0 = x0 > p ? boundary_slot(b, d.tp.tile_words, p, x0) : 0;
-                const int s1 = x1 < p + b.cost ? boundary_slot(b, d.tp.tile_words, p, x1)
+                const int words = own ? -1 : d.tp.tile_words;
+                const int s0 = x0 > p ? boundary_slot(b, words, p, x0) : 0;
+                const int s1 = x1 < p + b.cost ? boundary_slot(b, words, p, x1)
                                                : 32 * kCols * slot_rows(static_cast<int>(b.count));
                 const int most = d.tp.job_size & ~31;
                 for (int s = s0; s < s1; s += most)
