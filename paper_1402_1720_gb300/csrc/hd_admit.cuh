@@ -88,20 +88,61 @@ __device__ __forceinline__ void reserve_and_write(const TilePlan &tp, const Reco
     rec.status[i] = st;
 }
 
-// The end of an ingest block: its pair counts per bucket and in all.
-__device__ __forceinline__ void write_block_counts(int nh, const uint32_t *s_hist, unsigned *s_total,
-                                                   uint32_t *block_count, uint32_t *block_pairs)
+// The end of an ingest block: it reserves its pairs' places in every bucket
+// (block_base[b nh + t], by block b's atomic on the bucket's count; the order of
+// the blocks inside a bucket is the order they end in, which no count depends
+// on) and leaves its pairs in all.
+__device__ __forceinline__ void reserve_buckets(int nh, const uint32_t *s_hist, unsigned *s_total,
+                                                uint32_t *bucket_count, uint32_t *block_base,
+                                                uint32_t *block_pairs)
 {
     __syncthreads();
     unsigned mine = 0;
     for (int t = threadIdx.x; t < nh; t += blockDim.x) {
-        block_count[static_cast<size_t>(t) * gridDim.x + blockIdx.x] = s_hist[t];
-        mine += s_hist[t];
+        const unsigned c = s_hist[t];
+        if (c == 0) continue;
+        block_base[static_cast<size_t>(blockIdx.x) * nh + t] = atomicAdd(bucket_count + t, c);
+        mine += c;
     }
     mine = warp_sum_u32(mine);
     if ((threadIdx.x & 31u) == 0 && mine) atomicAdd(s_total, mine);
     __syncthreads();
     if (threadIdx.x == 0) block_pairs[blockIdx.x] = *s_total;
+}
+
+// The start of a scatter block: s_base[t], its first place in each of the nt
+// buckets it has pairs in, from the exclusive scan of the buckets' counts and
+// its reservations; block 0 also writes the buckets' first pairs.
+template <int kThreads>
+__device__ __forceinline__ void bucket_places(int nt, const Buckets &buckets,
+                                              const uint32_t *block_base, uint32_t *s_base)
+{
+    __shared__ unsigned s_warp[kThreads / 32];
+    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+    for (int t = threadIdx.x; t < nt; t += kThreads) s_base[t] = buckets.count[t];
+    __syncthreads();
+    const int per = (nt + kThreads - 1) / kThreads;
+    const int t0 = min(static_cast<int>(threadIdx.x) * per, nt), t1 = min(t0 + per, nt);
+    unsigned mine = 0;
+    for (int t = t0; t < t1; ++t) mine += s_base[t];
+    const unsigned incl = warp_incl_scan(mine);
+    if (lane == 31) s_warp[wid] = incl;
+    __syncthreads();
+    unsigned at = incl - mine;
+    for (unsigned w = 0; w < kThreads / 32; ++w) at += w < wid ? s_warp[w] : 0u;
+    for (int t = t0; t < t1; ++t) {
+        const unsigned c = s_base[t];
+        s_base[t] = at;
+        at += c;
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < nt; t += kThreads) {
+        const unsigned first = s_base[t];
+        if (blockIdx.x == 0) buckets.first[t] = first;
+        // nothing was reserved (and none of these is used) where the block has no pair
+        s_base[t] = first + block_base[static_cast<size_t>(blockIdx.x) * nt + t];
+    }
+    __syncthreads();
 }
 
 }  // namespace

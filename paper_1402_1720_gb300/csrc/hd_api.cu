@@ -132,8 +132,8 @@ struct hd_scan {
     hd::ScanDesc *desc_dev = nullptr;  // this scan's traversal descriptor
     hd::ScanDesc desc_host{};
     bool desc_dirty = true;
-    // kGroups * ntiles tile totals, then the ingest blocks' pair counts per tile
-    // (tile_count_words)
+    // kGroups * ntiles bucket totals, then the ingest blocks' places in the
+    // buckets (tile_count_words)
     uint32_t *tile_count = nullptr;
     uint32_t *tile_cursor = nullptr;  // kGroups * ntiles
     unsigned long long *tile_events = nullptr;  // kGroups * ntiles
@@ -356,8 +356,9 @@ size_t ingest_blocks_max(const hd_scan *s)
            static_cast<size_t>(hd::kIngestBlocksPerSm);
 }
 
-// Words of tile_count: the kGroups * ntiles totals, a column of pair counts per
-// group and tile for the most ingest blocks, then each block's pairs in all.
+// Words of tile_count: the kGroups * ntiles bucket totals, a row of the blocks'
+// first places in the buckets for the most ingest blocks, then each block's
+// pairs in all.
 size_t tile_count_words(const hd_scan *s)
 {
     const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
@@ -493,21 +494,21 @@ hd_status stage_prepare(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_
     const hd::Records rec = records_of(s, n);
     hd::TilePlan tp = s->tp;
     if (s->trace_grid <= 0) tp.ntiles = 0;
-    HD_CUDA(cudaMemsetAsync(&s->ctrl->n_global, 0, sizeof(hd::Ctrl) - offsetof(hd::Ctrl, n_global), st));
+    HD_CUDA(hd::launch_chunk_begin(s->ctrl, buckets_of(s), tp.ntiles, st));
     const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
-    uint32_t *block_count = s->tile_count + cols;
-    uint32_t *block_pairs = block_count + cols * ingest_blocks_max(s);
+    uint32_t *block_base = s->tile_count + cols;
+    uint32_t *block_pairs = block_base + cols * ingest_blocks_max(s);
     const hd::Pairs pairs = pairs_of(s);
     HD_CUDA(hd::launch_ingest(in, n, s->gq, s->cordic, s->params.wepl_miss_lt,
                               s->params.wepl_hit_gt, use_miss, use_hit, tp, rec, s->ctrl,
-                              tp.ntiles > 0 ? block_count : nullptr, block_pairs, pairs.stage,
+                              s->tile_count, tp.ntiles > 0 ? block_base : nullptr, block_pairs,
+                              pairs.stage,
                               s->inputs_on_host ? 1 : 0, s->sm_count, st));
-    s->launches += 1;
+    s->launches += 2;
     if (tp.ntiles > 0) {
-        HD_CUDA(hd::launch_plan(tp, n, block_count, buckets_of(s), s->sm_count, st));
-        HD_CUDA(hd::launch_scatter(tp, rec, n, s->ctrl, buckets_of(s), block_count, block_pairs,
+        HD_CUDA(hd::launch_scatter(tp, rec, n, s->ctrl, buckets_of(s), block_base, block_pairs,
                                    pairs, s->sm_count, st));
-        s->launches += 3;
+        s->launches += 1;
     }
     return HD_OK;
 }
@@ -569,8 +570,8 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
             int64_t most = euclid_pair_cap(s) / s->euclid_pairs & ~int64_t(3);
             if (most > (int64_t(1) << 23)) most = int64_t(1) << 23;  // a slot's bits in open_code
             const size_t cols = hd::kGroups * static_cast<size_t>(s->tp.ntiles);
-            uint32_t *block_count = s->tile_count + cols;
-            uint32_t *block_pairs = block_count + cols * ingest_blocks_max(s);
+            uint32_t *block_base = s->tile_count + cols;
+            uint32_t *block_pairs = block_base + cols * ingest_blocks_max(s);
             // equal chunks
             const int64_t parts = most > 0 ? (n + most - 1) / most : 0;
             const int64_t per = parts > 0 ? ((n + parts - 1) / parts + 3) & ~int64_t(3) : 0;
@@ -578,14 +579,12 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
                 const int64_t c = n - off < per ? n - off : per;
                 const hd::Inputs part{in.angle + off, in.u_in + off,  in.v_in + off,
                                       in.u_out + off, in.v_out + off, in.wepl + off};
-                HD_CUDA(cudaMemsetAsync(&s->ctrl->n_global, 0,
-                                        sizeof(hd::Ctrl) - offsetof(hd::Ctrl, n_global), st));
                 HD_CUDA(hd::launch_euclid_scan(
                     s->desc_dev, s->desc_host, part, c, &s->geom, s->gq, s->cordic,
                     s->params.wepl_miss_lt, s->params.wepl_hit_gt, (m & (HD_SC | HD_MSC)) ? 1 : 0,
-                    (m & HD_SM) ? 1 : 0, s->euclid_d0, records_of(s, c), block_count, block_pairs,
+                    (m & HD_SM) ? 1 : 0, s->euclid_d0, records_of(s, c), block_base, block_pairs,
                     s->thick_ws, s->trace_grid, s->sm_count, st));
-                s->launches += 12;
+                s->launches += 11;
             }
             if (per > 0) return HD_OK;
         }
@@ -1387,7 +1386,7 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
         }
         r = stage_prepare(s, round[i].in, round[i].n, ss);
         if (r != HD_OK) return r;
-        *kernels += 1 + ((s->tp.ntiles > 0 && s->trace_grid > 0) ? 2 : 0);
+        *kernels += 2 + ((s->tp.ntiles > 0 && s->trace_grid > 0) ? 1 : 0);
     }
     r = join();
     if (r != HD_OK) return r;

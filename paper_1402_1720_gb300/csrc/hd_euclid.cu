@@ -244,7 +244,7 @@ __device__ __forceinline__ void euclid_tiles(const TilePlan &tp, int klo, int kh
 __global__ void __launch_bounds__(kIngestThreads, 4) euclid_ingest_kernel(
     Inputs in, int64_t n, int64_t per_block, GeomQ g, Cordic cd, float tau_l, float tau_h,
     int use_miss, int use_hit, long long R, TilePlan tp, Records rec, Ctrl *ctrl,
-    uint32_t *block_count, uint32_t *block_pairs, uint32_t *stage)
+    uint32_t *bucket_count, uint32_t *block_base, uint32_t *block_pairs, uint32_t *stage)
 {
     extern __shared__ uint32_t s_hist[];  // kGroups * ntiles counters
     __shared__ unsigned s_demand, s_total;
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kIngestThreads, 4) euclid_ingest_kernel(
         const unsigned v = warp_sum_u32(sums[q]);
         if ((threadIdx.x & 31u) == 0 && v) atomicAdd(to[q], static_cast<unsigned long long>(v));
     }
-    write_block_counts(nh, s_hist, &s_total, block_count, block_pairs);
+    reserve_buckets(nh, s_hist, &s_total, bucket_count, block_base, block_pairs);
 }
 
 // Counting sort of the pairs (see scatter_kernel) with each pair's slice rows.
@@ -333,12 +333,8 @@ __global__ void __launch_bounds__(kSetupThreads, 2) euclid_setup_kernel(
     uint32_t *s_base = s_mem;          // this block's first position in each bucket
     uint32_t *s_next = s_mem + nt;     // pairs written per bucket so far
     uint32_t *s_events = s_next + nt;  // and their rows
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-        s_base[t] = buckets.first[t] + block_base[static_cast<size_t>(t) * gridDim.x + blockIdx.x];
-        s_next[t] = 0;
-        s_events[t] = 0;
-    }
-    __syncthreads();
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) s_next[t] = s_events[t] = 0;
+    bucket_places<kSetupThreads>(nt, buckets, block_base, s_base);
     const int64_t h0 = static_cast<int64_t>(blockIdx.x) * per_block;
     const unsigned npairs = block_pairs[blockIdx.x];
     const uint32_t *list = pairs.stage + static_cast<int64_t>(blockIdx.x) * per_block * tp.pairs_per_record;
@@ -462,7 +458,7 @@ int euclid_pairs_per_record(const hd_geometry *geom, float d0, const TilePlan &t
 cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, const Inputs &in,
                                int64_t n, const hd_geometry *geom, const GeomQ &g,
                                const Cordic &cd, float tau_l, float tau_h, int use_miss,
-                               int use_hit, float d0, const Records &rec, uint32_t *block_count,
+                               int use_hit, float d0, const Records &rec, uint32_t *block_base,
                                uint32_t *block_pairs, void *workspace, int grid, int sm_count,
                                cudaStream_t st)
 {
@@ -473,13 +469,13 @@ cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, c
     ra.rec = rec;
     const ChunkSplit sp = chunk_split(n, sm_count);
     const size_t cols = kGroups * static_cast<size_t>(tp.ntiles);
+    cudaError_t e = launch_chunk_begin(desc.ctrl, desc.buckets, tp.ntiles, st);
+    if (e != cudaSuccess) return e;
     euclid_ingest_kernel<<<static_cast<unsigned>(sp.blocks), kIngestThreads, 4 * cols, st>>>(
         in, n, sp.per_block, g, cd, tau_l, tau_h, use_miss, use_hit, ra.R, tp, rec, desc.ctrl,
-        block_count, block_pairs, desc.pairs.stage);
-    cudaError_t e = launch_plan(tp, n, block_count, desc.buckets, sm_count, st);
-    if (e != cudaSuccess) return e;
+        desc.buckets.count, block_base, block_pairs, desc.pairs.stage);
     euclid_setup_kernel<<<static_cast<unsigned>(sp.blocks), kSetupThreads, 12 * cols, st>>>(
-        tp, ra, sp.per_block, desc.buckets, block_count, block_pairs, desc.pairs);
+        tp, ra, sp.per_block, desc.buckets, block_base, block_pairs, desc.pairs);
     e = launch_trace_rows(desc_dev, tp.tile_words, tp.threads, grid, ra, st);
     if (e != cudaSuccess) return e;
     euclid_open_kernel<<<static_cast<unsigned>(grid * kOpenParts), 128, 0, st>>>(desc_dev, ra);

@@ -178,31 +178,30 @@ struct Inputs {
 
 // ---- launchers (stream-ordered; return the launch's cudaError_t) ----
 
-// Classification, records and pair counts of a chunk.  block_count (null
-// when tp.ntiles is 0) receives, per group-tile column c (kGroups tp.ntiles of
-// them) and ingest block b, the pairs of that block's records in that tile
-// at [c * blocks + b]; block_pairs[b] the block's pairs in all, listed in
-// stage (Pairs::stage).  Each block keeps to a pair budget of
+// Begins a chunk: clears the scan's lists (Ctrl from n_global on) and the
+// buckets' counts and events.
+cudaError_t launch_chunk_begin(Ctrl *ctrl, const Buckets &buckets, int ntiles, cudaStream_t s);
+
+// Classification, records and pair counts of a chunk.  Block b of the chunk
+// split adds its pairs to bucket_count (cleared before) and receives in
+// block_base[b kGroups ntiles + t] (null when tp.ntiles is 0) its first place in
+// bucket t, where it has pairs there; block_pairs[b] is its pairs in all, listed
+// in stage (Pairs::stage).  Each block keeps to a pair budget of
 // tp.pairs_per_record per history; its records beyond it take the global
 // path.  on_host: the inputs are page-locked host memory read in place.
 cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cordic &cordic,
                           float tau_l, float tau_h, int use_miss, int use_hit, const TilePlan &tp,
-                          const Records &rec, Ctrl *ctrl, uint32_t *block_count,
-                          uint32_t *block_pairs, uint32_t *stage, int on_host, int sm_count,
-                          cudaStream_t s);
+                          const Records &rec, Ctrl *ctrl, uint32_t *bucket_count,
+                          uint32_t *block_base, uint32_t *block_pairs, uint32_t *stage,
+                          int on_host, int sm_count, cudaStream_t s);
 
-// Per column: the exclusive prefix over blocks of block_count (in place) and
-// the column total into buckets.count; then the buckets' first pairs, and
-// their events cleared.
-cudaError_t launch_plan(const TilePlan &tp, int64_t n, uint32_t *block_count,
-                        const Buckets &buckets, int sm_count, cudaStream_t s);
-
-// Counting sort of the (record, tile) pairs by tile, with the walk set-up of
+// Counting sort of the (record, tile) pairs by bucket, with the walk set-up of
 // each pair; block b of the chunk split takes the block_pairs[b] pairs that
-// ingest block b listed and writes those of bucket c from
-// buckets.first[c] + block_count[c * blocks + b] on, adding their events.
+// ingest block b listed and writes them from its places in the buckets on (the
+// buckets' first pairs, an exclusive scan of their counts, are written here),
+// adding their events.
 cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ctrl *ctrl,
-                           const Buckets &buckets, const uint32_t *block_count,
+                           const Buckets &buckets, const uint32_t *block_base,
                            const uint32_t *block_pairs, const Pairs &pairs, int sm_count,
                            cudaStream_t s);
 

@@ -1,10 +1,9 @@
 // Bucketing of the (record, tile) pairs of a chunk for the tiled traversal,
-// after ingest has counted, per ingest block, its pairs in each tile:
-//   bases    per tile, exclusive scan over the blocks -> each block's offset
-//   plan     exclusive scan of the totals -> each bucket's first pair
-//   scatter  counting sort of the pairs by tile: block b of the ingest split
-//            writes its pairs from its offsets, with each pair's walk set-up
+// after the ingest blocks have reserved their places in each bucket
+// (reserve_buckets): a counting sort of the pairs by bucket, block b writing
+// those of ingest block b from its places on, with each pair's walk set-up.
 #include <cooperative_groups.h>
+#include "hd_admit.cuh"
 #include "hd_fallback.cuh"
 
 namespace cg = cooperative_groups;
@@ -15,76 +14,6 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kScatterThreads = 512;
-
-__device__ __forceinline__ unsigned warp_incl_scan_u(unsigned v)
-{
-    const unsigned lane = threadIdx.x & 31u;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned t = __shfl_up_sync(kFull, v, o);
-        if (lane >= static_cast<unsigned>(o)) v += t;
-    }
-    return v;
-}
-
-// Exclusive block scan of one value per thread (blockDim.x <= 1024).
-__device__ __forceinline__ unsigned block_excl_scan(unsigned v, unsigned *s_warp, unsigned &total)
-{
-    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-    const unsigned nw = blockDim.x >> 5;
-    const unsigned incl = warp_incl_scan_u(v);
-    if (lane == 31) s_warp[wid] = incl;
-    __syncthreads();
-    if (wid == 0) {
-        const unsigned x = lane < nw ? s_warp[lane] : 0u;
-        const unsigned xi = warp_incl_scan_u(x);
-        if (lane < nw) s_warp[lane] = xi - x;
-        if (lane == 31) s_warp[32] = xi;
-    }
-    __syncthreads();
-    const unsigned r = s_warp[wid] + incl - v;
-    total = s_warp[32];
-    __syncthreads();
-    return r;
-}
-
-
-// One warp per group-tile column: the exclusive prefix over the ingest
-// blocks of their pair counts (in place) and the column's total.
-__global__ void __launch_bounds__(256) bases_kernel(int ncols, int nblocks, uint32_t *counts,
-                                                    uint32_t *totals)
-{
-    const int c = static_cast<int>(blockIdx.x) * 8 + static_cast<int>(threadIdx.x >> 5);
-    const int lane = static_cast<int>(threadIdx.x & 31u);
-    if (c >= ncols) return;  // the whole warp
-    uint32_t *col = counts + static_cast<size_t>(c) * nblocks;
-    unsigned run = 0;
-    for (int b0 = 0; b0 < nblocks; b0 += 32) {
-        const int b = b0 + lane;
-        const unsigned v = b < nblocks ? col[b] : 0u;
-        const unsigned incl = warp_incl_scan_u(v);
-        if (b < nblocks) col[b] = run + incl - v;
-        run += __shfl_sync(kFull, incl, 31);
-    }
-    if (lane == 0) totals[c] = run;
-}
-
-// One block: the buckets' first pairs (exclusive scan of their counts).
-__global__ void __launch_bounds__(1024) plan_kernel(int nt, Buckets buckets)
-{
-    __shared__ unsigned s_warp[33];
-    const int per = (nt + blockDim.x - 1) / blockDim.x;
-    const int t0 = threadIdx.x * per;
-    unsigned my_pairs = 0;
-    for (int t = t0; t < t0 + per && t < nt; ++t) my_pairs += buckets.count[t];
-    unsigned tot_pairs;
-    unsigned off = block_excl_scan(my_pairs, s_warp, tot_pairs);
-    for (int t = t0; t < t0 + per && t < nt; ++t) {
-        buckets.first[t] = off;
-        buckets.events[t] = 0;
-        off += buckets.count[t];
-    }
-}
 
 // The general set-up of one (record, tile) pair: its packed event walk, an
 // empty walk, or (returns true) the general form for the fallback list.
@@ -111,10 +40,9 @@ __device__ __noinline__ bool general_setup(const int32_t gi[3], const int32_t go
     return fallback;
 }
 
-// Counting sort of (record, tile) pairs by tile.  Block b takes the pairs
-// ingest block b listed, one per thread, and writes those of tile c from
-// tile_start[c] + block_base[c * blocks + b] on (a shared-memory cursor per
-// tile orders them within the block).
+// Counting sort of (record, tile) pairs by bucket.  Block b takes the pairs
+// ingest block b listed, one per thread, and writes those of a bucket from its
+// places there on (a shared-memory cursor per bucket orders them).
 __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
     TilePlan tp, Records rec, int64_t per_block, Buckets buckets, const uint32_t *block_base,
     const uint32_t *block_pairs, Ctrl *ctrl, Pairs pairs)
@@ -124,12 +52,8 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
     uint32_t *s_base = s_mem;       // this block's first position in each bucket
     uint32_t *s_next = s_mem + nt;  // pairs written per bucket so far
     uint32_t *s_events = s_next + nt;  // and the events of their walks
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) {
-        s_base[t] = buckets.first[t] + block_base[static_cast<size_t>(t) * gridDim.x + blockIdx.x];
-        s_next[t] = 0;
-        s_events[t] = 0;
-    }
-    __syncthreads();
+    for (int t = threadIdx.x; t < nt; t += blockDim.x) s_next[t] = s_events[t] = 0;
+    bucket_places<kScatterThreads>(nt, buckets, block_base, s_base);
     const int64_t h0 = static_cast<int64_t>(blockIdx.x) * per_block;
     const unsigned npairs = block_pairs[blockIdx.x];
     unsigned runs = 0;
@@ -222,18 +146,6 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
 
 }  // namespace
 
-cudaError_t launch_plan(const TilePlan &tp, int64_t n, uint32_t *block_count,
-                        const Buckets &buckets, int sm_count, cudaStream_t s)
-{
-    const int ncols = kGroups * tp.ntiles;
-    const ChunkSplit sp = chunk_split(n, sm_count);
-    bases_kernel<<<static_cast<unsigned>((ncols + 7) / 8), 256, 0, s>>>(ncols, sp.blocks,
-                                                                        block_count,
-                                                                        buckets.count);
-    plan_kernel<<<1, 1024, 0, s>>>(ncols, buckets);
-    return cudaGetLastError();
-}
-
 cudaError_t init_scatter()
 {
     return cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -241,7 +153,7 @@ cudaError_t init_scatter()
 }
 
 cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ctrl *ctrl,
-                           const Buckets &buckets, const uint32_t *block_count,
+                           const Buckets &buckets, const uint32_t *block_base,
                            const uint32_t *block_pairs, const Pairs &pairs, int sm_count,
                            cudaStream_t s)
 {
@@ -249,7 +161,7 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
     const ChunkSplit sp = chunk_split(n, sm_count);
     const size_t smem = sizeof(uint32_t) * 3 * kGroups * static_cast<size_t>(tp.ntiles);
     scatter_kernel<<<static_cast<unsigned>(sp.blocks), kScatterThreads, smem, s>>>(
-        tp, rec, sp.per_block, buckets, block_count, block_pairs, ctrl, pairs);
+        tp, rec, sp.per_block, buckets, block_base, block_pairs, ctrl, pairs);
     return cudaGetLastError();
 }
 

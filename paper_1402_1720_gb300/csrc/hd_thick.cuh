@@ -129,7 +129,7 @@ int euclid_pairs_per_record(const hd_geometry *geom, float d0, const TilePlan &t
 cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, const Inputs &in,
                                int64_t n, const hd_geometry *geom, const GeomQ &g,
                                const Cordic &cd, float tau_l, float tau_h, int use_miss,
-                               int use_hit, float d0, const Records &rec, uint32_t *block_count,
+                               int use_hit, float d0, const Records &rec, uint32_t *block_base,
                                uint32_t *block_pairs, void *workspace, int grid, int sm_count,
                                cudaStream_t st);
 

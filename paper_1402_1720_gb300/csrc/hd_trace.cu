@@ -134,8 +134,8 @@ __device__ __forceinline__ void admit_and_write(const TilePlan &tp, const Record
 template <bool kWide>
 __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
     Inputs in, int64_t n, int64_t per_block, GeomQ g, Cordic cd, float tau_l, float tau_h,
-    int use_miss, int use_hit, TilePlan tp, Records rec, Ctrl *ctrl, uint32_t *block_count,
-    uint32_t *block_pairs, uint32_t *stage)
+    int use_miss, int use_hit, TilePlan tp, Records rec, Ctrl *ctrl, uint32_t *bucket_count,
+    uint32_t *block_base, uint32_t *block_pairs, uint32_t *stage)
 {
     extern __shared__ uint32_t s_hist[];  // kGroups * ntiles counters
     __shared__ unsigned s_demand, s_total;
@@ -219,8 +219,8 @@ __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
         if (a3) atomicAdd(&ctrl->n_none, static_cast<unsigned long long>(a3));
         if (a4) atomicAdd(&ctrl->n_reject, static_cast<unsigned long long>(a4));
     }
-    if (block_count == nullptr) return;
-    write_block_counts(nh, s_hist, &s_total, block_count, block_pairs);
+    if (block_base == nullptr) return;
+    reserve_buckets(nh, s_hist, &s_total, bucket_count, block_base, block_pairs);
 }
 
 // ---------------------------------------------------------------- traversal
@@ -264,18 +264,18 @@ __global__ void classify_kernel(const float *__restrict__ w, int64_t n, float ta
 
 cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cordic &cordic,
                           float tau_l, float tau_h, int use_miss, int use_hit, const TilePlan &tp,
-                          const Records &rec, Ctrl *ctrl, uint32_t *block_count,
-                          uint32_t *block_pairs, uint32_t *stage, int on_host, int sm_count,
+                          const Records &rec, Ctrl *ctrl, uint32_t *bucket_count,
+                          uint32_t *block_base, uint32_t *block_pairs, uint32_t *stage, int on_host, int sm_count,
                           cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
     const ChunkSplit sp = chunk_split(n, sm_count);
     // without the tiled path's buffers every record takes the global path
-    const bool tiled = tp.ntiles > 0 && block_count && block_pairs && stage;
+    const bool tiled = tp.ntiles > 0 && block_base && block_pairs && stage;
     TilePlan tpl = tp;
     if (!tiled) tpl.ntiles = 0;
     const size_t smem = sizeof(uint32_t) * kGroups * static_cast<size_t>(tpl.ntiles);
-    uint32_t *bc = tiled ? block_count : nullptr;
+    uint32_t *bb = tiled ? block_base : nullptr;
     uint32_t *bp = tiled ? block_pairs : nullptr;
     uint32_t *sg = tiled ? stage : nullptr;
     const uintptr_t bits =
@@ -284,12 +284,31 @@ cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cor
         reinterpret_cast<uintptr_t>(in.v_out) | reinterpret_cast<uintptr_t>(in.wepl);
     if (on_host && (bits & 15u) == 0)
         ingest_kernel<true><<<static_cast<unsigned>(sp.blocks), kIngestThreads, smem, s>>>(
-            in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl, bc,
-            bp, sg);
+            in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl,
+            bucket_count, bb, bp, sg);
     else
         ingest_kernel<false><<<static_cast<unsigned>(sp.blocks), kIngestThreads, smem, s>>>(
-            in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl, bc,
-            bp, sg);
+            in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl,
+            bucket_count, bb, bp, sg);
+    return cudaGetLastError();
+}
+
+// Clears a chunk's counters: the scan's lists and the buckets' pairs and events.
+__global__ void __launch_bounds__(1024) chunk_begin_kernel(Ctrl *ctrl, Buckets buckets, int ncols)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        ctrl->n_global = ctrl->n_fallback = ctrl->n_pair_fallback = ctrl->fb_next = 0u;
+    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ncols; t += gridDim.x * blockDim.x) {
+        buckets.count[t] = 0u;
+        buckets.events[t] = 0ull;
+    }
+}
+
+cudaError_t launch_chunk_begin(Ctrl *ctrl, const Buckets &buckets, int ntiles, cudaStream_t s)
+{
+    const int ncols = kGroups * ntiles;
+    chunk_begin_kernel<<<static_cast<unsigned>(ncols > 4096 ? (ncols + 4095) / 4096 : 1), 1024, 0, s>>>(
+        ctrl, buckets, ncols);
     return cudaGetLastError();
 }
 
