@@ -555,7 +555,7 @@ hd_status stage_finalize(hd_scan *scan, cudaStream_t st)
     return HD_OK;
 }
 
-int finalize_launches(const hd_scan *scan) { return (scan->params.methods & HD_SM) ? 3 : 1; }
+int finalize_launches(const hd_scan *scan) { return (scan->params.methods & HD_SM) ? 2 : 1; }
 
 // One chunk through the whole path on st.
 hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st)

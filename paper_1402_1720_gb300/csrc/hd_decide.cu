@@ -31,6 +31,7 @@ __global__ void __launch_bounds__(256) sm_slope_kernel(const uint32_t *__restric
                                                        int ny, int nz, int per_slice, int nbhd,
                                                        unsigned long long *slice_key)
 {
+    after_previous();
     const int z = blockIdx.y;
     const int plane = nx * ny;
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
@@ -69,26 +70,27 @@ __global__ void __launch_bounds__(256) sm_slope_kernel(const uint32_t *__restric
     }
 }
 
-__global__ void sm_threshold_kernel(const uint32_t *__restrict__ M, int nx, int ny, int nz,
-                                    int per_slice, const unsigned long long *slice_key,
-                                    uint32_t *mt, uint32_t *slope, long long *index)
-{
-    const int z = blockIdx.x * blockDim.x + threadIdx.x;
-    if (z >= nz) return;
-    const unsigned long long key = slice_key[per_slice ? z : 0];
-    const long long plane = static_cast<long long>(nx) * ny;
-    const long long id = static_cast<long long>(key & 0xffffffffull);
-    const long long v = per_slice ? z * plane + id : id;
-    slope[z] = static_cast<uint32_t>(key >> 32);
-    index[z] = v;
-    mt[z] = M[v];
-}
-
 __global__ void __launch_bounds__(256) decide_kernel(DecideArgs a)
 {
+    after_previous();
     const int z = blockIdx.y;
     const int plane = a.nx * a.ny;
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
+    uint32_t t = 0, slope = 0;
+    if (a.methods & HD_SM) {
+        // the slice's threshold M_t from its steepest drop (a kernel of its own
+        // for the nz of them cost a launch); one thread keeps it for the user
+        const unsigned long long key = a.slice_key[a.sm_per_slice ? z : 0];
+        const long long id = static_cast<long long>(key & 0xffffffffull);
+        const long long at = a.sm_per_slice ? static_cast<long long>(z) * plane + id : id;
+        slope = static_cast<uint32_t>(key >> 32);
+        t = a.M[at];
+        if (q == 0) {
+            a.slope[z] = slope;
+            a.index[z] = at;
+            a.mt[z] = t;
+        }
+    }
     if (q >= plane) return;
     const int x = q % a.nx, y = q / a.nx;
     const int64_t v = static_cast<int64_t>(z) * plane + q;
@@ -109,8 +111,7 @@ __global__ void __launch_bounds__(256) decide_kernel(DecideArgs a)
     }
     if (a.methods & HD_SM) {
         const uint32_t m = a.M[v];
-        const uint32_t t = a.mt[z];
-        const bool edge = a.slope[z] != 0;
+        const bool edge = slope != 0;
         a.H3[v] = edge && (a.sm_ge ? (m >= t) : (m > t));
     }
 }
@@ -253,18 +254,11 @@ cudaError_t launch_finalize(const DecideArgs &a, int sm_count, cudaStream_t s)
     if (a.methods & HD_SM) {
         cudaError_t e = cudaMemsetAsync(a.slice_key, 0, sizeof(unsigned long long) * a.nz, s);
         if (e != cudaSuccess) return e;
-        sm_slope_kernel<<<grid, 256, 0, s>>>(a.M, a.nx, a.ny, a.nz, a.sm_per_slice, a.nbhd,
-                                             a.slice_key);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        sm_threshold_kernel<<<(a.nz + 127) / 128, 128, 0, s>>>(a.M, a.nx, a.ny, a.nz,
-                                                               a.sm_per_slice, a.slice_key, a.mt,
-                                                               a.slope, a.index);
-        e = cudaGetLastError();
+        e = launch_chained(sm_slope_kernel, grid, 256, 0, s, a.M, a.nx, a.ny, a.nz, a.sm_per_slice,
+                           a.nbhd, a.slice_key);
         if (e != cudaSuccess) return e;
     }
-    decide_kernel<<<grid, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(decide_kernel, grid, 256, 0, s, a);
 }
 
 cudaError_t launch_pack_bits(const uint8_t *mask, int64_t V, uint32_t *bits, cudaStream_t s)

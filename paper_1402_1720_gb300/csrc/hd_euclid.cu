@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(kIngestThreads, 4) euclid_ingest_kernel(
         s_total = 0;
     }
     __syncthreads();
+    after_previous();
     EuCounts nc;
     bool tc_valid = false;
     float tc_ang = 0.0f;
@@ -334,6 +335,7 @@ __global__ void __launch_bounds__(kSetupThreads, 2) euclid_setup_kernel(
     uint32_t *s_next = s_mem + nt;     // pairs written per bucket so far
     uint32_t *s_events = s_next + nt;  // and their rows
     for (int t = threadIdx.x; t < nt; t += blockDim.x) s_next[t] = s_events[t] = 0;
+    after_previous();
     bucket_places<kSetupThreads>(nt, buckets, block_base, s_base);
     const int64_t h0 = static_cast<int64_t>(blockIdx.x) * per_block;
     const unsigned npairs = block_pairs[blockIdx.x];
@@ -393,6 +395,7 @@ constexpr int kOpenParts = 8;
 
 __global__ void __launch_bounds__(128) euclid_open_kernel(const ScanDesc *__restrict__ dp, RowsArgs ra)
 {
+    after_previous();
     const ScanDesc &d = *dp;
     const unsigned part = blockIdx.x / kOpenParts;
     const unsigned listed = d.pairs.fb_count[part];
@@ -471,14 +474,19 @@ cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, c
     const size_t cols = kGroups * static_cast<size_t>(tp.ntiles);
     cudaError_t e = launch_chunk_begin(desc.ctrl, desc.buckets, tp.ntiles, st);
     if (e != cudaSuccess) return e;
-    euclid_ingest_kernel<<<static_cast<unsigned>(sp.blocks), kIngestThreads, 4 * cols, st>>>(
-        in, n, sp.per_block, g, cd, tau_l, tau_h, use_miss, use_hit, ra.R, tp, rec, desc.ctrl,
-        desc.buckets.count, block_base, block_pairs, desc.pairs.stage);
-    euclid_setup_kernel<<<static_cast<unsigned>(sp.blocks), kSetupThreads, 12 * cols, st>>>(
-        tp, ra, sp.per_block, desc.buckets, block_base, block_pairs, desc.pairs);
+    e = launch_chained(euclid_ingest_kernel, static_cast<unsigned>(sp.blocks), kIngestThreads, 4 * cols,
+                       st, in, n, sp.per_block, g, cd, tau_l, tau_h, use_miss, use_hit, ra.R, tp,
+                       rec, desc.ctrl, desc.buckets.count, block_base, block_pairs,
+                       desc.pairs.stage);
+    if (e != cudaSuccess) return e;
+    e = launch_chained(euclid_setup_kernel, static_cast<unsigned>(sp.blocks), kSetupThreads, 12 * cols,
+                       st, tp, ra, sp.per_block, desc.buckets, block_base, block_pairs, desc.pairs);
+    if (e != cudaSuccess) return e;
     e = launch_trace_rows(desc_dev, tp.tile_words, tp.threads, grid, ra, st);
     if (e != cudaSuccess) return e;
-    euclid_open_kernel<<<static_cast<unsigned>(grid * kOpenParts), 128, 0, st>>>(desc_dev, ra);
+    e = launch_chained(euclid_open_kernel, static_cast<unsigned>(grid * kOpenParts), 128, 0, st, desc_dev,
+                       ra);
+    if (e != cudaSuccess) return e;
     // the records of the global path, when there are any
     e = launch_thick_clear(geom, workspace, desc.ctrl, sm_count, st);
     if (e != cudaSuccess) return e;

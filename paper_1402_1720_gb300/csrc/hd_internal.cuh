@@ -176,6 +176,37 @@ struct Inputs {
     const float *angle, *u_in, *v_in, *u_out, *v_out, *wepl;
 };
 
+// Launch of a kernel that begins with after_previous(): its blocks may come onto
+// the SMs, and do what needs none of the previous kernel's results, while that
+// one ends (the chain of a small chunk is mostly launches, ends and starts).
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
+                                  cudaStream_t s, const A &...args)
+{
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = grid;
+    c.blockDim = block;
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+#ifdef __CUDACC__
+// Waits until the previous kernel of the stream has ended and its writes are
+// visible; the next one may then be set up.  Every thread of a chained kernel
+// calls it before it reads or writes memory.
+__device__ __forceinline__ void after_previous()
+{
+    cudaGridDependencySynchronize();
+    cudaTriggerProgrammaticLaunchCompletion();
+}
+#endif
+
 // ---- launchers (stream-ordered; return the launch's cudaError_t) ----
 
 // Begins a chunk: clears the scan's lists (Ctrl from n_global on) and the

@@ -53,6 +53,7 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
     uint32_t *s_next = s_mem + nt;  // pairs written per bucket so far
     uint32_t *s_events = s_next + nt;  // and the events of their walks
     for (int t = threadIdx.x; t < nt; t += blockDim.x) s_next[t] = s_events[t] = 0;
+    after_previous();
     bucket_places<kScatterThreads>(nt, buckets, block_base, s_base);
     const int64_t h0 = static_cast<int64_t>(blockIdx.x) * per_block;
     const unsigned npairs = block_pairs[blockIdx.x];
@@ -160,9 +161,8 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
     if (n <= 0) return cudaSuccess;
     const ChunkSplit sp = chunk_split(n, sm_count);
     const size_t smem = sizeof(uint32_t) * 3 * kGroups * static_cast<size_t>(tp.ntiles);
-    scatter_kernel<<<static_cast<unsigned>(sp.blocks), kScatterThreads, smem, s>>>(
-        tp, rec, sp.per_block, buckets, block_base, block_pairs, ctrl, pairs);
-    return cudaGetLastError();
+    return launch_chained(scatter_kernel, static_cast<unsigned>(sp.blocks), kScatterThreads, smem, s, tp,
+                          rec, sp.per_block, buckets, block_base, block_pairs, ctrl, pairs);
 }
 
 }  // namespace hd

@@ -639,6 +639,10 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     __shared__ int s_slots[kPartList];      // slots of each group
     __shared__ int s_ngroups;
     __shared__ unsigned long long s_warp[32];
+    // each flush clears its box: the tile starts cleared once
+    for (int w = threadIdx.x; w < smem_words >> 2; w += blockDim.x)
+        reinterpret_cast<uint4 *>(tile)[w] = make_uint4(0u, 0u, 0u, 0u);
+    after_previous();
     // buckets of scan k are the launch's buckets [s_first[k], s_first[k + 1])
     if (threadIdx.x == 0) {
         s_next[1] = 0;
@@ -649,9 +653,6 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         }
         s_first[nscans] = acc;
     }
-    // each flush clears its box: the tile starts cleared once
-    for (int w = threadIdx.x; w < smem_words >> 2; w += blockDim.x)
-        reinterpret_cast<uint4 *>(tile)[w] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     const int nb = s_first[nscans];
     const int per = (nb + kThreads - 1) / kThreads;
@@ -849,20 +850,19 @@ static cudaError_t launch_trace(const ScanDesc *descs, int nscans, int tile_word
     const size_t smem = static_cast<size_t>(smem_words) * 4;
     switch (threads) {
     case 256:
-        trace_tiles_kernel<256, RowsT><<<grid, 256, smem, s>>>(descs, nscans, smem_words, ra);
-        break;
+        return launch_chained(trace_tiles_kernel<256, RowsT>, grid, 256, smem, s, descs, nscans,
+                              smem_words, ra);
     case 512:
-        trace_tiles_kernel<512, RowsT><<<grid, 512, smem, s>>>(descs, nscans, smem_words, ra);
-        break;
+        return launch_chained(trace_tiles_kernel<512, RowsT>, grid, 512, smem, s, descs, nscans,
+                              smem_words, ra);
     case 768:
-        trace_tiles_kernel<768, RowsT><<<grid, 768, smem, s>>>(descs, nscans, smem_words, ra);
-        break;
+        return launch_chained(trace_tiles_kernel<768, RowsT>, grid, 768, smem, s, descs, nscans,
+                              smem_words, ra);
     case 1024:
-        trace_tiles_kernel<1024, RowsT><<<grid, 1024, smem, s>>>(descs, nscans, smem_words, ra);
-        break;
+        return launch_chained(trace_tiles_kernel<1024, RowsT>, grid, 1024, smem, s, descs, nscans,
+                              smem_words, ra);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,

@@ -146,6 +146,7 @@ __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
         s_total = 0;
     }
     __syncthreads();
+    after_previous();
     LaneAcc acc;
     TrigCache tc;
     // the block's histories arrive grouped by gantry angle, so a thread's
@@ -229,6 +230,7 @@ __global__ void __launch_bounds__(256) trace_global_kernel(Records rec, Ctrl *ct
                                                            uint32_t *N, uint32_t *M,
                                                            int all_records)
 {
+    after_previous();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t total = rec.glist ? static_cast<int64_t>(ctrl->n_global) : rec.cap;
     unsigned taken = 0;
@@ -283,19 +285,18 @@ cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cor
         reinterpret_cast<uintptr_t>(in.v_in) | reinterpret_cast<uintptr_t>(in.u_out) |
         reinterpret_cast<uintptr_t>(in.v_out) | reinterpret_cast<uintptr_t>(in.wepl);
     if (on_host && (bits & 15u) == 0)
-        ingest_kernel<true><<<static_cast<unsigned>(sp.blocks), kIngestThreads, smem, s>>>(
-            in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl,
-            bucket_count, bb, bp, sg);
-    else
-        ingest_kernel<false><<<static_cast<unsigned>(sp.blocks), kIngestThreads, smem, s>>>(
-            in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit, tpl, rec, ctrl,
-            bucket_count, bb, bp, sg);
-    return cudaGetLastError();
+        return launch_chained(ingest_kernel<true>, static_cast<unsigned>(sp.blocks), kIngestThreads,
+                              smem, s, in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss,
+                              use_hit, tpl, rec, ctrl, bucket_count, bb, bp, sg);
+    return launch_chained(ingest_kernel<false>, static_cast<unsigned>(sp.blocks), kIngestThreads,
+                          smem, s, in, n, sp.per_block, g, cordic, tau_l, tau_h, use_miss, use_hit,
+                          tpl, rec, ctrl, bucket_count, bb, bp, sg);
 }
 
 // Clears a chunk's counters: the scan's lists and the buckets' pairs and events.
 __global__ void __launch_bounds__(1024) chunk_begin_kernel(Ctrl *ctrl, Buckets buckets, int ncols)
 {
+    after_previous();
     if (blockIdx.x == 0 && threadIdx.x == 0)
         ctrl->n_global = ctrl->n_fallback = ctrl->n_pair_fallback = ctrl->fb_next = 0u;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ncols; t += gridDim.x * blockDim.x) {
@@ -307,9 +308,8 @@ __global__ void __launch_bounds__(1024) chunk_begin_kernel(Ctrl *ctrl, Buckets b
 cudaError_t launch_chunk_begin(Ctrl *ctrl, const Buckets &buckets, int ntiles, cudaStream_t s)
 {
     const int ncols = kGroups * ntiles;
-    chunk_begin_kernel<<<static_cast<unsigned>(ncols > 4096 ? (ncols + 4095) / 4096 : 1), 1024, 0, s>>>(
-        ctrl, buckets, ncols);
-    return cudaGetLastError();
+    return launch_chained(chunk_begin_kernel, static_cast<unsigned>(ncols > 4096 ? (ncols + 4095) / 4096 : 1),
+                          1024, 0, s, ctrl, buckets, ncols);
 }
 
 cudaError_t init_ingest()
@@ -331,9 +331,8 @@ cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, c
     int64_t blocks = (upper + 255) / 256;
     const int64_t cap_blocks = static_cast<int64_t>(sm_count) * 8;
     if (blocks > cap_blocks) blocks = cap_blocks;
-    trace_global_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(rec, ctrl, g, N, M,
-                                                                       all_records);
-    return cudaGetLastError();
+    return launch_chained(trace_global_kernel, static_cast<unsigned>(blocks), 256, 0, s, rec, ctrl, g, N,
+                          M, all_records);
 }
 
 cudaError_t launch_classify(const float *wepl, int64_t n, float tau_l, float tau_h, uint8_t *cls,
