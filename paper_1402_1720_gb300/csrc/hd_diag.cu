@@ -4,14 +4,14 @@
 // H_2 of Eq. 3.6, whose excluded voxels form a shell around the object, it
 // keeps the region the shell encloses).
 //
-//   compare_kernel  one block per slice: block sums of the two counts
+//   compare_kernel  blocks over pieces of a slice: sums of the two counts
 //   fill_kernel     one block per slice: the mask and the exterior (mask
 //                   voxels joined to the slice border) as bitmaps in shared
-//                   memory, one row of words per voxel row; the exterior
-//                   grows by one voxel across words and rows and by whole
-//                   runs inside a word per sweep, until a sweep adds nothing
+//                   memory, one row of words per voxel row; the exterior grows
+//                   tile by tile (hd_grow.cuh)
 #include <cuda_runtime.h>
 
+#include "hd_grow.cuh"
 #include "hd_internal.cuh"
 
 namespace {
@@ -19,71 +19,59 @@ namespace {
 constexpr int kDiagThreads = 1024;
 constexpr int kFillMaxWords = 24 * 1024;  // two bitmaps of 96 KB
 
-__device__ __forceinline__ long long block_sum(long long v, long long *s_warp)
+constexpr int kCompareThreads = 256;
+constexpr int kComparePiece = 16 * kCompareThreads;  // voxels of a block
+
+// Nonzero bytes of h where o is zero, over four bytes.
+__device__ __forceinline__ unsigned only(unsigned h, unsigned o)
 {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) s_warp[warp] = v;
-    __syncthreads();
-    long long t = 0;
-    if (threadIdx.x == 0)
-        for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) t += s_warp[k];
-    __syncthreads();
-    return t;  // valid in thread 0
+    return static_cast<unsigned>(__popc(__vcmpne4(h, 0u) & __vcmpeq4(o, 0u))) >> 3;
 }
 
-__global__ void __launch_bounds__(kDiagThreads) compare_kernel(const uint8_t *hull,
-                                                               const uint8_t *object, int64_t plane,
-                                                               int nz, long long *counts)
+// A block per piece of a slice, 16 voxels a thread (one 16-byte load of each
+// volume where both slices allow it).  Latency-bound: a block per slice took 16 us
+// on the head-sized volume, in 40 steps of one voxel.
+__global__ void __launch_bounds__(kCompareThreads) compare_kernel(const uint8_t *hull,
+                                                                  const uint8_t *object,
+                                                                  int64_t plane, int nz,
+                                                                  unsigned long long *counts)
 {
-    __shared__ long long s_warp[32];
-    const int z = blockIdx.x;
+    const int z = blockIdx.y;
     const uint8_t *h = hull + static_cast<int64_t>(z) * plane;
     const uint8_t *o = object + static_cast<int64_t>(z) * plane;
-    long long extra = 0, missing = 0;
-    for (int64_t j = threadIdx.x; j < plane; j += blockDim.x) {
-        const bool hv = h[j] != 0, ov = o[j] != 0;
-        extra += hv && !ov ? 1 : 0;
-        missing += ov && !hv ? 1 : 0;
+    const int64_t j0 = static_cast<int64_t>(blockIdx.x) * kComparePiece;
+    unsigned extra = 0, missing = 0;
+    const int64_t j = j0 + 16 * static_cast<int>(threadIdx.x);
+    if (((reinterpret_cast<uintptr_t>(h) | reinterpret_cast<uintptr_t>(o)) & 15u) == 0 &&
+        j0 + kComparePiece <= plane) {
+        const uint4 a = *reinterpret_cast<const uint4 *>(h + j);
+        const uint4 b = *reinterpret_cast<const uint4 *>(o + j);
+        extra = only(a.x, b.x) + only(a.y, b.y) + only(a.z, b.z) + only(a.w, b.w);
+        missing = only(b.x, a.x) + only(b.y, a.y) + only(b.z, a.z) + only(b.w, a.w);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int64_t q = j0 + k * kCompareThreads + static_cast<int>(threadIdx.x);
+            const bool hv = q < plane && h[q] != 0, ov = q < plane && o[q] != 0;
+            extra += hv && !ov ? 1u : 0u;
+            missing += ov && !hv ? 1u : 0u;
+        }
     }
-    const long long e = block_sum(extra, s_warp);
-    const long long m = block_sum(missing, s_warp);
-    if (threadIdx.x == 0) {
-        counts[z] = e;
-        counts[nz + z] = m;
-        atomicAdd(reinterpret_cast<unsigned long long *>(counts + 2 * nz),
-                  static_cast<unsigned long long>(e));
-        atomicAdd(reinterpret_cast<unsigned long long *>(counts + 2 * nz + 1),
-                  static_cast<unsigned long long>(m));
+    extra = __reduce_add_sync(0xffffffffu, extra);
+    missing = __reduce_add_sync(0xffffffffu, missing);
+    __shared__ unsigned s_sum[2];
+    if (threadIdx.x < 2) s_sum[threadIdx.x] = 0u;
+    __syncthreads();
+    if ((threadIdx.x & 31u) == 0) {
+        atomicAdd(&s_sum[0], extra);
+        atomicAdd(&s_sum[1], missing);
     }
-}
-
-// Bits of g reachable from g through set bits of p, moving toward higher
-// bits (left) and toward lower bits (right) inside one word (Kogge-Stone).
-__device__ __forceinline__ uint32_t fill_word(uint32_t g, uint32_t p)
-{
-    uint32_t l = g, pl = p;
-    l |= pl & (l << 1);
-    pl &= pl << 1;
-    l |= pl & (l << 2);
-    pl &= pl << 2;
-    l |= pl & (l << 4);
-    pl &= pl << 4;
-    l |= pl & (l << 8);
-    pl &= pl << 8;
-    l |= pl & (l << 16);
-    uint32_t r = g, pr = p;
-    r |= pr & (r >> 1);
-    pr &= pr >> 1;
-    r |= pr & (r >> 2);
-    pr &= pr >> 2;
-    r |= pr & (r >> 4);
-    pr &= pr >> 4;
-    r |= pr & (r >> 8);
-    pr &= pr >> 8;
-    r |= pr & (r >> 16);
-    return l | r;
+    __syncthreads();
+    if (threadIdx.x < 2 && s_sum[threadIdx.x] != 0u) {
+        const unsigned long long c = s_sum[threadIdx.x];
+        atomicAdd(counts + static_cast<int64_t>(threadIdx.x) * nz + z, c);
+        atomicAdd(counts + 2 * static_cast<int64_t>(nz) + threadIdx.x, c);
+    }
 }
 
 // Bitmaps: word (y, w) = y * rw + w holds voxels x = 32 w .. 32 w + 31 of
@@ -100,11 +88,19 @@ __global__ void __launch_bounds__(kDiagThreads) fill_kernel(const uint8_t *mask,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int words = ny * rw;
     // mask bits, a warp per word (coalesced bytes, one ballot)
-    for (int k = warp; k < words; k += nwarps) {
-        const int y = k / rw, x = (k - y * rw) * 32 + lane;
-        const bool bit = x < nx && m[static_cast<int64_t>(y) * nx + x] != 0;
-        const uint32_t word = __ballot_sync(0xffffffffu, bit);
-        if (lane == 0) M[k] = word;
+    for (int k0 = warp; k0 < words; k0 += 8 * nwarps) {  // eight loads in flight
+        uint8_t v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = k0 + i * nwarps, y = k / rw, x = (k - y * rw) * 32 + lane;
+            v[i] = k < words && x < nx ? m[static_cast<int64_t>(y) * nx + x] : 0;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const int k = k0 + i * nwarps;
+            const uint32_t word = __ballot_sync(0xffffffffu, v[i] != 0);
+            if (lane == 0 && k < words) M[k] = word;
+        }
     }
     __syncthreads();
     // seeds: the mask voxels on the slice border
@@ -120,33 +116,14 @@ __global__ void __launch_bounds__(kDiagThreads) fill_kernel(const uint8_t *mask,
         E[k] = seed & M[k];
     }
     __syncthreads();
-    // sweeps until nothing changes; each sweep that changes adds a voxel, so
-    // at most nx ny + 1 sweeps run
-    const long long max_sweeps = plane + 1;
-    for (long long it = 0; it < max_sweeps; ++it) {
-        int changed = 0;
-        for (int k = threadIdx.x; k < words; k += blockDim.x) {
-            const int y = k / rw, w = k - y * rw;
-            const uint32_t e = E[k], mk = M[k];
-            uint32_t g = e | (e << 1) | (e >> 1);
-            if (w > 0) g |= E[k - 1] >> 31;
-            if (w + 1 < rw) g |= E[k + 1] << 31;
-            if (y > 0) g |= E[k - rw];
-            if (y + 1 < ny) g |= E[k + rw];
-            const uint32_t ne = fill_word(g & mk, mk);
-            if (ne != e) {
-                E[k] = ne;  // only this thread writes word k; neighbours may
-                changed = 1;  // read it old or new, both inside the exterior
-            }
-        }
-        if (!__syncthreads_or(changed)) break;
-    }
+    hd::grow_region<false>(M, E, rw, ny, plane);
     // enclosed = mask, not exterior
     uint8_t *o = out + static_cast<int64_t>(z) * plane;
-    for (int64_t j = threadIdx.x; j < plane; j += blockDim.x) {
-        const int y = static_cast<int>(j / nx), x = static_cast<int>(j - static_cast<int64_t>(y) * nx);
-        const int k = y * rw + (x >> 5);
-        o[j] = static_cast<uint8_t>(((M[k] & ~E[k]) >> (x & 31)) & 1u);
+    for (int k = warp; k < words; k += nwarps) {
+        const int y = k / rw, x = (k - y * rw) * 32 + lane;
+        if (x < nx)
+            o[static_cast<int64_t>(y) * nx + x] =
+                static_cast<uint8_t>(((M[k] & ~E[k]) >> lane) & 1u);
     }
 }
 
@@ -160,11 +137,14 @@ hd_status hd_hull_compare(const uint8_t *hull, const uint8_t *object, int32_t nx
     if (!hull || !object || !counts || nx < 1 || ny < 1 || nz < 1) return HD_ERR_ARG;
     if (nz > 65535) return HD_ERR_RANGE;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaMemsetAsync(counts + 2 * static_cast<int64_t>(nz), 0,
-                                    2 * sizeof(int64_t), st);
+    const int64_t plane = static_cast<int64_t>(nx) * ny;
+    const int64_t pieces = (plane + kComparePiece - 1) / kComparePiece;
+    if (pieces > 0x7fffffff) return HD_ERR_RANGE;
+    cudaError_t e = cudaMemsetAsync(counts, 0, (2 * static_cast<size_t>(nz) + 2) * sizeof(int64_t), st);
     if (e == cudaSuccess) {
-        compare_kernel<<<nz, kDiagThreads, 0, st>>>(hull, object, static_cast<int64_t>(nx) * ny,
-                                                    nz, reinterpret_cast<long long *>(counts));
+        compare_kernel<<<dim3(static_cast<unsigned>(pieces), static_cast<unsigned>(nz)), kCompareThreads,
+                         0, st>>>(hull, object, plane, nz,
+                                  reinterpret_cast<unsigned long long *>(counts));
         e = cudaGetLastError();
     }
     if (e != cudaSuccess) {
