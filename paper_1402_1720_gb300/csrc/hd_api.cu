@@ -1348,6 +1348,17 @@ void free_batch(hd_batch *b)
     delete b;
 }
 
+// The descriptor of a batch's item: its scan's, with the item's records.
+hd::ScanDesc item_desc(const hd_batch::Item &it)
+{
+    hd::ScanDesc d = it.scan->desc_host;
+    d.rec = records_of(it.scan, it.n);
+    d.nx = it.scan->geom.nx;
+    d.ny = it.scan->geom.ny;
+    d.nz = it.scan->geom.nz;
+    return d;
+}
+
 // One round: every item of `round` (distinct scans), issued on `st` with
 // the per-scan stages forked to the side streams.  Returns the number of
 // kernels issued through *kernels.
@@ -1363,13 +1374,17 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
             if (it.scan->tp.tile_words > max_words) max_words = it.scan->tp.tile_words;
         }
     }
+    // the stages of different scans run side by side on the side streams; a
+    // single scan needs none of them
+    const int sides = n_items == 1 ? 0 : (n_items < hd_batch::kSide ? n_items : hd_batch::kSide);
+    auto side_of = [&](int i) { return sides == 0 ? st : b->side[i % sides]; };
     auto fork = [&]() -> hd_status {
-        HD_CUDA(cudaEventRecord(b->fork, st));
-        for (int k = 0; k < hd_batch::kSide; ++k) HD_CUDA(cudaStreamWaitEvent(b->side[k], b->fork, 0));
+        if (sides > 0) HD_CUDA(cudaEventRecord(b->fork, st));
+        for (int k = 0; k < sides; ++k) HD_CUDA(cudaStreamWaitEvent(b->side[k], b->fork, 0));
         return HD_OK;
     };
     auto join = [&]() -> hd_status {
-        for (int k = 0; k < hd_batch::kSide; ++k) {
+        for (int k = 0; k < sides; ++k) {
             HD_CUDA(cudaEventRecord(b->join[k], b->side[k]));
             HD_CUDA(cudaStreamWaitEvent(st, b->join[k], 0));
         }
@@ -1377,9 +1392,14 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
     };
     hd_status r = fork();
     if (r != HD_OK) return r;
+    int64_t upper = 0;
+    bool any_finalize = false;
+    auto finalizes = [&](const hd_batch::Item &it) {
+        return (it.last && (flags & HD_BATCH_FINALIZE)) || (it.flags & HD_BATCH_FINALIZE);
+    };
     for (int i = 0; i < n_items; ++i) {
         hd_scan *s = round[i].scan;
-        cudaStream_t ss = b->side[i % hd_batch::kSide];
+        cudaStream_t ss = side_of(i);
         if ((round[i].first && (flags & HD_BATCH_RESET)) || (round[i].flags & HD_BATCH_RESET)) {
             r = stage_reset(s, ss);
             if (r != HD_OK) return r;
@@ -1387,6 +1407,8 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
         r = stage_prepare(s, round[i].in, round[i].n, ss);
         if (r != HD_OK) return r;
         *kernels += 2 + ((s->tp.ntiles > 0 && s->trace_grid > 0) ? 1 : 0);
+        if (round[i].n > upper) upper = round[i].n;
+        any_finalize = any_finalize || finalizes(round[i]);
     }
     r = join();
     if (r != HD_OK) return r;
@@ -1394,20 +1416,16 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
         HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, st));
         *kernels += 1;
     }
+    HD_CUDA(hd::launch_trace_global_batch(b->descs_dev, n_items, upper, b->sm_count, st));
+    *kernels += upper > 0 ? 1 : 0;
+    if (!any_finalize) return HD_OK;
     r = fork();
     if (r != HD_OK) return r;
     for (int i = 0; i < n_items; ++i) {
-        hd_scan *s = round[i].scan;
-        cudaStream_t ss = b->side[i % hd_batch::kSide];
-        r = stage_global(s, round[i].n, ss);
+        if (!finalizes(round[i])) continue;
+        r = stage_finalize(round[i].scan, side_of(i));
         if (r != HD_OK) return r;
-        *kernels += 1;
-        if ((round[i].last && (flags & HD_BATCH_FINALIZE)) ||
-            (round[i].flags & HD_BATCH_FINALIZE)) {
-            r = stage_finalize(s, ss);
-            if (r != HD_OK) return r;
-            *kernels += finalize_launches(s);
-        }
+        *kernels += finalize_launches(round[i].scan);
     }
     return join();
 }
@@ -1551,6 +1569,7 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
         key.push_back(static_cast<uintptr_t>(it.n));
         key.push_back(reinterpret_cast<uintptr_t>(it.scan->desc_dev));
         key.push_back(reinterpret_cast<uintptr_t>(it.scan->pair_buf));
+        key.push_back(reinterpret_cast<uintptr_t>(it.scan->rec_buf));
         key.push_back(static_cast<uintptr_t>(it.scan->tp.threads));
     }
     // the legacy default stream cannot be captured: run directly there
@@ -1574,7 +1593,7 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
         int64_t kernels = 0;
         if (graphable) {
             std::vector<hd::ScanDesc> descs;
-            for (const auto &it : rounds[0]) descs.push_back(it.scan->desc_host);
+            for (const auto &it : rounds[0]) descs.push_back(item_desc(it));
             HD_CUDA(cudaMemcpyAsync(batch->descs_dev, descs.data(),
                                     sizeof(hd::ScanDesc) * descs.size(), cudaMemcpyHostToDevice, st));
             HD_CUDA(cudaStreamSynchronize(st));
@@ -1606,12 +1625,13 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
             HD_CUDA(cudaGraphLaunch(batch->exec, st));
             batch->stats.graph_captures += 1;
         } else {
+            batch->key.clear();  // a captured graph's table of descriptors is overwritten
             for (size_t k = 0; k < rounds.size(); ++k) {
                 // stream-ordered upload of the table: the pinned staging may be
                 // refilled once the previous upload from it has run
                 HD_CUDA(cudaEventSynchronize(batch->descs_copied));
                 for (size_t i = 0; i < rounds[k].size(); ++i)
-                    batch->descs_pinned[i] = rounds[k][i].scan->desc_host;
+                    batch->descs_pinned[i] = item_desc(rounds[k][i]);
                 HD_CUDA(cudaMemcpyAsync(batch->descs_dev, batch->descs_pinned,
                                         sizeof(hd::ScanDesc) * rounds[k].size(),
                                         cudaMemcpyHostToDevice, st));

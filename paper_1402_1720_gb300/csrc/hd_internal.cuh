@@ -159,6 +159,9 @@ struct ScanDesc {
     Buckets buckets;
     Ctrl *ctrl;  // the scan's counters (added to) and fallback list (read)
     uint32_t *N, *M;
+    // of a batch's entries: the item's records and the grid they are walked in
+    Records rec;
+    int32_t nx, ny, nz;
 };
 
 constexpr int kMaxBatch = 64;  // scans per batched traversal launch
@@ -251,6 +254,12 @@ cudaError_t launch_trace_rows(const ScanDesc *desc, int tile_words, int threads,
 cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, const GeomQ &g,
                                 uint32_t *N, uint32_t *M, int all_records,
                                 int sm_count, cudaStream_t s);
+
+// The same for the chunks of nscans scans in one launch: most of them have no
+// such record, and a launch each, on forked streams, cost a server's thread more
+// than the work.  upper: the largest chunk's slots.
+cudaError_t launch_trace_global_batch(const ScanDesc *descs, int nscans, int64_t upper,
+                                      int sm_count, cudaStream_t s);
 
 // Once per device, before the first launch there: the shared memory ingest and
 // scatter may use for the most tiles a plan can have.

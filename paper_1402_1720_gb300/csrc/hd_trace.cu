@@ -226,11 +226,9 @@ __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
 
 // ---------------------------------------------------------------- traversal
 
-__global__ void __launch_bounds__(256) trace_global_kernel(Records rec, Ctrl *ctrl, GeomQ g,
-                                                           uint32_t *N, uint32_t *M,
-                                                           int all_records)
+__device__ __forceinline__ void trace_records(const Records &rec, Ctrl *ctrl, int nx, int ny, int nz,
+                                              uint32_t *N, uint32_t *M, int all_records)
 {
-    after_previous();
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t total = rec.glist ? static_cast<int64_t>(ctrl->n_global) : rec.cap;
     unsigned taken = 0;
@@ -244,11 +242,26 @@ __global__ void __launch_bounds__(256) trace_global_kernel(Records rec, Ctrl *ct
         const int32_t go[3] = {rec.g[3][i], rec.g[4][i], rec.g[5][i]};
         GlobalVisit v;
         v.vol = status_cls(stw) ? M : N;
-        walk_all(gi, go, g.nx, g.ny, g.nz, v);
+        walk_all(gi, go, nx, ny, nz, v);
         ++taken;
     }
     const unsigned tk = warp_sum_u32(taken);
     if ((threadIdx.x & 31u) == 0 && tk && !all_records) atomicAdd(&ctrl->n_fallback, tk);
+}
+
+__global__ void __launch_bounds__(256) trace_global_kernel(Records rec, Ctrl *ctrl, int nx, int ny,
+                                                           int nz, uint32_t *N, uint32_t *M,
+                                                           int all_records)
+{
+    after_previous();
+    trace_records(rec, ctrl, nx, ny, nz, N, M, all_records);
+}
+
+__global__ void __launch_bounds__(256) trace_global_batch_kernel(const ScanDesc *descs)
+{
+    after_previous();
+    const ScanDesc &d = descs[blockIdx.y];
+    trace_records(d.rec, d.ctrl, d.nx, d.ny, d.nz, d.N, d.M, 0);
 }
 
 __global__ void classify_kernel(const float *__restrict__ w, int64_t n, float tau_l, float tau_h,
@@ -331,8 +344,20 @@ cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, c
     int64_t blocks = (upper + 255) / 256;
     const int64_t cap_blocks = static_cast<int64_t>(sm_count) * 8;
     if (blocks > cap_blocks) blocks = cap_blocks;
-    return launch_chained(trace_global_kernel, static_cast<unsigned>(blocks), 256, 0, s, rec, ctrl, g, N,
-                          M, all_records);
+    return launch_chained(trace_global_kernel, static_cast<unsigned>(blocks), 256, 0, s, rec, ctrl,
+                          g.nx, g.ny, g.nz, N, M, all_records);
+}
+
+cudaError_t launch_trace_global_batch(const ScanDesc *descs, int nscans, int64_t upper,
+                                      int sm_count, cudaStream_t s)
+{
+    if (upper <= 0 || nscans < 1) return cudaSuccess;
+    int64_t blocks = (upper + 255) / 256;
+    const int64_t cap_blocks = (static_cast<int64_t>(sm_count) * 8 + nscans - 1) / nscans;
+    if (blocks > cap_blocks) blocks = cap_blocks;
+    return launch_chained(trace_global_batch_kernel,
+                          dim3(static_cast<unsigned>(blocks), static_cast<unsigned>(nscans)), 256, 0, s,
+                          descs);
 }
 
 cudaError_t launch_classify(const float *wepl, int64_t n, float tau_l, float tau_h, uint8_t *cls,
