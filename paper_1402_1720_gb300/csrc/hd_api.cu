@@ -149,6 +149,10 @@ struct hd_scan {
     bool inputs_on_host = false;  // the chunk being added is read in place from host memory
     float *staging = nullptr;  // copied host inputs: 6 columns of staging_half floats
     int64_t staging_half = 0;
+    // copies of page-locked inputs that run beside the chunks before (add_mapped)
+    static constexpr int kSlots = 3;
+    cudaStream_t up = nullptr;
+    cudaEvent_t up_begin = nullptr, up_copied[kSlots] = {}, up_free[kSlots] = {};
     uint32_t *compact_blocks = nullptr;
     unsigned long long *d_count = nullptr;
     int32_t *compact_out = nullptr;
@@ -212,9 +216,12 @@ void drain_profile(hd_scan *s)
     s->pending.clear();
 }
 
+void free_upload(hd_scan *s);
+
 void free_scan(hd_scan *s)
 {
     drain_profile(s);
+    free_upload(s);
     for (cudaEvent_t e : s->event_pool) cudaEventDestroy(e);
 
     void *ptrs[] = {s->N, s->M, s->H1, s->H2, s->H3, s->bits_out, s->slice_key,
@@ -334,6 +341,31 @@ bool all_mapped_host(const float *const src[6], int device)
             return false;
     }
     return true;
+}
+
+// The stream and events of add_mapped, made at its first use.
+bool ensure_upload(hd_scan *s)
+{
+    if (s->up_begin) return true;
+    bool ok = s->up || cudaStreamCreateWithFlags(&s->up, cudaStreamNonBlocking) == cudaSuccess;
+    auto event = [&](cudaEvent_t &e) {
+        ok = ok && (e || cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess);
+    };
+    for (auto &e : s->up_copied) event(e);
+    for (auto &e : s->up_free) event(e);
+    event(s->up_begin);
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
+void free_upload(hd_scan *s)
+{
+    if (s->up) cudaStreamDestroy(s->up);
+    if (s->up_begin) cudaEventDestroy(s->up_begin);
+    for (auto &e : s->up_copied)
+        if (e) cudaEventDestroy(e);
+    for (auto &e : s->up_free)
+        if (e) cudaEventDestroy(e);
 }
 
 // The records of a chunk of n histories: seven arrays of n slots and the
@@ -556,6 +588,99 @@ hd_status stage_finalize(hd_scan *scan, cudaStream_t st)
 }
 
 int finalize_launches(const hd_scan *scan) { return (scan->params.methods & HD_SM) ? 2 : 1; }
+
+hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st);
+
+// Page-locked inputs of many histories: copied in parts by the copy engine on a
+// stream of their own while the parts before are traversed, where reading them in
+// place kept the chip waiting for the host link (210 GB/s) with nothing beside
+// it.  Only the first copy is not hidden, and a history is traversed about as fast
+// as it is copied, so parts grow; each chunk has some 60 us of its own, so there
+// are few: three, each half as large again, or from kManyParts on four, a quarter
+// larger.  Head-sized scan: 9e6 histories 1951 us in place, 1665 in three parts,
+// 1567 in four; 4.5e6 1066, 953 and 1027; 2.7e6 711, 711 and 797.  taken stays
+// false when copying is not possible here (the stream is being captured, no
+// memory): the caller then reads in place.
+constexpr int64_t kOverlapLeast = int64_t(3) << 20;
+constexpr int64_t kManyParts = int64_t(6) << 20;
+constexpr int64_t kPartMost = int64_t(1) << 23;
+
+hd_status add_mapped(hd_scan *s, const float *const src[6], int64_t n, cudaStream_t st, bool &taken)
+{
+    taken = false;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return HD_OK;
+    }
+    constexpr int kSlots = hd_scan::kSlots;
+    std::vector<int64_t> parts;
+    const int grow = n < kManyParts ? 2 : 4;  // by a half or a quarter
+    int64_t part = n < kManyParts ? n / 5 : n * 9 / 50, left = n;
+    if (part > kPartMost / 4) part = kPartMost / 4;
+    int64_t most = 0, size[kSlots] = {};
+    while (left > 0) {
+        int64_t c = (part + 3) & ~int64_t(3);
+        if (left < c + c / 2) c = left;
+        if (c > kPartMost) c = kPartMost;
+        int64_t &slot = size[parts.size() % kSlots];
+        if (c > slot) slot = c;
+        if (c > most) most = c;
+        parts.push_back(c);
+        left -= c;
+        part = c + c / grow;
+    }
+    hd_status r = ensure_records(s, most, st);
+    if (r != HD_OK) return r;
+    if (!ensure_upload(s)) return HD_OK;
+    int64_t at[kSlots], cap_all = 0;
+    for (int k = 0; k < kSlots; ++k) {
+        at[k] = cap_all;
+        cap_all += (size[k] + 3) & ~int64_t(3);
+    }
+    r = ensure_staging(s, cap_all, st);
+    if (r != HD_OK) return r == HD_ERR_NOMEM ? HD_OK : r;
+    // evenly spaced columns are one strided copy per part
+    const int64_t pitch = src[1] - src[0];
+    bool rows = pitch >= n && pitch < (int64_t(1) << 28);
+    for (int a = 1; a < 5; ++a) rows = rows && src[a + 1] - src[a] == pitch;
+    auto copy = [&](float *to, int64_t width, int64_t off, int64_t c) {
+        if (rows)
+            return cudaMemcpy2DAsync(to, sizeof(float) * width, src[0] + off, sizeof(float) * pitch,
+                                     sizeof(float) * c, 6, cudaMemcpyHostToDevice, s->up);
+        cudaError_t e = cudaSuccess;
+        for (int a = 0; a < 6 && e == cudaSuccess; ++a)
+            e = cudaMemcpyAsync(to + a * width, src[a] + off, sizeof(float) * c,
+                                cudaMemcpyHostToDevice, s->up);
+        return e;
+    };
+    taken = true;
+    // after what st holds: the staging's last readers, the inputs' writers
+    HD_CUDA(cudaEventRecord(s->up_begin, st));
+    HD_CUDA(cudaStreamWaitEvent(s->up, s->up_begin, 0));
+    int64_t off = 0;
+    for (size_t k = 0; k < parts.size(); off += parts[k], ++k) {
+        const int64_t c = parts[k], w = (c + 3) & ~int64_t(3);  // columns on 16-byte boundaries
+        const int slot = static_cast<int>(k % kSlots);
+        float *const to = s->staging + 6 * at[slot];
+        cudaError_t e = k < kSlots ? cudaSuccess : cudaStreamWaitEvent(s->up, s->up_free[slot], 0);
+        if (e == cudaSuccess) e = copy(to, w, off, c);
+        if (e == cudaSuccess) e = cudaEventRecord(s->up_copied[slot], s->up);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->up_copied[slot], 0);
+        r = HD_OK;
+        if (e == cudaSuccess) {
+            const hd::Inputs in{to, to + w, to + 2 * w, to + 3 * w, to + 4 * w, to + 5 * w};
+            r = run_chunk(s, in, c, st);
+        }
+        if (e == cudaSuccess && r == HD_OK) e = cudaEventRecord(s->up_free[slot], st);
+        if (e != cudaSuccess || r != HD_OK) {
+            cudaStreamSynchronize(s->up);  // the inputs may be gone after this call
+            if (e != cudaSuccess) note_cuda(e, "hd_scan_add_histories: copies");
+            return e != cudaSuccess ? HD_ERR_CUDA : r;
+        }
+    }
+    return HD_OK;
+}
 
 // One chunk through the whole path on st.
 hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st)
@@ -817,14 +942,19 @@ hd_status hd_scan_add_histories(hd_scan *scan, const float *angle_deg, const flo
             if (r != HD_OK) return r;
         }
     } else if (all_mapped_host(src, scan->device)) {
-        // page-locked host arrays mapped into the device's address space: the
-        // ingest kernel reads them in place over the host link, so the
+        // page-locked host arrays mapped into the device's address space: many
+        // histories are copied beside the traversal of those before them; few
+        // are read in place by the ingest kernel, over the host link, so the
         // transfer happens inside the kernel that consumes it
+        hd_status r = HD_OK;
+        bool taken = false;
+        if (n >= kOverlapLeast) r = add_mapped(scan, src, n, st, taken);
+        const bool in_place = !taken;
         const int64_t chunk = n < kChunk ? n : kChunk;
-        hd_status r = ensure_records(scan, chunk, st);
+        if (r == HD_OK && in_place) r = ensure_records(scan, chunk, st);
         if (r != HD_OK) return r;
-        scan->inputs_on_host = true;
-        for (int64_t off = 0; off < n && r == HD_OK; off += chunk) {
+        scan->inputs_on_host = in_place;
+        for (int64_t off = 0; in_place && off < n && r == HD_OK; off += chunk) {
             const int64_t c = (n - off) < chunk ? (n - off) : chunk;
             const hd::Inputs in{src[0] + off, src[1] + off, src[2] + off,
                                 src[3] + off, src[4] + off, src[5] + off};
