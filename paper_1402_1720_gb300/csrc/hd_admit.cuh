@@ -71,16 +71,23 @@ __device__ __forceinline__ void reserve_and_write(const TilePlan &tp, const Reco
         if (path == 1) {
             int lo[3], hi[3];
             tiles(lo, hi);
-            const int off = (cls + 2 * type) * tp.ntiles;
-            for (int z = lo[2]; z <= hi[2]; ++z)
-                for (int y = lo[1]; y <= hi[1]; ++y)
-                    for (int x = lo[0]; x <= hi[0]; ++x)
-                        atomicAdd(&s_hist[off + x + tp.ntx * (y + tp.nty * z)], 1u);
+            uint32_t *const hist = s_hist + (cls + 2 * type) * tp.ntiles;
             // the record's pairs hold positions end - c .. end - 1 of the
             // block's list (all below its budget)
             const uint32_t code = static_cast<uint32_t>(i - h0) << kRecordTileBits;
-            const unsigned first = static_cast<unsigned>(end) - demand;
-            for (int j = 0; j < tcount; ++j) stage[first + j] = code | static_cast<uint32_t>(j);
+            uint32_t *const list = stage + (static_cast<unsigned>(end) - demand);
+            if (tp.ntx == 1 && tp.nty == 1) {  // whole planes: the tiles are consecutive
+                for (int j = 0; j < tcount; ++j) {
+                    atomicAdd(hist + lo[2] + j, 1u);
+                    list[j] = code | static_cast<uint32_t>(j);
+                }
+            } else {
+                for (int z = lo[2]; z <= hi[2]; ++z)
+                    for (int y = lo[1]; y <= hi[1]; ++y)
+                        for (int x = lo[0]; x <= hi[0]; ++x)
+                            atomicAdd(hist + x + tp.ntx * (y + tp.nty * z), 1u);
+                for (int j = 0; j < tcount; ++j) list[j] = code | static_cast<uint32_t>(j);
+            }
         }
 #pragma unroll
         for (int a = 0; a < 6; ++a) rec.g[a][i] = r[a];
