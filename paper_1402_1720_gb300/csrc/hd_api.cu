@@ -640,14 +640,9 @@ hd_status add_mapped(hd_scan *s, const float *const src[6], int64_t n, cudaStrea
     }
     r = ensure_staging(s, cap_all, st);
     if (r != HD_OK) return r == HD_ERR_NOMEM ? HD_OK : r;
-    // evenly spaced columns are one strided copy per part
-    const int64_t pitch = src[1] - src[0];
-    bool rows = pitch >= n && pitch < (int64_t(1) << 28);
-    for (int a = 1; a < 5; ++a) rows = rows && src[a + 1] - src[a] == pitch;
+    // a copy per column: even evenly spaced columns may lie in allocations of
+    // their own, which one strided copy must not span
     auto copy = [&](float *to, int64_t width, int64_t off, int64_t c) {
-        if (rows)
-            return cudaMemcpy2DAsync(to, sizeof(float) * width, src[0] + off, sizeof(float) * pitch,
-                                     sizeof(float) * c, 6, cudaMemcpyHostToDevice, s->up);
         cudaError_t e = cudaSuccess;
         for (int a = 0; a < 6 && e == cudaSuccess; ++a)
             e = cudaMemcpyAsync(to + a * width, src[a] + off, sizeof(float) * c,

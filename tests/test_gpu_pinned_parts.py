@@ -46,13 +46,15 @@ def _counts(hd, s):
 
 @pytest.mark.parametrize("n,how", [(LEAST, "thin"), (LEAST + 1, "thin"), (7_000_003, "thin"),
                                    (LEAST + 5, "thick"), (LEAST + 6, "distance")])
-@pytest.mark.parametrize("spaced", [True, False])
-def test_parts(hd, n, how, spaced):
+@pytest.mark.parametrize("columns", ["rows", "last apart", "all apart"])
+def test_parts(hd, n, how, columns):
     g = synth.Geometry(24, 20, 12, 1.0, 1.0, 2.0, 30.0)
     dev, host = _rows(n)
     cols = [host[k] for k in range(6)]
-    if not spaced:  # the last column elsewhere
+    if columns == "last apart":
         cols[5] = torch.empty(n, dtype=torch.float32, pin_memory=True).copy_(host[5])
+    if columns == "all apart":  # allocations of one size, which may lie evenly spaced
+        cols = [torch.empty(n, dtype=torch.float32, pin_memory=True).copy_(c) for c in cols]
     with hd.Scan(g) as a, hd.Scan(g) as b:
         for s in (a, b):
             if how == "thick":
