@@ -556,10 +556,7 @@ hd_status stage_global(hd_scan *s, int64_t n, cudaStream_t st)
 
 hd_status stage_reset(hd_scan *scan, cudaStream_t st)
 {
-    const size_t V = static_cast<size_t>(scan->V);
-    if (scan->N) HD_CUDA(cudaMemsetAsync(scan->N, 0, sizeof(uint32_t) * V, st));
-    if (scan->M) HD_CUDA(cudaMemsetAsync(scan->M, 0, sizeof(uint32_t) * V, st));
-    HD_CUDA(cudaMemsetAsync(scan->ctrl, 0, sizeof(hd::Ctrl), st));
+    HD_CUDA(hd::launch_reset(scan->N, scan->M, scan->V, scan->ctrl, scan->sm_count, st));
     return HD_OK;
 }
 

@@ -234,6 +234,37 @@ __global__ void __launch_bounds__(256) volume_sums_kernel(const uint32_t *__rest
 
 }  // namespace
 
+// Clears the counts of a new scan, N and M (either may be null; cudaMalloc's
+// alignment) and its counters, in one launch: three clearing copies were three
+// launches in turn.
+__global__ void __launch_bounds__(512) reset_kernel(uint32_t *N, uint32_t *M, int64_t V,
+                                                    unsigned *ctrl, int ctrl_words)
+{
+    after_previous();
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    if (blockIdx.x == 0 && static_cast<int>(threadIdx.x) < ctrl_words) ctrl[threadIdx.x] = 0u;
+    uint32_t *const vol[2] = {N, M};
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        if (vol[k] == nullptr) continue;
+        uint4 *v = reinterpret_cast<uint4 *>(vol[k]);
+        for (int64_t i = i0; i < V / 4; i += stride) v[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (i0 < (V & 3)) vol[k][(V & ~int64_t(3)) + i0] = 0u;
+    }
+}
+
+cudaError_t launch_reset(uint32_t *N, uint32_t *M, int64_t V, Ctrl *ctrl, int sm_count, cudaStream_t s)
+{
+    static_assert(sizeof(Ctrl) % 4 == 0 && sizeof(Ctrl) / 4 <= 512, "one block clears the counters");
+    int64_t blocks = (V / 4 + 511) / 512;
+    const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * 4;
+    if (blocks > cap) blocks = cap;
+    if (blocks < 1) blocks = 1;
+    return launch_chained(reset_kernel, static_cast<unsigned>(blocks), 512, 0, s, N, M, V,
+                          reinterpret_cast<unsigned *>(ctrl), static_cast<int>(sizeof(Ctrl) / 4));
+}
+
 cudaError_t launch_volume_sums(const uint32_t *N, const uint32_t *M, int64_t V,
                                unsigned long long *out, int sm_count, cudaStream_t s)
 {

@@ -285,6 +285,9 @@ struct DecideArgs {
     uint8_t *H1, *H2, *H3;
 };
 
+// A new scan: N and M (V words each, either null) and the counters cleared.
+cudaError_t launch_reset(uint32_t *N, uint32_t *M, int64_t V, Ctrl *ctrl, int sm_count, cudaStream_t s);
+
 cudaError_t launch_finalize(const DecideArgs &a, int sm_count, cudaStream_t s);
 
 // sum_v N(v) and sum_v M(v) (each 0 when its volume is null) into out[0],
