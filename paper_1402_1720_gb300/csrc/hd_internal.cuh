@@ -76,15 +76,29 @@ inline int64_t records_stride(int64_t n) { return (n + 3) & ~int64_t(3); }
 // [b per_block, min((b + 1) per_block, n)); per_block is a multiple of 4.
 constexpr int kIngestThreads = 256;
 constexpr int kIngestBlocksPerSm = 8;
+constexpr int kScatterBlocksPerSm = 2;  // resident
 struct ChunkSplit {
     int blocks;
     int64_t per_block;
 };
-inline ChunkSplit chunk_split(int64_t n, int sm_count)
+inline ChunkSplit chunk_split(int64_t n, int ntiles, int sm_count)
 {
     const int64_t units = (n + 3) / 4;  // groups of four histories
-    int64_t blocks = (units + kIngestThreads - 1) / kIngestThreads;
-    const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * kIngestBlocksPerSm;
+    // a block begins and ends with work per bucket: at least 1024 histories, and
+    // one for every two buckets; beyond one wave of the scatter in whole waves
+    int64_t least = kGroups * static_cast<int64_t>(ntiles) / 8;
+    if (least < 256) least = 256;
+    int64_t blocks = (units + least - 1) / least;
+    const int64_t sms = sm_count > 0 ? sm_count : 1;
+    const int64_t wave = sms * kScatterBlocksPerSm;
+    if (blocks > wave) blocks -= blocks % wave;
+    // but a small chunk is latency, and takes up to a wave of 256 histories each
+    // (60 chunks of 5064 histories: 2577 us in blocks of 1024, 2144 of 512, 1817
+    // of 256; fewer still exceed their pair budgets one by one)
+    int64_t fine = (units + 63) / 64;
+    if (fine > wave) fine = wave;
+    if (blocks < fine) blocks = fine;
+    const int64_t cap = sms * kIngestBlocksPerSm;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
     ChunkSplit c;
