@@ -470,7 +470,7 @@ cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, c
     ra.g = g;
     ra.R = 2 * q16_of(d0);
     ra.rec = rec;
-    const ChunkSplit sp = chunk_split(n, tp.ntiles, sm_count);
+    const ChunkSplit sp = chunk_split(n, sm_count, tp.ntiles);
     const size_t cols = kGroups * static_cast<size_t>(tp.ntiles);
     cudaError_t e = launch_chunk_begin(desc.ctrl, desc.buckets, tp.ntiles, st);
     if (e != cudaSuccess) return e;

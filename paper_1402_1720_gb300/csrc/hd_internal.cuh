@@ -81,7 +81,7 @@ struct ChunkSplit {
     int blocks;
     int64_t per_block;
 };
-inline ChunkSplit chunk_split(int64_t n, int ntiles, int sm_count)
+inline ChunkSplit chunk_split(int64_t n, int sm_count, int ntiles = 0)
 {
     const int64_t units = (n + 3) / 4;  // groups of four histories
     // a block begins and ends with work per bucket: at least 1024 histories, and

@@ -159,7 +159,7 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
                            cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    const ChunkSplit sp = chunk_split(n, tp.ntiles, sm_count);
+    const ChunkSplit sp = chunk_split(n, sm_count, tp.ntiles);
     const size_t smem = sizeof(uint32_t) * 3 * kGroups * static_cast<size_t>(tp.ntiles);
     return launch_chained(scatter_kernel, static_cast<unsigned>(sp.blocks), kScatterThreads, smem, s, tp,
                           rec, sp.per_block, buckets, block_base, block_pairs, ctrl, pairs);

@@ -288,7 +288,7 @@ cudaError_t launch_ingest(const Inputs &in, int64_t n, const GeomQ &g, const Cor
     const bool tiled = tp.ntiles > 0 && block_base && block_pairs && stage;
     TilePlan tpl = tp;
     if (!tiled) tpl.ntiles = 0;
-    const ChunkSplit sp = chunk_split(n, tpl.ntiles, sm_count);
+    const ChunkSplit sp = chunk_split(n, sm_count, tpl.ntiles);
     const size_t smem = sizeof(uint32_t) * kGroups * static_cast<size_t>(tpl.ntiles);
     uint32_t *bb = tiled ? block_base : nullptr;
     uint32_t *bp = tiled ? block_pairs : nullptr;

@@ -126,3 +126,11 @@ extern "C" int hx_events(const int32_t *seg, int dx, int dy, int dz, int thick, 
             }
     return n;
 }
+
+// The chunk split for a plan of ntiles tiles.
+extern "C" void hx_chunk_split(long long n, int sm_count, int ntiles, int *blocks, long long *per_block)
+{
+    const hd::ChunkSplit c = hd::chunk_split(n, sm_count, ntiles);
+    *blocks = c.blocks;
+    *per_block = c.per_block;
+}

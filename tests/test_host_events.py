@@ -109,3 +109,19 @@ def test_grid_coordinate_is_exact(hx, n, s):
                                                                        20000) * sq // 2])
     w = np.ascontiguousarray(w, dtype=np.int32)
     assert hx.hx_to_grid(n, ctypes.c_float(s), w.ctypes.data_as(I32P), ctypes.c_longlong(w.size)) == 0
+
+
+@pytest.mark.parametrize("ntiles", [0, 1, 33, 384, 2048])
+def test_chunk_split_with_tiles(hx, ntiles):
+    """The split of a plan with tiles covers [0, n) once, in multiples of four histories and at
+    most 8 blocks per SM."""
+    hx.hx_chunk_split.restype = None
+    blocks, per = ctypes.c_int(), ctypes.c_longlong()
+    rng = np.random.default_rng(ntiles)
+    ns = [1, 3, 4, 5, 255, 256, 257, 5064, 180000, 550000, 9000000, 1 << 25]
+    for sm in (1, 7, 152):
+        for n in ns + [int(x) for x in rng.integers(1, 1 << 25, 100)]:
+            hx.hx_chunk_split(ctypes.c_longlong(n), sm, ntiles, ctypes.byref(blocks), ctypes.byref(per))
+            b, p = blocks.value, per.value
+            assert p % 4 == 0 and p > 0 and 1 <= b <= 8 * sm, (n, sm, b, p)
+            assert b * p >= n and (b - 1) * p < n, (n, sm, b, p)
