@@ -182,8 +182,10 @@ HD_API hd_status hd_scan_reserve(hd_scan *scan, int64_t n, void *stream);
  * depends only on the multiset of histories.  on_device = 0 takes host
  * arrays: page-locked arrays mapped into the device's address space (as
  * cudaHostAlloc gives) are read in place by the first kernel over the host
- * link; other host memory is copied to a device staging buffer inside the
- * call.  Either way the arrays must stay unchanged until the work this call
+ * link, or, many of them, copied in parts beside the traversal (through a
+ * staging buffer of the scan, unless hd_scan_reserve covers the call or the
+ * stream is being captured); other host memory is copied to a device staging
+ * buffer inside the call.  Either way the arrays must stay unchanged until the work this call
  * queued on `stream` has completed.  n = 0 is a no-op.
  * HD_ERR_OVERFLOW if the scan would exceed 2^32 - 1 histories. */
 HD_API hd_status hd_scan_add_histories(hd_scan *scan, const float *angle_deg, const float *u_in,

@@ -151,6 +151,7 @@ struct hd_scan {
     int64_t staging_half = 0;
     // copies of page-locked inputs that run beside the chunks before (add_mapped)
     static constexpr int kSlots = 3;
+    int64_t reserved = 0;  // histories hd_scan_reserve made room for
     cudaStream_t up = nullptr;
     cudaEvent_t up_begin = nullptr, up_copied[kSlots] = {}, up_free[kSlots] = {};
     uint32_t *compact_blocks = nullptr;
@@ -597,7 +598,8 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
 // larger.  Head-sized scan: 9e6 histories 1951 us in place, 1665 in three parts,
 // 1567 in four; 4.5e6 1066, 953 and 1027; 2.7e6 711, 711 and 797.  taken stays
 // false when copying is not possible here (the stream is being captured, no
-// memory): the caller then reads in place.
+// memory, or an add that was reserved for and must not allocate): the caller
+// then reads in place.
 constexpr int64_t kOverlapLeast = int64_t(3) << 20;
 constexpr int64_t kManyParts = int64_t(6) << 20;
 constexpr int64_t kPartMost = int64_t(1) << 23;
@@ -627,14 +629,16 @@ hd_status add_mapped(hd_scan *s, const float *const src[6], int64_t n, cudaStrea
         left -= c;
         part = c + c / grow;
     }
-    hd_status r = ensure_records(s, most, st);
-    if (r != HD_OK) return r;
-    if (!ensure_upload(s)) return HD_OK;
     int64_t at[kSlots], cap_all = 0;
     for (int k = 0; k < kSlots; ++k) {
         at[k] = cap_all;
         cap_all += (size[k] + 3) & ~int64_t(3);
     }
+    // an add the user has reserved for neither allocates nor synchronises
+    if (n <= s->reserved && cap_all > s->staging_half) return HD_OK;
+    hd_status r = ensure_records(s, most, st);
+    if (r != HD_OK) return r;
+    if (!ensure_upload(s)) return HD_OK;
     r = ensure_staging(s, cap_all, st);
     if (r != HD_OK) return r == HD_ERR_NOMEM ? HD_OK : r;
     // a copy per column: even evenly spaced columns may lie in allocations of
@@ -906,7 +910,10 @@ hd_status hd_scan_reserve(hd_scan *scan, int64_t n, void *stream)
     if (n == 0) return HD_OK;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
-    return ensure_records(scan, n < kChunk ? n : kChunk, static_cast<cudaStream_t>(stream));
+    const hd_status r = ensure_records(scan, n < kChunk ? n : kChunk, static_cast<cudaStream_t>(stream));
+    // what is reserved must not grow in an add: see add_mapped
+    if (r == HD_OK && n > scan->reserved) scan->reserved = n;
+    return r;
 }
 
 hd_status hd_scan_add_histories(hd_scan *scan, const float *angle_deg, const float *u_in,

@@ -78,3 +78,24 @@ def test_parts(hd, n, how, columns):
             a.finalize()
             b.add(cols, st)  # the staging of the add before is used again
             b.finalize(st)
+
+
+def test_reserved_adds_allocate_nothing(hd):
+    """An add that was reserved for neither allocates nor changes its result."""
+    g = synth.Geometry(24, 20, 12, 1.0, 1.0, 2.0, 30.0)
+    n = LEAST + 7
+    dev, host = _rows(n)
+    with hd.Scan(g) as a, hd.Scan(g) as b:
+        a.add([dev[k] for k in range(6)])
+        a.finalize()
+        b.reserve(n)
+        b.add([dev[k][:8] for k in range(6)])
+        b.reset()
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        b.add([host[k] for k in range(6)])
+        b.finalize()
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+        for x, y in zip(_counts(hd, a), _counts(hd, b)):
+            assert np.array_equal(x, y)
