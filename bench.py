@@ -584,7 +584,10 @@ def run_rows(args):
             "nnz_per_s": nnz / (ms * 1e-3),
             "output": {"bytes_per_step": out_bytes,
                        "gbs": out_bytes / (ms * 1e-3) / 1e9, "hbm_peak_gbs": peaks["hbm_gbs"]},
-            "gpu_launches": 5 * args.steps, "clocks": clocks}
+            # pack, offset scan (3); per chunk of 2^22 histories set-up, counters, count
+            # and emit, and the set-up again when there are several
+            "gpu_launches": (4 + (-(-n // (1 << 22))) * (5 if n > 1 << 22 else 4)) * args.steps,
+            "clocks": clocks}
     print(json.dumps(line), flush=True)
     scan.close()
 
@@ -656,7 +659,7 @@ def run_binned(args):
                    "h2d_bytes_per_step": 24 * n, "d2h_bytes_per_step": int(out.numel())}
     peaks = _peaks()
     atomics = 7 * st["histories_binned"] + 2 * (st["histories_binned"] - st["histories_cut"])
-    l2_rate = hulld.hd_probe_atomics(hulld.HD_PROBE_L2_RANDOM)
+    smem_rate = hulld.hd_probe_atomics(hulld.HD_PROBE_SMEM_RANDOM)
     stats_atomics = 7 * st["histories_binned"]
     line = {"metric": "histories/s (SC with binning, data cuts and filter, as the paper ran it)",
             "value": n / (ms * 1e-3), "unit": UNIT, "n_gpus": 1, "steps": args.steps,
@@ -668,15 +671,18 @@ def run_binned(args):
             "phases_ms": {"statistics": t_stats, "cuts": t_cut, "carve_and_filter": t_fin},
             "atomic_rate": {"atomics_per_step": atomics,
                             "per_s": atomics / ((t_stats + t_cut) * 1e-3)},
-            "roofline": {"bound": "l2_atomic", "kernel": "binned_stats_kernel",
-                         "achieved": stats_atomics / (t_stats * 1e-3), "peak": l2_rate,
-                         "unit": "atomics/s", "frac": stats_atomics / (t_stats * 1e-3) / l2_rate,
+            # the bins of a gantry angle in shared memory: at least seven updates per
+            # history there (n, and the sums and low square words of three values)
+            "roofline": {"bound": "smem_atomic", "kernel": "binned_stats_tiles_kernel",
+                         "achieved": stats_atomics / (t_stats * 1e-3), "peak": smem_rate,
+                         "unit": "atomics/s", "frac": stats_atomics / (t_stats * 1e-3) / smem_rate,
                          "atomics_per_launch": stats_atomics,
-                         "peak_source": "hd_probe_atomics L2 random (measured in this run)"},
+                         "peak_source": "hd_probe_atomics shared-memory random (measured in this "
+                                        "run)"},
             "input": {"bytes_per_step": 2 * 24 * n,
                       "gbs": 2 * 24 * n / ((t_stats + t_cut) * 1e-3) / 1e9,
                       "hbm_peak_gbs": peaks["hbm_gbs"]},
-            "e2e": e2e, "gpu_launches": 5 * args.steps, "clocks": clocks}
+            "e2e": e2e, "gpu_launches": 4 * args.steps, "clocks": clocks}
     if not args.no_cpu_baseline:
         import oracle
         import time as _time
@@ -1117,7 +1123,7 @@ def run_large(args):
             "voxel_steps_per_scan": steps_per_scan,
             "voxel_steps_per_s": steps_per_scan / (ms * 1e-3),
             "smem_atomic_rate": smem_rate,
-            "gpu_launches": 6 * len(chunks) * args.steps, "clocks": clocks}
+            "gpu_launches": (5 * len(chunks) + 3) * args.steps, "clocks": clocks}
     print(json.dumps(line), flush=True)
 
 
@@ -1310,9 +1316,11 @@ def main():
         "voxel_steps_over_l2_random_ceiling": vsteps / probes["l2_random"],
         "runs_per_scan": runs,
         "voxels_per_run": steps_per_scan / runs if runs else None,
-        "trace_smem_atomics_per_s": 2.0 * runs / (trace_ms * 1e-3),
+        # one update per change of row and the two marks of a walk: one per run, and
+        # one per walk more (not counted here)
+        "trace_smem_atomics_per_s": runs / (trace_ms * 1e-3),
         "trace_smem_atomics_over_smem_random_ceiling":
-            2.0 * runs / (trace_ms * 1e-3) / probes["smem_random"]}
+            runs / (trace_ms * 1e-3) / probes["smem_random"]}
 
     # prepare = ingest + plan + scatter (everything before the traversal)
     phases = {"prepare_ms": prof["ms_ingest"] / args.steps, "trace_ms": trace_ms,

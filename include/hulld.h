@@ -167,7 +167,7 @@ HD_API hd_status hd_scan_destroy(hd_scan *scan);
  * new acquisition. */
 HD_API hd_status hd_scan_reset(hd_scan *scan, void *stream);
 
-/* Size the scan's per-chunk scratch (records, tile pairs, job table) for
+/* Size the scan's per-chunk scratch (records, tile pairs) for
  * calls of up to n histories now, so that later calls of that size allocate
  * nothing and never synchronise the stream to grow it.  Optional: the
  * scratch otherwise grows on demand.  May synchronise `stream`. */

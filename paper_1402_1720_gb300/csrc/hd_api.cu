@@ -121,7 +121,7 @@ struct hd_scan {
     uint32_t *mt = nullptr, *slope = nullptr;
     long long *index = nullptr;
     hd::Ctrl *ctrl = nullptr;
-    // scratch: traversal records, (record, tile) pairs, jobs, host staging
+    // scratch: traversal records, (record, tile) pairs, host staging
     hd::TilePlan tp{};
     hd_tuning tuning{1024, 12, 32767, 0};
     int trace_grid = 0;
