@@ -26,8 +26,9 @@ __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v)
 
 // Steepest drop per slice (or over the volume): max of the packed key
 // (S(v) << 32) | index, so the largest S wins and, among equal S, the
-// largest index, which is what the ">=" update of Alg. 3 leaves behind.
-__global__ void __launch_bounds__(256) sm_slope_kernel(const uint32_t *__restrict__ M, int nx,
+// largest index, which is what the ">=" update of Alg. 3 leaves behind.  (M is not
+// declared unaliased: a chained kernel's loads must not move above its wait.)
+__global__ void __launch_bounds__(256) sm_slope_kernel(const uint32_t *M, int nx,
                                                        int ny, int nz, int per_slice, int nbhd,
                                                        unsigned long long *slice_key)
 {
