@@ -1281,11 +1281,10 @@ def main():
     steps_per_scan = st["steps_miss"] + st["steps_hit"]
     value = ws * n / (ms * 1e-3)
 
-    # roofline of the dominant kernel (the traversal).  Its algorithmic work
-    # is one counter update per voxel-step (the oracle's exact sum |A_i|;
-    # one launch covers the whole scan), and the ceiling of a design that
-    # privatises the counts in shared memory is the random-address
-    # shared-memory atomic rate, measured here by the same process.
+    # roofline of the dominant kernel (the traversal).  Its unit of work is one
+    # shared-memory update per run of voxels (one launch covers the whole scan;
+    # the walks' marks, one more per walk, are not counted), and the ceiling the
+    # random-address shared-memory atomic rate, measured here by the same process.
     peaks = _peaks()
     trace_ms = prof["ms_trace"] / max(1, prof["trace_launches"])
     runs = st.get("runs", 0)
@@ -1297,12 +1296,13 @@ def main():
     vsteps = steps_per_scan / (trace_ms * 1e-3)
     traffic, traffic_note = _profiled_traffic()
     sms = torch.cuda.get_device_properties(local).multi_processor_count
-    roofline = {"bound": "smem_atomic", "achieved": vsteps, "peak": probes["smem_random"],
-                "unit": "atomics/s", "frac": vsteps / probes["smem_random"],
+    updates = runs / (trace_ms * 1e-3)
+    roofline = {"bound": "smem_atomic", "achieved": updates, "peak": probes["smem_random"],
+                "unit": "atomics/s", "frac": updates / probes["smem_random"],
                 "traffic": traffic, "traffic_source": traffic_note,
                 "kernel": "trace_tiles_kernel", "kernel_ms": trace_ms,
                 "voxel_steps_per_launch": steps_per_scan,
-                "work_per_unit": "one counter update per voxel-step (sum |A_i| of the scan)",
+                "work_per_unit": "one shared-memory update per run of voxels",
                 "peak_source": "hd_probe_atomics shared-memory random-address rate, measured "
                                "in this run (1024-thread blocks, xorshift addresses, best of 3)",
                 "sm_count": sms}
@@ -1316,11 +1316,9 @@ def main():
         "voxel_steps_over_l2_random_ceiling": vsteps / probes["l2_random"],
         "runs_per_scan": runs,
         "voxels_per_run": steps_per_scan / runs if runs else None,
-        # one update per change of row and the two marks of a walk: one per run, and
-        # one per walk more (not counted here)
-        "trace_smem_atomics_per_s": runs / (trace_ms * 1e-3),
-        "trace_smem_atomics_over_smem_random_ceiling":
-            runs / (trace_ms * 1e-3) / probes["smem_random"]}
+        "voxel_steps_over_smem_random_ceiling": vsteps / probes["smem_random"],
+        "trace_smem_atomics_per_s": updates,
+        "trace_smem_atomics_over_smem_random_ceiling": updates / probes["smem_random"]}
 
     # prepare = ingest + plan + scatter (everything before the traversal)
     phases = {"prepare_ms": prof["ms_ingest"] / args.steps, "trace_ms": trace_ms,
