@@ -266,6 +266,33 @@ cudaError_t launch_reset(uint32_t *N, uint32_t *M, int64_t V, Ctrl *ctrl, int sm
                           reinterpret_cast<unsigned *>(ctrl), static_cast<int>(sizeof(Ctrl) / 4));
 }
 
+// 16 bytes a thread and step where both addresses allow, else single bytes.
+__global__ void __launch_bounds__(256) copy_kernel(uint8_t *dst, const uint8_t *src, int64_t bytes)
+{
+    after_previous();
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    int64_t done = 0;
+    if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15u) == 0) {
+        const int64_t n = bytes / 16;
+        for (int64_t i = i0; i < n; i += stride)
+            reinterpret_cast<uint4 *>(dst)[i] = reinterpret_cast<const uint4 *>(src)[i];
+        done = 16 * n;
+    }
+    for (int64_t i = done + i0; i < bytes; i += stride) dst[i] = src[i];
+}
+
+cudaError_t launch_copy(void *dst, const void *src, size_t bytes, int sm_count, cudaStream_t s)
+{
+    int64_t blocks = static_cast<int64_t>((bytes / 16 + 255) / 256);
+    const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * 8;
+    if (blocks > cap) blocks = cap;
+    if (blocks < 1) blocks = 1;
+    return launch_chained(copy_kernel, static_cast<unsigned>(blocks), 256, 0, s,
+                          static_cast<uint8_t *>(dst), static_cast<const uint8_t *>(src),
+                          static_cast<int64_t>(bytes));
+}
+
 cudaError_t launch_volume_sums(const uint32_t *N, const uint32_t *M, int64_t V,
                                unsigned long long *out, int sm_count, cudaStream_t s)
 {

@@ -864,30 +864,6 @@ HD_HD bool run_begin(RunWalk &rw, const int32_t gi[3], const int32_t go[3], int 
     return true;
 }
 
-// Calls visit(v) for the voxels of the walk gi -> go over the whole grid in
-// path order: runs come in order, and a run is expanded in the direction
-// the major axis moves.
-template <class VisitT>
-HD_HD void walk_path(const int32_t r[6], int nx, int ny, int nz, VisitT &visit)
-{
-    const int32_t gi[3] = {r[0], r[1], r[2]};
-    const int32_t go[3] = {r[3], r[4], r[5]};
-    RunWalk w;
-    if (!run_begin(w, gi, go, nx, ny, nz)) return;
-    const bool ymaj = (w.flags >> 5) & 1;
-    const bool plus = w.flags & 1;
-    int row, lo, hi;
-    // a run's voxels are base + m stride: x-major rows are y + ny z (stride
-    // 1), y-major rows x + nx z (stride nx)
-    const int stride = ymaj ? nx : 1;
-    const int step = plus ? stride : -stride;
-    while (run_next(w, row, lo, hi)) {
-        const int base = ymaj ? row % nx + nx * ny * (row / nx) : nx * row;
-        int v = base + (plus ? lo : hi) * stride;
-        for (int k = hi - lo; k >= 0; --k, v += step) visit(static_cast<uint32_t>(v));
-    }
-}
-
 // -------------------------------------------------------------- path walk
 //
 // The whole-grid walk of one path as runs in path order, for segments with no
@@ -1395,13 +1371,6 @@ HD_HD int slab_lean(const int32_t gi[3], const int32_t go[3], int nx, int ny, Le
     const bool pm = (ymaj ? D[1] : D[0]) > 0, pc = (ymaj ? D[0] : D[1]) > 0;
     L.fl = (pm ? 1 : 0) | ((pc ? 1 : 0) << 1) | ((ymaj ? 1 : 0) << 2);
     return 1;
-}
-
-// A packed walk with no voxel.
-HD_HD void lean_pack_empty(uint32_t o[kLeanWords])
-{
-    for (int i = 0; i < kLeanWords; ++i) o[i] = 0;
-    o[5] = 8u << 16;
 }
 
 HD_HD void lean_unpack(const uint32_t o[kLeanWords], LeanWalk &L)

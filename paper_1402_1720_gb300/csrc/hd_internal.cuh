@@ -195,7 +195,9 @@ struct Inputs {
 
 // Launch of a kernel that begins with after_previous(): its blocks may come onto
 // the SMs, and do what needs none of the previous kernel's results, while that
-// one ends (the chain of a small chunk is mostly launches, ends and starts).
+// one ends (the chain of a small chunk is mostly launches, ends and starts).  Its
+// parameters are not declared unaliased where the previous kernel may write what
+// they point to: such a load could be moved above the wait.
 template <class... P, class... A>
 inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem,
                                   cudaStream_t s, const A &...args)
@@ -298,6 +300,9 @@ struct DecideArgs {
     long long *index;        // nz entries (SM)
     uint8_t *H1, *H2, *H3;
 };
+
+// bytes from src to dst, both on the device of s, by a chained kernel.
+cudaError_t launch_copy(void *dst, const void *src, size_t bytes, int sm_count, cudaStream_t s);
 
 // A new scan: N and M (V words each, either null) and the counters cleared.
 cudaError_t launch_reset(uint32_t *N, uint32_t *M, int64_t V, Ctrl *ctrl, int sm_count, cudaStream_t s);
