@@ -165,6 +165,31 @@ __device__ __forceinline__ bool keep_of(const BinQ &b, const unsigned long long 
     return keep;
 }
 
+// Clears 64-bit words: the bin table (16 bytes a thread and step: cudaMalloc's
+// alignment) and the counters.
+__global__ void __launch_bounds__(512) binned_clear_kernel(unsigned long long *acc, int64_t words,
+                                                           unsigned long long *ctr)
+{
+    after_previous();
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
+    for (int64_t i = i0; i < words / 2; i += stride)
+        reinterpret_cast<uint4 *>(acc)[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (i0 == 0 && (words & 1)) acc[words - 1] = 0ull;
+    if (i0 < kCtrWords) ctr[i0] = 0ull;
+}
+
+// Begins the image: nothing carved, its four counters cleared.
+__global__ void __launch_bounds__(512) binned_image_kernel(uint32_t *bits, int64_t words,
+                                                           unsigned long long *ctr)
+{
+    after_previous();
+    const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    for (int64_t i = i0; i < words; i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        bits[i] = 0xffffffffu;
+    if (i0 < 4) ctr[2 + i0] = 0ull;
+}
+
 // Histories i, i + stride, .. below end without a table, those of vertical bins
 // v0 .. v1 - 1: seven and two atomics each.  kAtOnce of them are in flight.
 template <int kAtOnce>
@@ -250,6 +275,7 @@ __device__ __forceinline__ unsigned cut_direct(const Inputs &in, int64_t i, int6
 __global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_stats_kernel(
     Inputs in, int64_t n, BinQ b, unsigned long long *acc, unsigned long long *ctr)
 {
+    after_previous();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     warp_add(stats_direct<1>(in, i, n, static_cast<int64_t>(gridDim.x) * blockDim.x, b, 0, b.n_v, acc),
              ctr + 0);
@@ -258,6 +284,7 @@ __global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_stats_ke
 __global__ void __launch_bounds__(kBinThreads, kPassBlocksPerSm) binned_cut_kernel(
     Inputs in, int64_t n, BinQ b, unsigned long long *acc, unsigned long long *ctr)
 {
+    after_previous();
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     warp_add(cut_direct<1>(in, i, n, static_cast<int64_t>(gridDim.x) * blockDim.x, b, 0, b.n_v, acc),
              ctr + 1);
@@ -335,6 +362,7 @@ __global__ void __launch_bounds__(kTileThreads) binned_stats_tiles_kernel(Inputs
     const int v0 = win * t.rows, v1 = min(b.n_v, v0 + t.rows);
     const int E = b.n_u * (v1 - v0);
     for (int e = threadIdx.x; e < kStatsWords * E; e += kTileThreads) s_tab[e] = 0u;
+    after_previous();
     unsigned long long binned = 0;
     TileAngle ang;
     auto flush = [&]() {
@@ -448,6 +476,7 @@ __global__ void __launch_bounds__(kTileThreads) binned_cut_tiles_kernel(Inputs i
     const int64_t i0 = n * seg / n_seg, i1 = n * (seg + 1) / n_seg;
     const int v0 = win * t.rows, v1 = min(b.n_v, v0 + t.rows);
     const int E = b.n_u * (v1 - v0);
+    after_previous();
     unsigned long long cut = 0;
     TileAngle ang;
     auto row_at = [&](int e) {
@@ -533,6 +562,7 @@ __global__ void __launch_bounds__(kBinThreads) binned_bins_kernel(const unsigned
                                                                   int64_t nb, long long miss_q8,
                                                                   unsigned long long *ctr)
 {
+    after_previous();
     unsigned long long used = 0, missed = 0;
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < nb;
@@ -614,6 +644,7 @@ __global__ void __launch_bounds__(kCarveThreads) binned_carve_kernel(
         s_cs[0] = c;
         s_cs[1] = sn;
     }
+    after_previous();
     const unsigned lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
     unsigned long long lines = 0, outside = 0, used = 0, missed = 0;
     for (int base = 0; base < b.n_u; base += kMaxLinesPerBlock) {
@@ -701,6 +732,7 @@ __global__ void __launch_bounds__(256) binned_filter_kernel(const uint32_t *bits
                                                             int ny, int r, int min_count,
                                                             uint8_t *mask, uint8_t *carved)
 {
+    after_previous();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -714,7 +746,7 @@ __global__ void __launch_bounds__(256) binned_filter_kernel(const uint32_t *bits
     for (int Y = max(y - r, 0); Y <= min(y + r, ny - 1); ++Y) {
         const uint32_t l = static_cast<uint32_t>(xl) + static_cast<uint32_t>(nx) * Y;
         const int w = static_cast<int>(l >> 5);
-        const uint32_t row = __funnelshift_r(__ldg(img + w), __ldg(img + min(w + 1, wps - 1)),
+        const uint32_t row = __funnelshift_r(img[w], img[min(w + 1, wps - 1)],
                                              l & 31u) & wmask;
         c += __popc(row);
         if (Y == y) own = row >> (x - xl);
@@ -862,6 +894,29 @@ hd_status check_inputs(const float *const *p, int k, bool &host)
     return HD_OK;
 }
 
+// Blocks of 512 threads for `items` of them, at most four per SM.
+unsigned blocks_of(const hd_binned *b, int64_t items)
+{
+    int64_t n = (items + 511) / 512;
+    const int64_t cap = 4 * int64_t(b->sm_count > 0 ? b->sm_count : 1);
+    if (n > cap) n = cap;
+    return static_cast<unsigned>(n < 1 ? 1 : n);
+}
+
+// To the caller's memory: on this device by a chained kernel up to 64 MB.
+cudaError_t copy_out(const hd_binned *b, void *dst, const void *src, size_t bytes,
+                     int32_t dst_on_device, cudaStream_t st)
+{
+    cudaPointerAttributes at{};
+    if (dst_on_device && bytes <= (size_t(64) << 20)) {
+        if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) cudaGetLastError();
+        else if (at.type == cudaMemoryTypeDevice && at.device == b->device)
+            return hd::launch_copy(dst, src, bytes, b->sm_count, st);
+    }
+    return cudaMemcpyAsync(dst, src, bytes,
+                           dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
+}
+
 // How a pass of n histories keeps an angle's bins in shared memory (words 32-bit
 // words each); n_win 0 when it does not: more than four windows (each reads every
 // history again), host inputs read twice, or too few histories to fill and empty
@@ -895,17 +950,14 @@ hd_status pass(hd_binned *b, const float *angle_deg, const float *u_in, const fl
     if (t.n_win > 0) {
         const unsigned blocks = static_cast<unsigned>(b->sm_count / t.n_win * t.n_win);
         const size_t smem = sizeof(uint32_t) * words * size_t(b->bq.n_u) * t.rows;
-        if (cut)
-            hd::binned_cut_tiles_kernel<<<blocks, hd::kTileThreads, smem, st>>>(in, n, b->bq, t,
-                                                                              b->acc, b->ctr);
-        else
-            hd::binned_stats_tiles_kernel<<<blocks, hd::kTileThreads, smem, st>>>(in, n, b->bq, t,
-                                                                                b->acc, b->ctr);
-    } else if (cut)
-        hd::binned_cut_kernel<<<grid, hd::kBinThreads, 0, st>>>(in, n, b->bq, b->acc, b->ctr);
-    else
-        hd::binned_stats_kernel<<<grid, hd::kBinThreads, 0, st>>>(in, n, b->bq, b->acc, b->ctr);
-    HB_CUDA(cudaGetLastError());
+        HB_CUDA(hd::launch_chained(cut ? hd::binned_cut_tiles_kernel : hd::binned_stats_tiles_kernel,
+                                   blocks, hd::kTileThreads, smem, st, in, n, b->bq, t, b->acc,
+                                   b->ctr));
+    } else {
+        HB_CUDA(hd::launch_chained(cut ? hd::binned_cut_kernel : hd::binned_stats_kernel,
+                                   static_cast<unsigned>(grid), hd::kBinThreads, 0, st, in, n, b->bq,
+                                   b->acc, b->ctr));
+    }
     return HD_OK;
 }
 
@@ -1093,8 +1145,9 @@ hd_status hd_binned_reset(hd_binned *b, void *stream)
     BinDevice g(b->device);
     if (!g.ok) return HD_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    HB_CUDA(cudaMemsetAsync(b->acc, 0, sizeof(unsigned long long) * hd::kAccWords * b->nb, st));
-    HB_CUDA(cudaMemsetAsync(b->ctr, 0, sizeof(unsigned long long) * hd::kCtrWords, st));
+    const int64_t words = hd::kAccWords * b->nb;
+    HB_CUDA(hd::launch_chained(hd::binned_clear_kernel, blocks_of(b, words / 2), 512, 0, st, b->acc,
+                               words, b->ctr));
     b->phase = 0;
     return HD_OK;
 }
@@ -1133,30 +1186,27 @@ hd_status hd_binned_finalize(hd_binned *b, void *stream)
     if (!g.ok) return HD_ERR_CUDA;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nz = b->geom.nz;
-    HB_CUDA(cudaMemsetAsync(b->ctr + 2, 0, sizeof(unsigned long long) * 4, st));
-    HB_CUDA(cudaMemsetAsync(b->bits, 0xff, sizeof(uint32_t) * size_t(b->wps) * nz, st));
+    const int64_t words = int64_t(b->wps) * nz;
+    HB_CUDA(hd::launch_chained(hd::binned_image_kernel, blocks_of(b, words), 512, 0, st, b->bits, words,
+                               b->ctr));
     if (b->count_apart)
-        hd::binned_bins_kernel<<<hd::grid_for(b->nb, b->sm_count), hd::kBinThreads, 0, st>>>(
-            b->acc, b->nb, b->bq.miss_q8, b->ctr);
-    HB_CUDA(cudaGetLastError());
+        HB_CUDA(hd::launch_chained(hd::binned_bins_kernel,
+                                   static_cast<unsigned>(hd::grid_for(b->nb, b->sm_count)),
+                                   hd::kBinThreads, 0, st, b->acc, b->nb, b->bq.miss_q8, b->ctr));
     const hd::LineTables t{b->tables, b->tables + b->bq.n_ang, b->tables + b->bq.n_ang + b->bq.n_u,
                            b->groups};
     const dim3 cg(static_cast<unsigned>(b->bq.n_ang), static_cast<unsigned>(b->n_groups));
     if (b->n_groups > 0) {
-        if (b->wps <= hd::kMaxSmemWords)
-            hd::binned_carve_kernel<true><<<cg, hd::kCarveThreads, sizeof(uint32_t) * b->wps, st>>>(
-                b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr);
-        else
-            hd::binned_carve_kernel<false><<<cg, hd::kCarveThreads, 0, st>>>(
-                b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr);
-        HB_CUDA(cudaGetLastError());
+        const bool shared = b->wps <= hd::kMaxSmemWords;
+        HB_CUDA(hd::launch_chained(shared ? hd::binned_carve_kernel<true> : hd::binned_carve_kernel<false>,
+                                   cg, hd::kCarveThreads, shared ? sizeof(uint32_t) * b->wps : 0, st,
+                                   b->acc, b->bq, b->gq, b->cordic, t, b->bits, b->wps, b->ctr));
     }
     const dim3 fb(32, 8);
     const dim3 fg(static_cast<unsigned>((b->geom.nx + 31) / 32),
                   static_cast<unsigned>((b->geom.ny + 7) / 8), static_cast<unsigned>(nz));
-    hd::binned_filter_kernel<<<fg, fb, 0, st>>>(b->bits, b->wps, b->geom.nx, b->geom.ny,
-                                                 b->bq.w / 2, b->bq.min_count, b->mask, b->carved);
-    HB_CUDA(cudaGetLastError());
+    HB_CUDA(hd::launch_chained(hd::binned_filter_kernel, fg, fb, 0, st, b->bits, b->wps, b->geom.nx,
+                               b->geom.ny, b->bq.w / 2, b->bq.min_count, b->mask, b->carved));
     b->phase = 2;
     return HD_OK;
 }
@@ -1181,9 +1231,8 @@ hd_status hd_binned_get_image(hd_binned *b, int32_t which, uint8_t *dst, int64_t
     if (b->phase != 2) return HD_ERR_STATE;
     BinDevice g(b->device);
     if (!g.ok) return HD_ERR_CUDA;
-    HB_CUDA(cudaMemcpyAsync(dst, which == HD_BINNED_HULL ? b->mask : b->carved, size_t(b->V),
-                            dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                            static_cast<cudaStream_t>(stream)));
+    HB_CUDA(copy_out(b, dst, which == HD_BINNED_HULL ? b->mask : b->carved, size_t(b->V),
+                     dst_on_device, static_cast<cudaStream_t>(stream)));
     return HD_OK;
 }
 
@@ -1193,9 +1242,8 @@ hd_status hd_binned_get_bins(hd_binned *b, int64_t *dst, int64_t n_bins, int32_t
     if (!b || !dst || n_bins < b->nb) return HD_ERR_ARG;
     BinDevice g(b->device);
     if (!g.ok) return HD_ERR_CUDA;
-    HB_CUDA(cudaMemcpyAsync(dst, b->acc, sizeof(int64_t) * hd::kAccWords * b->nb,
-                            dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
-                            static_cast<cudaStream_t>(stream)));
+    HB_CUDA(copy_out(b, dst, b->acc, sizeof(int64_t) * hd::kAccWords * b->nb, dst_on_device,
+                     static_cast<cudaStream_t>(stream)));
     return HD_OK;
 }
 
