@@ -95,8 +95,8 @@ __device__ __forceinline__ void general_pack(const int32_t gi[3], const int32_t 
 __device__ __forceinline__ uint32_t load_general(const Pairs &pairs, uint32_t pos, int32_t gi[3],
                                                  int32_t go[3])
 {
-    const uint4 a = __ldg(&pairs.v[2 * static_cast<size_t>(pos)]);
-    const uint4 b = __ldg(&pairs.v[2 * static_cast<size_t>(pos) + 1]);
+    const uint4 a = pairs.v[2 * static_cast<size_t>(pos)];
+    const uint4 b = pairs.v[2 * static_cast<size_t>(pos) + 1];
     gi[0] = static_cast<int32_t>(a.x);
     gi[1] = static_cast<int32_t>(a.y);
     gi[2] = static_cast<int32_t>(a.z);

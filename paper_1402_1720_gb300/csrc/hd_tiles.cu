@@ -116,7 +116,7 @@ __device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, N
     if (nw.walk) {
         nw.pos = t.first + static_cast<uint32_t>(k);
 #pragma unroll
-        for (int q = 0; q < kVec; ++q) nw.v[q] = __ldg(t.pairs + kVec * static_cast<size_t>(nw.pos) + q);
+        for (int q = 0; q < kVec; ++q) nw.v[q] = t.pairs[kVec * static_cast<size_t>(nw.pos) + q];
     }
 }
 
