@@ -1,4 +1,5 @@
 // C ABI of libhulld: scan objects, validation, memory and launch order.
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -132,6 +133,9 @@ struct hd_scan {
     hd::ScanDesc *desc_dev = nullptr;  // this scan's traversal descriptor
     hd::ScanDesc desc_host{};
     bool desc_dirty = true;
+    // names the scan's buffers, plan and parameters as they are now: no other scan
+    // of the process, and no earlier state of this one, has had this number
+    uint64_t plan = 0;
     // kGroups * ntiles bucket totals, then the ingest blocks' places in the
     // buckets (tile_count_words)
     uint32_t *tile_count = nullptr;
@@ -170,6 +174,15 @@ struct hd_scan {
 };
 
 namespace {
+
+// The scan's buffers or plan have changed (or are new): its descriptor is out of
+// date, and so is every captured graph that holds them.
+void renew_plan(hd_scan *s)
+{
+    static std::atomic<uint64_t> last{0};
+    s->plan = ++last;
+    s->desc_dirty = true;
+}
 
 cudaEvent_t take_event(hd_scan *s)
 {
@@ -263,6 +276,7 @@ hd_status ensure_records(hd_scan *s, int64_t n, cudaStream_t st)
 {
     if (n <= s->rec_cap) return HD_OK;
     HD_CUDA(cudaStreamSynchronize(st));
+    renew_plan(s);
     if (s->rec_buf) cudaFree(s->rec_buf);
     if (s->pair_buf) cudaFree(s->pair_buf);
     s->rec_buf = nullptr;
@@ -301,7 +315,6 @@ hd_status ensure_records(hd_scan *s, int64_t n, cudaStream_t st)
         return HD_ERR_NOMEM;
     }
     s->rec_cap = n;
-    s->desc_dirty = true;
     return HD_OK;
 }
 
@@ -869,6 +882,7 @@ hd_status hd_scan_create(const hd_geometry *geom, const hd_params *params, hd_sc
     if (m & HD_MSC) alloc(reinterpret_cast<void **>(&s->H2), V);
     alloc(reinterpret_cast<void **>(&s->bits_out), sizeof(uint32_t) * s->words);
     make_tile_plan(s);
+    renew_plan(s);
     if (hd::init_ingest() != cudaSuccess || hd::init_scatter() != cudaSuccess ||
         hd::init_euclid() != cudaSuccess)
         ok = false;
@@ -1293,7 +1307,7 @@ hd_status hd_scan_set_thick(hd_scan *scan, int32_t k)
     }
     scan->thick_k = k;
     scan->tp.thick = k;
-    scan->desc_dirty = true;
+    renew_plan(scan);
     if (k > 0) {
         scan->euclid_d0 = 0.0f;
         scan->euclid_pairs = 0;
@@ -1323,7 +1337,7 @@ hd_status hd_scan_set_thick_distance(hd_scan *scan, float d0_mm)
     }
     scan->euclid_pairs =
         d0_mm > 0.0f ? hd::euclid_pairs_per_record(&scan->geom, d0_mm, scan->tp) : 0;
-    scan->desc_dirty = true;
+    renew_plan(scan);
     return HD_OK;
 }
 
@@ -1340,6 +1354,7 @@ hd_status hd_scan_set_tuning(hd_scan *scan, const hd_tuning *t)
     if (!g.ok) return HD_ERR_CUDA;
     HD_CUDA(cudaDeviceSynchronize());
     // drop everything sized by the old plan; it regrows on the next add
+    renew_plan(scan);
     void *old[] = {scan->tile_count, scan->tile_cursor, scan->tile_events, scan->rec_buf,
                    scan->pair_buf};
     for (void *p : old)
@@ -1367,7 +1382,6 @@ hd_status hd_scan_set_tuning(hd_scan *scan, const hd_tuning *t)
         const int per_sm = hd::trace_tiles_occupancy(scan->tp.tile_words, scan->tp.threads);
         scan->trace_grid = per_sm > 0 ? per_sm * scan->sm_count : 0;
     }
-    scan->desc_dirty = true;
     return HD_OK;
 }
 
@@ -1688,6 +1702,7 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
         rounds[k].push_back(it);
     }
     // host-side preparation, outside any capture: buffers, limits, descriptors
+    // (all of it before the key is taken, so that the key names their final state)
     for (const auto &it : items) {
         hd_scan *s = it.scan;
         if (it.n > kChunk) return HD_ERR_RANGE;
@@ -1702,11 +1717,13 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
             if (it.scan == p.first) total += static_cast<uint64_t>(it.n);
         if (total > static_cast<uint64_t>(kMaxScanHistories)) return HD_ERR_OVERFLOW;
     }
+    // a graph holds the scans' buffers, plans and parameters by value: the scans
+    // enter the key by their plan's number (addresses can come again after a free)
     std::vector<uintptr_t> key;
     key.push_back(static_cast<uintptr_t>(flags));
     for (const auto &it : items) {
         key.push_back(static_cast<uintptr_t>(it.flags));
-        key.push_back(reinterpret_cast<uintptr_t>(it.scan));
+        key.push_back(static_cast<uintptr_t>(it.scan->plan));
         key.push_back(reinterpret_cast<uintptr_t>(it.in.angle));
         key.push_back(reinterpret_cast<uintptr_t>(it.in.u_in));
         key.push_back(reinterpret_cast<uintptr_t>(it.in.v_in));
@@ -1714,10 +1731,6 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
         key.push_back(reinterpret_cast<uintptr_t>(it.in.v_out));
         key.push_back(reinterpret_cast<uintptr_t>(it.in.wepl));
         key.push_back(static_cast<uintptr_t>(it.n));
-        key.push_back(reinterpret_cast<uintptr_t>(it.scan->desc_dev));
-        key.push_back(reinterpret_cast<uintptr_t>(it.scan->pair_buf));
-        key.push_back(reinterpret_cast<uintptr_t>(it.scan->rec_buf));
-        key.push_back(static_cast<uintptr_t>(it.scan->tp.threads));
     }
     // the legacy default stream cannot be captured: run directly there
     const bool graphable = batch->use_graph && rounds.size() == 1 && st != nullptr;
