@@ -342,7 +342,9 @@ HD_API hd_status hd_batch_add_item(hd_batch *batch, hd_scan *scan, const float *
 /* Run and then drop the queued items, stream-ordered on `stream`.
  * flags: HD_BATCH_RESET resets every scan of the batch first (as
  * hd_scan_reset); HD_BATCH_FINALIZE finalizes every scan afterwards (as
- * hd_scan_finalize).  May synchronise the stream when scan buffers grow. */
+ * hd_scan_finalize).  May synchronise the stream when scan buffers grow.
+ * HD_ERR_STATE, and nothing runs, when a queued scan has been set to thick rays
+ * since. */
 HD_API hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream);
 
 /* Enable (1, default) or disable (0) CUDA-graph capture and replay. */

@@ -1683,6 +1683,10 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
     auto items = batch->items;
     batch->items.clear();
     if (items.empty()) return HD_OK;
+    // a scan set to thick rays since its item was queued has other pairs and
+    // another layout of them than the thin paths run here
+    for (const auto &it : items)
+        if (it.scan->thick_k > 0 || it.scan->euclid_d0 > 0.0f) return HD_ERR_STATE;
     for (size_t i = 0; i < items.size(); ++i) {
         items[i].first = items[i].last = true;
         for (size_t j = 0; j < i; ++j)

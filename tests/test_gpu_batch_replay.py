@@ -90,3 +90,24 @@ def test_buffers_grown(hd, oracle_mod):
         _check(hd, s, oracle_mod.run(GRID, big))
         assert _run(hd, b, s, dev, st)
         _check(hd, s, ref)
+
+
+@pytest.mark.parametrize("graph", [True, False])
+@pytest.mark.parametrize("how", ["set_thick", "set_thick_distance"])
+def test_thick_rays_set_after_queueing(hd, oracle_mod, how, graph):
+    """Refused as at queueing; the scan and the batch work on."""
+    h, dev = _histories(2000)
+    ref, st = oracle_mod.run(GRID, h), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with hd.Batch() as b, hd.Scan(GRID) as s:
+        b.set_graph(graph)
+        for _ in range(2):
+            b.add(s, dev)
+            getattr(s, how)(2)
+            with pytest.raises(hd.HDError) as e:
+                b.run(hd.HD_BATCH_RESET | hd.HD_BATCH_FINALIZE, st)
+            assert e.value.status == hd.HD_ERR_STATE
+            getattr(s, how)(0)
+            _run(hd, b, s, dev, st)
+            _check(hd, s, ref)
+            s.reset()
