@@ -783,7 +783,7 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
     cudaEvent_t e1 = prof_begin(s, st);
     if (s->tp.ntiles > 0 && s->trace_grid > 0) {
         HD_CUDA(hd::launch_trace_tiles(s->desc_dev, 1, s->tp.tile_words, s->tp.threads,
-                                       s->trace_grid, st));
+                                       s->trace_grid, hd::kGroups * s->tp.ntiles, st));
         s->launches += 1;
         if (s->profiling) s->trace_launches += 1;
     }
@@ -1527,11 +1527,12 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
                       int grid, cudaStream_t st, int64_t *kernels)
 {
     const int n_items = static_cast<int>(round.size());
-    int max_words = 0;
+    int max_words = 0, buckets = 0;
     bool any_tiled = false;
     for (const auto &it : round) {
         if (it.scan->tp.ntiles > 0 && it.scan->trace_grid > 0) {
             any_tiled = true;
+            buckets += hd::kGroups * it.scan->tp.ntiles;
             if (it.scan->tp.tile_words > max_words) max_words = it.scan->tp.tile_words;
         }
     }
@@ -1574,7 +1575,7 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
     r = join();
     if (r != HD_OK) return r;
     if (any_tiled) {
-        HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, st));
+        HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, buckets, st));
         *kernels += 1;
     }
     HD_CUDA(hd::launch_trace_global_batch(b->descs_dev, n_items, upper, b->sm_count, st));

@@ -1689,6 +1689,102 @@ HD_HD int event_end(const EventCursor &c, int thick4)
     return e < c.endl ? e : c.endl;
 }
 
+// ------------------------------------------------------------ joined tiles
+//
+// Event walks of all four types in one tile: for tiles whose walks of a type
+// are too few to pay for a flush of their own.  One layout, x fastest in rows of
+// nx + 1 words and ny + 1 rows to a slice; the low half of a word holds the
+// difference counts of x-major runs along x, the high half those of y-major
+// runs along y, so that
+//   count(x, y) = sum_{x' <= x} low(x', y) + sum_{y' <= y} high(x, y').
+// An event then takes two updates: it ends its row's run past its major index
+// and begins the next row's there.  A walk adds at most one to a half of a word
+// and to a prefix sum of it, so both stay within the pairs of a job (32767).
+
+// How walks of one type lie in a joined tile (bytes from one index to the next,
+// the minor one's in the direction the walks go), and in their own layout.
+struct JoinedBox {
+    float rW;  // 1 / W
+    int major, minor, slice;
+    int16_t W, nminor;  // words per row and rows per slice of the own layout
+};
+
+HD_HD JoinedBox joined_box(int type, int dx, int dy)
+{
+    const bool ymaj = (type & 2) != 0;
+    JoinedBox b;
+    b.nminor = static_cast<int16_t>(ymaj ? dx : dy);
+    b.W = static_cast<int16_t>(tile_row_words(ymaj ? dy : dx, b.nminor));
+    b.rW = 1.0f / static_cast<float>(b.W);
+    const int row = 4 * (dx + 1);
+    b.major = ymaj ? row : 4;
+    b.minor = ymaj ? 4 : row;
+    if (type & 1) b.minor = -b.minor;
+    b.slice = row * (dy + 1);
+    return b;
+}
+
+// A walk in progress in a joined tile: an event at `addr` adds -v at addr + major
+// and v at addr + minor.
+struct JoinedCursor {
+    unsigned ad, Ru, rem;
+    int addr, step, left, endl;
+    int major, minor;
+    uint32_t v;
+};
+
+// Starts a packed event walk there; *first receives the address of its first
+// mark (v).  False when there is no walk.  The row of a word is a division by W
+// of a number below 2^16: (q + 1/2) / W is at least 1 / (2 W) from a whole
+// number, W <= 4098, its float error at most 2^-22 of it.
+HD_HD bool joined_start(const uint32_t o[kLeanWords], const JoinedBox &b, int base, JoinedCursor &c,
+                        int &first)
+{
+    c.ad = o[0];
+    c.Ru = o[1];
+    c.rem = o[2];
+    const bool walk = static_cast<int>(o[7]) >= 0;
+    c.left = walk ? static_cast<int>(o[7]) : 0;
+    const int f = static_cast<int>(o[6]) >> 2;
+    const int row = static_cast<int>((static_cast<float>(f) + 0.5f) * b.rW);
+    const int z = row < b.nminor ? 0 : row / b.nminor;
+    const int sgn = b.minor < 0 ? -1 : 1;  // rows per event
+    const int at = base + z * b.slice + (row - z * b.nminor) * sgn * b.minor;  // the first row's start
+    const int own = row * b.W;
+    first = at + (f - own) * b.major;
+    c.addr = at + ((static_cast<int>(o[4]) >> 2) - own) * b.major;
+    const int n = c.left * sgn;  // rows to the last one
+    c.endl = at + c.left * b.minor + ((static_cast<int>(o[5]) >> 2) - own - n * b.W) * b.major;
+    c.step = ((static_cast<int>(o[3]) >> 2) - sgn * b.W) * b.major + b.minor;
+    c.major = b.major;
+    c.minor = b.minor;
+    c.v = b.major == 4 ? 1u : 65536u;  // (a row has at least two words)
+    return walk;
+}
+
+// Moves past one event.
+HD_HD void joined_next(JoinedCursor &c)
+{
+    c.rem += c.Ru;
+    const bool carry = c.rem >= c.ad;
+    c.addr += c.step;
+    if (carry) {
+        c.rem -= c.ad;
+        c.addr += c.major;
+    }
+    --c.left;
+}
+
+// Address of the end mark (-v) once no event is left.
+HD_HD int joined_end(const JoinedCursor &c)
+{
+    const int e = c.addr + c.major;
+    return e < c.endl ? e : c.endl;
+}
+
+// The high half of a word, its low half being a signed count.
+HD_HD uint32_t joined_high(uint32_t w) { return (w + 0x8000u) >> 16; }
+
 // Packed run-walk state: 16 32-bit words, so a walk prepared by one kernel
 // can be resumed by another.  The row strides and the major size follow
 // from the box (nx, ny) and the flags.

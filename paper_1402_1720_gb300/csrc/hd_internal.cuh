@@ -183,7 +183,7 @@ constexpr int kMaxBatch = 64;  // scans per batched traversal launch
 // What the exact search of a row of Euclidean thick rays needs: the geometry,
 // R = 2 q16(d_0), and the chunk's records (world endpoints, mm * 2^16).
 struct RowsArgs {
-    static constexpr bool kRows = true;
+    static constexpr bool kRows = true, kCells = false;
     GeomQ g;
     long long R;
     Records rec;
@@ -257,9 +257,10 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
 
 // Traversal of the pairs of nscans scans (descs on the device) by `grid`
 // resident blocks.  tile_words is the largest tile of the scans; threads is
-// 256, 512, 768 or 1024.
+// 256, 512, 768 or 1024; buckets: kGroups ntiles of all scans together (0 for
+// dilated walks, whose buckets are never joined).
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
-                               int grid, cudaStream_t s);
+                               int grid, int buckets, cudaStream_t s);
 
 // The same over the pairs of Euclidean thick rays of one scan (hd_euclid.cu).
 cudaError_t launch_trace_rows(const ScanDesc *desc, int tile_words, int threads, int grid,

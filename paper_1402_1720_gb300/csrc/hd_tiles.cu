@@ -31,7 +31,11 @@ constexpr int kEventsPerStep = 8;  // events a traversal lane walks between refi
 
 // What the kernel of the thin and dilated walks needs besides the scans: nothing.
 struct NoRows {
-    static constexpr bool kRows = false;
+    static constexpr bool kRows = false, kCells = false;
+};
+// The same for launches that look for cells to join (see Cell).
+struct Cells {
+    static constexpr bool kRows = false, kCells = true;
 };
 
 // Shared-memory reduction (no value returned) at a shared-space byte address.
@@ -78,16 +82,37 @@ constexpr int kCols = 16;
 struct TilePart {
     const uint4 *pairs;  // the scan's pairs
     uint32_t first;      // the bucket's first one
-    int scan;
     int tile;    // tile id within its group
-    int group;   // bit 0 the class (missed: N, hit: M), bits 1-2 the walk type
     int count;   // the bucket's pairs
     int start;   // slots [start, end)
     int end;
     int words;   // of its tile
     int offset;  // of the tile in the block's shared memory, in words
     int slot0;   // slots of the group before this part's
+    int16_t scan;
+    int8_t group;   // bit 0 the class (missed: N, hit: M), bits 1-2 the walk type
+    int8_t form;    // kOwn, kJoined or kSame
+    JoinedBox box;  // unless kOwn
 };
+// A part's walks: in a tile of their type's layout; in a joined one; in the joined
+// one of the part before, which is flushed once for both.
+constexpr int8_t kOwn = 0, kJoined = 1, kSame = 2;
+
+struct TileBox {
+    int x0, y0, z0, dx, dy, dz;
+};
+
+__device__ __forceinline__ TileBox tile_box(const TilePlan &tp, int tile)
+{
+    TileBox b;
+    b.x0 = tile % tp.ntx * tp.tx;
+    b.y0 = (tile / tp.ntx) % tp.nty * tp.ty;
+    b.z0 = tile / (tp.ntx * tp.nty) * tp.tz;
+    b.dx = min(tp.tx, tp.nx - b.x0);
+    b.dy = min(tp.ty, tp.ny - b.y0);
+    b.dz = min(tp.tz, tp.nz - b.z0);
+    return b;
+}
 
 __device__ __forceinline__ int slot_rows(int count) { return (count + 32 * kCols - 1) / (32 * kCols); }
 
@@ -96,6 +121,7 @@ template <int kVec>
 struct NextWalk {
     uint4 v[kVec];
     int base;      // its tile's offset in bytes
+    int part;      // its part in the group
     uint32_t pos;  // the pair
     bool have;
     bool walk;  // false: a slot past its bucket's pairs
@@ -112,6 +138,7 @@ __device__ __forceinline__ void load_slot(const TilePart *parts, int n, int r, N
     const int v = p >> 5;
     const int k = 32 * ((v & (kCols - 1)) * slot_rows(t.count) + v / kCols) + (p & 31);
     nw.base = 4 * t.offset;
+    nw.part = j;
     nw.walk = k < t.count;
     if (nw.walk) {
         nw.pos = t.first + static_cast<uint32_t>(k);
@@ -140,7 +167,7 @@ __device__ __forceinline__ void first_walks(const TilePart *parts, int n, int to
 // events.  Out of line, so that nothing else in the kernel takes its registers.
 __device__ __noinline__ void walk_parts(uint32_t *tiles, int thick, const TilePart *parts, int n,
                                         int total, int refill, unsigned *s_next,
-                                        NextWalk<2> nw, const ScanDesc &, const NoRows &)
+                                        NextWalk<2> nw)
 {
     const unsigned lane = threadIdx.x & 31u;
     const int sbase = static_cast<int>(__cvta_generic_to_shared(tiles));
@@ -185,6 +212,74 @@ __device__ __noinline__ void walk_parts(uint32_t *tiles, int thick, const TilePa
     }
 }
 
+// event_step in a joined tile: the event's two updates.
+__device__ __forceinline__ void joined_step(JoinedCursor &c, int u, int cnt)
+{
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p, q;\n\t"
+        ".reg .b32 e, s, n;\n\t"
+        "setp.gt.s32 p, %3, %4;\n\t"
+        "add.s32 e, %0, %7;\n\t"
+        "add.s32 s, %0, %8;\n\t"
+        "neg.s32 n, %9;\n\t"
+        "@p red.shared.add.u32 [e], n;\n\t"
+        "@p red.shared.add.u32 [s], %9;\n\t"
+        "@p add.u32 %1, %1, %5;\n\t"
+        "setp.ge.and.u32 q, %1, %2, p;\n\t"
+        "@p add.s32 %0, %0, %6;\n\t"
+        "@q sub.u32 %1, %1, %2;\n\t"
+        "@q add.s32 %0, %0, %7;\n\t"
+        "}"
+        : "+r"(c.addr), "+r"(c.rem)
+        : "r"(c.ad), "r"(cnt), "r"(u), "r"(c.Ru), "r"(c.step), "r"(c.major), "r"(c.minor), "r"(c.v)
+        : "memory");
+}
+
+// walk_parts for joined tiles.
+__device__ __noinline__ void walk_joined(uint32_t *tiles, const TilePart *parts, int n, int total,
+                                         int refill, unsigned *s_next, NextWalk<2> nw)
+{
+    const unsigned lane = threadIdx.x & 31u;
+    const int sbase = static_cast<int>(__cvta_generic_to_shared(tiles));
+    JoinedCursor c{};
+    bool unmarked = false;  // the walk's end is still to be marked
+    for (;;) {
+        const unsigned idle = __ballot_sync(kFull, c.left == 0);
+        if (__popc(idle) >= refill) {
+            const unsigned want = __ballot_sync(kFull, c.left == 0 && nw.have);
+            if (c.left == 0) {
+                if (unmarked) smem_red_add(joined_end(c), 0u - c.v);
+                unmarked = false;
+                if (nw.have) {
+                    const uint32_t o[kLeanWords] = {nw.v[0].x, nw.v[0].y, nw.v[0].z, nw.v[0].w,
+                                                    nw.v[1].x, nw.v[1].y, nw.v[1].z, nw.v[1].w};
+                    int first = 0;
+                    if (nw.walk) unmarked = joined_start(o, parts[nw.part].box, sbase + nw.base, c, first);
+                    if (unmarked) smem_red_add(first, c.v);
+                    nw.have = false;
+                }
+            }
+            if (want != 0) {
+                unsigned base = 0;
+                if (lane == 0) base = atomicAdd(s_next, __popc(want));
+                base = __shfl_sync(kFull, base, 0);
+                if (want & (1u << lane)) {
+                    const unsigned r = base + __popc(want & ((1u << lane) - 1u));
+                    nw.have = r < static_cast<unsigned>(total);
+                    if (nw.have) load_slot(parts, n, static_cast<int>(r), nw);
+                }
+            } else if (idle == kFull) {
+                break;
+            }
+        }
+        const int cnt = min(c.left, kEventsPerStep);
+#pragma unroll
+        for (int u = 0; u < kEventsPerStep; ++u) joined_step(c, u, cnt);
+        c.left -= cnt;
+    }
+}
+
 // One row of a slice walk (slice_row): its interval's +1 and -1 in the row at
 // `at` (a byte address less 4 kWhole's bits, so that the whole_up form of an
 // index is added to it directly); nothing unless `on`.
@@ -212,7 +307,7 @@ constexpr int kRowsPerStep = 8;  // rows a lane takes between refill checks (4: 
 // one slice, one after the other, each a closed form of about 35 instructions
 // (slice_row) and two shared atomics.  What the closed form leaves open goes to
 // the scan's list, or is settled at once when that is full.
-__device__ __noinline__ void walk_parts(uint32_t *tiles, int, const TilePart *parts, int n, int total,
+__device__ __noinline__ void walk_parts(uint32_t *tiles, const TilePart *parts, int n, int total,
                                         int refill, unsigned *s_next, NextWalk<3> nw,
                                         const ScanDesc &d, const RowsArgs &ra)
 {
@@ -425,6 +520,74 @@ __device__ __noinline__ void flush_rows(uint32_t *tile, int dx, int dy, int dz, 
     }
 }
 
+// Flush of a joined tile.  A thread per column turns the high halves into their
+// sums along y (lanes along x); then a warp per row sums the low halves along x,
+// kPer words a lane at a time, and adds both to the volume, clearing the row.
+__device__ __noinline__ void flush_joined(uint32_t *tile, int dx, int dy, int dz, FlushTo to)
+{
+    constexpr int kPer = 7, kAhead = 8;
+    const int lane = static_cast<int>(threadIdx.x & 31u);
+    const int warp = static_cast<int>(threadIdx.x >> 5), nwarps = static_cast<int>(blockDim.x >> 5);
+    const int P = dx + 1, slice = P * (dy + 1);
+    for (int q = static_cast<int>(threadIdx.x); q < dx * dz; q += blockDim.x) {
+        const int z = dz == 1 ? 0 : q / dx;
+        uint32_t *col = tile + slice * z + q - z * dx;
+        uint32_t sum = 0u;
+        for (int y = 0; y < dy; y += kAhead, col += kAhead * P) {
+            uint32_t w[kAhead];
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) w[k] = y + k < dy ? col[k * P] : 0u;
+#pragma unroll
+            for (int k = 0; k < kAhead; ++k) {
+                sum += joined_high(w[k]);
+                if (y + k < dy) col[k * P] = (w[k] & 0xffffu) | (sum << 16);
+            }
+        }
+    }
+    __syncthreads();
+    for (int l = warp; l < dy * dz; l += nwarps) {
+        const int z = dz == 1 ? 0 : l / dy, y = l - z * dy;
+        uint32_t *row = tile + slice * z + P * y;
+        uint32_t *out = to.line(y, z);
+        uint32_t carry = 0u;
+        for (int m0 = 0; m0 < dx; m0 += 32 * kPer) {
+            const int b = m0 + lane * kPer;
+            uint32_t v[kPer], hi[kPer];
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) v[k] = b + k < dx ? row[b + k] : 0u;
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) hi[k] = v[k] >> 16;
+#pragma unroll
+            for (int k = 1; k < kPer; ++k) v[k] += v[k - 1];
+            uint32_t incl = v[kPer - 1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t t = __shfl_up_sync(kFull, incl, o);
+                if (lane >= o) incl += t;
+            }
+            const uint32_t before = incl - v[kPer - 1] + carry;
+            carry += __shfl_sync(kFull, incl, 31);
+#pragma unroll
+            for (int k = 0; k < kPer; ++k)
+                if (b + k < dx) row[b + k] = ((v[k] + before) & 0xffffu) + hi[k];
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < kPer; ++k) {
+                const int x = m0 + lane + 32 * k;
+                if (x < dx) {
+                    add_count(out + x, row[x]);
+                    row[x] = 0u;
+                }
+            }
+        }
+        if (lane == 0) row[dx] = 0u;
+    }
+    for (int q = static_cast<int>(threadIdx.x); q < P * dz; q += blockDim.x) {
+        const int z = dz == 1 ? 0 : q / P;
+        tile[slice * z + P * dy + q - z * P] = 0u;
+    }
+}
+
 // In-place inclusive prefix sum of a row of any length by a warp.
 __device__ __forceinline__ void prefix_row(uint32_t *row, int W)
 {
@@ -551,41 +714,85 @@ __device__ __forceinline__ unsigned long long flush_cost(int tile_words)
     return kPartCost + static_cast<unsigned long long>(kFlushCost) * static_cast<unsigned>(tile_words);
 }
 
-struct BucketCost {
-    unsigned long long cost;  // 0: no pairs
-    unsigned count;
+// A cell is one tile of one class with its four buckets, by walk type (bucket
+// (class + 2 type) ntiles + tile).  Each bucket with pairs is walked and flushed for
+// itself, or, joined, all of them into one tile that is flushed once.  An event
+// costs more there (two updates and a conversion of the walk) and so does the
+// flush (columns, then rows), but a cell of few walks in several directions
+// (histories of many angles, or in no order of angle, on many tiles) pays for
+// one flush instead of four.  400 x 400 x 128, 9e6 histories in no order: in 20
+// chunks 11.4 -> 6.7 ms (8.2 before walks were sorted by type), 2e5 of them in one
+// 769 -> 502 us (592); 236 x 236 x 60, 1e5 histories 168 -> 121 us.  Costs in event
+// units: kJoinedEvent quarters of one per event, kJoinedPair per walk, a quarter
+// more per flush.
+constexpr unsigned kJoinedEvent = 7, kJoinedPair = 16;
+
+// Launches of at most two buckets to a block do not look at it (launch_trace_tiles):
+// there the four flushes of a cell are spread over blocks that would have little
+// else to do, and a small scan waits for every instruction before its walks.
+struct Cell {
+    unsigned long long cost[4];  // of the parts made of each bucket (joined: cost[0], of all)
+    unsigned count[4];           // pairs
+    bool joined;
 };
 
-__device__ __forceinline__ BucketCost bucket_cost(const ScanDesc &d, int t, bool rows)
+// Pieces of 32 slots of a bucket.
+__device__ __forceinline__ int pieces_of(unsigned count) { return kCols * slot_rows(static_cast<int>(count)); }
+
+template <bool kRows>
+__device__ __forceinline__ unsigned long long bucket_cost(unsigned count, unsigned long long events,
+                                                          int tile_words)
 {
-    BucketCost b;
-    b.count = d.buckets.count[t];
-    b.cost = b.count == 0 ? 0ull
-                          : (rows ? 5ull : 1ull) * d.buckets.events[t] +
-                                static_cast<unsigned long long>(kPairCost) * b.count +
-                                flush_cost(d.tp.tile_words);
-    return b;
+    return count == 0 ? 0ull
+                      : (kRows ? 5ull : 1ull) * events + static_cast<unsigned long long>(kPairCost) * count +
+                            flush_cost(tile_words);
 }
 
-// Blocks of its own for a bucket, about two flushes' worth of work each.
-__device__ __forceinline__ unsigned long long own_blocks(const BucketCost &b, int tile_words)
+__device__ __forceinline__ Cell cell_of(const ScanDesc &d, int cell)
+{
+    const int step = 2 * d.tp.ntiles, words = d.tp.tile_words;
+    const unsigned long long flush = flush_cost(words);
+    unsigned long long e[4], events = 0, pairs = 0, split = 0;
+    Cell c;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        c.count[j] = d.buckets.count[cell + step * j];
+        e[j] = d.buckets.events[cell + step * j];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        c.cost[j] = bucket_cost<false>(c.count[j], e[j], words);
+        pairs += c.count[j];
+        events += e[j];
+        split += c.cost[j];
+    }
+    const unsigned long long all = kJoinedEvent * events / 4ull + kJoinedPair * pairs + flush + flush / 4ull;
+    c.joined = all < split;
+    if (c.joined) {
+        c.cost[0] = all;
+        c.cost[1] = c.cost[2] = c.cost[3] = 0ull;
+    }
+    return c;
+}
+
+// Blocks of its own for that cost, about two flushes' worth of work each.
+__device__ __forceinline__ unsigned long long own_blocks(unsigned long long cost, int tile_words)
 {
     const unsigned long long f = 2ull * flush_cost(tile_words);
-    return (b.cost + f - 1ull) / f;
+    return (cost + f - 1ull) / f;
 }
 
-// Where the boundary at cost x of the launch falls in a bucket whose cost
-// begins at p: pieces of 32 slots before it (0 .. all).  A part worth less
+// Where the boundary at cost x of the launch falls in `pieces` pieces of 32 slots
+// whose cost begins at p: slots before it (0 .. all).  A part worth less
 // than its own flush goes to the neighbour (tile_words -1: costs are blocks,
 // and a boundary stays where it falls).
-__device__ __forceinline__ int boundary_slot(const BucketCost &b, int tile_words,
+__device__ __forceinline__ int boundary_slot(unsigned long long cost, int pieces, int tile_words,
                                              unsigned long long p, unsigned long long x)
 {
-    const int pieces = kCols * slot_rows(static_cast<int>(b.count));
     const unsigned long long f = tile_words < 0 ? 0ull : flush_cost(tile_words);
     if (x <= p + f) return 0;
-    if (x + f >= p + b.cost) return 32 * pieces;
-    return 32 * static_cast<int>((x - p) * static_cast<unsigned long long>(pieces) / b.cost);
+    if (x + f >= p + cost) return 32 * pieces;
+    return 32 * static_cast<int>((x - p) * static_cast<unsigned long long>(pieces) / cost);
 }
 
 // Exclusive block scan of one 64-bit value per thread (blockDim.x <= 1024).
@@ -615,6 +822,99 @@ __device__ __forceinline__ unsigned long long block_excl_scan64(unsigned long lo
     return __shfl_sync(kFull, w - own, wid) + incl - v;
 }
 
+// The block's stretch [x0, x1) of the launch's costs, in blocks when `own`.
+struct Stretch {
+    unsigned long long before;  // of the thread's first bucket
+    unsigned long long x0, x1;
+    bool own;
+};
+
+__device__ __forceinline__ void fill_part(TilePart &j, const ScanDesc &d, int k, int t, int count,
+                                          int s0, int s1, int8_t form)
+{
+    j.pairs = d.pairs.v;
+    j.first = d.buckets.first[t];
+    j.scan = static_cast<int16_t>(k);
+    j.tile = t % d.tp.ntiles;
+    j.group = static_cast<int8_t>(t / d.tp.ntiles);
+    j.count = count;
+    j.start = s0;
+    j.end = s1;
+    j.words = d.tp.tile_words;
+    j.form = form;
+}
+
+// A pass over a thread's cells i0 .. i1 - 1 (of scan k those from s_first[k] / 4
+// on): the sum of their costs, or of the blocks of their own; or the parts in
+// the block's stretch, counted, or listed (the thread's first has number `rank`,
+// list begins at number j0): each at most job_size pairs, of a joined cell
+// in up to four, one to a bucket.
+enum CellPass { kCellCost, kCellBlocks, kCellCount, kCellList };
+
+template <CellPass pass>
+__device__ __forceinline__ unsigned long long cell_pass(const ScanDesc *__restrict__ descs,
+                                                        const int *s_first, int i0, int i1,
+                                                        const Stretch &st, unsigned long long rank,
+                                                        unsigned long long j0, TilePart *list)
+{
+    unsigned long long sum = 0, p = st.before;
+    int k = 0;
+    for (int i = i0; i < i1; ++i) {
+        while (4 * i >= s_first[k + 1]) ++k;
+        const ScanDesc &d = descs[k];
+        const int t0 = i - s_first[k] / 4, step = 2 * d.tp.ntiles, most = d.tp.job_size & ~31;
+        const Cell c = cell_of(d, t0);
+        auto take = [&](int u, int s0, int s1, bool same) {
+            if (pass == kCellList && rank >= j0 && rank < j0 + kPartList) {
+                TilePart &j = list[rank - j0];
+                fill_part(j, d, k, t0 + step * u, static_cast<int>(c.count[u]), s0, s1,
+                          !c.joined ? kOwn : (same ? kSame : kJoined));
+                if (c.joined) {
+                    const TileBox b = tile_box(d.tp, j.tile);
+                    j.box = joined_box(u, b.dx, b.dy);
+                }
+            }
+            ++rank;
+            ++sum;
+        };
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            if (pass == kCellCost || pass == kCellBlocks) {
+                sum += pass == kCellCost ? c.cost[j] : own_blocks(c.cost[j], d.tp.tile_words);
+                continue;
+            }
+            const unsigned long long cost = st.own ? own_blocks(c.cost[j], d.tp.tile_words) : c.cost[j];
+            if (cost != 0 && p < st.x1 && p + cost > st.x0) {
+                const int words = st.own ? -1 : d.tp.tile_words;
+                const int all = c.joined ? pieces_of(c.count[0]) + pieces_of(c.count[1]) +
+                                               pieces_of(c.count[2]) + pieces_of(c.count[3])
+                                         : pieces_of(c.count[j]);
+                const int s0 = st.x0 > p ? boundary_slot(cost, all, words, p, st.x0) : 0;
+                const int s1 = st.x1 < p + cost ? boundary_slot(cost, all, words, p, st.x1) : 32 * all;
+                for (int s = s0; s < s1; s += most) {
+                    const int e = min(s + most, s1);
+                    if (!c.joined) {
+                        take(j, s, e, false);
+                        continue;
+                    }
+                    int off = 0;
+                    bool same = false;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int len = 32 * pieces_of(c.count[u]);
+                        const int a = max(s - off, 0), z = min(e - off, len);
+                        if (a < z) take(u, a, z, same);
+                        same = same || a < z;
+                        off += len;
+                    }
+                }
+            }
+            p += cost;
+        }
+    }
+    return sum;
+}
+
 }  // namespace
 
 // The traversal: the buckets of all scans laid end to end by cost, one equal
@@ -629,7 +929,7 @@ template <int kThreads, class RowsT>
 __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     const ScanDesc *__restrict__ descs, int nscans, int smem_words, const RowsT ra)
 {
-    constexpr bool kRows = RowsT::kRows;
+    constexpr bool kRows = RowsT::kRows, kCells = RowsT::kCells;
     constexpr int kVec = kRows ? kSliceWords / 4 : kLeanWords / 4;
     extern __shared__ __align__(16) uint32_t tile[];
     __shared__ unsigned s_next[2];  // the next slot; entries of the block's list of open rows
@@ -655,84 +955,83 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     }
     __syncthreads();
     const int nb = s_first[nscans];
-    const int per = (nb + kThreads - 1) / kThreads;
-    const int i0 = min(static_cast<int>(threadIdx.x) * per, nb), i1 = min(i0 + per, nb);
-    // the thread's buckets i0 .. i1 - 1: visit(scan, bucket within it)
+    // the thread's buckets, or its cells (see cell_pass)
+    const int ni = kCells ? nb / 4 : nb, per = (ni + kThreads - 1) / kThreads;
+    const int i0 = min(static_cast<int>(threadIdx.x) * per, ni), i1 = min(i0 + per, ni);
+    // visit(scan, bucket within it, its cost and pairs)
     auto each = [&](auto visit) {
         int k = 0;
         for (int i = i0; i < i1; ++i) {
             while (i >= s_first[k + 1]) ++k;
-            visit(k, i - s_first[k]);
+            const ScanDesc &d = descs[k];
+            const int t = i - s_first[k];
+            const unsigned count = d.buckets.count[t];
+            visit(k, t, bucket_cost<kRows>(count, d.buckets.events[t], d.tp.tile_words), count);
         }
     };
+    Stretch st{};
     unsigned long long mine = 0, total;
-    each([&](int k, int t) { mine += bucket_cost(descs[k], t, kRows).cost; });
-    unsigned long long before = block_excl_scan64(mine, s_warp, total);
+    if constexpr (kCells) mine = cell_pass<kCellCost>(descs, s_first, i0, i1, st, 0, 0, nullptr);
+    else each([&](int, int, unsigned long long cost, unsigned) { mine += cost; });
+    st.before = block_excl_scan64(mine, s_warp, total);
     // the block's stretch: an equal share, but worth about two flushes
     unsigned long long blocks = total / (2ull * flush_cost(descs[0].tp.tile_words)) + 1ull;
-    unsigned long long share = 0, x0 = 0, x1 = 0;
+    unsigned long long share = 0;
     // a launch too small for that on every block: whole blocks for each bucket
     // instead, one for about two flushes' worth (a block of two small buckets
     // flushes twice, 11 000 cycles each)
-    bool own = blocks < gridDim.x;  // the same in all blocks and threads
-    if (own) {
+    st.own = blocks < gridDim.x;  // the same in all blocks and threads
+    if (st.own) {
         unsigned long long m = 0, all;
-        each([&](int k, int t) { m += own_blocks(bucket_cost(descs[k], t, kRows), descs[k].tp.tile_words); });
+        if constexpr (kCells) m = cell_pass<kCellBlocks>(descs, s_first, i0, i1, st, 0, 0, nullptr);
+        else
+            each([&](int k, int, unsigned long long cost, unsigned) {
+                m += own_blocks(cost, descs[k].tp.tile_words);
+            });
         const unsigned long long b = block_excl_scan64(m, s_warp, all);
-        own = all <= gridDim.x;
-        if (own) {
-            before = b;
+        st.own = all <= gridDim.x;
+        if (st.own) {
+            st.before = b;
             share = 1ull;
         }
     }
-    if (!own) {
+    if (!st.own) {
         if (blocks > gridDim.x) blocks = gridDim.x;
         share = (total + blocks - 1ull) / blocks;
     }
-    x0 = share * blockIdx.x;
-    x1 = x0 + share;
-    // the parts of the thread's buckets in that stretch, each at most
-    // job_size pairs (in whole pieces): count, then list
+    st.x0 = share * blockIdx.x;
+    st.x1 = st.x0 + share;
+    // the parts of the thread's buckets in that stretch, each at most job_size
+    // pairs (in whole pieces): count, then list
     auto parts = [&](auto take) {
-        unsigned long long p = before;
-        each([&](int k, int t) {
+        unsigned long long p = st.before;
+        each([&](int k, int t, unsigned long long cost, unsigned count) {
             const ScanDesc &d = descs[k];
-            BucketCost b = bucket_cost(d, t, kRows);
-            if (own) b.cost = own_blocks(b, d.tp.tile_words);
-            if (b.cost != 0 && p < x1 && p + b.cost > x0) {
-                const int words = own ? -1 : d.tp.tile_words;
-                const int s0 = x0 > p ? boundary_slot(b, words, p, x0) : 0;
-                const int s1 = x1 < p + b.cost ? boundary_slot(b, words, p, x1)
-                                               : 32 * kCols * slot_rows(static_cast<int>(b.count));
+            if (st.own) cost = own_blocks(cost, d.tp.tile_words);
+            if (cost != 0 && p < st.x1 && p + cost > st.x0) {
+                const int words = st.own ? -1 : d.tp.tile_words, all = pieces_of(count);
+                const int s0 = st.x0 > p ? boundary_slot(cost, all, words, p, st.x0) : 0;
+                const int s1 = st.x1 < p + cost ? boundary_slot(cost, all, words, p, st.x1) : 32 * all;
                 const int most = d.tp.job_size & ~31;
-                for (int s = s0; s < s1; s += most)
-                    take(k, t, static_cast<int>(b.count), s, min(s + most, s1));
+                for (int s = s0; s < s1; s += most) take(k, t, static_cast<int>(count), s, min(s + most, s1));
             }
-            p += b.cost;
+            p += cost;
         });
     };
     unsigned long long nmine = 0, nparts;
-    parts([&](int, int, int, int, int) { ++nmine; });
+    if constexpr (kCells) nmine = cell_pass<kCellCount>(descs, s_first, i0, i1, st, 0, 0, nullptr);
+    else parts([&](int, int, int, int, int) { ++nmine; });
     const unsigned long long rank0 = block_excl_scan64(nmine, s_warp, nparts);
     for (unsigned long long j0 = 0; j0 < nparts; j0 += kPartList) {
         if (nmine != 0) {
             unsigned long long r = rank0;
-            parts([&](int k, int t, int count, int s0, int s1) {
-                if (r >= j0 && r < j0 + kPartList) {
-                    TilePart &j = s_parts[r - j0];
-                    const ScanDesc &d = descs[k];
-                    j.pairs = d.pairs.v;
-                    j.first = d.buckets.first[t];
-                    j.scan = k;
-                    j.tile = t % d.tp.ntiles;
-                    j.group = t / d.tp.ntiles;
-                    j.count = count;
-                    j.start = s0;
-                    j.end = s1;
-                    j.words = d.tp.tile_words;
-                }
-                ++r;
-            });
+            if constexpr (kCells) cell_pass<kCellList>(descs, s_first, i0, i1, st, r, j0, s_parts);
+            else
+                parts([&](int k, int t, int count, int s0, int s1) {
+                    if (r >= j0 && r < j0 + kPartList)
+                        fill_part(s_parts[r - j0], descs[k], k, t, count, s0, s1, kOwn);
+                    ++r;
+                });
         }
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -741,15 +1040,24 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
             s_group[0] = 0;
             for (int q = 0; q < here; ++q) {
                 TilePart &j = s_parts[q];
-                if (q > s_group[g] && words + j.words > smem_words) {
-                    s_slots[g] = slots;
+                const int form = kCells ? j.form : kOwn;
+                j.slot0 = slots;
+                slots += j.end - j.start;
+                if (form == kSame && q > 0) {
+                    j.offset = s_parts[q - 1].offset;
+                    continue;
+                }
+                // (the first part of a list begins a tile in any case)
+                if (form == kSame) j.form = kJoined;
+                if (q > s_group[g] && (words + j.words > smem_words ||
+                                       (kCells && (form == kOwn) != (s_parts[q - 1].form == kOwn)))) {
+                    s_slots[g] = j.slot0;
                     s_group[++g] = q;
-                    words = slots = 0;
+                    slots -= j.slot0;
+                    j.slot0 = words = 0;
                 }
                 j.offset = words;
-                j.slot0 = slots;
                 words += j.words;
-                slots += j.end - j.start;
             }
             s_slots[g] = slots;
             s_group[++g] = here;
@@ -764,22 +1072,34 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
             if (threadIdx.x == 0) s_next[0] = blockDim.x;
             __syncthreads();
             const TilePlan &tp0 = descs[s_parts[q0].scan].tp;
-            walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, s_next, nw,
-                       descs[s_parts[q0].scan], ra);
+            bool joined = false;
+            if constexpr (kCells) {
+                joined = s_parts[q0].form != kOwn;
+                if (joined) walk_joined(tile, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, s_next, nw);
+            }
+            if constexpr (kRows)
+                walk_parts(tile, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, s_next, nw,
+                           descs[s_parts[q0].scan], ra);
+            else if (!joined)
+                walk_parts(tile, tp0.thick, s_parts + q0, q1 - q0, s_slots[g], tp0.refill, s_next, nw);
             if (g + 1 < ngroups)
                 first_walks(s_parts + q1, s_group[g + 2] - q1, s_slots[g + 1], nw);
             __syncthreads();
             for (int q = q0; q < q1; ++q) {
                 const TilePart &j = s_parts[q];
+                if (kCells && j.form == kSame) continue;
                 const ScanDesc &d = descs[j.scan];
                 const TilePlan &tp = d.tp;
-                const int tix = j.tile % tp.ntx;
-                const int tiy = (j.tile / tp.ntx) % tp.nty;
-                const int tiz = j.tile / (tp.ntx * tp.nty);
-                const int bx = tix * tp.tx, by = tiy * tp.ty, bz = tiz * tp.tz;
-                flush_tile<kRows>(tile + j.offset, min(tp.tx, tp.nx - bx), min(tp.ty, tp.ny - by),
-                           min(tp.tz, tp.nz - bz), j.group >> 1, tp.thick,
-                           (j.group & 1) == 0 ? d.N : d.M, tp.nx, tp.ny, bx, by, bz);
+                const TileBox b = tile_box(tp, j.tile);
+                uint32_t *const vol = (j.group & 1) == 0 ? d.N : d.M;
+                if (kCells && joined)
+                    flush_joined(tile + j.offset, b.dx, b.dy, b.dz,
+                                 FlushTo{vol + b.x0 + static_cast<long long>(tp.nx) *
+                                                          (b.y0 + static_cast<long long>(tp.ny) * b.z0),
+                                         tp.nx, tp.ny});
+                else
+                    flush_tile<kRows>(tile + j.offset, b.dx, b.dy, b.dz, j.group >> 1, tp.thick, vol,
+                                      tp.nx, tp.ny, b.x0, b.y0, b.z0);
             }
         }
         __syncthreads();
@@ -790,6 +1110,8 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         walk_fallback_lists(descs, nscans);
     }
 }
+
+static_assert(sizeof(TilePart) <= 64, "the block's lists leave room for the largest tile");
 
 // Shared memory of a launch whose largest tile has this many words: room for
 // up to eight tiles.
@@ -810,6 +1132,9 @@ int occupancy_of(int smem_words)
     // allow the largest tile once, so launches (also inside graph capture)
     // need no attribute change
     if (cudaFuncSetAttribute(trace_tiles_kernel<kThreads, NoRows>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
         cudaFuncSetAttribute(trace_tiles_kernel<rows_threads(kThreads), RowsArgs>,
@@ -866,8 +1191,9 @@ static cudaError_t launch_trace(const ScanDesc *descs, int nscans, int tile_word
 }
 
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
-                               int grid, cudaStream_t s)
+                               int grid, int buckets, cudaStream_t s)
 {
+    if (buckets > 2 * grid) return launch_trace(descs, nscans, tile_words, threads, grid, Cells{}, s);
     return launch_trace(descs, nscans, tile_words, threads, grid, NoRows{}, s);
 }
 
