@@ -191,7 +191,9 @@ __global__ void __launch_bounds__(512) binned_image_kernel(uint32_t *bits, int64
 }
 
 // Histories i, i + stride, .. below end without a table, those of vertical bins
-// v0 .. v1 - 1: seven and two atomics each.  kAtOnce of them are in flight.
+// v0 .. v1 - 1: seven and two atomics each.  kAtOnce of them are in flight.  (Plain
+// loads here and below: these kernels come right behind the caller's work, which
+// may still write the histories while they start.)
 template <int kAtOnce>
 __device__ __forceinline__ void load_histories(const Inputs &in, int64_t i, int64_t end,
                                                int64_t stride, float h[kAtOnce][6])
@@ -201,12 +203,12 @@ __device__ __forceinline__ void load_histories(const Inputs &in, int64_t i, int6
         const int64_t j = i + k * stride;
         h[k][0] = 2097152.0f;  // not binned
         if (j < end) {
-            h[k][0] = __ldg(in.angle + j);
-            h[k][1] = __ldg(in.u_in + j);
-            h[k][2] = __ldg(in.v_in + j);
-            h[k][3] = __ldg(in.u_out + j);
-            h[k][4] = __ldg(in.v_out + j);
-            h[k][5] = __ldg(in.wepl + j);
+            h[k][0] = in.angle[j];
+            h[k][1] = in.u_in[j];
+            h[k][2] = in.v_in[j];
+            h[k][3] = in.u_out[j];
+            h[k][4] = in.v_out[j];
+            h[k][5] = in.wepl[j];
         }
     }
 }
@@ -345,9 +347,9 @@ __device__ __forceinline__ void load_chunk(const Inputs &in, int64_t c0, int64_t
                                            float h[kTileUnroll][6], float s[3])
 {
     if (c0 >= i1) return;
-    s[0] = __ldg(in.angle + c0);
-    s[1] = __ldg(in.angle + min(c0 + kTileChunk / 2, i1 - 1));
-    s[2] = __ldg(in.angle + min(c0 + kTileChunk, i1) - 1);
+    s[0] = in.angle[c0];
+    s[1] = in.angle[min(c0 + kTileChunk / 2, i1 - 1)];
+    s[2] = in.angle[min(c0 + kTileChunk, i1) - 1];
     load_histories<kTileUnroll>(in, c0 + threadIdx.x, i1, kTileThreads, h);
 }
 
