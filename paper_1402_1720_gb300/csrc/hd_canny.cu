@@ -153,11 +153,12 @@ __global__ void __launch_bounds__(kSliceThreads) canny_slice_kernel(
     const long long mmax = block_max(mloc, s_red);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int words = ny * rw;
+    const hd::WordRows row_of(rw);
     for (int k0 = warp; k0 < words; k0 += 8 * nwarps) {  // a ballot per word, eight loads in flight
         long long a[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int k = k0 + i * nwarps, y = k / rw, x = (k - y * rw) * 32 + lane;
+            const int k = k0 + i * nwarps, y = row_of(k), x = (k - y * rw) * 32 + lane;
             a[i] = k < words && x < nx ? mg[static_cast<int64_t>(y) * nx + x] : 0;
         }
 #pragma unroll
@@ -180,7 +181,7 @@ __global__ void __launch_bounds__(kSliceThreads) canny_slice_kernel(
     if (threadIdx.x == 0) s_n = 0;
     __syncthreads();
     for (int k = threadIdx.x; k < words; k += blockDim.x) {
-        const int y = k / rw, x0 = (k - y * rw) * 32;
+        const int y = row_of(k), x0 = (k - y * rw) * 32;
         for (uint32_t bits = E[k]; bits != 0; bits &= bits - 1u) {
             const int slot = atomicAdd(&s_n, 1);
             if (slot < kListCap) L[slot] = m[static_cast<int64_t>(y) * nx + x0 + __ffs(bits) - 1];
@@ -216,7 +217,7 @@ __global__ void __launch_bounds__(kSliceThreads) canny_slice_kernel(
             }
         } else {
             for (int k = threadIdx.x; k < words; k += blockDim.x) {
-                const int y = k / rw, x0 = (k - y * rw) * 32;
+                const int y = row_of(k), x0 = (k - y * rw) * 32;
                 for (uint32_t bits = E[k]; bits != 0; bits &= bits - 1u) {
                     const uint32_t v = m[static_cast<int64_t>(y) * nx + x0 + __ffs(bits) - 1];
                     if ((v & above) == prefix) atomicAdd(&s_hist[(v >> b) & 255u], 1);

@@ -87,12 +87,13 @@ __global__ void __launch_bounds__(kDiagThreads) fill_kernel(const uint8_t *mask,
     const uint8_t *m = mask + static_cast<int64_t>(z) * plane;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int words = ny * rw;
+    const hd::WordRows row_of(rw);
     // mask bits, a warp per word (coalesced bytes, one ballot)
     for (int k0 = warp; k0 < words; k0 += 8 * nwarps) {  // eight loads in flight
         uint8_t v[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const int k = k0 + i * nwarps, y = k / rw, x = (k - y * rw) * 32 + lane;
+            const int k = k0 + i * nwarps, y = row_of(k), x = (k - y * rw) * 32 + lane;
             v[i] = k < words && x < nx ? m[static_cast<int64_t>(y) * nx + x] : 0;
         }
 #pragma unroll
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(kDiagThreads) fill_kernel(const uint8_t *mask,
     __syncthreads();
     // seeds: the mask voxels on the slice border
     for (int k = threadIdx.x; k < words; k += blockDim.x) {
-        const int y = k / rw, w = k - y * rw;
+        const int y = row_of(k), w = k - y * rw;
         uint32_t seed = 0;
         if (y == 0 || y == ny - 1) {
             seed = 0xffffffffu;
@@ -120,7 +121,7 @@ __global__ void __launch_bounds__(kDiagThreads) fill_kernel(const uint8_t *mask,
     // enclosed = mask, not exterior
     uint8_t *o = out + static_cast<int64_t>(z) * plane;
     for (int k = warp; k < words; k += nwarps) {
-        const int y = k / rw, x = (k - y * rw) * 32 + lane;
+        const int y = row_of(k), x = (k - y * rw) * 32 + lane;
         if (x < nx)
             o[static_cast<int64_t>(y) * nx + x] =
                 static_cast<uint8_t>(((M[k] & ~E[k]) >> lane) & 1u);
