@@ -382,25 +382,6 @@ void free_upload(hd_scan *s)
         if (e) cudaEventDestroy(e);
 }
 
-// A volume of the scan to the caller's memory: on this device by a chained kernel
-// up to kCopyKernel (a copy of the copy engine's kind takes about 4 us more: the
-// five of a small scan 78 -> 65 us of the whole, those of a batch of 12 scans 2379
-// -> 2261; at 20 to 80 MB a volume no difference).
-constexpr size_t kCopyKernel = size_t(64) << 20;
-
-cudaError_t copy_out(const hd_scan *s, void *dst, const void *src, size_t bytes, int32_t dst_on_device,
-                     cudaStream_t st)
-{
-    cudaPointerAttributes at{};
-    if (dst_on_device && bytes <= kCopyKernel) {
-        if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) cudaGetLastError();
-        else if (at.type == cudaMemoryTypeDevice && at.device == s->device)
-            return hd::launch_copy(dst, src, bytes, s->sm_count, st);
-    }
-    return cudaMemcpyAsync(dst, src, bytes,
-                           dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
-}
-
 // The records of a chunk of n histories: seven arrays of n slots and the
 // global path's list, each starting on a 16-byte boundary.
 hd::Records records_of(const hd_scan *s, int64_t n)
@@ -1149,7 +1130,7 @@ hd_status hd_scan_get_mask(hd_scan *scan, int32_t method, int32_t layout, void *
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (layout == HD_MASK_U8) {
-        HD_CUDA(copy_out(scan, dst, src, need, dst_on_device, st));
+        HD_CUDA(hd::copy_out(dst, src, need, dst_on_device, scan->device, scan->sm_count, st));
     } else {
         uint32_t *bits = dst_on_device ? static_cast<uint32_t *>(dst) : scan->bits_out;
         HD_CUDA(hd::launch_pack_bits(src, scan->V, bits, st));
@@ -1170,8 +1151,8 @@ hd_status hd_scan_get_counts(hd_scan *scan, int32_t method, uint32_t *dst, int64
     if (n < scan->V) return HD_ERR_ARG;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
-    HD_CUDA(copy_out(scan, dst, src, sizeof(uint32_t) * static_cast<size_t>(scan->V), dst_on_device,
-                     static_cast<cudaStream_t>(stream)));
+    HD_CUDA(hd::copy_out(dst, src, sizeof(uint32_t) * static_cast<size_t>(scan->V), dst_on_device,
+                         scan->device, scan->sm_count, static_cast<cudaStream_t>(stream)));
     return HD_OK;
 }
 

@@ -905,20 +905,6 @@ unsigned blocks_of(const hd_binned *b, int64_t items)
     return static_cast<unsigned>(n < 1 ? 1 : n);
 }
 
-// To the caller's memory: on this device by a chained kernel up to 64 MB.
-cudaError_t copy_out(const hd_binned *b, void *dst, const void *src, size_t bytes,
-                     int32_t dst_on_device, cudaStream_t st)
-{
-    cudaPointerAttributes at{};
-    if (dst_on_device && bytes <= (size_t(64) << 20)) {
-        if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) cudaGetLastError();
-        else if (at.type == cudaMemoryTypeDevice && at.device == b->device)
-            return hd::launch_copy(dst, src, bytes, b->sm_count, st);
-    }
-    return cudaMemcpyAsync(dst, src, bytes,
-                           dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st);
-}
-
 // How a pass of n histories keeps an angle's bins in shared memory (words 32-bit
 // words each); n_win 0 when it does not: more than four windows (each reads every
 // history again), too few histories to fill and empty a block's table, or host
@@ -1235,8 +1221,8 @@ hd_status hd_binned_get_image(hd_binned *b, int32_t which, uint8_t *dst, int64_t
     if (b->phase != 2) return HD_ERR_STATE;
     BinDevice g(b->device);
     if (!g.ok) return HD_ERR_CUDA;
-    HB_CUDA(copy_out(b, dst, which == HD_BINNED_HULL ? b->mask : b->carved, size_t(b->V),
-                     dst_on_device, static_cast<cudaStream_t>(stream)));
+    HB_CUDA(hd::copy_out(dst, which == HD_BINNED_HULL ? b->mask : b->carved, size_t(b->V), dst_on_device,
+                         b->device, b->sm_count, static_cast<cudaStream_t>(stream)));
     return HD_OK;
 }
 
@@ -1246,8 +1232,8 @@ hd_status hd_binned_get_bins(hd_binned *b, int64_t *dst, int64_t n_bins, int32_t
     if (!b || !dst || n_bins < b->nb) return HD_ERR_ARG;
     BinDevice g(b->device);
     if (!g.ok) return HD_ERR_CUDA;
-    HB_CUDA(copy_out(b, dst, b->acc, sizeof(int64_t) * hd::kAccWords * b->nb, dst_on_device,
-                     static_cast<cudaStream_t>(stream)));
+    HB_CUDA(hd::copy_out(dst, b->acc, sizeof(int64_t) * hd::kAccWords * b->nb, dst_on_device, b->device,
+                         b->sm_count, static_cast<cudaStream_t>(stream)));
     return HD_OK;
 }
 

@@ -282,15 +282,25 @@ __global__ void __launch_bounds__(256) copy_kernel(uint8_t *dst, const uint8_t *
     for (int64_t i = done + i0; i < bytes; i += stride) dst[i] = src[i];
 }
 
-cudaError_t launch_copy(void *dst, const void *src, size_t bytes, int sm_count, cudaStream_t s)
+cudaError_t copy_out(void *dst, const void *src, size_t bytes, int32_t dst_on_device, int device,
+                     int sm_count, cudaStream_t s)
 {
-    int64_t blocks = static_cast<int64_t>((bytes / 16 + 255) / 256);
-    const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * 8;
-    if (blocks > cap) blocks = cap;
-    if (blocks < 1) blocks = 1;
-    return launch_chained(copy_kernel, static_cast<unsigned>(blocks), 256, 0, s,
-                          static_cast<uint8_t *>(dst), static_cast<const uint8_t *>(src),
-                          static_cast<int64_t>(bytes));
+    cudaPointerAttributes at{};
+    if (dst_on_device && copy_by_kernel(dst, src, bytes)) {
+        if (cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+            cudaGetLastError();
+        } else if (at.type == cudaMemoryTypeDevice && at.device == device) {
+            int64_t blocks = static_cast<int64_t>((bytes / 16 + 255) / 256);
+            const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * 8;
+            if (blocks > cap) blocks = cap;
+            if (blocks < 1) blocks = 1;
+            return launch_chained(copy_kernel, static_cast<unsigned>(blocks), 256, 0, s,
+                                  static_cast<uint8_t *>(dst), static_cast<const uint8_t *>(src),
+                                  static_cast<int64_t>(bytes));
+        }
+    }
+    return cudaMemcpyAsync(dst, src, bytes,
+                           dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, s);
 }
 
 cudaError_t launch_volume_sums(const uint32_t *N, const uint32_t *M, int64_t V,
