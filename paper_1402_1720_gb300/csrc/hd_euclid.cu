@@ -239,6 +239,12 @@ __device__ __forceinline__ void euclid_tiles(const TilePlan &tp, int klo, int kh
     hi[2] = khi;
 }
 
+// The strips along y of a record's tiles, as its status word holds them in place of
+// its last slice (euclid_setup_kernel names the tiles from there: computed twice, in
+// float, the two kernels' strips would have to agree to the bit).
+__device__ __forceinline__ int strips_code(int lo, int hi) { return lo | ((hi - lo + 1) << 4); }
+static_assert(kOpenStrips <= 16 && (kOpenStrips << 4 | (kOpenStrips - 1)) < 4096, "12 bits");
+
 // Classification and records of a chunk (see ingest_kernel): world endpoints
 // at the histories' slots, the walk type 2 for rows along y.
 __global__ void __launch_bounds__(kIngestThreads, 4) euclid_ingest_kernel(
@@ -303,14 +309,15 @@ __global__ void __launch_bounds__(kIngestThreads, 4) euclid_ingest_kernel(
                 }
             }
         }
-        int c = 0;
+        int c = 0, strips = 0;
         if (ok) {
             int lo[3], hi[3];
             euclid_tiles(tp, klo, khi, ylo, yhi, lo, hi);
             c = (hi[1] - lo[1] + 1) * (hi[2] - lo[2] + 1);
+            strips = strips_code(lo[1], hi[1]);
         }
         reserve_and_write(tp, rec, ctrl, s_hist, &s_demand, budget, h0, i, h1, list, cls, type, ok,
-                          closed && c <= tp.max_tiles ? c : -1, klo, khi, w6,
+                          closed && c <= tp.max_tiles ? c : -1, klo, strips, w6,
                           [&](int lo[3], int hi[3]) { euclid_tiles(tp, klo, khi, ylo, yhi, lo, hi); });
     }
     const unsigned sums[5] = {nc.n_in, nc.n_miss, nc.n_hit, nc.n_none, nc.n_reject};
@@ -351,15 +358,8 @@ __global__ void __launch_bounds__(kSetupThreads, 2) euclid_setup_kernel(
         const int klo = status_zlo(stw);
         int y = 0, k = klo + j;
         if (tp.nty > 1) {
-            long long W[6];
-#pragma unroll
-            for (int a = 0; a < 6; ++a) W[a] = w[a];
-            int kl, kh, ylo, yhi, lo[3], hi[3];
-            bool closed;
-            euclid_range(ra.g, W, ra.R, kl, kh, ylo, yhi, closed);
-            euclid_tiles(tp, kl, kh, ylo, yhi, lo, hi);
-            const int ey = hi[1] - lo[1] + 1;
-            y = lo[1] + j % ey;
+            const int strips = status_zhi(stw), ey = strips >> 4;
+            y = (strips & 15) + j % ey;
             k = klo + j / ey;
         }
         const int t = status_group(stw) * tp.ntiles + y + tp.nty * k;
