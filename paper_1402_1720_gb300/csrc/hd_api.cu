@@ -1068,20 +1068,21 @@ hd_status hd_scan_system_rows(hd_scan *scan, int32_t method, const float *angle_
             return HD_ERR_NOMEM;
         }
     }
-    const int64_t chunk = n < hd::kRowsChunk ? n : hd::kRowsChunk;
-    if (chunk > scan->rows_walks_cap) {
+    if ((n < hd::kRowsChunk ? n : hd::kRowsChunk) > scan->rows_walks_cap) {
         HD_CUDA(cudaStreamSynchronize(st));
         if (scan->rows_walks) cudaFree(scan->rows_walks);
         scan->rows_walks = nullptr;
-        scan->rows_walks_cap = 0;
         // the walks, then the passes' counters
-        if (cudaMalloc(&scan->rows_walks, sizeof(uint32_t) * hd::kPathWords *
-                                              static_cast<size_t>(chunk) + 64) != cudaSuccess) {
+        scan->rows_walks_cap = hd::rows_walks_room(n, [&](int64_t walks) {
+            const size_t bytes = sizeof(uint32_t) * hd::kPathWords * static_cast<size_t>(walks) + 64;
+            if (cudaMalloc(&scan->rows_walks, bytes) == cudaSuccess) return true;
             cudaGetLastError();
-            return HD_ERR_NOMEM;
-        }
-        scan->rows_walks_cap = chunk;
+            scan->rows_walks = nullptr;
+            return false;
+        });
+        if (scan->rows_walks_cap == 0) return HD_ERR_NOMEM;
     }
+    const int64_t chunk = n < scan->rows_walks_cap ? n : scan->rows_walks_cap;
     HD_CUDA(hd::launch_pack_bits(hull, scan->V, scan->rows_bits, st));
     unsigned *counters = scan->rows_walks + hd::kPathWords * scan->rows_walks_cap;
     auto setup = [&](int64_t off, int64_t c) {

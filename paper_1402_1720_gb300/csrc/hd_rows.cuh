@@ -13,6 +13,21 @@
 namespace hd {
 
 constexpr int64_t kRowsChunk = int64_t(1) << 22;  // 268 MB of walks
+constexpr int64_t kRowsLeast = int64_t(1) << 10;  // 64 KB
+
+// Walks to allocate for calls of n histories: a chunk's when there is room, else
+// half as many, and so on (more chunks, each set up once more for the second pass).
+// try_alloc(walks) allocates; 0 when not even kRowsLeast of them fit.
+template <class TryAlloc>
+int64_t rows_walks_room(int64_t n, TryAlloc try_alloc)
+{
+    int64_t walks = n < kRowsChunk ? n : kRowsChunk;
+    while (!try_alloc(walks)) {
+        if (walks <= kRowsLeast) return 0;
+        walks = walks / 2 > kRowsLeast ? walks / 2 : kRowsLeast;
+    }
+    return walks;
+}
 
 int64_t rows_hull_words(int64_t V);
 cudaError_t launch_rows_setup(const Inputs &in, int64_t n, const GeomQ &g, const Cordic &cd,
