@@ -561,6 +561,7 @@ def run_rows(args):
         for _ in range(args.warmup):
             step()
         torch.cuda.synchronize()
+        launches = scan.profile()["kernel_launches"]
         sampler = ClockSampler(local)
         sampler.start()
         e0 = torch.cuda.Event(enable_timing=True)
@@ -571,6 +572,7 @@ def run_rows(args):
         e1.record(stream)
         torch.cuda.synchronize()
         clocks = sampler.stop()
+    launches = scan.profile()["kernel_launches"] - launches
     ms = e0.elapsed_time(e1) / args.steps
     peaks = _peaks()
     out_bytes = 4.0 * nnz + 8.0 * (n + 1)
@@ -584,10 +586,7 @@ def run_rows(args):
             "nnz_per_s": nnz / (ms * 1e-3),
             "output": {"bytes_per_step": out_bytes,
                        "gbs": out_bytes / (ms * 1e-3) / 1e9, "hbm_peak_gbs": peaks["hbm_gbs"]},
-            # pack, offset scan (3); per chunk of 2^22 histories set-up, counters, count
-            # and emit, and the set-up again when there are several
-            "gpu_launches": (4 + (-(-n // (1 << 22))) * (5 if n > 1 << 22 else 4)) * args.steps,
-            "clocks": clocks}
+            "gpu_launches": launches, "clocks": clocks}
     print(json.dumps(line), flush=True)
     scan.close()
 
@@ -661,6 +660,12 @@ def run_binned(args):
     atomics = 7 * st["histories_binned"] + 2 * (st["histories_binned"] - st["histories_cut"])
     smem_rate = hulld.hd_probe_atomics(hulld.HD_PROBE_SMEM_RANDOM)
     stats_atomics = 7 * st["histories_binned"]
+    # enough histories for every SM's table of an angle's bins, else atomics in L2
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
+    tiled = n >= 2 * sms * b.params.n_u * b.params.n_v
+    stats_kernel = ("smem_atomic", "binned_stats_tiles_kernel", smem_rate, "shared-memory") if tiled \
+        else ("l2_atomic", "binned_stats_kernel",
+              hulld.hd_probe_atomics(hulld.HD_PROBE_L2_RANDOM), "L2")
     line = {"metric": "histories/s (SC with binning, data cuts and filter, as the paper ran it)",
             "value": n / (ms * 1e-3), "unit": UNIT, "n_gpus": 1, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True,
@@ -673,16 +678,18 @@ def run_binned(args):
                             "per_s": atomics / ((t_stats + t_cut) * 1e-3)},
             # the bins of a gantry angle in shared memory: at least seven updates per
             # history there (n, and the sums and low square words of three values)
-            "roofline": {"bound": "smem_atomic", "kernel": "binned_stats_tiles_kernel",
-                         "achieved": stats_atomics / (t_stats * 1e-3), "peak": smem_rate,
-                         "unit": "atomics/s", "frac": stats_atomics / (t_stats * 1e-3) / smem_rate,
+            "roofline": {"bound": stats_kernel[0], "kernel": stats_kernel[1],
+                         "achieved": stats_atomics / (t_stats * 1e-3), "peak": stats_kernel[2],
+                         "unit": "atomics/s",
+                         "frac": stats_atomics / (t_stats * 1e-3) / stats_kernel[2],
                          "atomics_per_launch": stats_atomics,
-                         "peak_source": "hd_probe_atomics shared-memory random (measured in this "
+                         "peak_source": f"hd_probe_atomics {stats_kernel[3]} random (measured in this "
                                         "run)"},
             "input": {"bytes_per_step": 2 * 24 * n,
                       "gbs": 2 * 24 * n / ((t_stats + t_cut) * 1e-3) / 1e9,
                       "hbm_peak_gbs": peaks["hbm_gbs"]},
-            "e2e": e2e, "gpu_launches": 4 * args.steps, "clocks": clocks}
+            # clearing, statistics, cuts, the image's start, carving, filter
+            "e2e": e2e, "gpu_launches": 6 * args.steps, "clocks": clocks}
     if not args.no_cpu_baseline:
         import oracle
         import time as _time
@@ -761,6 +768,7 @@ def run_thick(args):
         for _ in range(args.warmup):
             scan_step()
         torch.cuda.synchronize()
+        launches = scan.profile()["kernel_launches"]
         sampler = ClockSampler(local)
         sampler.start()
         f0 = torch.cuda.Event(enable_timing=True)
@@ -771,6 +779,7 @@ def run_thick(args):
         f1.record(stream)
         torch.cuda.synchronize()
         clocks_scan = sampler.stop()
+    launches = scan.profile()["kernel_launches"] - launches
     ms_scan = f0.elapsed_time(f1) / args.steps
     scan_stats = scan.stats()
     scan.close()
@@ -796,7 +805,7 @@ def run_thick(args):
                                         "peak_source": "hd_probe_atomics L2 random "
                                                        "(measured in this run)",
                                         "hbm_peak_gbs": peaks["hbm_gbs"]}},
-            "gpu_launches": 12 * args.steps, "clocks": clocks_scan,
+            "gpu_launches": launches, "clocks": clocks_scan,
             "clocks_standalone": clocks}
     if not args.no_cpu_baseline:
         import oracle
@@ -873,7 +882,9 @@ def run_euclid(args):
         for _ in range(args.warmup):
             scan_step()
         torch.cuda.synchronize()
+        launches = scan.profile()["kernel_launches"]
         ms_scan = timed(scan_step, args.steps)
+        launches = scan.profile()["kernel_launches"] - launches
     scan.close()
     line = {"metric": f"histories/s (SC+MSC+SM on Euclidean thick rays, d_0 = {d0:g} mm)",
             "value": n / (ms_scan * 1e-3), "unit": UNIT, "n_gpus": 1, "steps": args.steps,
@@ -889,7 +900,7 @@ def run_euclid(args):
                            "thick_voxels_per_s": voxels / (ms * 1e-3),
                            "rows_per_s": n_rows / (ms * 1e-3), "rows_per_step": n_rows,
                            "voxels_per_row": voxels / n_rows if n_rows else None},
-            "gpu_launches": 4 * args.steps, "clocks": clocks}
+            "gpu_launches": launches, "clocks": clocks}
     if not args.no_cpu_baseline:
         import oracle
         import time as _time
@@ -1099,6 +1110,7 @@ def run_large(args):
         for _ in range(args.warmup):
             step()
         torch.cuda.synchronize()
+        launches = s.profile()["kernel_launches"]
         sampler = ClockSampler(local)
         sampler.start()
         e0 = torch.cuda.Event(enable_timing=True)
@@ -1109,6 +1121,7 @@ def run_large(args):
         e1.record(stream)
         torch.cuda.synchronize()
         clocks = sampler.stop()
+        launches = s.profile()["kernel_launches"] - launches
         st = s.stats()
     ms = e0.elapsed_time(e1) / args.steps
     steps_per_scan = (st["steps_miss"] + st["steps_hit"])
@@ -1123,7 +1136,7 @@ def run_large(args):
             "voxel_steps_per_scan": steps_per_scan,
             "voxel_steps_per_s": steps_per_scan / (ms * 1e-3),
             "smem_atomic_rate": smem_rate,
-            "gpu_launches": (5 * len(chunks) + 3) * args.steps, "clocks": clocks}
+            "gpu_launches": launches, "clocks": clocks}
     print(json.dumps(line), flush=True)
 
 

@@ -130,7 +130,7 @@ typedef struct {
  * CUDA-event time on the scan's stream of each phase, summed over calls,
  * and the number of kernels the library launched (always counted). */
 typedef struct {
-    int64_t kernel_launches;  /* kernels launched by this scan since create */
+    int64_t kernel_launches;  /* kernels launched by calls on this scan since create */
     int64_t trace_launches;   /* traversal kernel launches (profiled window) */
     double ms_ingest;         /* classification, geometry, bucketing by tile */
     double ms_trace;          /* voxel traversal and accumulation (shared-memory tiles) */

@@ -175,6 +175,14 @@ struct hd_scan {
 
 namespace {
 
+// Adds the kernels launched while it lives to a count.
+struct CountLaunches {
+    int64_t &to;
+    const int64_t from = hd::kernels_launched();
+    explicit CountLaunches(int64_t &t) : to(t) {}
+    ~CountLaunches() { to += hd::kernels_launched() - from; }
+};
+
 // The scan's buffers or plan have changed (or are new): its descriptor is out of
 // date, and so is every captured graph that holds them.
 void renew_plan(hd_scan *s)
@@ -550,11 +558,9 @@ hd_status stage_prepare(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_
                               s->tile_count, tp.ntiles > 0 ? block_base : nullptr, block_pairs,
                               pairs.stage,
                               s->inputs_on_host ? 1 : 0, s->sm_count, st));
-    s->launches += 2;
     if (tp.ntiles > 0) {
         HD_CUDA(hd::launch_scatter(tp, rec, n, s->ctrl, buckets_of(s), block_base, block_pairs,
                                    pairs, s->sm_count, st));
-        s->launches += 1;
     }
     return HD_OK;
 }
@@ -564,7 +570,6 @@ hd_status stage_global(hd_scan *s, int64_t n, cudaStream_t st)
 {
     HD_CUDA(hd::launch_trace_global(records_of(s, n), s->ctrl, n, s->gq, s->N, s->M, 0,
                                     s->sm_count, st));
-    s->launches += 1;
     return HD_OK;
 }
 
@@ -597,8 +602,6 @@ hd_status stage_finalize(hd_scan *scan, cudaStream_t st)
     HD_CUDA(hd::launch_finalize(a, scan->sm_count, st));
     return HD_OK;
 }
-
-int finalize_launches(const hd_scan *scan) { return (scan->params.methods & HD_SM) ? 2 : 1; }
 
 hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st);
 
@@ -718,7 +721,6 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
                     s->params.wepl_miss_lt, s->params.wepl_hit_gt, (m & (HD_SC | HD_MSC)) ? 1 : 0,
                     (m & HD_SM) ? 1 : 0, s->euclid_d0, records_of(s, c), block_base, block_pairs,
                     s->thick_ws, s->trace_grid, s->sm_count, st));
-                s->launches += 11;
             }
             if (per > 0) return HD_OK;
         }
@@ -727,7 +729,6 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
                                   s->params.wepl_hit_gt, (m & (HD_SC | HD_MSC)) ? 1 : 0,
                                   (m & HD_SM) ? 1 : 0, s->euclid_d0, s->thick_ws, s->N, s->M,
                                   &s->ctrl->n_in, nullptr, s->sm_count, st));
-        s->launches += 4;
         return HD_OK;
     }
     if (s->thick_k > 0) {
@@ -743,7 +744,6 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
                                           s->gq, s->thick_k, s->thick_ws, s->N, s->M,
                                           tp.tile_words, tp.threads, s->trace_grid, s->sm_count,
                                           st));
-            s->launches += 4;
             return HD_OK;
         }
         // other plans: a lane per history over the whole grid
@@ -752,7 +752,6 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
                                  s->params.wepl_hit_gt, (m & (HD_SC | HD_MSC)) ? 1 : 0,
                                  (m & HD_SM) ? 1 : 0, s->thick_k, s->thick_ws, s->N, s->M,
                                  &s->ctrl->n_in, nullptr, s->sm_count, st));
-        s->launches += 1;
         return HD_OK;
     }
     hd_status r = upload_desc(s, st);
@@ -765,7 +764,6 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
     if (s->tp.ntiles > 0 && s->trace_grid > 0) {
         HD_CUDA(hd::launch_trace_tiles(s->desc_dev, 1, s->tp.tile_words, s->tp.threads,
                                        s->trace_grid, hd::kGroups * s->tp.ntiles, st));
-        s->launches += 1;
         if (s->profiling) s->trace_launches += 1;
     }
     prof_end(s, 1, e1, st);
@@ -911,6 +909,7 @@ hd_status hd_scan_reset(hd_scan *scan, void *stream)
     if (!scan) return HD_ERR_ARG;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     const hd_status r = stage_reset(scan, static_cast<cudaStream_t>(stream));
     if (r != HD_OK) return r;
     scan->n_total = 0;
@@ -941,6 +940,7 @@ hd_status hd_scan_add_histories(hd_scan *scan, const float *angle_deg, const flo
         return HD_ERR_OVERFLOW;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *src[6] = {angle_deg, u_in, v_in, u_out, v_out, wepl};
     if (on_device) {
@@ -1006,11 +1006,11 @@ hd_status hd_scan_finalize(hd_scan *scan, void *stream)
     if (!scan) return HD_ERR_ARG;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaEvent_t e0 = prof_begin(scan, st);
     const hd_status r = stage_finalize(scan, st);
     if (r != HD_OK) return r;
-    scan->launches += finalize_launches(scan);
     prof_end(scan, 2, e0, st);
     scan->finalized = true;
     return HD_OK;
@@ -1039,6 +1039,7 @@ hd_status hd_scan_system_rows(hd_scan *scan, int32_t method, const float *angle_
         return HD_ERR_STATE;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     *nnz = 0;
     if (n == 0) {
@@ -1128,6 +1129,7 @@ hd_status hd_scan_get_mask(hd_scan *scan, int32_t method, int32_t layout, void *
     if (dst_bytes < need) return HD_ERR_ARG;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const cudaMemcpyKind kind = dst_on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     if (layout == HD_MASK_U8) {
@@ -1152,6 +1154,7 @@ hd_status hd_scan_get_counts(hd_scan *scan, int32_t method, uint32_t *dst, int64
     if (n < scan->V) return HD_ERR_ARG;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     HD_CUDA(hd::copy_out(dst, src, sizeof(uint32_t) * static_cast<size_t>(scan->V), dst_on_device,
                          scan->device, scan->sm_count, static_cast<cudaStream_t>(stream)));
     return HD_OK;
@@ -1198,6 +1201,7 @@ hd_status hd_scan_get_stats(hd_scan *scan, hd_stats *out, void *stream)
     if (!scan || !out) return HD_ERR_ARG;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     hd::Ctrl c;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     // voxel memberships: sum_v N(v) = sum over missed histories of |A_i|
@@ -1229,6 +1233,7 @@ hd_status hd_scan_get_hull_indices(hd_scan *scan, int32_t method, int32_t *dst,
         return HD_ERR_STATE;
     DeviceGuard g(scan->device);
     if (!g.ok) return HD_ERR_CUDA;
+    const CountLaunches counted(scan->launches);
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t nb = (scan->V + 1023) / 1024;
     if (!scan->compact_blocks) {
@@ -1503,10 +1508,9 @@ hd::ScanDesc item_desc(const hd_batch::Item &it)
 }
 
 // One round: every item of `round` (distinct scans), issued on `st` with
-// the per-scan stages forked to the side streams.  Returns the number of
-// kernels issued through *kernels.
+// the per-scan stages forked to the side streams.
 hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int flags,
-                      int grid, cudaStream_t st, int64_t *kernels)
+                      int grid, cudaStream_t st)
 {
     const int n_items = static_cast<int>(round.size());
     int max_words = 0, buckets = 0;
@@ -1550,7 +1554,6 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
         }
         r = stage_prepare(s, round[i].in, round[i].n, ss);
         if (r != HD_OK) return r;
-        *kernels += 2 + ((s->tp.ntiles > 0 && s->trace_grid > 0) ? 1 : 0);
         if (round[i].n > upper) upper = round[i].n;
         any_finalize = any_finalize || finalizes(round[i]);
     }
@@ -1558,10 +1561,8 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
     if (r != HD_OK) return r;
     if (any_tiled) {
         HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, buckets, st));
-        *kernels += 1;
     }
     HD_CUDA(hd::launch_trace_global_batch(b->descs_dev, n_items, upper, b->sm_count, st));
-    *kernels += upper > 0 ? 1 : 0;
     if (!any_finalize) return HD_OK;
     r = fork();
     if (r != HD_OK) return r;
@@ -1569,7 +1570,6 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
         if (!finalizes(round[i])) continue;
         r = stage_finalize(round[i].scan, side_of(i));
         if (r != HD_OK) return r;
-        *kernels += finalize_launches(round[i].scan);
     }
     return join();
 }
@@ -1737,7 +1737,7 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
     } else {
         // descriptor table of the (single-round) traversal; multi-round runs
         // upload one table per round below
-        int64_t kernels = 0;
+        const int64_t before = hd::kernels_launched();
         if (graphable) {
             std::vector<hd::ScanDesc> descs;
             for (const auto &it : rounds[0]) descs.push_back(item_desc(it));
@@ -1749,7 +1749,7 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
                 batch->exec = nullptr;
             }
             HD_CUDA(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-            hd_status r = issue_round(batch, rounds[0], flags, grid, st, &kernels);
+            hd_status r = issue_round(batch, rounds[0], flags, grid, st);
             cudaGraph_t graph = nullptr;
             const cudaError_t ec = cudaStreamEndCapture(st, &graph);
             if (r != HD_OK) {
@@ -1768,7 +1768,7 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
                 return HD_ERR_CUDA;
             }
             batch->key = key;
-            batch->graph_kernels = kernels;
+            batch->graph_kernels = hd::kernels_launched() - before;
             HD_CUDA(cudaGraphLaunch(batch->exec, st));
             batch->stats.graph_captures += 1;
         } else {
@@ -1783,11 +1783,11 @@ hd_status hd_batch_run(hd_batch *batch, int32_t flags, void *stream)
                                         sizeof(hd::ScanDesc) * rounds[k].size(),
                                         cudaMemcpyHostToDevice, st));
                 HD_CUDA(cudaEventRecord(batch->descs_copied, st));
-                hd_status r = issue_round(batch, rounds[k], flags, grid, st, &kernels);
+                hd_status r = issue_round(batch, rounds[k], flags, grid, st);
                 if (r != HD_OK) return r;
             }
         }
-        batch->stats.kernel_launches += kernels;
+        batch->stats.kernel_launches += hd::kernels_launched() - before;
     }
     for (const auto &p : seen) {
         hd_scan *s = p.first;

@@ -311,6 +311,7 @@ cudaError_t launch_volume_sums(const uint32_t *N, const uint32_t *M, int64_t V,
     int64_t blocks = (V + 255) / 256;
     const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * 4;
     if (blocks > cap) blocks = cap;
+    count_kernels(1);
     volume_sums_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(N, M, V, out);
     return cudaGetLastError();
 }
@@ -335,6 +336,7 @@ cudaError_t launch_pack_bits(const uint8_t *mask, int64_t V, uint32_t *bits, cud
     const int64_t threads = ((V + 31) / 32) * 32;
     int64_t blocks = (threads + 255) / 256;
     if (blocks > 65535) blocks = 65535;
+    count_kernels(1);
     pack_bits_kernel<<<static_cast<unsigned>(blocks), 256, 0, s>>>(mask, V, bits);
     return cudaGetLastError();
 }
@@ -343,6 +345,7 @@ cudaError_t launch_compact(const uint8_t *mask, int64_t V, int32_t *out, int64_t
                            uint32_t *block_counts, unsigned long long *d_count, cudaStream_t s)
 {
     const int64_t nb = (V + kCompactBlock - 1) / kCompactBlock;
+    count_kernels(3);
     compact_count_kernel<<<static_cast<unsigned>(nb), kCompactBlock, 0, s>>>(mask, V,
                                                                             block_counts);
     cudaError_t e = cudaGetLastError();

@@ -427,6 +427,7 @@ cudaError_t launch_euclid(const Inputs &in, int64_t n, const hd_geometry *geom, 
         const int64_t want = (n + kEuGroup * (kEuThreads / 32) - 1) /
                              (kEuGroup * (kEuThreads / 32));
         if (blocks > want) blocks = want;
+        count_kernels(1);
         euclid_kernel<<<static_cast<unsigned>(blocks), kEuThreads, 0, st>>>(
             in, n, g, cd, tau_l, tau_h, use_miss, use_hit, R2, td, cnt, cnt + 8, nullptr, nullptr);
         e = cudaGetLastError();
@@ -491,6 +492,7 @@ cudaError_t launch_euclid_scan(const ScanDesc *desc_dev, const ScanDesc &desc, c
     e = launch_thick_clear(geom, workspace, desc.ctrl, sm_count, st);
     if (e != cudaSuccess) return e;
     unsigned long long *cnt = thick_counters_of(geom, workspace);
+    count_kernels(1);
     euclid_kernel<<<static_cast<unsigned>((sm_count > 0 ? sm_count : 1) * kEuBlocksPerSm), kEuThreads, 0,
                     st>>>(in, n, g, cd, tau_l, tau_h, use_miss, use_hit, ra.R,
                           thick_diff_of(geom, workspace), cnt, cnt + 8, rec.glist,

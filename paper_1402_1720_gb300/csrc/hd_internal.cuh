@@ -193,6 +193,15 @@ struct Inputs {
     const float *angle, *u_in, *v_in, *u_out, *v_out, *wepl;
 };
 
+// Kernels the calling thread has launched on the paths of scans and batches, which
+// count theirs by the difference over a call (launch_chained counts itself).
+inline int64_t &kernels_launched()
+{
+    static thread_local int64_t n = 0;
+    return n;
+}
+inline void count_kernels(int n) { kernels_launched() += n; }
+
 // Launch of a kernel that begins with after_previous(): its blocks may come onto
 // the SMs, and do what needs none of the previous kernel's results, while that
 // one ends (the chain of a small chunk is mostly launches, ends and starts).  Its
@@ -212,6 +221,7 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
     c.stream = s;
     c.attrs = &at;
     c.numAttrs = 1;
+    count_kernels(1);
     return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 

@@ -511,6 +511,7 @@ cudaError_t launch_rows_setup(const Inputs &in, int64_t n, const GeomQ &g, const
     int64_t blocks = (n + kSetupThreads - 1) / kSetupThreads;
     const int64_t cap = static_cast<int64_t>(sm_count > 0 ? sm_count : 1) * 16;
     if (blocks > cap) blocks = cap;
+    count_kernels(1);
     rows_setup_kernel<<<static_cast<unsigned>(blocks), kSetupThreads, 0, s>>>(
         in, n, g, cd, reinterpret_cast<uint4 *>(walks));
     return cudaGetLastError();
@@ -520,6 +521,7 @@ cudaError_t launch_rows_count(const uint32_t *walks, int64_t n, const GeomQ &g,
                               const uint32_t *hull_bits, unsigned *counters, int64_t *row_ptr,
                               bool first, int sm_count, cudaStream_t s)
 {
+    count_kernels(2);
     rows_first_kernel<<<1, 1, 0, s>>>(counters, first ? row_ptr : nullptr);
     const int64_t words = rows_hull_words(int64_t(g.nx) * g.ny * g.nz);
     const int sms = sm_count > 0 ? sm_count : 1;
@@ -540,6 +542,7 @@ cudaError_t launch_rows_scan(int64_t *a, int64_t n, int64_t *scratch, cudaStream
 {
     if (n <= 0) return cudaSuccess;
     const int64_t nb = rows_scan_scratch(n);
+    count_kernels(3);
     scan_tiles_kernel<<<static_cast<unsigned>(nb), kScanThreads, 0, s>>>(a, n, scratch);
     scan_sums_kernel<<<1, kScanThreads, 0, s>>>(scratch, nb);
     scan_add_kernel<<<static_cast<unsigned>(nb), kScanThreads, 0, s>>>(a, n, scratch);
@@ -553,6 +556,7 @@ cudaError_t launch_rows_emit(const uint32_t *walks, int64_t n, const GeomQ &g,
     const int64_t words = rows_hull_words(int64_t(g.nx) * g.ny * g.nz);
     const int sms = sm_count > 0 ? sm_count : 1;
     const uint4 *w = reinterpret_cast<const uint4 *>(walks);
+    count_kernels(1);
     auto ring = [](int threads) { return sizeof(int32_t) * kRing * static_cast<size_t>(threads); };
     const size_t bits = 4 * static_cast<size_t>(words + 1);
     if (words < kMaxHullWords) {

@@ -385,6 +385,7 @@ cudaError_t launch_thick(const Inputs &in, int64_t n, const hd_geometry *geom, c
         int64_t blocks = (n + kThickThreads - 1) / kThickThreads;
         const int64_t cap = int64_t(sm_count > 0 ? sm_count : 1) * 4;
         if (blocks > cap) blocks = cap;  // resident, persistent
+        count_kernels(1);
         thick_kernel<<<static_cast<unsigned>(blocks), kThickThreads, 0, st>>>(
             in, n, g, cd, tau_l, tau_h, use_miss, use_hit, k, ws, ws.stats);
         e = cudaGetLastError();
@@ -394,6 +395,7 @@ cudaError_t launch_thick(const Inputs &in, int64_t n, const hd_geometry *geom, c
         uint32_t *out = c == 0 ? (use_miss ? N : nullptr) : (use_hit ? M : nullptr);
         if (!out) continue;
         const int64_t rx = int64_t(geom->ny) * geom->nz, ry = int64_t(geom->nx) * geom->nz;
+        count_kernels(2);
         thick_rows_kernel<<<static_cast<unsigned>((rx + 255) / 256), 256, 0, st>>>(
             ws.dx[c], rx, geom->nx, 1, geom->ny, plane, 0, out, nullptr);
         thick_rows_kernel<<<static_cast<unsigned>((ry + 255) / 256), 256, 0, st>>>(
@@ -401,6 +403,7 @@ cudaError_t launch_thick(const Inputs &in, int64_t n, const hd_geometry *geom, c
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && (stats || intervals)) {
+        count_kernels(1);
         thick_stats_kernel<<<1, 32, 0, st>>>(ws.stats, stats, intervals);
         e = cudaGetLastError();
     }
@@ -436,6 +439,7 @@ static cudaError_t launch_thick_rows(const hd_geometry *geom, const ThickWs &ws,
         uint32_t *out = c == 0 ? N : M;
         if (!out) continue;
         const int64_t rx = int64_t(geom->ny) * geom->nz, ry = int64_t(geom->nx) * geom->nz;
+        count_kernels(2);
         thick_rows_kernel<<<static_cast<unsigned>((rx + 255) / 256), 256, 0, st>>>(
             ws.dx[c], rx, geom->nx, 1, geom->ny, plane, 0, out, ctrl);
         thick_rows_kernel<<<static_cast<unsigned>((ry + 255) / 256), 256, 0, st>>>(
@@ -452,6 +456,7 @@ cudaError_t launch_thick_finish(const hd_geometry *geom, void *workspace, uint32
     thick_layout(geom, workspace, &ws);
     cudaError_t e = launch_thick_rows(geom, ws, N, M, nullptr, st);
     if (e == cudaSuccess && (stats || intervals)) {
+        count_kernels(1);
         thick_stats_kernel<<<1, 32, 0, st>>>(ws.stats, stats, intervals);
         e = cudaGetLastError();
     }
@@ -463,6 +468,7 @@ cudaError_t launch_thick_clear(const hd_geometry *geom, void *workspace, const C
 {
     // the workspace is a multiple of 256 bytes (thick_layout)
     const int64_t need = static_cast<int64_t>(thick_workspace_bytes(geom));
+    count_kernels(1);
     thick_clear_kernel<<<static_cast<unsigned>(sm_count > 0 ? 8 * sm_count : 8), kThickThreads, 0, st>>>(
         static_cast<uint4 *>(workspace), need / 16, ctrl);
     return cudaGetLastError();
@@ -489,6 +495,7 @@ cudaError_t launch_thick_scan(const ScanDesc *desc_dev, const hd_geometry *geom,
         if (blocks > cap) blocks = cap;
         e = launch_thick_clear(geom, workspace, ctrl, sm_count, st);
         if (e != cudaSuccess) return e;
+        count_kernels(2);
         thick_fallback_kernel<<<static_cast<unsigned>(sm_count > 0 ? 4 * sm_count : 4), 32 * kFbWarps, 0,
                                 st>>>(desc_dev, k);
         thick_records_kernel<<<static_cast<unsigned>(blocks), kThickThreads, 0, st>>>(rec, ctrl, g,
