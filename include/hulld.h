@@ -264,7 +264,8 @@ typedef struct {
 
 /* Set the scan's traversal parameters.  Only while the scan holds no
  * histories (after create or reset): HD_ERR_STATE otherwise; HD_ERR_ARG for
- * values outside the ranges above. */
+ * values outside the ranges above.  Drops the per-chunk scratch, and with it
+ * what hd_scan_reserve made room for. */
 HD_API hd_status hd_scan_set_tuning(hd_scan *scan, const hd_tuning *tuning);
 HD_API hd_status hd_scan_get_tuning(hd_scan *scan, hd_tuning *out);
 

@@ -1351,6 +1351,7 @@ hd_status hd_scan_set_tuning(hd_scan *scan, const hd_tuning *t)
     scan->rec_buf = nullptr;
     scan->pair_buf = nullptr;
     scan->rec_cap = 0;
+    scan->reserved = 0;
     scan->tuning = *t;
     make_tile_plan(scan);
     scan->euclid_pairs = scan->euclid_d0 > 0.0f
