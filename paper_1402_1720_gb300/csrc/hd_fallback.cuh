@@ -14,19 +14,20 @@ struct GlobalVisit {
 };
 
 // A lane's part of a segment in a box of dx x dy voxels (in-plane), for walks
-// shared by a warp: the box becomes the lane's strip of it along the segment's
-// longer in-plane axis, (ox, oy) its corner, and a, b the segment relative to
+// shared by `lanes` lanes of a warp (a power of two): the box becomes the lane's
+// strip of it along the segment's longer in-plane axis, (ox, oy) its corner, and a, b the segment relative to
 // that.  The strips' parts are a partition of the segment's voxels in the box
 // (A_i is a set of points).  False when the lane has no strip.  (With a lane
 // per segment instead the last walks alone took 0.1 ms at the end of the
 // head-sized traversal.)
 __device__ __forceinline__ bool warp_strip(const int32_t gi[3], const int32_t go[3], int &dx,
-                                           int &dy, int &ox, int &oy, int32_t a[3], int32_t b[3])
+                                           int &dy, int &ox, int &oy, int32_t a[3], int32_t b[3],
+                                           int lanes = 32)
 {
     const bool along_y = abs(go[1] - gi[1]) > abs(go[0] - gi[0]);
     const int n = along_y ? dy : dx;
-    const int strip = (n + 31) >> 5;
-    const int s0 = static_cast<int>(threadIdx.x & 31u) * strip, len = min(strip, n - s0);
+    const int strip = (n + lanes - 1) / lanes;
+    const int s0 = (static_cast<int>(threadIdx.x) & (lanes - 1)) * strip, len = min(strip, n - s0);
     if (len <= 0) return false;
     ox = along_y ? 0 : s0;
     oy = along_y ? s0 : 0;
@@ -41,10 +42,10 @@ __device__ __forceinline__ bool warp_strip(const int32_t gi[3], const int32_t go
 }
 
 // The voxels of a segment clipped to one tile of tp (gi, go relative to the
-// tile's origin, grid Q16), by a warp with the general run walk, visited with
+// tile's origin, grid Q16), by `lanes` lanes with the general run walk, visited with
 // global indices.
 __device__ void walk_tile_global(const TilePlan &tp, const int32_t gi[3], const int32_t go[3],
-                                 int tile, const GlobalVisit &visit)
+                                 int tile, int lanes, const GlobalVisit &visit)
 {
     const int tix = tile % tp.ntx;
     const int tiy = (tile / tp.ntx) % tp.nty;
@@ -55,7 +56,7 @@ __device__ void walk_tile_global(const TilePlan &tp, const int32_t gi[3], const 
     const int dz = min(tp.tz, tp.nz - z0);
     int ox, oy;
     int32_t a[3], b[3];
-    if (!warp_strip(gi, go, dx, dy, ox, oy, a, b)) return;
+    if (!warp_strip(gi, go, dx, dy, ox, oy, a, b, lanes)) return;
     x0 += ox;
     y0 += oy;
     RunWalk w;

@@ -677,25 +677,36 @@ __device__ __forceinline__ void flush_tile(uint32_t *tile, int dx, int dy, int d
 }
 
 // The pairs without an event walk (the fallback lists), walked with the general
-// run walk in global memory, a warp per pair, by the blocks as they run out of
-// parts.  Out of line, so its registers do not weigh on the event loop.
+// run walk in global memory by the blocks as they run out of parts: a warp per
+// pair while there are no more of them than warps (the last walks end sooner), else
+// fewer lanes for each, whose strips are set up fewer times (deep slabs list every
+// walk that crosses z inside one: 64 x 64 x 64 in slabs of four, 1e6 histories 275
+// -> 248 us, 250 with a lane for each, which ends 0.1 ms late where they are few).
+// Out of line, so its registers do not weigh on
+// the event loop.
 __device__ __noinline__ void walk_fallback_lists(const ScanDesc *__restrict__ descs, int nscans)
 {
+    const unsigned lane = threadIdx.x & 31u;
+    const unsigned warps = gridDim.x * (blockDim.x >> 5);
     for (int k = 0; k < nscans; ++k) {
         const ScanDesc &d = descs[k];
         if (d.tp.thick > 0) continue;  // dilated by a kernel of their own
         const unsigned nf = d.ctrl->n_pair_fallback;
         if (nf == 0) continue;
+        const int lanes = nf <= warps ? 32 : (nf <= 4u * warps ? 8 : 2);
         for (;;) {
             unsigned i = 0;
-            if ((threadIdx.x & 31u) == 0) i = atomicAdd(&d.ctrl->fb_next, 1u);
+            if (lane == 0) i = atomicAdd(&d.ctrl->fb_next, 32u / lanes);
             i = __shfl_sync(kFull, i, 0);
             if (i >= nf) break;
-            int32_t gi[3], go[3];
-            const uint32_t id = load_general(d.pairs, d.pairs.fb[i].x, gi, go);
-            GlobalVisit v;
-            v.vol = (id & 1u) == 0 ? d.N : d.M;
-            walk_tile_global(d.tp, gi, go, static_cast<int>(id >> 1), v);
+            i += lane / lanes;
+            if (i < nf) {
+                int32_t gi[3], go[3];
+                const uint32_t id = load_general(d.pairs, d.pairs.fb[i].x, gi, go);
+                GlobalVisit v;
+                v.vol = (id & 1u) == 0 ? d.N : d.M;
+                walk_tile_global(d.tp, gi, go, static_cast<int>(id >> 1), lanes, v);
+            }
             __syncwarp();
         }
     }
