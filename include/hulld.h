@@ -253,7 +253,8 @@ HD_API hd_status hd_scan_get_hull_indices(hd_scan *scan, int32_t method, int32_t
  * autotuner (paper_1402_1720_gb300/autotune.py) or left at their defaults:
  *   threads     threads per block of the traversal: 256, 512, 768 or 1024 (1024)
  *   refill      idle lanes of a warp that trigger taking new walks, 1..32 (12)
- *   job_size    (record, tile) pairs per job, 256..32767 (32767)
+ *   job_size    most (record, tile) pairs walked into a tile between two
+ *               flushes of it, 256..32767 (32767)
  *   slab_depth  z-slices per shared-memory tile when whole x-y planes fit,
  *               at most as many as fit; 0 = one slice (0).  Walks that cross
  *               z inside a deeper slab take the general walk in global memory
@@ -299,8 +300,8 @@ HD_API hd_status hd_scan_get_profile(hd_scan *scan, hd_profile *out);
  * A batch collects work items (a scan and a chunk of its histories, device
  * SoA arrays) without launching anything; hd_batch_run then runs every item:
  * classification, geometry and bucketing of each item on its own stream (they
- * overlap on the GPU), ONE persistent traversal launch whose blocks take the
- * jobs of all scans from a device job counter, the global-memory pass, and
+ * overlap on the GPU), ONE traversal launch whose blocks share the pairs of all
+ * scans by their counted cost, ONE global-memory pass over all scans, and
  * (with HD_BATCH_FINALIZE) each scan's decisions.  With graph replay on (the
  * default), the first run of a batch shape is captured into a CUDA graph and
  * later runs with the same items (same scans, pointers and sizes) replay it.

@@ -568,7 +568,7 @@ hd_status stage_prepare(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_
 // Records outside the tiled path, walked with global-memory updates.
 hd_status stage_global(hd_scan *s, int64_t n, cudaStream_t st)
 {
-    HD_CUDA(hd::launch_trace_global(records_of(s, n), s->ctrl, n, s->gq, s->N, s->M, 0,
+    HD_CUDA(hd::launch_trace_global(records_of(s, n), s->ctrl, n, s->gq, s->N, s->M,
                                     s->sm_count, st));
     return HD_OK;
 }

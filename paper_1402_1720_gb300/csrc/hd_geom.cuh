@@ -111,8 +111,8 @@ HD_HD long long floordiv_small(long long a, long long b)
 
 // floor(a / b) for b > 0 and |a / b| < 2^20: a correctly rounded float
 // quotient estimate (relative error below 2^-21) is within one of the
-// floor, so one correction step each way settles it; unlike floordiv_small
-// it needs no loop, which keeps the lanes of a warp together.
+// floor, so one correction step each way settles it.  The 64-bit form of fdiv32,
+// which the kernels use; the host tests compare it with the floor.
 HD_HD long long fdiv_small(long long a, long long b)
 {
 #ifdef __CUDA_ARCH__
@@ -1476,8 +1476,9 @@ HD_HD bool lean_step(LeanWalk &L, int &row, int &lo, int &hi, unsigned &steps)
     return true;
 }
 
-// The tiled traversal's form of a lean walk: the same runs as lean_run, as
-// byte offsets into a tile box of dx x dy x dz voxels stored one 32-bit
+// The updates of a joined tile (below) stated run by run, as the host tests check
+// them; the traversal itself takes them from event walks (JoinedCursor).  The
+// same runs as lean_run, as byte offsets into a tile box of dx x dy x dz voxels stored one 32-bit
 // word per voxel, x fastest, with one padding column and one padding row:
 // word(x, y, z) = x + Wx (y + Hy z), Wx = dx + 1, Hy = dy + 1.  A run adds
 // inc (1 for runs along x, 65536 for runs along y: the two halves of a
@@ -1575,7 +1576,7 @@ HD_HD bool tile_cursor_run(TileCursor &c, int &at_prev, int &at_cur)
 //   count(m, row) = SP(m, row) + SE(m, row - s) - SE(m - 1, row)
 // SE and SP the prefix sums of E and P along the major axis (P is +1 at the
 // walk's first voxel, -1 just past its last).  A row of a walk holds at most
-// one event, so SE and SP stay within the pairs of a job (32767).
+// one event, so SE and SP stay within the pairs of a part (32767).
 //
 // Rays dilated by t voxels in-plane decode from the same events: the
 // dilated set's interval in a row runs from where the run t rows earlier began,
@@ -1699,7 +1700,7 @@ HD_HD int event_end(const EventCursor &c, int thick4)
 //   count(x, y) = sum_{x' <= x} low(x', y) + sum_{y' <= y} high(x, y').
 // An event then takes two updates: it ends its row's run past its major index
 // and begins the next row's there.  A walk adds at most one to a half of a word
-// and to a prefix sum of it, so both stay within the pairs of a job (32767).
+// and to a prefix sum of it, so both stay within the pairs of a part (32767).
 
 // How walks of one type lie in a joined tile (bytes from one index to the next,
 // the minor one's in the direction the walks go), and in their own layout.

@@ -12,7 +12,6 @@ constexpr int64_t kQ16 = 65536;
 constexpr int kMaxN = 4096;
 constexpr int kMaxTiles = 2048;       // tiles per group for the shared-memory path
 constexpr int kGroups = 8;            // groups of records: class + 2 * walk type (hd_geom.cuh)
-constexpr int kTraceThreads = 512;    // threads per block of the tiled traversal
 constexpr int kTileSmemBytes = 224 * 1024;  // shared memory per block for a private tile
 
 // Gantry-rotation constants: theta[i] = round(atan(2^-i) * 180/pi * 2^30)
@@ -49,7 +48,6 @@ struct Ctrl {
     unsigned long long pairs_general;  // pairs sent to the fallback list (cumulative)
     unsigned long long runs;           // runs walked by the tiled pass (cumulative)
     unsigned int n_global;    // records listed for the global path (Records::glist)
-    unsigned int n_fallback;  // records traversed by the global-memory path
     unsigned int n_pair_fallback;  // entries of the pair fallback list
     unsigned int fb_next;          // next fallback entry to hand out
 };
@@ -116,7 +114,7 @@ struct TilePlan {
     int ntiles;         // tiles per group (0: tiled path off)
     int max_tiles;      // records touching more tiles take the global path
     int pairs_per_record;  // pair budget per history (pair_cap = this * slots)
-    int job_size;       // most pairs between two flushes of a tile
+    int job_size;       // most walks in a tile between two flushes
     long long pair_cap;
     int tile_words;     // 32-bit words of shared memory per block
     int refill;         // idle lanes that trigger a warp refill
@@ -127,11 +125,11 @@ struct TilePlan {
 
 // (record, tile) pairs sorted by group and tile: the packed event walk of the
 // record clipped to the tile, 32 bytes per pair (two uint4: one 32-byte
-// sector; group and tile come from the job).  A pair whose walk has no lean form
+// sector; group and tile come from the part).  A pair whose walk has no lean form
 // (a tie, a pending start, or a z crossing inside the tile) holds instead
 // its tile-local endpoints, tile and class, marked empty for the lean pass,
 // and its position goes to the fallback list; traversal blocks that run out
-// of jobs walk those with the general run walk in global memory.
+// of parts walk those with the general run walk in global memory.
 struct Pairs {
     uint4 *v;   // 2 per pair
     uint2 *fb;  // fallback list: (pair position, 0), pair_cap entries
@@ -276,11 +274,10 @@ cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words
 cudaError_t launch_trace_rows(const ScanDesc *desc, int tile_words, int threads, int grid,
                               const RowsArgs &ra, cudaStream_t s);
 
-// Global-memory traversal of the records whose path is 2 (or of every
-// record when all_records is set); upper is the chunk's slot count.
+// Global-memory traversal of the records whose path is 2; upper is the chunk's
+// slot count.
 cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, const GeomQ &g,
-                                uint32_t *N, uint32_t *M, int all_records,
-                                int sm_count, cudaStream_t s);
+                                uint32_t *N, uint32_t *M, int sm_count, cudaStream_t s);
 
 // The same for the chunks of nscans scans in one launch: most of them have no
 // such record, and a launch each, on forked streams, cost a server's thread more

@@ -656,7 +656,7 @@ __device__ __noinline__ void flush_general(uint32_t *tile, int dx, int dy, int d
 }
 
 // Adds the tile's counts to the volume (one global atomic per nonzero voxel,
-// lanes along x whichever axis the rows follow) and clears it for the next job.
+// lanes along x whichever axis the rows follow) and clears it for the next part.
 template <bool kPlain>
 __device__ __forceinline__ void flush_tile(uint32_t *tile, int dx, int dy, int dz, int type,
                                            int thick, uint32_t *vol, int nx, int ny, int x0,
@@ -931,7 +931,7 @@ __device__ __forceinline__ unsigned long long cell_pass(const ScanDesc *__restri
 // The traversal: the buckets of all scans laid end to end by cost, one equal
 // stretch per block (static: the costs are counted, not estimated, so the
 // blocks end within a few per cent of each other, and a bucket is flushed once
-// per block that has a part of it; a queue of four jobs per SM flushed twice
+// per block that has a part of it; a queue of four pieces per SM flushed twice
 // as often and left the SMs 10 % apart).  Each part is walked into the block's
 // shared-memory tile and flushed; then the blocks walk the fallback lists.
 // smem_words: the dynamic shared memory of the launch, at least the

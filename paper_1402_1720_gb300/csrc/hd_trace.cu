@@ -226,42 +226,36 @@ __global__ void __launch_bounds__(kIngestThreads, 4) ingest_kernel(
 
 // ---------------------------------------------------------------- traversal
 
-__device__ __forceinline__ void trace_records(const Records &rec, Ctrl *ctrl, int nx, int ny, int nz,
-                                              uint32_t *N, uint32_t *M, int all_records)
+__device__ __forceinline__ void trace_records(const Records &rec, const Ctrl *ctrl, int nx, int ny,
+                                              int nz, uint32_t *N, uint32_t *M)
 {
     const int64_t stride = static_cast<int64_t>(gridDim.x) * blockDim.x;
     const int64_t total = rec.glist ? static_cast<int64_t>(ctrl->n_global) : rec.cap;
-    unsigned taken = 0;
     for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < total;
          k += stride) {
         const int64_t i = rec.glist ? static_cast<int64_t>(rec.glist[k]) : k;
         const int32_t stw = rec.status[i];
-        const int path = status_path(stw);
-        if (all_records ? path == 0 : path != 2) continue;
+        if (status_path(stw) != 2) continue;
         const int32_t gi[3] = {rec.g[0][i], rec.g[1][i], rec.g[2][i]};
         const int32_t go[3] = {rec.g[3][i], rec.g[4][i], rec.g[5][i]};
         GlobalVisit v;
         v.vol = status_cls(stw) ? M : N;
         walk_all(gi, go, nx, ny, nz, v);
-        ++taken;
     }
-    const unsigned tk = warp_sum_u32(taken);
-    if ((threadIdx.x & 31u) == 0 && tk && !all_records) atomicAdd(&ctrl->n_fallback, tk);
 }
 
-__global__ void __launch_bounds__(256) trace_global_kernel(Records rec, Ctrl *ctrl, int nx, int ny,
-                                                           int nz, uint32_t *N, uint32_t *M,
-                                                           int all_records)
+__global__ void __launch_bounds__(256) trace_global_kernel(Records rec, const Ctrl *ctrl, int nx,
+                                                           int ny, int nz, uint32_t *N, uint32_t *M)
 {
     after_previous();
-    trace_records(rec, ctrl, nx, ny, nz, N, M, all_records);
+    trace_records(rec, ctrl, nx, ny, nz, N, M);
 }
 
 __global__ void __launch_bounds__(256) trace_global_batch_kernel(const ScanDesc *descs)
 {
     after_previous();
     const ScanDesc &d = descs[blockIdx.y];
-    trace_records(d.rec, d.ctrl, d.nx, d.ny, d.nz, d.N, d.M, 0);
+    trace_records(d.rec, d.ctrl, d.nx, d.ny, d.nz, d.N, d.M);
 }
 
 __global__ void classify_kernel(const float *__restrict__ w, int64_t n, float tau_l, float tau_h,
@@ -311,7 +305,7 @@ __global__ void __launch_bounds__(1024) chunk_begin_kernel(Ctrl *ctrl, Buckets b
 {
     after_previous();
     if (blockIdx.x == 0 && threadIdx.x == 0)
-        ctrl->n_global = ctrl->n_fallback = ctrl->n_pair_fallback = ctrl->fb_next = 0u;
+        ctrl->n_global = ctrl->n_pair_fallback = ctrl->fb_next = 0u;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < ncols; t += gridDim.x * blockDim.x) {
         buckets.count[t] = 0u;
         buckets.events[t] = 0ull;
@@ -337,15 +331,14 @@ cudaError_t init_ingest()
 }
 
 cudaError_t launch_trace_global(const Records &rec, Ctrl *ctrl, int64_t upper, const GeomQ &g,
-                                uint32_t *N, uint32_t *M, int all_records,
-                                int sm_count, cudaStream_t s)
+                                uint32_t *N, uint32_t *M, int sm_count, cudaStream_t s)
 {
     if (upper <= 0) return cudaSuccess;
     int64_t blocks = (upper + 255) / 256;
     const int64_t cap_blocks = static_cast<int64_t>(sm_count) * 8;
     if (blocks > cap_blocks) blocks = cap_blocks;
     return launch_chained(trace_global_kernel, static_cast<unsigned>(blocks), 256, 0, s, rec, ctrl,
-                          g.nx, g.ny, g.nz, N, M, all_records);
+                          g.nx, g.ny, g.nz, N, M);
 }
 
 cudaError_t launch_trace_global_batch(const ScanDesc *descs, int nscans, int64_t upper,
