@@ -14,6 +14,10 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 constexpr int kScatterThreads = 512;
+// Buckets whose events a block sums in shared memory: with more of them, beside the
+// positions, only one block per SM would be resident, and two updates of one bucket
+// are then rare (64 x 64 x 2000: 160 us).
+constexpr int kLocalEvents = 12 * 1024;
 
 // The general set-up of one (record, tile) pair: its packed event walk, an
 // empty walk, or (returns true) the general form for the fallback list.
@@ -49,12 +53,12 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
 {
     extern __shared__ uint32_t s_mem[];
     const int nt = kGroups * tp.ntiles;
-    uint32_t *s_base = s_mem;       // this block's first position in each bucket
-    uint32_t *s_next = s_mem + nt;  // pairs written per bucket so far
-    uint32_t *s_events = s_next + nt;  // and the events of their walks
-    for (int t = threadIdx.x; t < nt; t += blockDim.x) s_next[t] = s_events[t] = 0;
+    uint32_t *s_next = s_mem;         // this block's next position in each bucket
+    uint32_t *s_events = s_mem + nt;  // the events of the walks written there
+    const bool local = nt <= kLocalEvents;
+    for (int t = threadIdx.x; local && t < nt; t += blockDim.x) s_events[t] = 0;
     after_previous();
-    bucket_places<kScatterThreads>(nt, buckets, block_base, s_base);
+    bucket_places<kScatterThreads>(nt, buckets, block_base, s_next);
     const int64_t h0 = static_cast<int64_t>(blockIdx.x) * per_block;
     const unsigned npairs = block_pairs[blockIdx.x];
     unsigned runs = 0;
@@ -84,7 +88,7 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
         }
         const int tile = x + tp.ntx * (y + tp.nty * z);
         const int t = status_group(stw) * tp.ntiles + tile;
-        const uint32_t pos = s_base[t] + atomicAdd(&s_next[t], 1u);
+        const uint32_t pos = atomicAdd(&s_next[t], 1u);
         // set up the walk of this record clipped to this tile
         const int x0 = x * tp.tx, y0 = y * tp.ty, z0 = z * tp.tz;
         const int dx = min(tp.tx, tp.nx - x0), dy = min(tp.ty, tp.ny - y0),
@@ -117,7 +121,10 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
         }
         if (static_cast<int>(p1.w) >= 0) {
             runs += p1.w + 1u;  // a walk's runs: one more than its events
-            if (p1.w != 0u) atomicAdd(&s_events[t], p1.w);
+            if (p1.w != 0u) {
+                if (local) atomicAdd(&s_events[t], p1.w);
+                else atomicAdd(&buckets.events[t], static_cast<unsigned long long>(p1.w));
+            }
         }
         pairs.v[2 * static_cast<size_t>(pos)] = p0;
         pairs.v[2 * static_cast<size_t>(pos) + 1] = p1;
@@ -140,7 +147,7 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
     for (int o = 16; o > 0; o >>= 1) all += __shfl_xor_sync(kFull, all, o);
     if ((threadIdx.x & 31u) == 0 && all) atomicAdd(&ctrl->runs, all);
     __syncthreads();
-    for (int t = threadIdx.x; t < nt; t += blockDim.x)
+    for (int t = threadIdx.x; local && t < nt; t += blockDim.x)
         if (s_events[t])
             atomicAdd(&buckets.events[t], static_cast<unsigned long long>(s_events[t]));
 }
@@ -150,7 +157,7 @@ __global__ void __launch_bounds__(kScatterThreads, 2) scatter_kernel(
 cudaError_t init_scatter()
 {
     return cudaFuncSetAttribute(scatter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                static_cast<int>(sizeof(uint32_t)) * 3 * kGroups * kMaxTiles);
+                                static_cast<int>(sizeof(uint32_t)) * 2 * kGroups * kMaxTiles);
 }
 
 cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ctrl *ctrl,
@@ -160,7 +167,8 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
 {
     if (n <= 0) return cudaSuccess;
     const ChunkSplit sp = chunk_split(n, sm_count, tp.ntiles);
-    const size_t smem = sizeof(uint32_t) * 3 * kGroups * static_cast<size_t>(tp.ntiles);
+    const size_t nt = kGroups * static_cast<size_t>(tp.ntiles);
+    const size_t smem = sizeof(uint32_t) * (nt <= kLocalEvents ? 2 * nt : nt);
     return launch_chained(scatter_kernel, static_cast<unsigned>(sp.blocks), kScatterThreads, smem, s, tp,
                           rec, sp.per_block, buckets, block_base, block_pairs, ctrl, pairs);
 }

@@ -520,71 +520,96 @@ __device__ __noinline__ void flush_rows(uint32_t *tile, int dx, int dy, int dz, 
     }
 }
 
-// Flush of a joined tile.  A thread per column turns the high halves into their
-// sums along y (lanes along x); then a warp per row sums the low halves along x,
-// kPer words a lane at a time, and adds both to the volume, clearing the row.
-__device__ __noinline__ void flush_joined(uint32_t *tile, int dx, int dy, int dz, FlushTo to)
+// Flush of a group's n parts in joined tiles, all tiles at once (small ones leave
+// most warps without a column).  A thread per column turns the high halves into
+// their sums along y (lanes along x); then a warp per row sums the low halves along
+// x, kPer words a lane at a time, and adds both to the volume, clearing the row.
+__device__ __noinline__ void flush_joined(uint32_t *tiles, const TilePart *parts, int n,
+                                          const ScanDesc *__restrict__ descs)
 {
     constexpr int kPer = 7, kAhead = 8;
     const int lane = static_cast<int>(threadIdx.x & 31u);
     const int warp = static_cast<int>(threadIdx.x >> 5), nwarps = static_cast<int>(blockDim.x >> 5);
-    const int P = dx + 1, slice = P * (dy + 1);
-    for (int q = static_cast<int>(threadIdx.x); q < dx * dz; q += blockDim.x) {
-        const int z = dz == 1 ? 0 : q / dx;
-        uint32_t *col = tile + slice * z + q - z * dx;
-        uint32_t sum = 0u;
-        for (int y = 0; y < dy; y += kAhead, col += kAhead * P) {
-            uint32_t w[kAhead];
+    int mine = warp;  // this warp's next piece of 32 columns, or row, of the tile at hand
+    for (int t = 0; t < n; ++t) {
+        const TilePart &j = parts[t];
+        if (j.form == kSame) continue;
+        const TileBox b = tile_box(descs[j.scan].tp, j.tile);
+        const int P = b.dx + 1, slice = P * (b.dy + 1), pieces = (b.dx * b.dz + 31) >> 5;
+        for (; mine < pieces; mine += nwarps) {
+            const int q = 32 * mine + lane;
+            if (q >= b.dx * b.dz) continue;
+            const int z = b.dz == 1 ? 0 : q / b.dx;
+            uint32_t *col = tiles + j.offset + slice * z + q - z * b.dx;
+            uint32_t sum = 0u;
+            for (int y = 0; y < b.dy; y += kAhead, col += kAhead * P) {
+                uint32_t w[kAhead];
 #pragma unroll
-            for (int k = 0; k < kAhead; ++k) w[k] = y + k < dy ? col[k * P] : 0u;
+                for (int k = 0; k < kAhead; ++k) w[k] = y + k < b.dy ? col[k * P] : 0u;
 #pragma unroll
-            for (int k = 0; k < kAhead; ++k) {
-                sum += joined_high(w[k]);
-                if (y + k < dy) col[k * P] = (w[k] & 0xffffu) | (sum << 16);
-            }
-        }
-    }
-    __syncthreads();
-    for (int l = warp; l < dy * dz; l += nwarps) {
-        const int z = dz == 1 ? 0 : l / dy, y = l - z * dy;
-        uint32_t *row = tile + slice * z + P * y;
-        uint32_t *out = to.line(y, z);
-        uint32_t carry = 0u;
-        for (int m0 = 0; m0 < dx; m0 += 32 * kPer) {
-            const int b = m0 + lane * kPer;
-            uint32_t v[kPer], hi[kPer];
-#pragma unroll
-            for (int k = 0; k < kPer; ++k) v[k] = b + k < dx ? row[b + k] : 0u;
-#pragma unroll
-            for (int k = 0; k < kPer; ++k) hi[k] = v[k] >> 16;
-#pragma unroll
-            for (int k = 1; k < kPer; ++k) v[k] += v[k - 1];
-            uint32_t incl = v[kPer - 1];
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t t = __shfl_up_sync(kFull, incl, o);
-                if (lane >= o) incl += t;
-            }
-            const uint32_t before = incl - v[kPer - 1] + carry;
-            carry += __shfl_sync(kFull, incl, 31);
-#pragma unroll
-            for (int k = 0; k < kPer; ++k)
-                if (b + k < dx) row[b + k] = ((v[k] + before) & 0xffffu) + hi[k];
-            __syncwarp();
-#pragma unroll
-            for (int k = 0; k < kPer; ++k) {
-                const int x = m0 + lane + 32 * k;
-                if (x < dx) {
-                    add_count(out + x, row[x]);
-                    row[x] = 0u;
+                for (int k = 0; k < kAhead; ++k) {
+                    sum += joined_high(w[k]);
+                    if (y + k < b.dy) col[k * P] = (w[k] & 0xffffu) | (sum << 16);
                 }
             }
         }
-        if (lane == 0) row[dx] = 0u;
+        mine -= pieces;
     }
-    for (int q = static_cast<int>(threadIdx.x); q < P * dz; q += blockDim.x) {
-        const int z = dz == 1 ? 0 : q / P;
-        tile[slice * z + P * dy + q - z * P] = 0u;
+    __syncthreads();
+    mine = warp;
+    for (int t = 0; t < n; ++t) {
+        const TilePart &j = parts[t];
+        if (j.form == kSame) continue;
+        const ScanDesc &d = descs[j.scan];
+        const TileBox b = tile_box(d.tp, j.tile);
+        uint32_t *const tile = tiles + j.offset;
+        const int P = b.dx + 1, slice = P * (b.dy + 1), rows = b.dy * b.dz;
+        const FlushTo to{((j.group & 1) == 0 ? d.N : d.M) + b.x0 +
+                             static_cast<long long>(d.tp.nx) *
+                                 (b.y0 + static_cast<long long>(d.tp.ny) * b.z0),
+                         d.tp.nx, d.tp.ny};
+        for (; mine < rows; mine += nwarps) {
+            const int z = b.dz == 1 ? 0 : mine / b.dy, y = mine - z * b.dy;
+            uint32_t *row = tile + slice * z + P * y;
+            uint32_t *out = to.line(y, z);
+            uint32_t carry = 0u;
+            for (int m0 = 0; m0 < b.dx; m0 += 32 * kPer) {
+                const int a = m0 + lane * kPer;
+                uint32_t v[kPer], hi[kPer];
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) v[k] = a + k < b.dx ? row[a + k] : 0u;
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) hi[k] = v[k] >> 16;
+#pragma unroll
+                for (int k = 1; k < kPer; ++k) v[k] += v[k - 1];
+                uint32_t incl = v[kPer - 1];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t u = __shfl_up_sync(kFull, incl, o);
+                    if (lane >= o) incl += u;
+                }
+                const uint32_t before = incl - v[kPer - 1] + carry;
+                carry += __shfl_sync(kFull, incl, 31);
+#pragma unroll
+                for (int k = 0; k < kPer; ++k)
+                    if (a + k < b.dx) row[a + k] = ((v[k] + before) & 0xffffu) + hi[k];
+                __syncwarp();
+#pragma unroll
+                for (int k = 0; k < kPer; ++k) {
+                    const int x = m0 + lane + 32 * k;
+                    if (x < b.dx) {
+                        add_count(out + x, row[x]);
+                        row[x] = 0u;
+                    }
+                }
+            }
+            if (lane == 0) row[b.dx] = 0u;
+        }
+        mine -= rows;
+        for (int q = static_cast<int>(threadIdx.x); q < P * b.dz; q += blockDim.x) {
+            const int z = b.dz == 1 ? 0 : q / P;
+            tile[slice * z + P * b.dy + q - z * P] = 0u;
+        }
     }
 }
 
@@ -1096,21 +1121,15 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
             if (g + 1 < ngroups)
                 first_walks(s_parts + q1, s_group[g + 2] - q1, s_slots[g + 1], nw);
             __syncthreads();
-            for (int q = q0; q < q1; ++q) {
+            if constexpr (kCells)
+                if (joined) flush_joined(tile, s_parts + q0, q1 - q0, descs);
+            for (int q = q0; q < q1 && !joined; ++q) {
                 const TilePart &j = s_parts[q];
-                if (kCells && j.form == kSame) continue;
                 const ScanDesc &d = descs[j.scan];
                 const TilePlan &tp = d.tp;
                 const TileBox b = tile_box(tp, j.tile);
-                uint32_t *const vol = (j.group & 1) == 0 ? d.N : d.M;
-                if (kCells && joined)
-                    flush_joined(tile + j.offset, b.dx, b.dy, b.dz,
-                                 FlushTo{vol + b.x0 + static_cast<long long>(tp.nx) *
-                                                          (b.y0 + static_cast<long long>(tp.ny) * b.z0),
-                                         tp.nx, tp.ny});
-                else
-                    flush_tile<kRows>(tile + j.offset, b.dx, b.dy, b.dz, j.group >> 1, tp.thick, vol,
-                                      tp.nx, tp.ny, b.x0, b.y0, b.z0);
+                flush_tile<kRows>(tile + j.offset, b.dx, b.dy, b.dz, j.group >> 1, tp.thick,
+                                  (j.group & 1) == 0 ? d.N : d.M, tp.nx, tp.ny, b.x0, b.y0, b.z0);
             }
         }
         __syncthreads();
