@@ -579,7 +579,7 @@ HD_HD void k_range(const CapF &cf, int a, int blo2, int bhi2, int &klo, int &khi
 // ------------------------------------------------------ rows of one slice
 //
 // The tiled form takes a history's rows one slice (fixed k) at a time.  When
-// every centre of the grid projects onto the segment's interior (the trackers
+// every centre of its slices projects onto the segment's interior (the trackers
 // stand outside the grid), the capsule is a cylinder there, and its rows have
 // a closed form: with h^2 = u_1^2 + u_2^2, row a of the slice lies at the
 // signed distance e R from the line in the plane of axes 1 and 2, linear in a,
@@ -612,7 +612,8 @@ constexpr float kEps = 5.9604644775390625e-8f;  // 2^-24
 
 // Where a record's rows can lie: false when no voxel centre of the grid is
 // inside; else the slices klo .. khi and the extent of axis y (ylo .. yhi, for
-// tiles that are strips), and whether the closed form above holds.  In float,
+// tiles that are strips), and whether the closed form above holds in those slices
+// (asked of the whole grid it failed in tall ones for any path a little inclined).  In float,
 // widened by 2^-14 S, far beyond its roundings.
 HD_HD bool euclid_range(const GeomQ &g, const long long W[6], long long R, int &klo, int &khi,
                         int &ylo, int &yhi, bool &closed)
@@ -624,19 +625,10 @@ HD_HD bool euclid_range(const GeomQ &g, const long long W[6], long long R, int &
     const float H[3] = {static_cast<float>((g.nx - 1LL) * g.sx), static_cast<float>((g.ny - 1LL) * g.sy),
                         static_cast<float>((g.nz - 1LL) * g.sz)};
     const float Rf = static_cast<float>(R);
-    float S = Rf, uu = 0.0f, dmin = 0.0f, dmax = 0.0f;
+    float S = Rf;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        S += H[a] + fabsf(P[a]) + fabsf(D[a]);
-        uu = fmaf(D[a], D[a], uu);
-        const float lo = (-H[a] - P[a]) * D[a], hi = (H[a] - P[a]) * D[a];
-        dmin += fminf(lo, hi);
-        dmax += fmaxf(lo, hi);
-    }
+    for (int a = 0; a < 3; ++a) S += H[a] + fabsf(P[a]) + fabsf(D[a]);
     const float m = S * (1.0f / 16384.0f);
-    const float mu = m * (fabsf(D[0]) + fabsf(D[1]) + fabsf(D[2]));
-    // off both in-plane axes (h > 0 either way round) and interior
-    closed = W[0] != W[3] && W[1] != W[4] && dmin > mu && dmax < uu - mu;
     float t0 = 0.0f, t1 = 1.0f;
 #pragma unroll
     for (int a = 0; a < 2; ++a) {
@@ -664,6 +656,21 @@ HD_HD bool euclid_range(const GeomQ &g, const long long W[6], long long R, int &
     if (yh < 0.0f || yl > static_cast<float>(g.ny - 1)) return false;
     ylo = static_cast<int>(ceilf(fmaxf(yl, 0.0f)));
     yhi = static_cast<int>(floorf(fminf(yh, static_cast<float>(g.ny - 1))));
+    // off both in-plane axes (h > 0 either way round), and the centres of its
+    // slices interior
+    const float zc[2] = {static_cast<float>((2LL * klo + 1 - g.nz) * g.sz),
+                         static_cast<float>((2LL * khi + 1 - g.nz) * g.sz)};
+    float uu = 0.0f, dmin = 0.0f, dmax = 0.0f;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        uu = fmaf(D[a], D[a], uu);
+        const float lo = ((a < 2 ? -H[a] : zc[0]) - P[a]) * D[a],
+                    hi = ((a < 2 ? H[a] : zc[1]) - P[a]) * D[a];
+        dmin += fminf(lo, hi);
+        dmax += fmaxf(lo, hi);
+    }
+    const float mu = m * (fabsf(D[0]) + fabsf(D[1]) + fabsf(D[2]));
+    closed = W[0] != W[3] && W[1] != W[4] && dmin > mu && dmax < uu - mu;
     return klo <= khi && ylo <= yhi;
 }
 

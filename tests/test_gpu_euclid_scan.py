@@ -58,6 +58,7 @@ def _check(hd, s, ref):
     (G(24, 24, 24, 1 / 64, 1 / 64, 1 / 64, 1.0), 1500, 0.02),
     (G(12, 10, 6, 64.0, 64.0, 64.0, 4000.0), 1500, 63.9),
     (G(40, 30, 6, 1.0, 1.0, 1.0, 12.0), 1500, 1.0),         # trackers inside the grid
+    (G(24, 28, 300, 1.0, 1.0, 4.0, 40.0), 1500, 1.5),       # tall: far slices beyond the ends
 ])
 @pytest.mark.parametrize("few", [False, True])
 def test_scattered_paths(hd, oracle_mod, g, n, d0, few):
