@@ -612,7 +612,8 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
 // as it is copied, so parts grow; each chunk has some 60 us of its own, so there
 // are few: three, each half as large again, or from kManyParts on four, a quarter
 // larger.  Head-sized scan: 9e6 histories 1951 us in place, 1665 in three parts,
-// 1567 in four; 4.5e6 1066, 953 and 1027; 2.7e6 711, 711 and 797.  taken stays
+// 1567 in four (1600 to 1630 on other machines); 4.5e6 1066, 953 and 1027; 2.7e6
+// 711, 711 and 797.  taken stays
 // false when copying is not possible here (the stream is being captured, no
 // memory, or an add that was reserved for and must not allocate): the caller
 // then reads in place.

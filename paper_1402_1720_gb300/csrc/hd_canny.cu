@@ -15,7 +15,7 @@
 //                        the quantile by a radix select of four 8-bit steps
 //   canny_hull_kernel    thread per voxel: the hull
 //
-// Latency-bound on volumes of tens of slices.  Head-sized volume: 255 -> 86 us
+// Latency-bound on volumes of tens of slices.  Head-sized volume: 255 -> 78 us
 // (before, three passes over 64-bit volumes, and in the slice's block a step of
 // the select per bit, a barrier per row of the hysteresis and the hull).
 #include <cuda_runtime.h>

@@ -14,7 +14,7 @@
 // records without the closed form (trackers inside the grid, axis-parallel
 // paths, too many tiles) to the kernel below, which the standalone
 // accumulation and other plans use for every history.  Head-sized scan,
-// 2.7e6 histories, d_0 = 2.5 mm, all hulls: 12.46 -> 1.46 ms.
+// 2.7e6 histories, d_0 = 2.5 mm, all hulls: 12.46 -> 1.33 ms.
 //
 // euclid_kernel.  A warp takes groups of 32 consecutive histories (so each lane's
 // gantry cos/sin rarely change); each lane classifies one history and sets
