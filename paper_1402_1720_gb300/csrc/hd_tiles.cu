@@ -33,10 +33,16 @@ constexpr int kEventsPerStep = 8;  // events a traversal lane walks between refi
 struct NoRows {
     static constexpr bool kRows = false, kCells = false;
 };
-// The same for launches that look for cells to join (see Cell).
+// The same for launches that look for cells to join (see Cell), with more cells
+// than threads or not (see scan_types).
+template <bool kMany>
 struct Cells {
     static constexpr bool kRows = false, kCells = true;
 };
+template <class T>
+constexpr bool kManyCells = false;
+template <>
+constexpr bool kManyCells<Cells<true>> = true;
 
 // Shared-memory reduction (no value returned) at a shared-space byte address.
 __device__ __forceinline__ void smem_red_add(int addr, uint32_t v)
@@ -880,20 +886,83 @@ __device__ __forceinline__ void fill_part(TilePart &j, const ScanDesc &d, int k,
     j.form = form;
 }
 
-// A pass over a thread's cells i0 .. i1 - 1 (of scan k those from s_first[k] / 4
-// on): the sum of their costs, or of the blocks of their own; or the parts in
-// the block's stretch, counted, or listed (the thread's first has number `rank`,
-// list begins at number j0): each at most job_size pairs, of a joined cell
-// in up to four, one to a bucket.
-enum CellPass { kCellCost, kCellBlocks, kCellCount, kCellList };
-
-template <CellPass pass>
-__device__ __forceinline__ unsigned long long cell_pass(const ScanDesc *__restrict__ descs,
-                                                        const int *s_first, int i0, int i1,
-                                                        const Stretch &st, unsigned long long rank,
-                                                        unsigned long long j0, TilePart *list)
+// Passes over a thread's cells i0 .. i1 - 1 (of scan k those from s_first[k] / 4
+// on): the sums of their costs by type, or of the blocks of their own.
+template <bool kBlocks>
+__device__ __forceinline__ void cell_sums(const ScanDesc *__restrict__ descs, const int *s_first,
+                                          int i0, int i1, unsigned long long sum[4])
 {
-    unsigned long long sum = 0, p = st.before;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) sum[j] = 0ull;
+    int k = 0;
+    for (int i = i0; i < i1; ++i) {
+        while (4 * i >= s_first[k + 1]) ++k;
+        const ScanDesc &d = descs[k];
+        const Cell c = cell_of(d, i - s_first[k] / 4);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            sum[j] += kBlocks ? own_blocks(c.cost[j], d.tp.tile_words) : c.cost[j];
+    }
+}
+
+// Exclusive block scan of them in the order of the launch's costs, with four words
+// of s for each warp.  Many cells: all buckets of type 0, then of type 1, and so on.
+// With a cell's types close together, blocks beside one another go through the same
+// tiles in step and their flushes meet (a batch of 48 scans 27.3 ms, 26.5 so).  At
+// most a cell per thread: of the cells of a warp all of type 0, then of type 1, ..,
+// a scan instead of four (1 us of a chunk of the large streamed scan).
+template <bool many>
+__device__ __forceinline__ void scan_types(const unsigned long long sum[4], unsigned long long *s,
+                                           unsigned long long before[4], unsigned long long &total)
+{
+    const unsigned lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    unsigned long long types = 0;  // of the warp's types so far
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        unsigned long long incl = sum[j];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(kFull, incl, o);
+            if (lane >= static_cast<unsigned>(o)) incl += t;
+        }
+        before[j] = incl - sum[j] + (many ? 0ull : types);
+        types += __shfl_sync(kFull, incl, 31);
+        if (lane == 31) s[4 * wid + j] = many ? incl : types;
+    }
+    __syncthreads();
+    total = 0ull;
+    // every warp scans the warps' sums for itself
+#pragma unroll
+    for (int j = many ? 0 : 3; j < 4; ++j) {
+        unsigned long long w = lane < nw ? s[4 * lane + j] : 0ull;
+        const unsigned long long own = w;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long t = __shfl_up_sync(kFull, w, o);
+            if (lane >= static_cast<unsigned>(o)) w += t;
+        }
+        const unsigned long long base = total + __shfl_sync(kFull, w - own, wid);
+        total += __shfl_sync(kFull, w, 31);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (!many || q == j) before[q] += base;
+    }
+    __syncthreads();  // s is free again
+}
+
+// The parts of a thread's cells in the block's stretch, counted, or listed (kList:
+// the thread's first has number `rank`, list begins at number j0): each at most
+// job_size pairs, of a joined cell in up to four, one to a bucket.  before: of the
+// thread's first cell, by type.
+template <bool kList>
+__device__ __forceinline__ unsigned long long cell_parts(const ScanDesc *__restrict__ descs,
+                                                         const int *s_first, int i0, int i1,
+                                                         const Stretch &st,
+                                                         const unsigned long long before[4],
+                                                         unsigned long long rank,
+                                                         unsigned long long j0, TilePart *list)
+{
+    unsigned long long n = 0, p[4] = {before[0], before[1], before[2], before[3]};
     int k = 0;
     for (int i = i0; i < i1; ++i) {
         while (4 * i >= s_first[k + 1]) ++k;
@@ -901,7 +970,7 @@ __device__ __forceinline__ unsigned long long cell_pass(const ScanDesc *__restri
         const int t0 = i - s_first[k] / 4, step = 2 * d.tp.ntiles, most = d.tp.job_size & ~31;
         const Cell c = cell_of(d, t0);
         auto take = [&](int u, int s0, int s1, bool same) {
-            if (pass == kCellList && rank >= j0 && rank < j0 + kPartList) {
+            if (kList && rank >= j0 && rank < j0 + kPartList) {
                 TilePart &j = list[rank - j0];
                 fill_part(j, d, k, t0 + step * u, static_cast<int>(c.count[u]), s0, s1,
                           !c.joined ? kOwn : (same ? kSame : kJoined));
@@ -911,22 +980,18 @@ __device__ __forceinline__ unsigned long long cell_pass(const ScanDesc *__restri
                 }
             }
             ++rank;
-            ++sum;
+            ++n;
         };
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (pass == kCellCost || pass == kCellBlocks) {
-                sum += pass == kCellCost ? c.cost[j] : own_blocks(c.cost[j], d.tp.tile_words);
-                continue;
-            }
             const unsigned long long cost = st.own ? own_blocks(c.cost[j], d.tp.tile_words) : c.cost[j];
-            if (cost != 0 && p < st.x1 && p + cost > st.x0) {
+            if (cost != 0 && p[j] < st.x1 && p[j] + cost > st.x0) {
                 const int words = st.own ? -1 : d.tp.tile_words;
                 const int all = c.joined ? pieces_of(c.count[0]) + pieces_of(c.count[1]) +
                                                pieces_of(c.count[2]) + pieces_of(c.count[3])
                                          : pieces_of(c.count[j]);
-                const int s0 = st.x0 > p ? boundary_slot(cost, all, words, p, st.x0) : 0;
-                const int s1 = st.x1 < p + cost ? boundary_slot(cost, all, words, p, st.x1) : 32 * all;
+                const int s0 = st.x0 > p[j] ? boundary_slot(cost, all, words, p[j], st.x0) : 0;
+                const int s1 = st.x1 < p[j] + cost ? boundary_slot(cost, all, words, p[j], st.x1) : 32 * all;
                 for (int s = s0; s < s1; s += most) {
                     const int e = min(s + most, s1);
                     if (!c.joined) {
@@ -945,10 +1010,10 @@ __device__ __forceinline__ unsigned long long cell_pass(const ScanDesc *__restri
                     }
                 }
             }
-            p += cost;
+            p[j] += cost;
         }
     }
-    return sum;
+    return n;
 }
 
 }  // namespace
@@ -981,7 +1046,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     after_previous();
     // buckets of scan k are the launch's buckets [s_first[k], s_first[k + 1])
     if (threadIdx.x == 0) {
-        s_next[1] = 0;
+        s_next[0] = s_next[1] = 0;
         int acc = 0;
         for (int k = 0; k < nscans; ++k) {
             s_first[k] = acc;
@@ -991,7 +1056,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     }
     __syncthreads();
     const int nb = s_first[nscans];
-    // the thread's buckets, or its cells (see cell_pass)
+    // the thread's buckets, or its cells (see cell_parts)
     const int ni = kCells ? nb / 4 : nb, per = (ni + kThreads - 1) / kThreads;
     const int i0 = min(static_cast<int>(threadIdx.x) * per, ni), i1 = min(i0 + per, ni);
     // visit(scan, bucket within it, its cost and pairs)
@@ -1006,10 +1071,17 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         }
     };
     Stretch st{};
-    unsigned long long mine = 0, total;
-    if constexpr (kCells) mine = cell_pass<kCellCost>(descs, s_first, i0, i1, st, 0, 0, nullptr);
-    else each([&](int, int, unsigned long long cost, unsigned) { mine += cost; });
-    st.before = block_excl_scan64(mine, s_warp, total);
+    unsigned long long total, before[4];  // before: of a cell's types
+    if constexpr (kCells) {
+        unsigned long long mine[4];
+        cell_sums<false>(descs, s_first, i0, i1, mine);
+        scan_types<kManyCells<RowsT>>(mine, reinterpret_cast<unsigned long long *>(s_parts), before,
+                                      total);
+    } else {
+        unsigned long long mine = 0;
+        each([&](int, int, unsigned long long cost, unsigned) { mine += cost; });
+        st.before = block_excl_scan64(mine, s_warp, total);
+    }
     // the block's stretch: an equal share, but worth about two flushes
     unsigned long long blocks = total / (2ull * flush_cost(descs[0].tp.tile_words)) + 1ull;
     unsigned long long share = 0;
@@ -1018,16 +1090,22 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     // flushes twice, 11 000 cycles each)
     st.own = blocks < gridDim.x;  // the same in all blocks and threads
     if (st.own) {
-        unsigned long long m = 0, all;
-        if constexpr (kCells) m = cell_pass<kCellBlocks>(descs, s_first, i0, i1, st, 0, 0, nullptr);
-        else
+        unsigned long long m = 0, all, b = 0, bs[4];
+        if constexpr (kCells) {
+            unsigned long long ms[4];
+            cell_sums<true>(descs, s_first, i0, i1, ms);
+            scan_types<kManyCells<RowsT>>(ms, reinterpret_cast<unsigned long long *>(s_parts), bs, all);
+        } else {
             each([&](int k, int, unsigned long long cost, unsigned) {
                 m += own_blocks(cost, descs[k].tp.tile_words);
             });
-        const unsigned long long b = block_excl_scan64(m, s_warp, all);
+            b = block_excl_scan64(m, s_warp, all);
+        }
         st.own = all <= gridDim.x;
         if (st.own) {
             st.before = b;
+            if constexpr (kCells)
+                for (int j = 0; j < 4; ++j) before[j] = bs[j];
             share = 1ull;
         }
     }
@@ -1054,14 +1132,21 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
             p += cost;
         });
     };
-    unsigned long long nmine = 0, nparts;
-    if constexpr (kCells) nmine = cell_pass<kCellCount>(descs, s_first, i0, i1, st, 0, 0, nullptr);
-    else parts([&](int, int, int, int, int) { ++nmine; });
-    const unsigned long long rank0 = block_excl_scan64(nmine, s_warp, nparts);
+    unsigned long long nmine = 0, nparts, rank0 = 0;
+    if constexpr (kCells) {
+        // (the order of the parts does not matter: numbers from a counter, no scan)
+        nmine = cell_parts<false>(descs, s_first, i0, i1, st, before, 0, 0, nullptr);
+        if (nmine != 0) rank0 = atomicAdd(&s_next[0], static_cast<unsigned>(nmine));
+        __syncthreads();
+        nparts = s_next[0];
+    } else {
+        parts([&](int, int, int, int, int) { ++nmine; });
+        rank0 = block_excl_scan64(nmine, s_warp, nparts);
+    }
     for (unsigned long long j0 = 0; j0 < nparts; j0 += kPartList) {
         if (nmine != 0) {
             unsigned long long r = rank0;
-            if constexpr (kCells) cell_pass<kCellList>(descs, s_first, i0, i1, st, r, j0, s_parts);
+            if constexpr (kCells) cell_parts<true>(descs, s_first, i0, i1, st, before, r, j0, s_parts);
             else
                 parts([&](int k, int t, int count, int s0, int s1) {
                     if (r >= j0 && r < j0 + kPartList)
@@ -1142,6 +1227,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
 }
 
 static_assert(sizeof(TilePart) <= 64, "the block's lists leave room for the largest tile");
+static_assert(kPartList * sizeof(TilePart) >= 4 * 32 * sizeof(unsigned long long), "scan_types");
 
 // Shared memory of a launch whose largest tile has this many words: room for
 // up to eight tiles.
@@ -1164,7 +1250,10 @@ int occupancy_of(int smem_words)
     if (cudaFuncSetAttribute(trace_tiles_kernel<kThreads, NoRows>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells>,
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<false>>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<true>>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
         cudaFuncSetAttribute(trace_tiles_kernel<rows_threads(kThreads), RowsArgs>,
@@ -1223,7 +1312,10 @@ static cudaError_t launch_trace(const ScanDesc *descs, int nscans, int tile_word
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
                                int grid, int buckets, cudaStream_t s)
 {
-    if (buckets > 2 * grid) return launch_trace(descs, nscans, tile_words, threads, grid, Cells{}, s);
+    if (buckets / 4 > threads && buckets > 2 * grid)
+        return launch_trace(descs, nscans, tile_words, threads, grid, Cells<true>{}, s);
+    if (buckets > 2 * grid)
+        return launch_trace(descs, nscans, tile_words, threads, grid, Cells<false>{}, s);
     return launch_trace(descs, nscans, tile_words, threads, grid, NoRows{}, s);
 }
 
