@@ -459,6 +459,13 @@ hd::Buckets buckets_of(const hd_scan *s)
     return b;
 }
 
+// Cells of the tiled traversal: the tiles of each class the scan counts.
+int cells_of(const hd_scan *s)
+{
+    const uint32_t m = s->params.methods;
+    return s->tp.ntiles * (((m & (HD_SC | HD_MSC)) ? 1 : 0) + ((m & HD_SM) ? 1 : 0));
+}
+
 // Tiles: one or more z-slices of the full x-y plane when they fit in the
 // shared-memory budget, otherwise x-y strips of one slice.
 void make_tile_plan(hd_scan *s)
@@ -764,7 +771,7 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
     cudaEvent_t e1 = prof_begin(s, st);
     if (s->tp.ntiles > 0 && s->trace_grid > 0) {
         HD_CUDA(hd::launch_trace_tiles(s->desc_dev, 1, s->tp.tile_words, s->tp.threads,
-                                       s->trace_grid, hd::kGroups * s->tp.ntiles, st));
+                                       s->trace_grid, hd::kGroups * s->tp.ntiles, cells_of(s), st));
         if (s->profiling) s->trace_launches += 1;
     }
     prof_end(s, 1, e1, st);
@@ -1515,12 +1522,13 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
                       int grid, cudaStream_t st)
 {
     const int n_items = static_cast<int>(round.size());
-    int max_words = 0, buckets = 0;
+    int max_words = 0, buckets = 0, cells = 0;
     bool any_tiled = false;
     for (const auto &it : round) {
         if (it.scan->tp.ntiles > 0 && it.scan->trace_grid > 0) {
             any_tiled = true;
             buckets += hd::kGroups * it.scan->tp.ntiles;
+            cells += cells_of(it.scan);
             if (it.scan->tp.tile_words > max_words) max_words = it.scan->tp.tile_words;
         }
     }
@@ -1562,7 +1570,8 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
     r = join();
     if (r != HD_OK) return r;
     if (any_tiled) {
-        HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, buckets, st));
+        HD_CUDA(hd::launch_trace_tiles(b->descs_dev, n_items, max_words, b->threads, grid, buckets, cells,
+                                       st));
     }
     HD_CUDA(hd::launch_trace_global_batch(b->descs_dev, n_items, upper, b->sm_count, st));
     if (!any_finalize) return HD_OK;

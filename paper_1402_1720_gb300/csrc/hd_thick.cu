@@ -488,7 +488,7 @@ cudaError_t launch_thick_scan(const ScanDesc *desc_dev, const hd_geometry *geom,
                               int threads, int grid, int sm_count, cudaStream_t st)
 {
     const ThickDiff td = thick_diff_of(geom, workspace);
-    cudaError_t e = launch_trace_tiles(desc_dev, 1, smem_words, threads, grid, 0, st);
+    cudaError_t e = launch_trace_tiles(desc_dev, 1, smem_words, threads, grid, 0, 0, st);
     if (e == cudaSuccess && upper > 0) {
         int64_t blocks = (upper + kThickThreads - 1) / kThickThreads;
         const int64_t cap = int64_t(sm_count > 0 ? sm_count : 1) * 8;

@@ -766,12 +766,17 @@ __device__ __forceinline__ unsigned long long flush_cost(int tile_words)
 // chunks 11.4 -> 6.7 ms (8.2 before walks were sorted by type), 2e5 of them in one
 // 769 -> 502 us (592); 236 x 236 x 60, 1e5 histories 168 -> 121 us.  Costs in event
 // units: kJoinedEvent quarters of one per event, kJoinedPair per walk, a quarter
-// more per flush.
-constexpr unsigned kJoinedEvent = 7, kJoinedPair = 16;
+// more per flush.  What a flush saves is less than what one costs (it also waits
+// while others walk): kSavedPart and kSavedWord, from both forms of 17 grids at
+// four chunk sizes each (in every direction they are alike at 8 events per word of
+// the tile; joined takes 0.5 to 0.9 of the time at one).
+constexpr unsigned kJoinedEvent = 7, kJoinedPair = 16, kSavedPart = 2500, kSavedWord = 3;
 
-// Launches of at most two buckets to a block do not look at it (launch_trace_tiles):
-// there the four flushes of a cell are spread over blocks that would have little
-// else to do, and a small scan waits for every instruction before its walks.
+// Launches of fewer cells than three to four blocks do not look at it
+// (launch_trace_tiles): their cells are cut into parts, each with a flush, and the
+// four flushes of a cell are spread over blocks that would have little else to do
+// (64 x 64 x 50 joined takes 1.1 times as long at any chunk size); and a small scan
+// waits for every instruction before its walks.
 struct Cell {
     unsigned long long cost[4];  // of the parts made of each bucket (joined: cost[0], of all)
     unsigned count[4];           // pairs
@@ -794,7 +799,8 @@ __device__ __forceinline__ Cell cell_of(const ScanDesc &d, int cell)
 {
     const int step = 2 * d.tp.ntiles, words = d.tp.tile_words;
     const unsigned long long flush = flush_cost(words);
-    unsigned long long e[4], events = 0, pairs = 0, split = 0;
+    unsigned long long e[4], events = 0, pairs = 0;
+    int types = 0;
     Cell c;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -806,10 +812,13 @@ __device__ __forceinline__ Cell cell_of(const ScanDesc &d, int cell)
         c.cost[j] = bucket_cost<false>(c.count[j], e[j], words);
         pairs += c.count[j];
         events += e[j];
-        split += c.cost[j];
+        types += c.count[j] != 0u ? 1 : 0;
     }
     const unsigned long long all = kJoinedEvent * events / 4ull + kJoinedPair * pairs + flush + flush / 4ull;
-    c.joined = all < split;
+    const unsigned long long more = (kJoinedEvent - 4u) * events + 4u * (kJoinedPair - kPairCost) * pairs;
+    const unsigned long long saved = kSavedPart + static_cast<unsigned long long>(kSavedWord) *
+                                                      static_cast<unsigned>(words);
+    c.joined = types > 1 && more < static_cast<unsigned>(4 * types - 5) * saved;  // quarters
     if (c.joined) {
         c.cost[0] = all;
         c.cost[1] = c.cost[2] = c.cost[3] = 0ull;
@@ -1310,11 +1319,11 @@ static cudaError_t launch_trace(const ScanDesc *descs, int nscans, int tile_word
 }
 
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
-                               int grid, int buckets, cudaStream_t s)
+                               int grid, int buckets, int cells, cudaStream_t s)
 {
-    if (buckets / 4 > threads && buckets > 2 * grid)
+    if (4 * cells >= 3 * grid && buckets / 4 > threads)
         return launch_trace(descs, nscans, tile_words, threads, grid, Cells<true>{}, s);
-    if (buckets > 2 * grid)
+    if (4 * cells >= 3 * grid)
         return launch_trace(descs, nscans, tile_words, threads, grid, Cells<false>{}, s);
     return launch_trace(descs, nscans, tile_words, threads, grid, NoRows{}, s);
 }
