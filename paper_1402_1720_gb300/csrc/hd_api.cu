@@ -459,11 +459,18 @@ hd::Buckets buckets_of(const hd_scan *s)
     return b;
 }
 
-// Cells of the tiled traversal: the tiles of each class the scan counts.
-int cells_of(const hd_scan *s)
+// Cells of the tiled traversal that n histories may leave so few walks in that they
+// are joined: the tiles of each class the scan counts, or none.  A history is one
+// class's and makes (nx + ny) / 2 events if it crosses the grid; half of that is
+// asked for, and a cell is joined up to 11/3 events per word of its tile.
+int cells_of(const hd_scan *s, int64_t n)
 {
     const uint32_t m = s->params.methods;
-    return s->tp.ntiles * (((m & (HD_SC | HD_MSC)) ? 1 : 0) + ((m & HD_SM) ? 1 : 0));
+    const int64_t cells =
+        int64_t(s->tp.ntiles) * (((m & (HD_SC | HD_MSC)) ? 1 : 0) + ((m & HD_SM) ? 1 : 0));
+    return n * (int64_t(s->geom.nx) + s->geom.ny) / 4 <= 4 * cells * s->tp.tile_words
+               ? static_cast<int>(cells)
+               : 0;
 }
 
 // Tiles: one or more z-slices of the full x-y plane when they fit in the
@@ -771,7 +778,7 @@ hd_status run_chunk(hd_scan *s, const hd::Inputs &in, int64_t n, cudaStream_t st
     cudaEvent_t e1 = prof_begin(s, st);
     if (s->tp.ntiles > 0 && s->trace_grid > 0) {
         HD_CUDA(hd::launch_trace_tiles(s->desc_dev, 1, s->tp.tile_words, s->tp.threads,
-                                       s->trace_grid, hd::kGroups * s->tp.ntiles, cells_of(s), st));
+                                       s->trace_grid, hd::kGroups * s->tp.ntiles, cells_of(s, n), st));
         if (s->profiling) s->trace_launches += 1;
     }
     prof_end(s, 1, e1, st);
@@ -1528,7 +1535,7 @@ hd_status issue_round(hd_batch *b, const std::vector<hd_batch::Item> &round, int
         if (it.scan->tp.ntiles > 0 && it.scan->trace_grid > 0) {
             any_tiled = true;
             buckets += hd::kGroups * it.scan->tp.ntiles;
-            cells += cells_of(it.scan);
+            cells += cells_of(it.scan, it.n);
             if (it.scan->tp.tile_words > max_words) max_words = it.scan->tp.tile_words;
         }
     }

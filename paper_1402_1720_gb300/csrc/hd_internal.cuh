@@ -266,8 +266,8 @@ cudaError_t launch_scatter(const TilePlan &tp, const Records &rec, int64_t n, Ct
 // Traversal of the pairs of nscans scans (descs on the device) by `grid`
 // resident blocks.  tile_words is the largest tile of the scans; threads is
 // 256, 512, 768 or 1024; buckets: kGroups ntiles of all scans together; cells: a
-// tile's buckets of one class, those of the classes that are counted (0 for dilated
-// walks, which are never joined).
+// tile's buckets of one class, those of the classes that are counted and that may be
+// joined (0: dilated walks, which never are, and chunks of too many histories).
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
                                int grid, int buckets, int cells, cudaStream_t s);
 

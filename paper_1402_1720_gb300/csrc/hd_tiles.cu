@@ -4,6 +4,8 @@
 // its private tile into N or M once per part of a bucket (the pairs of one
 // group and tile, sorted in hd_scatter.cu) that it has walked; warps refill
 // idle lanes from the parts' pairs, so lanes do not wait for the longest path.
+#include <type_traits>
+
 #include "hd_euclid.cuh"
 #include "hd_fallback.cuh"
 
@@ -33,16 +35,21 @@ constexpr int kEventsPerStep = 8;  // events a traversal lane walks between refi
 struct NoRows {
     static constexpr bool kRows = false, kCells = false;
 };
-// The same for launches that look for cells to join (see Cell), with more cells
-// than threads or not (see scan_types).
-template <bool kMany>
+// The same for launches that look for cells to join (see Cell): a bucket per thread
+// where there are threads enough, else a cell per thread, or several.
+enum PlanBy { kByBucket, kByCell, kByCells };
+template <PlanBy kPlanBy>
 struct Cells {
     static constexpr bool kRows = false, kCells = true;
+    static constexpr PlanBy kBy = kPlanBy;
 };
-template <class T>
-constexpr bool kManyCells = false;
-template <>
-constexpr bool kManyCells<Cells<true>> = true;
+
+template <class RowsT>
+constexpr PlanBy plan_by()
+{
+    if constexpr (RowsT::kCells) return RowsT::kBy;
+    else return kByBucket;
+}
 
 // Shared-memory reduction (no value returned) at a shared-space byte address.
 __device__ __forceinline__ void smem_red_add(int addr, uint32_t v)
@@ -763,20 +770,24 @@ __device__ __forceinline__ unsigned long long flush_cost(int tile_words)
 // flush (columns, then rows), but a cell of few walks in several directions
 // (histories of many angles, or in no order of angle, on many tiles) pays for
 // one flush instead of four.  400 x 400 x 128, 9e6 histories in no order: in 20
-// chunks 11.4 -> 6.7 ms (8.2 before walks were sorted by type), 2e5 of them in one
-// 769 -> 502 us (592); 236 x 236 x 60, 1e5 histories 168 -> 121 us.  Costs in event
+// chunks 11.4 -> 6.8 ms (8.2 before walks were sorted by type), 2e5 of them in one
+// 765 -> 510 us (592); 236 x 236 x 60, 1e5 histories 167 -> 119 us.  Costs in event
 // units: kJoinedEvent quarters of one per event, kJoinedPair per walk, a quarter
-// more per flush.  What a flush saves is less than what one costs (it also waits
-// while others walk): kSavedPart and kSavedWord, from both forms of 17 grids at
-// four chunk sizes each (in every direction they are alike at 8 events per word of
-// the tile; joined takes 0.5 to 0.9 of the time at one).
-constexpr unsigned kJoinedEvent = 7, kJoinedPair = 16, kSavedPart = 2500, kSavedWord = 3;
+// more per flush.  What a flush saves is far less than what one costs (it also
+// waits while others walk): kSavedPart and kSavedWord, with four types joined up to
+// 3.7 events per word of the tile.  In 17 grids at four chunk sizes joined takes 0.5
+// to 0.9 of the time at one event per word, and the forms are alike at 8; but
+// joined up to 11, 48 scans in one launch took 27.2 ms, and 25.6 up to 3.7 or not
+// joined at all.
+constexpr unsigned kJoinedEvent = 7, kJoinedPair = 16, kSavedPart = 1000, kSavedWord = 1;
 
 // Launches of fewer cells than three to four blocks do not look at it
 // (launch_trace_tiles): their cells are cut into parts, each with a flush, and the
 // four flushes of a cell are spread over blocks that would have little else to do
 // (64 x 64 x 50 joined takes 1.1 times as long at any chunk size); and a small scan
-// waits for every instruction before its walks.
+// waits for every instruction before its walks.  Nor do those of too many histories
+// per cell, which the host knows: 3 to 5 us of 140 to 300 (1e6 histories on 100 x 100
+// x 100 to 400 x 400 x 64, nine chunks 2 % slower with it).
 struct Cell {
     unsigned long long cost[4];  // of the parts made of each bucket (joined: cost[0], of all)
     unsigned count[4];           // pairs
@@ -959,10 +970,64 @@ __device__ __forceinline__ void scan_types(const unsigned long long sum[4], unsi
     __syncthreads();  // s is free again
 }
 
-// The parts of a thread's cells in the block's stretch, counted, or listed (kList:
-// the thread's first has number `rank`, list begins at number j0): each at most
-// job_size pairs, of a joined cell in up to four, one to a bucket.  before: of the
-// thread's first cell, by type.
+// The parts of bucket j of cell t0 of scan k (cost c.cost[j], beginning at p) in the
+// block's stretch, counted in n, or listed (kList: the thread's next has number
+// rank, list begins at number j0): each at most job_size pairs, of a joined cell in
+// up to four, one to a bucket.
+template <bool kList>
+struct PartTaker {
+    const Stretch &st;
+    unsigned long long rank, j0;
+    TilePart *list;
+    unsigned long long n = 0;
+
+    __device__ __forceinline__ void put(const ScanDesc &d, int k, const Cell &c, int t0, int u, int s0,
+                                        int s1, bool same)
+    {
+        if (kList && rank >= j0 && rank < j0 + kPartList) {
+            TilePart &j = list[rank - j0];
+            fill_part(j, d, k, t0 + 2 * d.tp.ntiles * u, static_cast<int>(c.count[u]), s0, s1,
+                      !c.joined ? kOwn : (same ? kSame : kJoined));
+            if (c.joined) {
+                const TileBox b = tile_box(d.tp, j.tile);
+                j.box = joined_box(u, b.dx, b.dy);
+            }
+        }
+        ++rank;
+        ++n;
+    }
+    // (j a constant after unrolling)
+    __device__ __forceinline__ void take(const ScanDesc &d, int k, const Cell &c, int t0, int j,
+                                         unsigned long long cost, unsigned long long p)
+    {
+        if (cost == 0 || p >= st.x1 || p + cost <= st.x0) return;
+        const int words = st.own ? -1 : d.tp.tile_words, most = d.tp.job_size & ~31;
+        const int all = c.joined ? pieces_of(c.count[0]) + pieces_of(c.count[1]) +
+                                       pieces_of(c.count[2]) + pieces_of(c.count[3])
+                                 : pieces_of(c.count[j]);
+        const int s0 = st.x0 > p ? boundary_slot(cost, all, words, p, st.x0) : 0;
+        const int s1 = st.x1 < p + cost ? boundary_slot(cost, all, words, p, st.x1) : 32 * all;
+        for (int s = s0; s < s1; s += most) {
+            const int e = min(s + most, s1);
+            if (!c.joined) {
+                put(d, k, c, t0, j, s, e, false);
+                continue;
+            }
+            int off = 0;
+            bool same = false;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int len = 32 * pieces_of(c.count[u]);
+                const int a = max(s - off, 0), z = min(e - off, len);
+                if (a < z) put(d, k, c, t0, u, a, z, same);
+                same = same || a < z;
+                off += len;
+            }
+        }
+    }
+};
+
+// The parts of a thread's cells i0 .. i1 - 1; before: of the first, by type.
 template <bool kList>
 __device__ __forceinline__ unsigned long long cell_parts(const ScanDesc *__restrict__ descs,
                                                          const int *s_first, int i0, int i1,
@@ -971,58 +1036,40 @@ __device__ __forceinline__ unsigned long long cell_parts(const ScanDesc *__restr
                                                          unsigned long long rank,
                                                          unsigned long long j0, TilePart *list)
 {
-    unsigned long long n = 0, p[4] = {before[0], before[1], before[2], before[3]};
+    PartTaker<kList> taker{st, rank, j0, list};
+    unsigned long long p[4] = {before[0], before[1], before[2], before[3]};
     int k = 0;
     for (int i = i0; i < i1; ++i) {
         while (4 * i >= s_first[k + 1]) ++k;
         const ScanDesc &d = descs[k];
-        const int t0 = i - s_first[k] / 4, step = 2 * d.tp.ntiles, most = d.tp.job_size & ~31;
+        const int t0 = i - s_first[k] / 4;
         const Cell c = cell_of(d, t0);
-        auto take = [&](int u, int s0, int s1, bool same) {
-            if (kList && rank >= j0 && rank < j0 + kPartList) {
-                TilePart &j = list[rank - j0];
-                fill_part(j, d, k, t0 + step * u, static_cast<int>(c.count[u]), s0, s1,
-                          !c.joined ? kOwn : (same ? kSame : kJoined));
-                if (c.joined) {
-                    const TileBox b = tile_box(d.tp, j.tile);
-                    j.box = joined_box(u, b.dx, b.dy);
-                }
-            }
-            ++rank;
-            ++n;
-        };
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             const unsigned long long cost = st.own ? own_blocks(c.cost[j], d.tp.tile_words) : c.cost[j];
-            if (cost != 0 && p[j] < st.x1 && p[j] + cost > st.x0) {
-                const int words = st.own ? -1 : d.tp.tile_words;
-                const int all = c.joined ? pieces_of(c.count[0]) + pieces_of(c.count[1]) +
-                                               pieces_of(c.count[2]) + pieces_of(c.count[3])
-                                         : pieces_of(c.count[j]);
-                const int s0 = st.x0 > p[j] ? boundary_slot(cost, all, words, p[j], st.x0) : 0;
-                const int s1 = st.x1 < p[j] + cost ? boundary_slot(cost, all, words, p[j], st.x1) : 32 * all;
-                for (int s = s0; s < s1; s += most) {
-                    const int e = min(s + most, s1);
-                    if (!c.joined) {
-                        take(j, s, e, false);
-                        continue;
-                    }
-                    int off = 0;
-                    bool same = false;
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        const int len = 32 * pieces_of(c.count[u]);
-                        const int a = max(s - off, 0), z = min(e - off, len);
-                        if (a < z) take(u, a, z, same);
-                        same = same || a < z;
-                        off += len;
-                    }
-                }
-            }
+            taker.take(d, k, c, t0, j, cost, p[j]);
             p[j] += cost;
         }
     }
-    return n;
+    return taker.n;
+}
+
+// Bucket i of the launch with its cell; visit(scan's number, scan, cell, its number, type).
+template <class VisitT>
+__device__ __forceinline__ void with_bucket(const ScanDesc *__restrict__ descs, const int *s_first,
+                                            int i, VisitT visit)
+{
+    int k = 0;
+    while (i >= s_first[k + 1]) ++k;
+    const ScanDesc &d = descs[k];
+    const int t = i - s_first[k], type = t / (2 * d.tp.ntiles), t0 = t - 2 * d.tp.ntiles * type;
+    visit(k, d, cell_of(d, t0), t0, type);
+}
+
+__device__ __forceinline__ unsigned long long cost_of(const Cell &c, int type)
+{
+    const unsigned long long a = type & 1 ? c.cost[1] : c.cost[0], b = type & 1 ? c.cost[3] : c.cost[2];
+    return type & 2 ? b : a;
 }
 
 }  // namespace
@@ -1066,7 +1113,8 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     __syncthreads();
     const int nb = s_first[nscans];
     // the thread's buckets, or its cells (see cell_parts)
-    const int ni = kCells ? nb / 4 : nb, per = (ni + kThreads - 1) / kThreads;
+    constexpr bool kByBuckets = plan_by<RowsT>() == kByBucket;
+    const int ni = kByBuckets ? nb : nb / 4, per = (ni + kThreads - 1) / kThreads;
     const int i0 = min(static_cast<int>(threadIdx.x) * per, ni), i1 = min(i0 + per, ni);
     // visit(scan, bucket within it, its cost and pairs)
     auto each = [&](auto visit) {
@@ -1081,14 +1129,22 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     };
     Stretch st{};
     unsigned long long total, before[4];  // before: of a cell's types
-    if constexpr (kCells) {
+    if constexpr (!kByBuckets) {
         unsigned long long mine[4];
         cell_sums<false>(descs, s_first, i0, i1, mine);
-        scan_types<kManyCells<RowsT>>(mine, reinterpret_cast<unsigned long long *>(s_parts), before,
-                                      total);
+        scan_types<plan_by<RowsT>() == kByCells>(mine, reinterpret_cast<unsigned long long *>(s_parts),
+                                                 before, total);
     } else {
         unsigned long long mine = 0;
-        each([&](int, int, unsigned long long cost, unsigned) { mine += cost; });
+        if constexpr (kCells) {
+            if (i0 < i1)
+                with_bucket(descs, s_first, i0,
+                            [&](int, const ScanDesc &, const Cell &c, int, int type) {
+                                mine = cost_of(c, type);
+                            });
+        } else {
+            each([&](int, int, unsigned long long cost, unsigned) { mine += cost; });
+        }
         st.before = block_excl_scan64(mine, s_warp, total);
     }
     // the block's stretch: an equal share, but worth about two flushes
@@ -1100,10 +1156,18 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     st.own = blocks < gridDim.x;  // the same in all blocks and threads
     if (st.own) {
         unsigned long long m = 0, all, b = 0, bs[4];
-        if constexpr (kCells) {
+        if constexpr (!kByBuckets) {
             unsigned long long ms[4];
             cell_sums<true>(descs, s_first, i0, i1, ms);
-            scan_types<kManyCells<RowsT>>(ms, reinterpret_cast<unsigned long long *>(s_parts), bs, all);
+            scan_types<plan_by<RowsT>() == kByCells>(ms, reinterpret_cast<unsigned long long *>(s_parts),
+                                                     bs, all);
+        } else if constexpr (kCells) {
+            if (i0 < i1)
+                with_bucket(descs, s_first, i0,
+                            [&](int, const ScanDesc &d, const Cell &c, int, int type) {
+                                m = own_blocks(cost_of(c, type), d.tp.tile_words);
+                            });
+            b = block_excl_scan64(m, s_warp, all);
         } else {
             each([&](int k, int, unsigned long long cost, unsigned) {
                 m += own_blocks(cost, descs[k].tp.tile_words);
@@ -1113,7 +1177,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
         st.own = all <= gridDim.x;
         if (st.own) {
             st.before = b;
-            if constexpr (kCells)
+            if constexpr (!kByBuckets)
                 for (int j = 0; j < 4; ++j) before[j] = bs[j];
             share = 1ull;
         }
@@ -1141,10 +1205,29 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
             p += cost;
         });
     };
+    // the same of launches that join cells
+    auto planned = [&](auto list, unsigned long long rank, unsigned long long j0) {
+        constexpr bool kList = decltype(list)::value;
+        if constexpr (!kByBuckets) {
+            return cell_parts<kList>(descs, s_first, i0, i1, st, before, rank, j0, s_parts);
+        } else {
+            PartTaker<kList> taker{st, rank, j0, s_parts};
+            if (i0 < i1)
+                with_bucket(descs, s_first, i0,
+                            [&](int k, const ScanDesc &d, const Cell &c, int t0, int type) {
+                                unsigned long long cost = cost_of(c, type);
+                                if (st.own) cost = own_blocks(cost, d.tp.tile_words);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    if (j == type) taker.take(d, k, c, t0, j, cost, st.before);
+                            });
+            return taker.n;
+        }
+    };
     unsigned long long nmine = 0, nparts, rank0 = 0;
     if constexpr (kCells) {
         // (the order of the parts does not matter: numbers from a counter, no scan)
-        nmine = cell_parts<false>(descs, s_first, i0, i1, st, before, 0, 0, nullptr);
+        nmine = planned(std::false_type{}, 0, 0);
         if (nmine != 0) rank0 = atomicAdd(&s_next[0], static_cast<unsigned>(nmine));
         __syncthreads();
         nparts = s_next[0];
@@ -1155,7 +1238,7 @@ __global__ void __launch_bounds__(kThreads, 1) trace_tiles_kernel(
     for (unsigned long long j0 = 0; j0 < nparts; j0 += kPartList) {
         if (nmine != 0) {
             unsigned long long r = rank0;
-            if constexpr (kCells) cell_parts<true>(descs, s_first, i0, i1, st, before, r, j0, s_parts);
+            if constexpr (kCells) planned(std::true_type{}, r, j0);
             else
                 parts([&](int k, int t, int count, int s0, int s1) {
                     if (r >= j0 && r < j0 + kPartList)
@@ -1259,10 +1342,13 @@ int occupancy_of(int smem_words)
     if (cudaFuncSetAttribute(trace_tiles_kernel<kThreads, NoRows>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<false>>,
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<kByBucket>>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<true>>,
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<kByCell>>,
+                             cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
+            cudaSuccess ||
+        cudaFuncSetAttribute(trace_tiles_kernel<kThreads, Cells<kByCells>>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, kTileSmemBytes) !=
             cudaSuccess ||
         cudaFuncSetAttribute(trace_tiles_kernel<rows_threads(kThreads), RowsArgs>,
@@ -1321,10 +1407,13 @@ static cudaError_t launch_trace(const ScanDesc *descs, int nscans, int tile_word
 cudaError_t launch_trace_tiles(const ScanDesc *descs, int nscans, int tile_words, int threads,
                                int grid, int buckets, int cells, cudaStream_t s)
 {
-    if (4 * cells >= 3 * grid && buckets / 4 > threads)
-        return launch_trace(descs, nscans, tile_words, threads, grid, Cells<true>{}, s);
-    if (4 * cells >= 3 * grid)
-        return launch_trace(descs, nscans, tile_words, threads, grid, Cells<false>{}, s);
+    if (4 * cells >= 3 * grid) {
+        if (buckets <= threads)
+            return launch_trace(descs, nscans, tile_words, threads, grid, Cells<kByBucket>{}, s);
+        if (buckets / 4 <= threads)
+            return launch_trace(descs, nscans, tile_words, threads, grid, Cells<kByCell>{}, s);
+        return launch_trace(descs, nscans, tile_words, threads, grid, Cells<kByCells>{}, s);
+    }
     return launch_trace(descs, nscans, tile_words, threads, grid, NoRows{}, s);
 }
 
