@@ -777,8 +777,8 @@ __device__ __forceinline__ unsigned long long flush_cost(int tile_words)
 // waits while others walk): kSavedPart and kSavedWord, with four types joined up to
 // 3.7 events per word of the tile.  In 17 grids at four chunk sizes joined takes 0.5
 // to 0.9 of the time at one event per word, and the forms are alike at 8; but
-// joined up to 11, 48 scans in one launch took 27.2 ms, and 25.6 up to 3.7 or not
-// joined at all.
+// joined up to 11, 48 head-sized scans in one launch of this kernel took 27.2 ms,
+// and 25.6 up to 3.7 or not joined at all.
 constexpr unsigned kJoinedEvent = 7, kJoinedPair = 16, kSavedPart = 1000, kSavedWord = 1;
 
 // Launches of fewer cells than three to four blocks do not look at it
